@@ -415,7 +415,7 @@ trdq_status trdq_prepare_weights(const trdq_rotation* rot, const void* W_bf16, i
     for (int i = 0; i < kNumTileN; ++i) {
       const trdq_status st = wbits == 8
                                  ? encode_tmap_u8_sw128(&gw.tmap_b[i], gw.codes, row_bytes, N, row_bytes, box_bytes, kTileN[i])
-                                 : encode_tmap_2d(&gw.tmap_b[i], gw.codes, 1, row_bytes, N, row_bytes, box_bytes, 128, 0);
+                                 : encode_tmap_2d(&gw.tmap_b[i], gw.codes, 1, row_bytes, N, row_bytes, box_bytes, 64, 0);
       if (st != TRDQ_OK) {
         trdq_weights_destroy(w);
         return st;

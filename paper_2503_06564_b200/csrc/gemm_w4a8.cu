@@ -2,20 +2,31 @@
 // fp32 scale per (output channel, 128 consecutive k):
 //     y[m, n] = sx[m] * sum_kg sw4[n, kg] * ( sum_{k in kg} q[m, k] * q4[n, k] ) + bias[n]
 //
+// The product is formed TRANSPOSED: the weights are the M operand of the tensor core (128 output channels = the 128
+// lanes of tensor memory) and the activation codes the N operand (128 tokens = columns).  A drain thread then owns ONE
+// output channel for 64 tokens, so the group's scale is one register per k-block instead of a table look-up per column.
+//
 // The k-block of the pipeline is exactly one scale group.  Per k-block:
-//   warp 0       TMA: 128 x 128-byte tile of activation codes and 128 x 64-byte tile of packed nibbles
-//   warps 2-3    unpack in registers: 16 bytes of nibbles -> 32 int8 (nibble << 4, i.e. 16 * q4, which is
-//                sign-correct without any sign extension) written in the 128-byte-swizzled K-major
-//                layout the tensor core reads
-//   warp 1       four tcgen05.mma kind::i8 (128 x 128 x 32) into a FRESH tensor-memory accumulator
-//                (four accumulators of 128 columns rotate)
-//   warps 4-11   drain that accumulator: acc64[n] += acc32[n] * mult[kg][n] with 64-bit integer
-//                multiply-adds.  mult are the group scales of a channel on a common power-of-two grid
-//                (sw4[n,kg] = mult[kg][n] * base[n]), so the sum over groups is EXACT integer arithmetic
-//                and no cancellation between groups can lose bits.
+//   warp 0       TMA of the 128 x 128-byte tile of activation codes
+//   warp 1       four tcgen05.mma kind::i8 (128 x 128 x 32) into a FRESH accumulator of 128 tensor-memory columns; two
+//                k-blocks are handed to the drain at a time
+//   warps 2-7    two warps per k-block, three k-blocks in turn: TMA of the packed nibbles of 64 channels (weights are
+//                constants: the first tiles are requested before the kernel that produces the codes has finished),
+//                unpacked in registers: 16 bytes of nibbles -> 32 int8 (nibble << 4, i.e. 16 * q4, which is sign-correct
+//                without any sign extension) written in the 128-byte-swizzled K-major layout the tensor core reads
+//   warps 8-15   drain: acc64[m] += acc32[m] * mult[kg][n] with 64-bit integer multiply-adds.  mult are the group
+//                scales of a channel on a common power-of-two grid (sw4[n,kg] = mult[kg][n] * base[n]), so the sum over
+//                groups is EXACT integer arithmetic and no cancellation between groups can lose bits.
 // At the end of a tile the 64-bit sums are converted once: y = fma(float(S), sx * base[n], bias[n]),
-// with the same cancellation check against the bias as the 8-bit kernel, staged in shared memory and
-// written by TMA stores.  Every wait is bounded.
+// with the same cancellation check against the bias as the 8-bit kernel, transposed through a staging tile in shared
+// memory and written by TMA stores.  Every wait is bounded.
+//
+// What bounds it: the drain.  A 32 x 32 -> 64-bit multiply-add issues at a quarter of the fp32 rate, 512 clocks per k-block
+// and scheduler for its 128 x 128 values against 256 clocks of tensor pipe; alone the drain takes 740 clocks per k-block,
+// beside the other warps' traffic 1130.  M = 16384, microseconds with the weights as the N operand (multipliers read from
+// a shared-memory table per column, one k-block per hand-over) -> now: 1152 -> 4608 323 -> 221, 4608 -> 1152 247 -> 170,
+// 1152 -> 1152 84 -> 59, 1152 -> 3456 244 -> 168.  Measured and not better: a CTA pair sharing the codes (211 / 186 / 64 / 167: the
+// 256-channel tile pads N = 1152 by 11 %) and sixteen drain warps of 32 tokens (218 / 175 / 58 / 166).
 #include <cuda_bf16.h>
 
 #include "epilogue.cuh"
@@ -25,30 +36,44 @@
 namespace trdq {
 namespace {
 
-constexpr int kTileM = 128;
-constexpr int kTileNW4 = 128;
+constexpr int kTileTok = 128;    // tokens per tile: N of the MMA
+constexpr int kTileCh = 128;     // output channels per tile: M of the MMA, lanes of tensor memory
 constexpr int kTileK = 128;
-constexpr int kThreads = 384;
-constexpr int kEpilogueThreads = 256;
-constexpr int kUnpackThreads = 64;
-constexpr int kAccStages = 4;
+constexpr int kUnpackWarps = 6;
+constexpr int kUnpackSplit = 2;    // warps that share a k-block
+constexpr int kUnpackTurns = kUnpackWarps / kUnpackSplit;
+constexpr int kDrainWarps = 8;   // 4 lane quarters x 2 groups of 64 tokens
+constexpr int kThreads = 32 * (2 + kUnpackWarps + kDrainWarps);
+constexpr int kTokPerWarp = kTileTok / (kDrainWarps / 4);
+constexpr int kHandoff = 2;      // k-blocks per hand-over to the drain
+constexpr int kSlots = 2;        // hand-overs in flight: kSlots * kHandoff accumulators of 128 columns
 constexpr int kTmemCols = 512;
-constexpr int kABytes = kTileM * kTileK;       // 16 KB int8
-constexpr int kBPackedBytes = kTileNW4 * 64;     // 8 KB nibbles
-constexpr int kB8Bytes = kTileNW4 * kTileK;      // 16 KB int8 after unpacking
-constexpr int kStageBytes = kABytes + kB8Bytes + kBPackedBytes;  // A and B8 first: both need 1024-byte alignment
+constexpr int kW8Bytes = kTileCh * kTileK;         // 16 KB int8 weights after unpacking
+constexpr int kTokBytes = kTileTok * kTileK;       // 16 KB activation codes
+constexpr int kStageBytes = kW8Bytes + kTokBytes;
 constexpr int kStages = 4;
-constexpr int kOutStageBytes = (kEpilogueThreads / 32) * 2048;
-constexpr int kParamBytes = kTileNW4 * 12;
-constexpr int kBarrierBytes = 256;
-constexpr int kFixedSmemBytes = 1024 + kStages * kStageBytes + kOutStageBytes + kParamBytes + kBarrierBytes;
-// The tile's multipliers ([K/128][128] int32) are staged in shared memory when they fit.
-constexpr int kMaxSmemGroups = (227 * 1024 - kFixedSmemBytes) / (kTileNW4 * 4);
+constexpr int kPackedBytes = kTileCh / kUnpackSplit * 64;  // 4 KB nibbles of one unpack warp
+constexpr int kPackedDepth = 2;                    // packed tiles in flight per unpack warp
+constexpr int kPackedStages = kPackedDepth * kUnpackWarps;
+constexpr int kOutStageBytes = kDrainWarps * kTokPerWarp * 64;  // per drain warp 64 tokens x 32 channels bf16
+constexpr int kSxBytes = kDrainWarps * kTokPerWarp * 4;
+constexpr int kBarrierBytes = 512;
+constexpr int kPackedOff = kStages * kStageBytes;
+constexpr int kOutOff = kPackedOff + kPackedStages * kPackedBytes;
+constexpr int kSxOff = kOutOff + kOutStageBytes;
+constexpr int kBarOff = kSxOff + kSxBytes;
+constexpr int kSmemBytes = 1024 + kBarOff + kBarrierBytes;
+static_assert(kSmemBytes <= 227 * 1024, "shared memory");
+static_assert(kSlots * kHandoff * kTileTok <= kTmemCols, "tensor memory");
+// Registers: 512 threads are launched with 128 each.  The two drain warpgroups need the 128 of their 64-bit sums plus a
+// double-buffered tensor-memory load, the other two few: 128 * (2 * 192 + 2 * 64) = the 512 * 128 of the launch.
+constexpr int kRegsLaunch = 128, kRegsDrain = 192, kRegsOther = 64;
+static_assert(kDrainWarps * 32 * kRegsDrain + (kThreads - kDrainWarps * 32) * kRegsOther <= kThreads * kRegsLaunch, "register split exceeds the launch's allocation");
 
 struct alignas(64) W4Params {
-  CUtensorMap tmap_a[2];
-  CUtensorMap tmap_b;
-  CUtensorMap tmap_out[2];
+  CUtensorMap tmap_a[2];    // codes of each segment, box 128 B x 128 rows, 128-byte swizzle
+  CUtensorMap tmap_b;       // packed weights, box 64 B x 64 rows
+  CUtensorMap tmap_out[2];  // bf16 output, box 32 channels x 64 tokens, 64-byte swizzle
   const float* sx[2];
   int32_t M[2];
   int32_t tiles_m[2];
@@ -56,7 +81,6 @@ struct alignas(64) W4Params {
   const float* base;      // [n_pad]
   const __nv_bfloat16* bias;
   int32_t N, K, tiles_n, n_pad;
-  int32_t mult_in_smem;  // 1: all K/128 multiplier rows of a tile fit the shared-memory table
   uint32_t* status;
 };
 
@@ -70,9 +94,27 @@ __device__ __forceinline__ TileCoord tile_coord(const W4Params& p, int tile) {
   TileCoord c;
   c.seg = mt >= p.tiles_m[0] ? 1 : 0;
   if (c.seg) mt -= p.tiles_m[0];
-  c.m0 = mt * kTileM;
-  c.n0 = nt * kTileNW4;
+  c.m0 = mt * kTileTok;
+  c.n0 = nt * kTileCh;
   return c;
+}
+
+struct Ring {
+  int idx = 0;
+  uint32_t phase = 0;
+  __device__ __forceinline__ void advance(int n) {
+    if (++idx == n) {
+      idx = 0;
+      phase ^= 1;
+    }
+  }
+};
+
+// Waits for this thread's tensor-memory loads; every use of the registers stays behind the wait.
+__device__ __forceinline__ void tmem_wait_ld_regs(uint32_t (&r)[16]) {
+  tmem_wait_ld();
+#pragma unroll
+  for (int i = 0; i < 16; ++i) asm volatile("" : "+r"(r[i]));
 }
 
 // ACT: GELU (tanh form) on the dequantized value before the bf16 rounding.
@@ -81,18 +123,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_con
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t out_stage_base = smem_base + kStages * kStageBytes;
-  float2* param_buf = reinterpret_cast<float2*>(smem + kStages * kStageBytes + kOutStageBytes);  // (base, bias)[128]
-  float* thr_buf = reinterpret_cast<float*>(param_buf + kTileNW4);                                 // 2^-10 |bias|
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes + kOutStageBytes + kParamBytes);
-  // barriers: raw[S] (TMA landed), b8[S] (unpacked), empty[S], tfull[4], tempty[4]
-  const uint32_t bar_raw = smem_u32(bars);
-  const uint32_t bar_b8 = bar_raw + 8 * kStages;
-  const uint32_t bar_empty = bar_b8 + 8 * kStages;
-  const uint32_t bar_tfull = bar_empty + 8 * kStages;
-  const uint32_t bar_tempty = bar_tfull + 8 * kAccStages;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * kStages + 2 * kAccStages);
-  int32_t* mult_smem = reinterpret_cast<int32_t*>(smem + kStages * kStageBytes + kOutStageBytes + kParamBytes + kBarrierBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kBarOff);
+  const uint32_t bar_full = smem_u32(bars);                // [kStages]        codes landed and weights unpacked
+  const uint32_t bar_empty = bar_full + 8 * kStages;       // [kStages]        the MMAs have read the stage
+  const uint32_t bar_praw = bar_empty + 8 * kStages;       // [kPackedStages]  nibbles landed
+  const uint32_t bar_tfull = bar_praw + 8 * kPackedStages; // [kSlots]         accumulators complete
+  const uint32_t bar_tempty = bar_tfull + 8 * kSlots;      // [kSlots]         accumulators drained
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + kPackedStages + 2 * kSlots);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -101,17 +138,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_con
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(bar_raw + 8 * s, 1);
-      mbar_init(bar_b8 + 8 * s, kUnpackThreads / 32);
+      mbar_init(bar_full + 8 * s, 1 + kUnpackSplit);  // one arrive.expect_tx for the codes, the unpack warps
       mbar_init(bar_empty + 8 * s, 1);
     }
-    for (int a = 0; a < kAccStages; ++a) {
+    for (int s = 0; s < kPackedStages; ++s) mbar_init(bar_praw + 8 * s, 1);
+    for (int a = 0; a < kSlots; ++a) {
       mbar_init(bar_tfull + 8 * a, 1);
-      mbar_init(bar_tempty + 8 * a, kEpilogueThreads / 32);
+      mbar_init(bar_tempty + 8 * a, kDrainWarps);
     }
     fence_mbar_init();
   }
-  if (warp == 1) {
+  if (warp == 2) {
     tmem_alloc(smem_u32(tmem_slot), kTmemCols);
     tmem_relinquish();
   }
@@ -120,226 +157,250 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_con
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();
-  griddep_wait();  // codes, scales and weights may come from the kernel before; Y may still be read by it
+  const int my_tiles = static_cast<int>(blockIdx.x) < total_tiles ? (total_tiles - 1 - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x) + 1 : 0;
+  const int total_kb = my_tiles * num_kb;
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    if (elect_one()) {
-      prefetch_tensormap(&p.tmap_a[0]);
-      prefetch_tensormap(&p.tmap_a[1]);
-      prefetch_tensormap(&p.tmap_b);
-      prefetch_tensormap(&p.tmap_out[0]);
-      prefetch_tensormap(&p.tmap_out[1]);
-      BoundedWaiter w(p.status, kStatusTimeoutProducer);
-      int stage = 0;
-      uint32_t phase = 0;
-      for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-        const TileCoord tc = tile_coord(p, tile);
-        for (int kb = 0; kb < num_kb; ++kb) {
-          w.wait(bar_empty + 8 * stage, phase ^ 1);
-          const uint32_t a_dst = smem_base + stage * kStageBytes;
-          const uint32_t bp_dst = a_dst + kABytes + kB8Bytes;
-          mbar_arrive_expect_tx(bar_raw + 8 * stage, kABytes + kBPackedBytes);
-          tma_load_2d(a_dst, &p.tmap_a[tc.seg], kb * kTileK, tc.m0, bar_raw + 8 * stage);
-          tma_load_2d(bp_dst, &p.tmap_b, kb * (kTileK / 2), tc.n0, bar_raw + 8 * stage);
-          if (++stage == kStages) {
-            stage = 0;
-            phase ^= 1;
-          }
-        }
-      }
-      w.settle();
-    }
-  } else if (warp == 1) {
-    // -------------------------------------------------------------- MMA issuer
-    if (elect_one()) {
-      BoundedWaiter w(p.status, kStatusTimeoutMma);
-      constexpr uint32_t idesc = umma_idesc_s8(kTileNW4);
-      int stage = 0;
-      uint32_t phase = 0;
-      int acc = 0;
-      uint32_t acc_phase = 0;
-      for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-        for (int kb = 0; kb < num_kb; ++kb) {
-          w.wait(bar_tempty + 8 * acc, acc_phase ^ 1);  // accumulator drained
-          w.wait(bar_b8 + 8 * stage, phase);            // A landed and B unpacked
-          tc_fence_after();
-          const uint32_t a_addr = smem_base + stage * kStageBytes;
-          const uint64_t a_desc = umma_desc_k_sw128(a_addr);
-          const uint64_t b_desc = umma_desc_k_sw128(a_addr + kABytes);
-          const uint32_t d_tmem = tmem_base + acc * kTileNW4;
-#pragma unroll
-          for (int k = 0; k < kTileK / 32; ++k) umma_i8(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, k != 0 ? 1u : 0u);
-          umma_commit(bar_empty + 8 * stage);
-          umma_commit(bar_tfull + 8 * acc);
-          if (++stage == kStages) {
-            stage = 0;
-            phase ^= 1;
-          }
-          if (++acc == kAccStages) {
-            acc = 0;
-            acc_phase ^= 1;
-          }
-        }
-      }
-      w.settle();
-    }
-  } else if (warp == 2 || warp == 3) {
-    // ------------------------------------------------- unpack nibbles -> int8
-    const int ut = threadIdx.x - 64;  // 0..63
-    BoundedWaiter w(p.status, kStatusTimeoutUnpack);
-    int stage = 0;
-    uint32_t phase = 0;
-    for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-      for (int kb = 0; kb < num_kb; ++kb) {
-        w.wait(bar_raw + 8 * stage, phase);
-        __syncwarp();
-        const uint8_t* bp = smem + stage * kStageBytes + kABytes + kB8Bytes;
-        const uint32_t b8 = smem_base + stage * kStageBytes + kABytes;
-#pragma unroll
-        for (int i = 0; i < (kTileNW4 * 4) / kUnpackThreads; ++i) {
-          const int id = ut + kUnpackThreads * i;  // 16-byte source chunk: row = id / 4, chunk = id % 4
-          const int row = id >> 2, sc = id & 3;
-          const uint4 src = *reinterpret_cast<const uint4*>(bp + row * 64 + sc * 16);
-          const uint32_t wsrc[4] = {src.x, src.y, src.z, src.w};
-          uint32_t o[8];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t even = (wsrc[j] << 4) & 0xF0F0F0F0u;  // k even: low nibble moved to the high half
-            const uint32_t odd = wsrc[j] & 0xF0F0F0F0u;          // k odd: already in the high half
-            o[2 * j] = __byte_perm(even, odd, 0x5140);
-            o[2 * j + 1] = __byte_perm(even, odd, 0x7362);
-          }
-          const uint32_t dst_row = b8 + row * 128;
-          st_shared_v4(dst_row + (((2 * sc) ^ (row & 7)) << 4), o[0], o[1], o[2], o[3]);
-          st_shared_v4(dst_row + (((2 * sc + 1) ^ (row & 7)) << 4), o[4], o[5], o[6], o[7]);
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_b8 + 8 * stage);
-        if (++stage == kStages) {
-          stage = 0;
-          phase ^= 1;
-        }
-      }
-    }
-    w.settle();
-  } else {
-    // ---------------------------------------------------------------- epilogue
-    const int ew = warp - 4;
-    const int q = ew & 3;
-    const int half = ew >> 2;
-    const int et = threadIdx.x - 4 * 32;
-    const uint32_t my_stage = out_stage_base + ew * 2048;
+  if (warp >= kThreads / 32 - kDrainWarps) {
+    // ------------------------------------------------------------------- drain
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsDrain));
+    griddep_wait();
+    const int dw = warp - (kThreads / 32 - kDrainWarps);
+    const int q = dw & 3;           // = warp % 4: the lane quarter of tensor memory this warp may read
+    const int tok_off = (dw >> 2) * kTokPerWarp;
+    const uint32_t my_stage = smem_base + kOutOff + dw * (kTokPerWarp * 64);
+    float* my_sx = reinterpret_cast<float*>(smem + kSxOff) + dw * kTokPerWarp;
+    const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + tok_off;
     BoundedWaiter w(p.status, kStatusTimeoutEpilogue);
-    int acc = 0;
-    uint32_t acc_phase = 0;
+    Ring slot;
+    const int lane_n = q * 32 + lane;
+    int32_t m_next = my_tiles > 0 ? __ldg(p.mult_t + tile_coord(p, blockIdx.x).n0 + lane_n) : 0;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
       const TileCoord tc = tile_coord(p, tile);
-      // all epilogue threads are past the previous tile's parameter reads before these writes
-      asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory");
-      for (int c = et; c < kTileNW4; c += kEpilogueThreads) {
-        const int n = tc.n0 + c;
-        float2 v = make_float2(0.0f, 0.0f);
-        if (n < p.N) {
-          v.x = __ldg(p.base + n);
-          v.y = p.bias ? __bfloat162float(p.bias[n]) : 0.0f;
-        }
-        param_buf[c] = v;
-        thr_buf[c] = fabsf(v.y) * 0.0009765625f;
-      }
-      if (p.mult_in_smem) {
-        // this tile's multipliers for every scale group: [num_kb][128] int32
-        const int4* src = reinterpret_cast<const int4*>(p.mult_t + tc.n0);
-        for (int i = et; i < num_kb * (kTileNW4 / 4); i += kEpilogueThreads) {
-          const int kb = i / (kTileNW4 / 4), c4 = i % (kTileNW4 / 4);
-          reinterpret_cast<int4*>(mult_smem)[i] = __ldg(src + static_cast<int64_t>(kb) * (p.n_pad / 4) + c4);
-        }
-      }
-      asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory");
-      const int row = tc.m0 + q * 32 + lane;
-      const bool row_ok = row < p.M[tc.seg];
-      const float sxm = row_ok ? __ldg(p.sx[tc.seg] + row) : 0.0f;
-
-      long long sum[64];
+      const int n = tc.n0 + lane_n;  // < n_pad
+      const int32_t* mp = p.mult_t + n;
+      // requested here, used after the last k-block: an L2 round trip is about as long as a k-block
+      const float base = __ldg(p.base + n);
+      const uint16_t bias_bits = p.bias && n < p.N ? __ldg(reinterpret_cast<const uint16_t*>(p.bias) + n) : 0;
+      float sx_reg[kTokPerWarp / 32];
 #pragma unroll
-      for (int j = 0; j < 64; ++j) sum[j] = 0;
-      const int col0 = half * 64;
+      for (int i = 0; i < kTokPerWarp / 32; ++i) {
+        const int row = tc.m0 + tok_off + 32 * i + lane;
+        sx_reg[i] = row < p.M[tc.seg] ? __ldg(p.sx[tc.seg] + row) : 0.0f;
+      }
+      long long sum[kTokPerWarp];
+#pragma unroll
+      for (int j = 0; j < kTokPerWarp; ++j) sum[j] = 0;
+      // Two register buffers: a tensor-memory load is always in flight behind the multiply-adds, across k-blocks too.
+      uint32_t r[2][16];
+      w.wait(bar_tfull + 8 * slot.idx, slot.phase);
+      __syncwarp();
+      tc_fence_after();
+      uint32_t t_row = t_lane + slot.idx * (kHandoff * kTileTok);
+      tmem_ld_32x16(t_row, r[0]);
       for (int kb = 0; kb < num_kb; ++kb) {
-        const int4* mrow = p.mult_in_smem ? reinterpret_cast<const int4*>(mult_smem + kb * kTileNW4 + col0)
-                                          : reinterpret_cast<const int4*>(p.mult_t + static_cast<int64_t>(kb) * p.n_pad + tc.n0 + col0);
-        w.wait(bar_tfull + 8 * acc, acc_phase);
-        __syncwarp();
-        tc_fence_after();
-        const uint32_t t_row = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kTileNW4 + col0;
-        // two register buffers: the load of chunk ch + 1 is in flight while chunk ch is accumulated
-        uint32_t r[2][16];
-        tmem_ld_32x16(t_row, r[0]);
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          tmem_wait_ld();
-          if (ch < 3) tmem_ld_32x16(t_row + (ch + 1) * 16, r[(ch + 1) & 1]);
-#pragma unroll
-          for (int j4 = 0; j4 < 4; ++j4) {
-            const int4 m = mrow[ch * 4 + j4];
-            const int mv[4] = {m.x, m.y, m.z, m.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              sum[ch * 16 + j4 * 4 + e] +=
-                  static_cast<long long>(static_cast<int32_t>(r[ch & 1][j4 * 4 + e])) * static_cast<long long>(mv[e]);
-          }
+        int32_t mult = m_next;
+        asm volatile("" : "+r"(mult));  // stays a 32-bit factor: widened ahead of the loop it would cost a 64 x 64 product
+        if (kb + 1 < num_kb) {
+          mp += p.n_pad;
+          m_next = __ldg(mp);
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_tempty + 8 * acc);
-        if (++acc == kAccStages) {
-          acc = 0;
-          acc_phase ^= 1;
+        const bool hand_back = kb % kHandoff == kHandoff - 1 || kb + 1 == num_kb;
+#pragma unroll
+        for (int ch = 0; ch < kTokPerWarp / 16; ++ch) {
+          tmem_wait_ld_regs(r[ch & 1]);
+          if (ch + 1 < kTokPerWarp / 16) {
+            tmem_ld_32x16(t_row + (ch + 1) * 16, r[(ch + 1) & 1]);
+          } else if (!hand_back) {
+            t_row += kTileTok;
+            tmem_ld_32x16(t_row, r[0]);
+          } else {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_tempty + 8 * slot.idx);
+            slot.advance(kSlots);
+            if (kb + 1 < num_kb) {
+              w.wait(bar_tfull + 8 * slot.idx, slot.phase);
+              __syncwarp();
+              tc_fence_after();
+              t_row = t_lane + slot.idx * (kHandoff * kTileTok);
+              tmem_ld_32x16(t_row, r[0]);
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            sum[ch * 16 + j] += static_cast<long long>(static_cast<int32_t>(r[ch & 1][j])) * static_cast<long long>(mult);
         }
       }
 
       // final conversion: y = float(S) * (sx * base) + bias   (base is a power of two: the product is exact)
+      if (tile + static_cast<int>(gridDim.x) < total_tiles) m_next = __ldg(p.mult_t + tile_coord(p, tile + gridDim.x).n0 + lane_n);
+      const float bias = __uint_as_float(static_cast<uint32_t>(bias_bits) << 16);
+      const float thr = fabsf(bias) * 0.0009765625f;
+      // byte of this lane's channel inside a staging row (64 bytes, 64-byte swizzle: 16-byte chunk index xor row bits 1..2)
+      const uint32_t lane_chunk = lane >> 3, lane_byte = (lane & 7) * 2;
+      if (lane == 0) bulk_wait_group_read<0>();  // the previous store has finished reading the staging tile
 #pragma unroll
-      for (int c2 = 0; c2 < 2; ++c2) {
-        uint32_t packed[16];
+      for (int i = 0; i < kTokPerWarp / 32; ++i) my_sx[32 * i + lane] = sx_reg[i];
+      __syncwarp();
+      // Eight tokens at a time without a branch between them (a branch per value serialises conversion, product and
+      // store); the rare cancellation against the bias is repaired for the whole group.
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-          float y[2];
+      for (int j0 = 0; j0 < kTokPerWarp; j0 += 8) {
+        float v[8];
+        bool cancels = false;
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int col = col0 + c2 * 32 + j + e;
-            const float2 pb = param_buf[col];
-            const long long S = sum[c2 * 32 + j + e];
-            const float sf = __ll2float_rn(S);
-            const float cm = __fmul_rn(sxm, pb.x);
-            float v = __fmaf_rn(sf, cm, pb.y);
-            if (fabsf(v) < thr_buf[col]) v = __fmaf_rn(__ll2float_rn(S - __float2ll_rz(sf)), cm, v);  // the part fp32 dropped
-            y[e] = ACT ? gelu_tanh(v) : v;
+        for (int e = 0; e < 8; ++e) {
+          v[e] = __fmaf_rn(__ll2float_rn(sum[j0 + e]), __fmul_rn(my_sx[j0 + e], base), bias);
+          cancels |= fabsf(v[e]) < thr;
+        }
+        if (cancels) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const long long S = sum[j0 + e];
+            // the part of the sum that fp32 dropped
+            if (fabsf(v[e]) < thr) v[e] = __fmaf_rn(__ll2float_rn(S - __float2ll_rz(__ll2float_rn(S))), __fmul_rn(my_sx[j0 + e], base), v[e]);
           }
-          const __nv_bfloat162 h = __floats2bfloat162_rn(y[0], y[1]);
-          packed[j / 2] = *reinterpret_cast<const uint32_t*>(&h);
         }
-        if (lane == 0) bulk_wait_group_read<0>();
-        __syncwarp();
 #pragma unroll
-        for (int v = 0; v < 4; ++v)
-          st_shared_v4(my_stage + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4), packed[4 * v], packed[4 * v + 1], packed[4 * v + 2],
-                       packed[4 * v + 3]);
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          tma_store_2d(&p.tmap_out[tc.seg], tc.n0 + col0 + c2 * 32, tc.m0 + q * 32, my_stage);
-          bulk_commit_group();
+        for (int e = 0; e < 8; ++e) {
+          const int j = j0 + e;
+          const uint16_t h = __bfloat16_as_ushort(__float2bfloat16_rn(ACT ? gelu_tanh(v[e]) : v[e]));
+          asm volatile("st.shared.u16 [%0], %1;" ::"r"(my_stage + j * 64 + ((lane_chunk ^ ((j >> 1) & 3)) << 4) + lane_byte), "h"(h) : "memory");
         }
+      }
+      fence_proxy_async_smem();
+      __syncwarp();  // (the reads of my_sx are done as well)
+      if (lane == 0) {
+        tma_store_2d(&p.tmap_out[tc.seg], tc.n0 + q * 32, tc.m0 + tok_off, my_stage);  // rows >= M and columns >= N are clipped
+        bulk_commit_group();
       }
     }
     if (lane == 0) bulk_wait_group_read<0>();  // the staging tiles have been read; the stores complete before the grid does
     w.settle();
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
+    if (warp == 0) {
+      // ------------------------------------------------- TMA of the activation codes
+      if (elect_one()) {
+        prefetch_tensormap(&p.tmap_a[0]);
+        prefetch_tensormap(&p.tmap_a[1]);
+        prefetch_tensormap(&p.tmap_out[0]);
+        prefetch_tensormap(&p.tmap_out[1]);
+        griddep_wait();  // the codes come from the kernel before
+        BoundedWaiter w(p.status, kStatusTimeoutProducer);
+        Ring st;
+        for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
+          const TileCoord tc = tile_coord(p, tile);
+          for (int kb = 0; kb < num_kb; ++kb) {
+            w.wait(bar_empty + 8 * st.idx, st.phase ^ 1);
+            mbar_arrive_expect_tx(bar_full + 8 * st.idx, kTokBytes);
+            tma_load_2d(smem_base + st.idx * kStageBytes + kW8Bytes, &p.tmap_a[tc.seg], kb * kTileK, tc.m0, bar_full + 8 * st.idx);
+            st.advance(kStages);
+          }
+        }
+        w.settle();
+      }
+    } else if (warp == 1) {
+      // ------------------------------------------------- MMA issuer
+      if (elect_one()) {
+        BoundedWaiter w(p.status, kStatusTimeoutMma);
+        constexpr uint32_t idesc = umma_idesc_s8(kTileTok);
+        Ring st, slot;
+        for (int t = 0; t < my_tiles; ++t) {
+          for (int kb = 0; kb < num_kb; ++kb) {
+            const int h = kb % kHandoff;
+            if (h == 0) w.wait(bar_tempty + 8 * slot.idx, slot.phase ^ 1);  // accumulators drained
+            w.wait(bar_full + 8 * st.idx, st.phase);                        // codes landed, weights unpacked
+            tc_fence_after();
+            const uint32_t w_addr = smem_base + st.idx * kStageBytes;
+            const uint64_t a_desc = umma_desc_k_sw128(w_addr);
+            const uint64_t b_desc = umma_desc_k_sw128(w_addr + kW8Bytes);
+            const uint32_t d_tmem = tmem_base + (slot.idx * kHandoff + h) * kTileTok;
+#pragma unroll
+            for (int k = 0; k < kTileK / 32; ++k) umma_i8(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, k != 0 ? 1u : 0u);
+            umma_commit(bar_empty + 8 * st.idx);
+            st.advance(kStages);
+            if (h == kHandoff - 1 || kb + 1 == num_kb) {
+              umma_commit(bar_tfull + 8 * slot.idx);
+              slot.advance(kSlots);
+            }
+          }
+        }
+        w.settle();
+      }
+    } else {
+      // ------------------------------------------------- unpack nibbles -> int8, k-blocks i = turn (mod 3), 64 of the tile's channels
+      // The nibbles are requested without waiting for the kernel before: the weights are constants of the prepared
+      // object, and the last kernel of their preparation (w4_multipliers_kernel, an ordinary launch) is complete before
+      // this kernel's predecessor can start.
+      const int uw = warp - 2;
+      const int turn = uw / kUnpackSplit, part = uw % kUnpackSplit;
+      BoundedWaiter w(p.status, kStatusTimeoutUnpack);
+      const uint32_t my_packed = smem_base + kPackedOff + uw * kPackedDepth * kPackedBytes;
+      const uint32_t my_praw = bar_praw + 8 * uw * kPackedDepth;
+      auto request = [&](int i, int slot_idx) {  // lane 0: the nibbles of this CTA's k-block i
+        const int t = i / num_kb;
+        const TileCoord tc = tile_coord(p, blockIdx.x + t * gridDim.x);
+        mbar_arrive_expect_tx(my_praw + 8 * slot_idx, kPackedBytes);
+        tma_load_2d(my_packed + slot_idx * kPackedBytes, &p.tmap_b, (i - t * num_kb) * (kTileK / 2), tc.n0 + part * (kTileCh / kUnpackSplit), my_praw + 8 * slot_idx);
+      };
+      if (lane == 0) {
+        prefetch_tensormap(&p.tmap_b);
+        for (int d = 0; d < kPackedDepth; ++d)
+          if (turn + d * kUnpackTurns < total_kb) request(turn + d * kUnpackTurns, d);
+      }
+      __syncwarp();
+      Ring ps;
+      for (int i = turn; i < total_kb; i += kUnpackTurns) {
+        w.wait(my_praw + 8 * ps.idx, ps.phase);
+        const int st_idx = i % kStages;
+        w.wait(bar_empty + 8 * st_idx, ((i / kStages) & 1) ^ 1);
+        __syncwarp();
+        const uint32_t bp = my_packed + ps.idx * kPackedBytes;
+        const uint32_t w8 = smem_base + st_idx * kStageBytes + part * (kW8Bytes / kUnpackSplit);
+#pragma unroll 1
+        for (int c = 0; c < 4 / kUnpackSplit; ++c) {
+          // 16-byte source chunks: channel = id / 4, chunk = id % 4, id = lane + 32 (4 c + i); four in flight at once
+          uint4 src[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(src[k].x), "=r"(src[k].y), "=r"(src[k].z), "=r"(src[k].w)
+                         : "r"(bp + (lane + 32 * (4 * c + k)) * 16)
+                         : "memory");
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int id = lane + 32 * (4 * c + k);
+            const int row = id >> 2, sc = id & 3;
+            const uint32_t wsrc[4] = {src[k].x, src[k].y, src[k].z, src[k].w};
+            uint32_t o[8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t even = (wsrc[j] << 4) & 0xF0F0F0F0u;  // k even: low nibble moved to the high half
+              const uint32_t odd = wsrc[j] & 0xF0F0F0F0u;          // k odd: already in the high half
+              o[2 * j] = __byte_perm(even, odd, 0x5140);
+              o[2 * j + 1] = __byte_perm(even, odd, 0x7362);
+            }
+            const uint32_t dst_row = w8 + row * 128;
+            st_shared_v4(dst_row + (((2 * sc) ^ (row & 7)) << 4), o[0], o[1], o[2], o[3]);
+            st_shared_v4(dst_row + (((2 * sc + 1) ^ (row & 7)) << 4), o[4], o[5], o[6], o[7]);
+          }
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(bar_full + 8 * st_idx);
+          if (i + kPackedDepth * kUnpackTurns < total_kb) request(i + kPackedDepth * kUnpackTurns, ps.idx);
+        }
+        ps.advance(kPackedDepth);
+      }
+      w.settle();
+    }
   }
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) {
+  if (warp == 2) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
@@ -385,17 +446,17 @@ trdq_status launch_gemm_w4(const trdq_weights* w, int g, const GemmSegment seg[2
   for (int s = 0; s < 2; ++s) {
     p.sx[s] = seg[s].sx;
     p.M[s] = seg[s].M;
-    p.tiles_m[s] = (seg[s].M + kTileM - 1) / kTileM;
+    p.tiles_m[s] = (seg[s].M + kTileTok - 1) / kTileTok;
     tiles_m += p.tiles_m[s];
   }
   if (tiles_m == 0) return TRDQ_OK;
   for (int s = 0; s < 2; ++s) {
     const GemmSegment& src = seg[s].M > 0 ? seg[s] : seg[1 - s];
     trdq_status st = encode_tmap_u8_sw128(&p.tmap_a[s], src.codes, static_cast<uint64_t>(w->K), static_cast<uint64_t>(src.M),
-                                          static_cast<uint64_t>(w->K), kTileK, kTileM);
+                                          static_cast<uint64_t>(w->K), kTileK, kTileTok);
     if (st != TRDQ_OK) return st;
     st = encode_tmap_2d(&p.tmap_out[s], src.out, 2, static_cast<uint64_t>(w->N), static_cast<uint64_t>(src.M),
-                        static_cast<uint64_t>(src.ld) * 2, 32, 32, 64);
+                        static_cast<uint64_t>(src.ld) * 2, 32, kTokPerWarp, 64);
     if (st != TRDQ_OK) return st;
   }
   p.tmap_b = w->groups[g].tmap_b[0];
@@ -404,25 +465,21 @@ trdq_status launch_gemm_w4(const trdq_weights* w, int g, const GemmSegment seg[2
   p.bias = static_cast<const __nv_bfloat16*>(bias_bf16);
   p.N = w->N;
   p.K = w->K;
-  p.tiles_n = (w->N + kTileNW4 - 1) / kTileNW4;
-  p.n_pad = p.tiles_n * kTileNW4;
+  p.tiles_n = (w->N + kTileCh - 1) / kTileCh;
+  p.n_pad = p.tiles_n * kTileCh;
   p.status = device_status_word();
   if (!p.status) return TRDQ_ERR_CUDA;
-  const int groups = w->K / kTileK;
-  p.mult_in_smem = groups <= kMaxSmemGroups ? 1 : 0;
-  const int smem_bytes = kFixedSmemBytes + (p.mult_in_smem ? groups * kTileNW4 * 4 : 0);
   const int64_t total = tiles_m * p.tiles_n;
   const int grid = static_cast<int>(total < sms ? total : sms);
   static PerDeviceFlag configured;
   if (!configured.get(dev)) {
-    const int max_smem = kFixedSmemBytes + kMaxSmemGroups * kTileNW4 * 4;
-    if (cudaFuncSetAttribute(gemm_w4a8_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w4a8_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(gemm_w4a8_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_w4a8_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
       return TRDQ_ERR_CUDA;
     configured.set(dev, true);
   }
-  const cudaError_t e = act ? launch_overlapped(gemm_w4a8_kernel<true>, dim3(grid), dim3(kThreads), smem_bytes, stream, p)
-                            : launch_overlapped(gemm_w4a8_kernel<false>, dim3(grid), dim3(kThreads), smem_bytes, stream, p);
+  const cudaError_t e = act ? launch_overlapped(gemm_w4a8_kernel<true>, dim3(grid), dim3(kThreads), kSmemBytes, stream, p)
+                            : launch_overlapped(gemm_w4a8_kernel<false>, dim3(grid), dim3(kThreads), kSmemBytes, stream, p);
   return e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA;
 }
 

@@ -34,7 +34,7 @@ constexpr int kTileN[kNumTileN] = {128, 192, 256};
 struct GroupWeights {
   void* codes = nullptr;                // dev int8 [N,K] or packed uint8 [N,K/2]
   float* scales = nullptr;              // dev fp32 [N] or [N,K/128]
-  CUtensorMap tmap_b[kNumTileN];        // TMA descriptors of `codes`, one per tile width (4-bit: only [0], 128 rows x 64 bytes)
+  CUtensorMap tmap_b[kNumTileN];        // TMA descriptors of `codes`, one per tile width (4-bit: only [0], 64 rows x 64 bytes)
   CUtensorMap tmap_b_half[kNumTileN];   // 8-bit only: boxes of half a tile width (64 / 96 / 128 rows) for the CTA-pair kernel
   // 4-bit weights only: the scales of an output channel as integers on a common power-of-two grid,
   //   scales[n][kg] = mult_t[kg][n] * base[n]   (exact whenever the exponents of a channel span < 7 bits)
