@@ -44,7 +44,7 @@ struct Cfg {
   static constexpr int kStageBytes = kABytes + kBBytes;
   // parameters staged for the epilogue: (sw, bias) and the cancellation threshold per column, one
   // buffer per accumulator stage
-  static constexpr int kParamBytes = 2 * BN * 16;  // (sw, bias), threshold and (asymmetric mode) weight column sums
+  static constexpr int kParamBytes = 2 * (ColumnParamLayout<BN>::kBytes + BN * 4);  // two sets: column parameters and (asymmetric mode) weight column sums
   static constexpr int kBarrierBytes = 256;
   // output staging: one 32-row x 32-column bf16 tile (2 KB, 64-byte swizzle) per epilogue warp
   static constexpr int kOutStageBytes = (kEpilogueThreads / 32) * 2048;
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w8a8_kernel(const __grid_con
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
   const uint32_t out_stage_base = smem_base + C::kStages * C::kStageBytes;
-  float2* param_buf = reinterpret_cast<float2*>(smem + C::kStages * C::kStageBytes + C::kOutStageBytes);
+  float* param_buf = reinterpret_cast<float*>(smem + C::kStages * C::kStageBytes + C::kOutStageBytes);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes + C::kOutStageBytes + C::kParamBytes);
   // barrier layout: full[S], empty[S], tmem_full[2], tmem_empty[2], then the tensor-memory base address
   const uint32_t bar_full = smem_u32(bars);
@@ -244,11 +244,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w8a8_kernel(const __grid_con
     uint32_t acc_phase = 0;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
       const TileCoord tc = tile_coord(p, tile, BN);
-      float2* pb = param_buf + acc * BN;                                           // (sw, bias)
-      float* thr = reinterpret_cast<float*>(param_buf + 2 * BN) + acc * BN;        // 2^-10 * |bias|
-      int32_t* csum = reinterpret_cast<int32_t*>(reinterpret_cast<float*>(param_buf + 2 * BN) + 2 * BN) + acc * BN;
+      constexpr int kParamFloats = ColumnParamLayout<BN>::kFloats;
+      ColumnParams cp = {};
+      int32_t* csum = reinterpret_cast<int32_t*>(param_buf + 2 * kParamFloats) + acc * BN;
       if (MODE != 1) {
-        stage_column_params(pb, thr, p.sw, p.bias, tc.n0, p.N, BN, et, kEpilogueThreads);
+        cp = stage_column_params<BN>(param_buf + acc * kParamFloats, p.sw, p.bias, tc.n0, p.N, et, kEpilogueThreads);
         if (MODE == 2)
           for (int c = et; c < BN; c += kEpilogueThreads) csum[c] = tc.n0 + c < p.N ? __ldg(p.colsum + tc.n0 + c) : 0;
         asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory");
@@ -275,10 +275,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w8a8_kernel(const __grid_con
           for (int j = 0; j < 32; ++j) r[j] = static_cast<uint32_t>(static_cast<int32_t>(r[j]) - zrow * csum[c * 32 + j]);
         }
         if (MODE != 1) {
-          const float4* pb4 = reinterpret_cast<const float4*>(pb + c * 32);
-          const float4* thr4 = reinterpret_cast<const float4*>(thr + c * 32);
           uint32_t packed[16];
-          dequant_row32<MODE == 3>(r, sxm, pb4, thr4, packed);
+          dequant_row32<MODE == 3>(r, sxm, cp, c, packed);
           // staging tile: row = lane, 64 bytes per row, 16-byte chunk j stored at j ^ ((lane >> 1) & 3)
           if (lane == 0) bulk_wait_group_read<0>();  // the previous store has finished reading the tile
           __syncwarp();

@@ -38,7 +38,7 @@ struct Cfg2 {
   static constexpr int kABytes = kTileM * kTileKBytes;
   static constexpr int kBBytes = (BN / 2) * kTileKBytes;  // this CTA's half of the weight tile
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kParamBytes = 2 * BN * 12;
+  static constexpr int kParamBytes = 2 * ColumnParamLayout<BN>::kBytes;
   static constexpr int kBarrierBytes = 256;
   static constexpr int kOutStageBytes = (kEpilogueThreads / 32) * 4096;  // one 32 x 64 bf16 tile per warp
   static constexpr int kStages = (kSmemBudget - 1024 - kOutStageBytes - kParamBytes - kBarrierBytes) / kStageBytes;
@@ -154,7 +154,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
   const uint32_t out_stage_base = smem_base + C::kStages * C::kStageBytes;
-  float2* param_buf = reinterpret_cast<float2*>(smem + C::kStages * C::kStageBytes + C::kOutStageBytes);
+  float* param_buf = reinterpret_cast<float*>(smem + C::kStages * C::kStageBytes + C::kOutStageBytes);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes + C::kOutStageBytes + C::kParamBytes);
   const uint32_t bar_full = smem_u32(bars);                  // [S]   used in the leader
   const uint32_t bar_empty = bar_full + 8 * C::kStages;      // [S]   each CTA's own
@@ -298,9 +298,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
     for (int tile = cluster_id; tile < total_tiles; tile += num_clusters) {
       const TileCoord tc = pair_tile_coord(p, tile, BN);
       const int m0 = tc.m0 + rank * kTileM;
-      float2* pb = param_buf + acc * BN;
-      float* thr = reinterpret_cast<float*>(param_buf + 2 * BN) + acc * BN;
-      stage_column_params(pb, thr, p.sw, p.bias, tc.n0, p.N, BN, et, kEpilogueThreads);
+      const ColumnParams cp =
+          stage_column_params<BN>(param_buf + acc * ColumnParamLayout<BN>::kFloats, p.sw, p.bias, tc.n0, p.N, et, kEpilogueThreads);
       asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory");
       const int row = m0 + q * 32 + lane;
       const float sxm = row < p.M[tc.seg] ? __ldg(p.sx[tc.seg] + row) : 0.0f;
@@ -319,8 +318,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
           tmem_ld_32x32(t_row + (c + h2) * 32, r);
           tmem_wait_ld();
           uint32_t packed[16];
-          dequant_row32<ACT>(r, sxm, reinterpret_cast<const float4*>(pb + (c + h2) * 32), reinterpret_cast<const float4*>(thr + (c + h2) * 32),
-                             packed);
+          dequant_row32<ACT>(r, sxm, cp, c + h2, packed);
           if (h2 == 0) {
             if (lane == 0) bulk_wait_group_read<0>();  // the previous store has finished reading the tile
             __syncwarp();
@@ -344,7 +342,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
         tmem_ld_32x32(t_row + c * 32, r);
         tmem_wait_ld();
         uint32_t packed[16];
-        dequant_row32<ACT>(r, sxm, reinterpret_cast<const float4*>(pb + c * 32), reinterpret_cast<const float4*>(thr + c * 32), packed);
+        dequant_row32<ACT>(r, sxm, cp, c, packed);
         if (lane == 0) bulk_wait_group_read<0>();
         __syncwarp();
 #pragma unroll
