@@ -22,17 +22,26 @@ __device__ __forceinline__ float dequant_one(int32_t a, float sxm, float swn, fl
   return v;
 }
 
-// GELU in its tanh form, the activation between the two MLP linears of a DiT block:
+// GELU in its tanh form, the activation between the two MLP linears of a DiT block, two values at a time:
 //   gelu(x) = 0.5 x (1 + tanh(u)) = x / (1 + exp(-2u)) = x exp(2u) / (1 + exp(2u)),   u = sqrt(2/pi) (x + 0.044715 x^3).
 // With e = exp(-|2u|) in (0, 1] the denominator 1 + e stays in [1, 2] on both sides, so nothing overflows and the
 // fast division is in its defined range.  exp through ex2.approx: relative error near 1e-6, far inside a bf16
 // rounding step; results below about 1e-37 in magnitude (x < -10) flush to zero.
-__device__ __forceinline__ float gelu_tanh(float x) {
+// The two special-function results per value (an eighth of a warp per clock each) bound the epilogue with GELU.  One
+// reciprocal shared by four quotients was measured: 22.3 against 25.8 us (30.3 with a scalar form and the column-by-column epilogue) (1152 -> 4608, M = 4096), but one bf16 result in
+// 10^5 then rounds the other way, and repairing exactly those costs more than is gained (33 us).
+__device__ __forceinline__ float2 gelu_tanh2(float2 x) {
   const float k = 1.5957691216057308f;  // 2 sqrt(2/pi)
-  const float t = __fmul_rn(x, __fmaf_rn(__fmul_rn(x, x), 0.044715f * k, k));  // 2u, same sign as x
-  const float e = __expf(-fabsf(t));
-  const float num = t >= 0.0f ? x : __fmul_rn(x, e);
-  return __fdividef(num, __fadd_rn(1.0f, e));
+  const float2 t = __fmul2_rn(x, __ffma2_rn(__fmul2_rn(x, x), make_float2(0.044715f * k, 0.044715f * k), make_float2(k, k)));  // 2u, sign of x
+  const float2 e = make_float2(__expf(-fabsf(t.x)), __expf(-fabsf(t.y)));
+  const float2 m = __fmul2_rn(x, e);
+  const float2 d = __fadd2_rn(e, make_float2(1.0f, 1.0f));
+  return make_float2(__fdividef(t.x >= 0.0f ? x.x : m.x, d.x), __fdividef(t.y >= 0.0f ? x.y : m.y, d.y));
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float2 v) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 // min(|a|, |b|, |c|) in one instruction
@@ -59,7 +68,8 @@ struct ColumnParamLayout {  // [sw BN][bias BN][thr BN / 32], 16-byte aligned
 // packed to bf16 pairs.  Packed fp32x2 arithmetic, the same roundings as dequant_one; the cancellation against the bias is
 // looked for once per row and chunk (smallest |y| against the chunk's largest threshold) and repaired column by column
 // only where it may have happened.  Per column: one conversion, 2.5 instructions of arithmetic and half a 16-byte
-// shared-memory read, against about 6 and 0.75 when every column is tested by itself.
+// shared-memory read, against about 6 and 0.75 when every column is tested by itself: the 8-bit GEMM at M = 4096,
+// 1152 -> 3456 / 4608 / 1152 went from 16.2 / 19.1 / 9.2 to 14.9 / 17.9 / 8.7 us, at M = 16384, 1152 -> 3456 from 62 to 54 us.
 template <bool ACT = false>
 __device__ __forceinline__ void dequant_row32(const uint32_t (&r)[32], float sxm, const ColumnParams& cp, int c, uint32_t (&packed)[16]) {
   const float4* sw4 = reinterpret_cast<const float4*>(cp.sw + c * 32);
@@ -77,7 +87,7 @@ __device__ __forceinline__ void dequant_row32(const uint32_t (&r)[32], float sxm
     lowest = min3_abs(lowest, v[2 * j].x, v[2 * j].y);
     lowest = min3_abs(lowest, v[2 * j + 1].x, v[2 * j + 1].y);
   }
-  if (lowest < cp.thr[c]) {
+  if (!(lowest >= cp.thr[c])) {  // also when a NaN bias made the threshold one
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
       const float bn = cp.bias[c * 32 + j];
@@ -89,11 +99,7 @@ __device__ __forceinline__ void dequant_row32(const uint32_t (&r)[32], float sxm
     }
   }
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    if (ACT) v[j] = make_float2(gelu_tanh(v[j].x), gelu_tanh(v[j].y));
-    const __nv_bfloat162 h = __floats2bfloat162_rn(v[j].x, v[j].y);
-    packed[j] = *reinterpret_cast<const uint32_t*>(&h);
-  }
+  for (int j = 0; j < 16; ++j) packed[j] = pack_bf16(ACT ? gelu_tanh2(v[j]) : v[j]);
 }
 
 // Stages the epilogue parameters of BN columns starting at n0 (see ColumnParamLayout).  Called by whole warps with
@@ -110,7 +116,7 @@ __device__ __forceinline__ ColumnParams stage_column_params(float* dst, const fl
     }
     dst[c] = s;
     dst[BN + c] = b;
-    // non-negative floats order like their bit patterns (a NaN bias sends the chunk to the column-by-column path)
+    // non-negative floats order like their bit patterns (a NaN bias gives a NaN threshold)
     const unsigned int top = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(b) * 0.0009765625f));
     if ((c & 31) == 0) dst[2 * BN + c / 32] = __uint_as_float(top);
   }

@@ -261,10 +261,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_con
             if (fabsf(v[e]) < thr) v[e] = __fmaf_rn(__ll2float_rn(S - __float2ll_rz(__ll2float_rn(S))), __fmul_rn(my_sx[j0 + e], base), v[e]);
           }
         }
+        uint32_t packed[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const float2 two = make_float2(v[2 * g], v[2 * g + 1]);
+          packed[g] = pack_bf16(ACT ? gelu_tanh2(two) : two);
+        }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const int j = j0 + e;
-          const uint16_t h = __bfloat16_as_ushort(__float2bfloat16_rn(ACT ? gelu_tanh(v[e]) : v[e]));
+          const uint16_t h = static_cast<uint16_t>(packed[e / 2] >> (16 * (e & 1)));
           asm volatile("st.shared.u16 [%0], %1;" ::"r"(my_stage + j * 64 + ((lane_chunk ^ ((j >> 1) & 3)) << 4) + lane_byte), "h"(h) : "memory");
         }
       }
