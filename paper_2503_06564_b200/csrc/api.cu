@@ -77,10 +77,16 @@ static trdq_status encode_cached(CUtensorMap* out, CUtensorMapDataType dt, uint3
     key.box[i] = box[i];
     if (i + 1 < rank) key.strides[i] = strides[i];
   }
-  uint64_t h = 1469598103934665603ull;
-  const unsigned char* kb = reinterpret_cast<const unsigned char*>(&key);
-  for (size_t i = 0; i < sizeof key; ++i) h = (h ^ kb[i]) * 1099511628211ull;
-  TmapEntry& slot = g_tmap_cache[h & 511u];
+  // word by word (the key is a dozen words; byte by byte the hash alone took 0.15 us a map); the top bits are the mixed ones
+  static_assert(sizeof(TmapKey) % 8 == 0, "hashed in words");
+  uint64_t words[sizeof(TmapKey) / 8];
+  std::memcpy(words, &key, sizeof key);
+  uint64_t h = 0;
+  for (const uint64_t word : words) {
+    h = (h ^ word) * 0x9E3779B97F4A7C15ull;
+    h ^= h >> 32;
+  }
+  TmapEntry& slot = g_tmap_cache[(h * 0x9E3779B97F4A7C15ull) >> 55];
   {
     std::lock_guard<std::mutex> lock(g_tmap_mutex);
     if (slot.valid && std::memcmp(&slot.key, &key, sizeof key) == 0) {

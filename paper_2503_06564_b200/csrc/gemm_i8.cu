@@ -406,17 +406,23 @@ static trdq_status launch_gemm_w8_mode(const trdq_weights* w, int g, const GemmS
   const int ti = choose_tile_n(tiles_m, w->N, sms);
   const int bn = kTileN[ti];
   for (int s = 0; s < 2; ++s) {
-    // an empty segment still needs a valid descriptor object; reuse the other segment's
-    const GemmSegment& src = seg[s].M > 0 ? seg[s] : seg[1 - s];
+    if (seg[s].M == 0) continue;
+    const GemmSegment& src = seg[s];
     trdq_status st = encode_tmap_u8_sw128(&p.tmap_a[s], src.codes, static_cast<uint64_t>(w->K), static_cast<uint64_t>(src.M),
                                           static_cast<uint64_t>(w->K), kTileKBytes, kTileM);
     if (st != TRDQ_OK) return st;
   }
   for (int s = 0; s < 2 && !raw_i32; ++s) {
-    const GemmSegment& src = seg[s].M > 0 ? seg[s] : seg[1 - s];
+    if (seg[s].M == 0) continue;
+    const GemmSegment& src = seg[s];
     trdq_status st = encode_tmap_2d(&p.tmap_out[s], src.out, 2, static_cast<uint64_t>(w->N), static_cast<uint64_t>(src.M),
                                     static_cast<uint64_t>(src.ld) * 2, 32, 32, 64);
     if (st != TRDQ_OK) return st;
+  }
+  for (int s = 0; s < 2; ++s) {
+    if (seg[s].M > 0) continue;  // an empty segment's maps are never used, only prefetched: the other segment's
+    p.tmap_a[s] = p.tmap_a[1 - s];
+    p.tmap_out[s] = p.tmap_out[1 - s];
   }
   if (raw_i32) p.tmap_out[0] = p.tmap_out[1] = p.tmap_a[0];  // unused by the raw-accumulator mode
   p.tmap_b = w->groups[g].tmap_b[ti];

@@ -573,7 +573,8 @@ trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment 
   if (best < 0) return TRDQ_ERR_SHAPE;
   const int bn = kTileN[best];
   for (int s = 0; s < 2; ++s) {
-    const GemmSegment& src = seg[s].M > 0 ? seg[s] : seg[1 - s];
+    if (seg[s].M == 0) continue;
+    const GemmSegment& src = seg[s];
     trdq_status st = encode_tmap_u8_sw128(&p.tmap_a[s], src.codes, static_cast<uint64_t>(w->K), static_cast<uint64_t>(src.M),
                                           static_cast<uint64_t>(w->K), kTileKBytes, kTileM);
     if (st != TRDQ_OK) return st;
@@ -583,6 +584,12 @@ trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment 
     st = encode_tmap_2d(&p.tmap_out32[s], src.out, 2, static_cast<uint64_t>(w->N), static_cast<uint64_t>(src.M),
                         static_cast<uint64_t>(src.ld) * 2, 32, 32, 64);
     if (st != TRDQ_OK) return st;
+  }
+  for (int s = 0; s < 2; ++s) {
+    if (seg[s].M > 0) continue;  // an empty segment's maps are never used, only prefetched: the other segment's
+    p.tmap_a[s] = p.tmap_a[1 - s];
+    p.tmap_out[s] = p.tmap_out[1 - s];
+    p.tmap_out32[s] = p.tmap_out32[1 - s];
   }
   p.tmap_b = w->groups[g].tmap_b_half[best];
   p.sw = w->groups[g].scales;
