@@ -378,87 +378,91 @@ trdq_status trdq_prepare_weights(const trdq_rotation* rot, const void* W_bf16, i
     delete w;
     return TRDQ_ERR_CUDA;
   }
-  const size_t code_bytes = wbits == 8 ? static_cast<size_t>(N) * K : static_cast<size_t>(N) * K / 2;
-  const size_t scale_count = wbits == 8 ? static_cast<size_t>(N) : static_cast<size_t>(N) * (K / TRDQ_BLOCK);
-  const uint64_t row_bytes = wbits == 8 ? K : K / 2;
-  const uint32_t box_bytes = wbits == 8 ? 128 : 64;
+  const bool eight = wbits == 8;
+  const int scale_groups = K / TRDQ_BLOCK;
+  const int n_pad = (N + 127) / 128 * 128;
+  const size_t code_bytes = eight ? static_cast<size_t>(N) * K : static_cast<size_t>(N) * K / 2;
+  const size_t scale_count = eight ? static_cast<size_t>(N) : static_cast<size_t>(N) * scale_groups;
+  const uint64_t row_bytes = eight ? K : K / 2;
+  const uint32_t box_bytes = eight ? 128 : 64;
+
+  // ONE device allocation holds every table of every group (a cudaMalloc and its cudaFree cost 0.1 - 0.3 ms each: three a
+  // group made up nearly all of the 3 ms that five groups of 4608 x 1152 took), table after table, group after group, so
+  // that the kernels below run over all groups in one launch.
+  size_t total = 0;
+  auto place = [&total](size_t bytes) {
+    const size_t at = total;
+    total += (bytes + 511) / 512 * 512;
+    return at;
+  };
+  const size_t codes_at = place(G * code_bytes);  // code_bytes is a multiple of 1024: every group's codes stay aligned
+  const size_t scales_at = place(G * scale_count * sizeof(float));
+  const size_t colsum_at = eight ? place(static_cast<size_t>(G) * N * sizeof(int32_t)) : 0;
+  const size_t mult_at = eight ? 0 : place(static_cast<size_t>(G) * scale_groups * n_pad * sizeof(int32_t));
+  const size_t base_at = eight ? 0 : place(static_cast<size_t>(G) * n_pad * sizeof(float));
+  if (cudaMalloc(&w->tables, total) != cudaSuccess) {
+    cudaGetLastError();
+    trdq_weights_destroy(w);
+    return TRDQ_ERR_NOMEM;
+  }
+  uint8_t* const tables = static_cast<uint8_t*>(w->tables);
+  float* const scales = reinterpret_cast<float*>(tables + scales_at);
   for (int g = 0; g < G; ++g) {
     GroupWeights& gw = w->groups[g];
-    if (cudaMalloc(&gw.codes, code_bytes) != cudaSuccess || cudaMalloc(&gw.scales, scale_count * sizeof(float)) != cudaSuccess) {
+    gw.codes = tables + codes_at + g * code_bytes;
+    gw.scales = scales + g * scale_count;
+    if (eight) {
+      gw.colsum = reinterpret_cast<int32_t*>(tables + colsum_at) + static_cast<size_t>(g) * N;
+    } else {
+      gw.mult_t = reinterpret_cast<int32_t*>(tables + mult_at) + static_cast<size_t>(g) * scale_groups * n_pad;
+      gw.base = reinterpret_cast<float*>(tables + base_at) + static_cast<size_t>(g) * n_pad;
+    }
+  }
+
+  cudaStream_t const cs = static_cast<cudaStream_t>(stream);
+  cudaError_t e = cudaSuccess;
+  if (rot->dense) {
+    // dense blocks (Eq. 6-8): W S^-1 into an fp32 scratch, then the quantizer; the groups take turns with the scratch
+    float* wr = nullptr;
+    if (cudaMalloc(&wr, static_cast<size_t>(N) * K * sizeof(float)) != cudaSuccess) {
       cudaGetLastError();
       trdq_weights_destroy(w);
       return TRDQ_ERR_NOMEM;
     }
-    if (rot->dense) {
-      // dense blocks (Eq. 6-8): W S^-1 into an fp32 scratch, then the quantizer
-      float* wr = nullptr;
-      if (cudaMalloc(&wr, static_cast<size_t>(N) * K * sizeof(float)) != cudaSuccess) {
-        cudaGetLastError();
-        trdq_weights_destroy(w);
-        return TRDQ_ERR_NOMEM;
-      }
-      const size_t per_group = static_cast<size_t>(K / TRDQ_BLOCK) * TRDQ_BLOCK * TRDQ_BLOCK;
-      const cudaError_t ed = launch_dense_prepare(W_bf16, N, K, rot->dense_inv_t + static_cast<size_t>(g) * per_group, wbits, wr, gw.codes,
-                                                  gw.scales, static_cast<cudaStream_t>(stream));
-      const cudaError_t es = ed == cudaSuccess ? cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) : ed;  // the scratch is freed next
-      cudaFree(wr);
-      if (es != cudaSuccess) {
-        trdq_weights_destroy(w);
-        return TRDQ_ERR_CUDA;
-      }
+    const size_t per_group = static_cast<size_t>(scale_groups) * TRDQ_BLOCK * TRDQ_BLOCK;
+    for (int g = 0; g < G && e == cudaSuccess; ++g)
+      e = launch_dense_prepare(W_bf16, N, K, rot->dense_inv_t + static_cast<size_t>(g) * per_group, wbits, wr, w->groups[g].codes,
+                               w->groups[g].scales, cs);
+    const cudaError_t es = cudaStreamSynchronize(cs);  // the scratch is freed next
+    if (e == cudaSuccess) e = es;
+    cudaFree(wr);
+  } else if (rot->perm) {
+    for (int g = 0; g < G && e == cudaSuccess; ++g)
+      e = launch_rotate2_quantize(W_bf16, K, N, K, rot->weight_vec + static_cast<size_t>(g) * K, rot->perm + static_cast<size_t>(g) * K,
+                                  rot->vec2 + static_cast<size_t>(g) * K, eight ? 0 : 1, w->groups[g].codes, w->groups[g].scales, cs);
+  } else {
+    e = launch_rotate_quantize_groups(W_bf16, K, N, K, rot->weight_vec, G, eight ? 0 : 1, tables + codes_at, scales, cs);
+  }
+  // The kernel below ends the preparation and MUST stay an ordinary launch (full stream dependency, no early trigger of
+  // dependents): the GEMM kernels request weight tiles before their dependent-launch wait, which orders them only against
+  // the kernel directly before them, so the codes have to be complete before that kernel starts.
+  if (e == cudaSuccess)
+    e = eight ? launch_weight_colsum(reinterpret_cast<const int8_t*>(tables + codes_at), G * static_cast<int64_t>(N), K,
+                                     reinterpret_cast<int32_t*>(tables + colsum_at), cs)
+              : launch_w4_multipliers(scales, N, scale_groups, n_pad, G, reinterpret_cast<int32_t*>(tables + mult_at),
+                                      reinterpret_cast<float*>(tables + base_at), cs);
+  trdq_status st = e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA;
+  for (int g = 0; g < G && st == TRDQ_OK; ++g) {
+    GroupWeights& gw = w->groups[g];
+    if (!eight) st = encode_tmap_2d(&gw.tmap_b[0], gw.codes, 1, row_bytes, N, row_bytes, box_bytes, 64, 0);
+    for (int i = 0; i < kNumTileN && eight && st == TRDQ_OK; ++i) {
+      st = encode_tmap_u8_sw128(&gw.tmap_b[i], gw.codes, row_bytes, N, row_bytes, box_bytes, kTileN[i]);
+      if (st == TRDQ_OK) st = encode_tmap_u8_sw128(&gw.tmap_b_half[i], gw.codes, row_bytes, N, row_bytes, box_bytes, kTileN[i] / 2);
     }
-    const cudaError_t e =
-        rot->dense ? cudaSuccess :
-        rot->perm ? launch_rotate2_quantize(W_bf16, K, N, K, rot->weight_vec + static_cast<size_t>(g) * K, rot->perm + static_cast<size_t>(g) * K,
-                                            rot->vec2 + static_cast<size_t>(g) * K, wbits == 8 ? 0 : 1, gw.codes, gw.scales,
-                                            static_cast<cudaStream_t>(stream))
-                  : launch_rotate_quantize(W_bf16, K, N, K, rot->weight_vec + static_cast<size_t>(g) * K, wbits == 8 ? 0 : 1, gw.codes,
-                                           gw.scales, static_cast<cudaStream_t>(stream));
-    if (e != cudaSuccess) {
-      trdq_weights_destroy(w);
-      return TRDQ_ERR_CUDA;
-    }
-    for (int i = 0; i < kNumTileN; ++i) {
-      const trdq_status st = wbits == 8
-                                 ? encode_tmap_u8_sw128(&gw.tmap_b[i], gw.codes, row_bytes, N, row_bytes, box_bytes, kTileN[i])
-                                 : encode_tmap_2d(&gw.tmap_b[i], gw.codes, 1, row_bytes, N, row_bytes, box_bytes, 64, 0);
-      if (st != TRDQ_OK) {
-        trdq_weights_destroy(w);
-        return st;
-      }
-      if (wbits == 8 && encode_tmap_u8_sw128(&gw.tmap_b_half[i], gw.codes, row_bytes, N, row_bytes, box_bytes, kTileN[i] / 2) != TRDQ_OK) {
-        trdq_weights_destroy(w);
-        return TRDQ_ERR_CUDA;
-      }
-    }
-    // The kernels below end the group's preparation and MUST stay ordinary launches (full stream dependency, no early
-    // trigger of dependents): the GEMM kernels request weight tiles before their dependent-launch wait, which orders
-    // them only against the kernel directly before them, so the codes have to be complete before that kernel starts.
-    if (wbits == 8) {
-      if (cudaMalloc(&gw.colsum, static_cast<size_t>(N) * sizeof(int32_t)) != cudaSuccess) {
-        cudaGetLastError();
-        trdq_weights_destroy(w);
-        return TRDQ_ERR_NOMEM;
-      }
-      if (launch_weight_colsum(static_cast<const int8_t*>(gw.codes), N, K, gw.colsum, static_cast<cudaStream_t>(stream)) != cudaSuccess) {
-        trdq_weights_destroy(w);
-        return TRDQ_ERR_CUDA;
-      }
-    }
-    if (wbits == 4) {
-      const int n_pad = (N + 127) / 128 * 128;
-      const int groups = K / TRDQ_BLOCK;
-      if (cudaMalloc(&gw.mult_t, static_cast<size_t>(groups) * n_pad * sizeof(int32_t)) != cudaSuccess ||
-          cudaMalloc(&gw.base, static_cast<size_t>(n_pad) * sizeof(float)) != cudaSuccess) {
-        cudaGetLastError();
-        trdq_weights_destroy(w);
-        return TRDQ_ERR_NOMEM;
-      }
-      if (launch_w4_multipliers(gw.scales, N, groups, n_pad, gw.mult_t, gw.base, static_cast<cudaStream_t>(stream)) != cudaSuccess) {
-        trdq_weights_destroy(w);
-        return TRDQ_ERR_CUDA;
-      }
-    }
+  }
+  if (st != TRDQ_OK) {
+    trdq_weights_destroy(w);
+    return st;
   }
   *out = w;
   return TRDQ_OK;
@@ -466,13 +470,7 @@ trdq_status trdq_prepare_weights(const trdq_rotation* rot, const void* W_bf16, i
 
 trdq_status trdq_weights_destroy(trdq_weights* w) {
   if (!w) return TRDQ_OK;
-  for (auto& gw : w->groups) {
-    if (gw.codes) cudaFree(gw.codes);
-    if (gw.scales) cudaFree(gw.scales);
-    if (gw.colsum) cudaFree(gw.colsum);
-    if (gw.mult_t) cudaFree(gw.mult_t);
-    if (gw.base) cudaFree(gw.base);
-  }
+  if (w->tables) cudaFree(w->tables);
   delete w;
   return TRDQ_OK;
 }

@@ -469,11 +469,11 @@ trdq_status launch_gemm_w8_asym(const trdq_weights* w, int g, const GemmSegment 
 
 // Row sums of the int8 weight codes, one warp per output channel.
 namespace {
-__global__ void weight_colsum_kernel(const int8_t* __restrict__ codes, int32_t N, int32_t K, int32_t* __restrict__ colsum) {
-  const int n = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  if (n >= N) return;
+__global__ void weight_colsum_kernel(const int8_t* __restrict__ codes, int64_t rows, int32_t K, int32_t* __restrict__ colsum) {
+  const int64_t n = static_cast<int64_t>(blockIdx.x) * (blockDim.x / 32) + (threadIdx.x >> 5);
+  if (n >= rows) return;
   const int lane = threadIdx.x & 31;
-  const int4* row = reinterpret_cast<const int4*>(codes + static_cast<int64_t>(n) * K);
+  const int4* row = reinterpret_cast<const int4*>(codes + n * K);
   int32_t s = 0;
   for (int i = lane; i < K / 16; i += 32) {
     const int4 v = row[i];
@@ -486,8 +486,8 @@ __global__ void weight_colsum_kernel(const int8_t* __restrict__ codes, int32_t N
 }
 }  // namespace
 
-cudaError_t launch_weight_colsum(const int8_t* codes, int32_t N, int32_t K, int32_t* colsum, cudaStream_t stream) {
-  weight_colsum_kernel<<<(N + 7) / 8, 256, 0, stream>>>(codes, N, K, colsum);
+cudaError_t launch_weight_colsum(const int8_t* codes, int64_t rows, int32_t K, int32_t* colsum, cudaStream_t stream) {
+  weight_colsum_kernel<<<static_cast<unsigned>((rows + 7) / 8), 256, 0, stream>>>(codes, rows, K, colsum);
   return cudaGetLastError();
 }
 

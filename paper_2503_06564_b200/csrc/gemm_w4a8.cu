@@ -412,11 +412,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_con
   }
 }
 
-// One thread per output channel: put the channel's group scales on a common power-of-two grid.
+// One thread per output channel (and time-step group, blockIdx.y): put the channel's group scales on a common power-of-two grid.
 __global__ void w4_multipliers_kernel(const float* __restrict__ scales, int32_t N, int32_t groups, int32_t n_pad,
                                       int32_t* __restrict__ mult_t, float* __restrict__ base) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= n_pad) return;
+  scales += static_cast<int64_t>(blockIdx.y) * N * groups;
+  mult_t += static_cast<int64_t>(blockIdx.y) * groups * n_pad;
+  base += static_cast<int64_t>(blockIdx.y) * n_pad;
   if (n >= N) {
     for (int g = 0; g < groups; ++g) mult_t[static_cast<int64_t>(g) * n_pad + n] = 0;
     base[n] = 0.0f;
@@ -437,9 +440,9 @@ __global__ void w4_multipliers_kernel(const float* __restrict__ scales, int32_t 
 
 }  // namespace
 
-cudaError_t launch_w4_multipliers(const float* scales, int32_t N, int32_t groups, int32_t n_pad, int32_t* mult_t, float* base,
+cudaError_t launch_w4_multipliers(const float* scales, int32_t N, int32_t groups, int32_t n_pad, int sets, int32_t* mult_t, float* base,
                                   cudaStream_t stream) {
-  w4_multipliers_kernel<<<(n_pad + 127) / 128, 128, 0, stream>>>(scales, N, groups, n_pad, mult_t, base);
+  w4_multipliers_kernel<<<dim3((n_pad + 127) / 128, sets), 128, 0, stream>>>(scales, N, groups, n_pad, mult_t, base);
   return cudaGetLastError();
 }
 

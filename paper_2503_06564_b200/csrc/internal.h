@@ -49,6 +49,7 @@ struct trdq_weights {
   int32_t N = 0, K = 0, wbits = 8, num_groups = 0;
   int device = 0;
   std::vector<int32_t> t_bounds;
+  void* tables = nullptr;  // dev: the one allocation all tables of all groups point into
   std::vector<trdq::GroupWeights> groups;
 };
 
@@ -77,6 +78,10 @@ uint32_t* device_status_word();  // device address of the status word of the cur
 // mode 0: per-row int8 codes + fp32 scale per row; mode 1: per-128-block int4 codes packed + scale per block
 cudaError_t launch_rotate_quantize(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, int mode,
                                    void* codes, float* scales, cudaStream_t stream);
+
+// the same for `groups` fused vectors one after the other (vec + g K), codes and scales of group g behind those of g - 1
+cudaError_t launch_rotate_quantize_groups(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, int groups, int mode,
+                                          void* codes, float* scales, cudaStream_t stream);
 
 cudaError_t launch_rotate2_quantize(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec1, const int32_t* perm,
                                     const float* vec2, int mode, void* codes, float* scales, cudaStream_t stream);
@@ -114,7 +119,7 @@ trdq_status launch_gemm_w4(const trdq_weights* w, int g, const GemmSegment seg[2
                            cudaStream_t stream, int act = 0);
 trdq_status launch_gemm_w8_asym(const trdq_weights* w, int g, const GemmSegment seg[2], const int32_t* const zp[2],
                                 const void* bias_bf16, cudaStream_t stream);
-cudaError_t launch_weight_colsum(const int8_t* codes, int32_t N, int32_t K, int32_t* colsum, cudaStream_t stream);
+cudaError_t launch_weight_colsum(const int8_t* codes, int64_t rows, int32_t K, int32_t* colsum, cudaStream_t stream);
 cudaError_t launch_rotate_quantize_asym(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, uint8_t* codes,
                                         float* scales, int32_t* zero_points, cudaStream_t stream);
 // split-K (8-bit weights, one segment): partial int32 sums in `workspace` (splits * M * N), then reduce + epilogue
@@ -132,7 +137,8 @@ trdq_status launch_mma_ceiling(int32_t mmas_per_cluster, int32_t* clusters_out, 
 // gemm_i8_2cta.cu: CTA-pair kernel; TRDQ_ERR_SHAPE means "not applicable here, use the single-CTA kernel"
 trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment seg[2], const void* bias_bf16,
                                 cudaStream_t stream, int act = 0);
-cudaError_t launch_w4_multipliers(const float* scales, int32_t N, int32_t groups, int32_t n_pad, int32_t* mult_t, float* base,
+// for `sets` time-step groups, the tables of one behind the other
+cudaError_t launch_w4_multipliers(const float* scales, int32_t N, int32_t groups, int32_t n_pad, int sets, int32_t* mult_t, float* base,
                                   cudaStream_t stream);
 
 // tensor maps (driver entry point fetched through the runtime; no link-time libcuda dependency)

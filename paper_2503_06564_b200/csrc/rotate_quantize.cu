@@ -250,6 +250,10 @@ __global__ void __launch_bounds__(320, MIN_CTAS)
 rotate_quantize_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t ldx, int32_t M, int32_t K, const float* __restrict__ vec,
                             int8_t* __restrict__ codes, float* __restrict__ scales, int32_t rows_per_tile, float zero) {
   extern __shared__ float svec[];  // the group's fused vector, K floats
+  // weight preparation runs all time-step groups in one launch: blockIdx.y is the group
+  vec += static_cast<int64_t>(blockIdx.y) * K;
+  codes += static_cast<int64_t>(blockIdx.y) * M * K;
+  scales += static_cast<int64_t>(blockIdx.y) * M;
   __shared__ unsigned int row_max[3][32];
   const int nb = K / TRDQ_BLOCK;
   const int lane4 = threadIdx.x & (kFastLanes - 1);
@@ -509,7 +513,7 @@ rotate_quantize_rows_asym_kernel(const __nv_bfloat16* __restrict__ x, int64_t ld
   }
 }
 
-cudaError_t launch_rows_fast(const void* x, int64_t ldx, int32_t M, int32_t K, const float* vec, void* codes, float* scales,
+cudaError_t launch_rows_fast(const void* x, int64_t ldx, int32_t M, int32_t K, const float* vec, int groups, void* codes, float* scales,
                              cudaStream_t stream) {
   const int nb = K / TRDQ_BLOCK;
   int dev = 0, sms = 148;
@@ -524,7 +528,7 @@ cudaError_t launch_rows_fast(const void* x, int64_t ldx, int32_t M, int32_t K, c
   const int num_tiles = (M + rows - 1) / rows;
   const int grid = min(num_tiles, sms * 2);
   const size_t smem = static_cast<size_t>(K) * sizeof(float);
-  return launch_overlapped(rotate_quantize_rows_kernel<2>, dim3(grid), dim3(threads), smem, stream, static_cast<const __nv_bfloat16*>(x),
+  return launch_overlapped(rotate_quantize_rows_kernel<2>, dim3(grid, groups), dim3(threads), smem, stream, static_cast<const __nv_bfloat16*>(x),
                            ldx, M, K, vec, static_cast<int8_t*>(codes), scales, rows, 0.0f);
 }
 
@@ -648,14 +652,25 @@ void describe_rotate_quantize_kernel(int32_t M, int32_t K, char* name, size_t ca
 
 cudaError_t launch_rotate_quantize(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, int mode,
                                    void* codes, float* scales, cudaStream_t stream) {
+  return launch_rotate_quantize_groups(x_bf16, ldx, M, K, vec, 1, mode, codes, scales, stream);
+}
+
+cudaError_t launch_rotate_quantize_groups(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, int groups, int mode,
+                                          void* codes, float* scales, cudaStream_t stream) {
   if (M == 0) return cudaSuccess;
-  if (mode == 0) {
-    // fast path: the whole tile of a CTA fits 320 threads and the vector fits the default shared memory
-    if (K / TRDQ_BLOCK <= 80 && static_cast<size_t>(K) * sizeof(float) <= 40 * 1024)
-      return launch_rows_fast(x_bf16, ldx, M, K, vec, codes, scales, stream);
-    return dispatch<0>(x_bf16, ldx, M, K, vec, codes, scales, stream);
+  // fast path: the whole tile of a CTA fits 320 threads and the vector fits the default shared memory
+  if (mode == 0 && K / TRDQ_BLOCK <= 80 && static_cast<size_t>(K) * sizeof(float) <= 40 * 1024 && groups <= 65535)
+    return launch_rows_fast(x_bf16, ldx, M, K, vec, groups, codes, scales, stream);
+  const int64_t code_bytes = mode == 0 ? static_cast<int64_t>(M) * K : static_cast<int64_t>(M) * K / 2;
+  const int64_t scale_count = mode == 0 ? M : static_cast<int64_t>(M) * (K / TRDQ_BLOCK);
+  for (int g = 0; g < groups; ++g) {
+    const float* v = vec + static_cast<int64_t>(g) * K;
+    uint8_t* c = static_cast<uint8_t*>(codes) + g * code_bytes;
+    float* s = scales + g * scale_count;
+    const cudaError_t e = mode == 0 ? dispatch<0>(x_bf16, ldx, M, K, v, c, s, stream) : dispatch<1>(x_bf16, ldx, M, K, v, c, s, stream);
+    if (e != cudaSuccess) return e;
   }
-  return dispatch<1>(x_bf16, ldx, M, K, vec, codes, scales, stream);
+  return cudaSuccess;
 }
 
 }  // namespace trdq
