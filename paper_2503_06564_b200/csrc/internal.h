@@ -91,6 +91,11 @@ bool rotate_quantize_prefers_team(int32_t M, int32_t K);
 trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, int8_t* codes,
                                         float* scales, cudaStream_t stream);
 
+// rotate2_quantize_team.cu: full transform, per-row int8 path in the same form
+bool rotate2_prefers_team(int32_t M, int32_t K);
+trdq_status launch_rotate2_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec1, const int32_t* perm,
+                                         const float* vec2, int8_t* codes, float* scales, cudaStream_t stream);
+
 // norm_rotate_quantize.cu: LayerNorm + per-sample modulation in front of the rotation (K <= 8192)
 cudaError_t launch_norm_rotate_quantize(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, const void* shift_bf16,
                                         const void* scale_bf16, int32_t rows_per_sample, float eps, int8_t* codes, float* scales,

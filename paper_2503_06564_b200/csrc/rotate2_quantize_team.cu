@@ -1,0 +1,253 @@
+// Full balancing transform (Eq. 9 / Eq. 10) + per-token quantizer, ONE THREAD PER 128-BLOCK, the CTA split into teams of
+// warps that hold whole rows (see rotate_quantize_team.cu for the idea, team.cuh for the shared steps):
+//     v1 = blockWHT(x o vec1),  v2[j] = fl32(v1[perm[j]] * vec2[j]),  v3 = blockWHT(v2),  codes of v3.
+// Both butterflies are register-to-register.  Between them the rotated row is parked in shared memory as fp32, already
+// times the second rotation's factor (vec2 is looked up at the SOURCE channel, where a whole block is written with 16-byte
+// stores, instead of at each gathered value: the product is the same), and every thread gathers its 128 permuted channels;
+// the table of byte offsets is 16 bits per channel, eight per load.
+//
+// What bounds it: shared memory.  Of about 27 wavefronts per block and row (tile in, vectors, row out, gather, codes) the
+// gather of 128 scalars at arbitrary banks takes 16; 15 instructions per element come to 0.6 of that time.  The row
+// buffer is swizzled (16-byte chunk index xor block) and rows are 48 bytes apart modulo 128, so that the writes of a
+// quarter warp and the three rows of one channel fall into different banks.
+// One input stage (the next tile is requested as soon as this one is in registers, most of a tile's time before its use)
+// and codes staged in the row buffer after the last gather leave room for ten teams at K = 1152 and two at K = 4608.
+#include <cuda_bf16.h>
+
+#include "internal.h"
+#include "team.cuh"
+
+namespace trdq {
+namespace {
+
+constexpr int kRowPadBytes = 48;
+
+struct alignas(64) Team2Params {
+  CUtensorMap tmap_x;      // bf16: (64, M, K/64), box 64 x R x K/64
+  CUtensorMap tmap_codes;  // int8: (128, M, K/128), box 128 x R x K/128
+  const float* vec1;       // fused vector of the group, K floats
+  const int32_t* perm;     // (v P)[j] = v[perm[j]]
+  const float* vec2;       // factors of the second rotation, by destination channel
+  float* scales;           // [M]
+  int32_t M, K;
+  int32_t R, team_warps, teams;
+  float zero;              // 0.0f, see quantize_store_block
+  uint32_t* status;
+};
+
+// Byte offset of channel c inside a row of the row buffer.
+__device__ __forceinline__ uint32_t row_offset(int c) {
+  const int b = c >> 7;
+  return static_cast<uint32_t>(b) * 512 + (((static_cast<uint32_t>(c) >> 2 & 31) ^ (b & 7)) << 4) + (c & 3) * 4;
+}
+__host__ __device__ constexpr uint32_t row_buffer_bytes(int K, int R) { return (static_cast<uint32_t>(R) * (4 * K + kRowPadBytes) + 127) / 128 * 128; }
+
+__device__ __forceinline__ float lds32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+
+__global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate2_quantize_team_kernel(const __grid_constant__ Team2Params p) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t smem_base = (smem_u32(smem_raw) + 127u) & ~127u;
+  uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
+  const int nb = p.K / TRDQ_BLOCK;
+  const int R = p.R;
+  const uint32_t box_bytes = R * 128;
+  const uint32_t in_bytes = 2 * nb * box_bytes;
+  const uint32_t row_stride = 4 * p.K + kRowPadBytes;
+  const uint32_t team_bytes = in_bytes + row_buffer_bytes(p.K, R);
+  const int vec_floats = nb * (TRDQ_BLOCK + kVecPadFloats);
+  float* svec1 = reinterpret_cast<float*>(smem + p.teams * team_bytes);
+  float* svec2 = svec1 + vec_floats;                                              // by SOURCE channel
+  uint16_t* soff = reinterpret_cast<uint16_t*>(svec2 + vec_floats);               // [K] byte offsets, block b at b * (128 + 8)
+  unsigned int* row_max_all = reinterpret_cast<unsigned int*>(soff + nb * (TRDQ_BLOCK + 8));  // [teams][3][R]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(row_max_all + ((p.teams * 3 * R + 1) & ~1));   // [teams]
+
+  const int tid = threadIdx.x;
+  const int team_threads = p.team_warps * 32;
+  const int team = tid / team_threads;
+  const int tt = tid - team * team_threads;
+  const uint32_t team_base = smem_base + team * team_bytes;
+  const uint32_t rows_base = team_base + in_bytes;  // row buffer, later the code tile
+  unsigned int* row_max = row_max_all + team * 3 * R;
+  const uint32_t bar_full = smem_u32(bars + team);
+
+  if (tt == 0) {
+    mbar_init(bar_full, 1);
+    fence_mbar_init();
+  }
+  stage_vector(svec1, p.vec1, p.K, tid, blockDim.x);
+  for (int j = tid; j < p.K; j += blockDim.x) {
+    const int c = __ldg(p.perm + j);
+    svec2[(c >> 7) * (TRDQ_BLOCK + kVecPadFloats) + (c & 127)] = __ldg(p.vec2 + j);
+    soff[(j >> 7) * (TRDQ_BLOCK + 8) + (j & 127)] = static_cast<uint16_t>(row_offset(c));
+  }
+  for (int i = tid; i < p.teams * 3 * R; i += blockDim.x) row_max_all[i] = 0u;
+  if (tid == 0) {
+    prefetch_tensormap(&p.tmap_x);
+    prefetch_tensormap(&p.tmap_codes);
+  }
+  __syncthreads();
+  griddep_launch_dependents();
+  griddep_wait();  // X may be written, and the code buffer still read, by the kernel before (the tables are constant)
+
+  const int num_tiles = (p.M + R - 1) / R;
+  const int stride = gridDim.x * p.teams;
+  const int first = team * gridDim.x + blockIdx.x;
+  if (tt == 0 && first < num_tiles) {
+    mbar_arrive_expect_tx(bar_full, in_bytes);
+    tma_load_3d(team_base, &p.tmap_x, 0, first * R, 0, bar_full);
+  }
+
+  const bool active = tt < R * nb;
+  const int b = active ? tt / R : 0;
+  const int r = active ? tt - b * R : 0;
+  const float4* sv1 = reinterpret_cast<const float4*>(svec1 + b * (TRDQ_BLOCK + kVecPadFloats));
+  const float4* sv2 = reinterpret_cast<const float4*>(svec2 + b * (TRDQ_BLOCK + kVecPadFloats));
+  const uint32_t off_base = smem_u32(soff + b * (TRDQ_BLOCK + 8));
+  const uint32_t my_row = rows_base + r * row_stride;
+
+  BoundedWaiter w(p.status, kStatusTimeoutEpilogue);
+  int it = 0;
+  for (int tile = first; tile < num_tiles; tile += stride, ++it) {
+    const int buf = it % 3;
+    if (tt < R) row_max[((it + 1) % 3) * R + tt] = 0u;
+    w.wait(bar_full, it & 1);
+    float2 v[64];
+    load_scaled_block(team_base, box_bytes, b, r, sv1, v);
+    wht128_thread(v);  // first rotation
+
+    if (tt == 0) bulk_wait_group_read<0>();  // the previous tile's codes have left the row buffer
+    team_barrier(team, team_threads);        // every thread of the team has read the input stage
+    if (tt == 0 && tile + stride < num_tiles) {
+      mbar_arrive_expect_tx(bar_full, in_bytes);
+      tma_load_3d(team_base, &p.tmap_x, 0, (tile + stride) * R, 0, bar_full);
+    }
+    if (active) {
+#pragma unroll
+      for (int q = 0; q < 32; ++q) {
+        const float4 f = sv2[q];
+        const float2 lo = __fmul2_rn(v[2 * q], make_float2(f.x, f.y)), hi = __fmul2_rn(v[2 * q + 1], make_float2(f.z, f.w));
+        st_shared_v4(my_row + b * 512 + ((q ^ (b & 7)) << 4), __float_as_uint(lo.x), __float_as_uint(lo.y), __float_as_uint(hi.x), __float_as_uint(hi.y));
+      }
+    }
+    team_barrier(team, team_threads);
+    // permutation: eight 16-bit offsets per load
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const uint4 o = lds128(off_base + q * 16);
+      const uint32_t wd[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[4 * q + i] = make_float2(lds32(my_row + (wd[i] & 0xFFFFu)), lds32(my_row + (wd[i] >> 16)));
+    }
+    wht128_thread(v);  // second rotation
+    const float m = absmax_thread(v);
+    if (active) atomicMax(&row_max[buf * R + r], __float_as_uint(m));
+    team_barrier(team, team_threads);  // row maxima complete; every gather of the tile is done, the row buffer takes the codes
+
+    const float amax = __uint_as_float(row_max[buf * R + r]);
+    const float inv = amax > 0.0f ? __fdiv_rn(127.0f, amax) : 0.0f;
+    if (active) {
+      quantize_store_block(v, inv, p.zero, rows_base + b * box_bytes + r * 128);
+      const int64_t row = static_cast<int64_t>(tile) * R + r;
+      if (b == 0 && row < p.M) p.scales[row] = __fdiv_rn(amax, 127.0f);
+    }
+    fence_proxy_async_smem();
+    team_barrier(team, team_threads);
+    if (tt == 0) {
+      tma_store_3d(&p.tmap_codes, 0, tile * R, 0, rows_base);  // all nb column boxes; rows >= M are clipped
+      bulk_commit_group();
+    }
+  }
+  if (tt == 0) bulk_wait_group_read<0>();
+  w.settle();
+}
+
+struct Team2Shape {
+  int R, team_warps, teams;
+  size_t smem;
+  double use;  // fraction of the twelve warps' lanes that hold a block
+};
+
+size_t team2_smem_bytes(int K, int R, int teams) {
+  const size_t nb = K / TRDQ_BLOCK;
+  return 128 + teams * (static_cast<size_t>(2) * R * K + row_buffer_bytes(K, R)) + nb * (TRDQ_BLOCK + kVecPadFloats) * 8 + nb * (TRDQ_BLOCK + 8) * 2 +
+         (static_cast<size_t>(teams) * 3 * R + 2) * 4 + static_cast<size_t>(teams) * 8 + 16;
+}
+
+// The team size with the best use of the lanes of twelve warps (the fuller teams of two that are alike); at least two teams, so that one can transform while
+// another waits (rows of up to 72 blocks; offsets of 16 bits would reach 128).
+bool choose_team2_shape(int K, Team2Shape* out) {
+  const int nb = K / TRDQ_BLOCK;
+  Team2Shape best = {0, 0, 0, 0, 0.0};
+  for (int tw = 1; tw <= kTeamMaxWarps / 2; ++tw)
+    for (int rows = tw * 32 / nb < 32 ? tw * 32 / nb : 32; rows >= 1; --rows) {
+      int teams = kTeamMaxWarps / tw;
+      while (teams > 0 && team2_smem_bytes(K, rows, teams) > 227u * 1024u) --teams;
+      if (teams < 2) continue;
+      const double use = static_cast<double>(rows) * nb * teams / (32 * kTeamMaxWarps);
+      const double lanes = static_cast<double>(rows) * nb / (32 * tw), best_lanes = static_cast<double>(best.R) * nb / (32 * best.team_warps + 1e-9);
+      if (use > best.use + 1e-9 || (use > best.use - 1e-9 && lanes > best_lanes + 1e-9)) best = Team2Shape{rows, tw, teams, team2_smem_bytes(K, rows, teams), use};
+    }
+  if (best.teams == 0) return false;
+  *out = best;
+  return true;
+}
+
+}  // namespace
+
+// The team kernel serves rows that keep at least 0.45 of the lanes of twelve warps busy (K = 7680: 72 -> 64 us at M = 4096;
+// K = 8192, 0.33 of the lanes: 75 against 84 us) once there is a tile per SM.  Below that the lane-group kernel, whose CTAs
+// are smaller and start sooner, finishes first (M = 256, K = 1152: 5.0 against 5.6 us; M = 448: 5.9 against 5.6).
+// M = 4096, K = 1152 / 4608: 14.2 / 44.3 -> 10.0 / 35.0 us; M = 16384: 43.8 / 166 -> 28.7 / 115 us.
+bool rotate2_prefers_team(int32_t M, int32_t K) {
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  Team2Shape s;
+  return choose_team2_shape(K, &s) && s.use >= 0.45 && (M + s.R - 1) / s.R >= sms;
+}
+
+trdq_status launch_rotate2_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec1, const int32_t* perm,
+                                         const float* vec2, int8_t* codes, float* scales, cudaStream_t stream) {
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) != cudaSuccess) return TRDQ_ERR_CUDA;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  Team2Shape shape;
+  if (!choose_team2_shape(K, &shape)) return TRDQ_ERR_SHAPE;
+  const int nb = K / TRDQ_BLOCK;
+  Team2Params p;
+  trdq_status st = encode_tmap_boxes(&p.tmap_x, x_bf16, 2, 64, static_cast<uint64_t>(M), static_cast<uint64_t>(ldx) * 2,
+                                     static_cast<uint32_t>(2 * nb), static_cast<uint32_t>(shape.R));
+  if (st != TRDQ_OK) return st;
+  st = encode_tmap_boxes(&p.tmap_codes, codes, 1, 128, static_cast<uint64_t>(M), static_cast<uint64_t>(K), static_cast<uint32_t>(nb),
+                         static_cast<uint32_t>(shape.R));
+  if (st != TRDQ_OK) return st;
+  p.vec1 = vec1;
+  p.perm = perm;
+  p.vec2 = vec2;
+  p.scales = scales;
+  p.M = M;
+  p.K = K;
+  p.R = shape.R;
+  p.team_warps = shape.team_warps;
+  p.teams = shape.teams;
+  p.zero = 0.0f;
+  p.status = device_status_word();
+  if (!p.status) return TRDQ_ERR_CUDA;
+  static PerDeviceFlag configured;
+  if (!configured.get(dev)) {
+    if (cudaFuncSetAttribute(rotate2_quantize_team_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
+      return TRDQ_ERR_CUDA;
+    configured.set(dev, true);
+  }
+  const int num_tiles = (M + shape.R - 1) / shape.R;
+  const int grid = num_tiles < sms ? num_tiles : sms;
+  const cudaError_t e = launch_overlapped(rotate2_quantize_team_kernel, dim3(grid), dim3(shape.teams * shape.team_warps * 32), shape.smem,
+                                          stream, p);
+  return e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA;
+}
+
+}  // namespace trdq

@@ -592,6 +592,10 @@ cudaError_t launch_rotate2_quantize(const void* x_bf16, int64_t ldx, int32_t M, 
   if (M == 0) return cudaSuccess;
   const int nb = K / TRDQ_BLOCK;
   if (nb > 128) return cudaErrorInvalidValue;
+  if (mode == 0 && rotate2_prefers_team(M, K))
+    return launch_rotate2_quantize_team(x_bf16, ldx, M, K, vec1, perm, vec2, static_cast<int8_t*>(codes), scales, stream) == TRDQ_OK
+               ? cudaSuccess
+               : cudaErrorUnknown;
   if (mode == 0 && nb <= 72) {
     // four lanes per block, packed arithmetic: about 72 lane groups per CTA, two CTAs per SM
     int rows2 = 72 / nb;

@@ -15,14 +15,10 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
-#include "lane_group.cuh"
-#include "ptx.cuh"
+#include "team.cuh"
 
 namespace trdq {
 namespace {
-
-constexpr int kMaxWarps = 12;        // 12 x 32 threads x <= 168 registers fill the register file
-constexpr int kVecPadFloats = 4;     // the fused vector of block b starts at float b * (128 + 4): see the staging loop
 
 struct alignas(64) TeamParams {
   // Both maps view a row as K/64 (K/128) column boxes: dims (column in box, row, box), so that ONE copy moves a tile of R
@@ -35,31 +31,11 @@ struct alignas(64) TeamParams {
   int32_t R;               // rows per team tile
   int32_t team_warps;      // warps per team (R * K/128 <= 32 * team_warps)
   int32_t teams;           // teams per CTA
-  float zero;              // 0.0f, see the quantizer below
+  float zero;              // 0.0f, see quantize_store_block
   uint32_t* status;
 };
 
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-  uint4 v;
-  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-  return v;
-}
-
-// max(|a|, |b|, |c|) in one instruction
-__device__ __forceinline__ float max3_abs(float a, float b, float c) {
-  float r;
-  asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-
-__device__ __forceinline__ void team_barrier(int team, int team_threads) {
-  if (team_threads == 32)
-    __syncwarp();
-  else
-    asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(team_threads) : "memory");
-}
-
-__global__ void __launch_bounds__(kMaxWarps * 32, 1) rotate_quantize_team_kernel(const __grid_constant__ TeamParams p) {
+__global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_kernel(const __grid_constant__ TeamParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 127u) & ~127u;  // TMA destinations need 128 bytes; the swizzle is a function of the address
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -87,12 +63,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) rotate_quantize_team_kernel
     mbar_init(bar_full + 8, 1);
     fence_mbar_init();
   }
-  // The fused vector, block b at float b * 132: lanes of a quarter warp that hold different blocks then read different
-  // bank groups with their 16-byte loads (same block: same address, a broadcast).
-  for (int i = tid; i < p.K / 4; i += blockDim.x) {
-    const int b = i >> 5;
-    reinterpret_cast<float4*>(svec + b * (TRDQ_BLOCK + kVecPadFloats))[i & 31] = __ldg(reinterpret_cast<const float4*>(p.vec) + i);
-  }
+  stage_vector(svec, p.vec, p.K, tid, blockDim.x);
   for (int i = tid; i < p.teams * 3 * R; i += blockDim.x) row_max_all[i] = 0u;
   if (tid == 0) {
     prefetch_tensormap(&p.tmap_x);
@@ -119,7 +90,6 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) rotate_quantize_team_kernel
   const int b = active ? tt / R : 0;
   const int r = active ? tt - b * R : 0;
   const float4* sv4 = reinterpret_cast<const float4*>(svec + b * (TRDQ_BLOCK + kVecPadFloats));
-  const float2 neg1 = make_float2(-1.0f, -1.0f);
 
   BoundedWaiter w(p.status, kStatusTimeoutEpilogue);
   int it = 0;
@@ -134,44 +104,10 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) rotate_quantize_team_kernel
       mbar_arrive_expect_tx(bar_full + 8, in_bytes);
       tma_load_3d(team_base + in_bytes, &p.tmap_x, 0, (tile + stride) * R, 0, bar_full + 8);
     }
-    // v[32h + 4j + i] = elements (2i, 2i+1) of 16-byte chunk j of half h, times the fused vector
     float2 v[64];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const uint32_t in_row = team_base + s * in_bytes + (2 * b + h) * box_bytes + r * 128;
-      const uint32_t swz = (in_row >> 7) & 7u;  // 128-byte swizzle: chunk index xor address bits 7..9
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const uint4 raw = lds128(in_row + ((j ^ swz) << 4));
-        const float4 s0 = sv4[h * 16 + j * 2], s1 = sv4[h * 16 + j * 2 + 1];
-        const uint32_t wd[4] = {raw.x, raw.y, raw.z, raw.w};
-        const float2 sc[4] = {make_float2(s0.x, s0.y), make_float2(s0.z, s0.w), make_float2(s1.x, s1.y), make_float2(s1.z, s1.w)};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          // bf16 -> fp32 is exact: the 16 bits become the high half of the fp32 pattern
-          const float2 xv = make_float2(__uint_as_float(wd[i] << 16), __uint_as_float(wd[i] & 0xFFFF0000u));
-          v[h * 32 + j * 4 + i] = __fmul2_rn(xv, sc[i]);
-        }
-      }
-    }
-
-    // h = 1: inside a pair; h = 2 .. 64: pair index bits 0 .. 5
-#pragma unroll
-    for (int q = 0; q < 64; ++q) v[q] = make_float2(__fadd_rn(v[q].x, v[q].y), __fsub_rn(v[q].x, v[q].y));
-#pragma unroll
-    for (int hb = 1; hb < 64; hb <<= 1) {
-#pragma unroll
-      for (int q = 0; q < 64; ++q) {
-        if ((q & hb) == 0) {
-          const float2 a = v[q], c = v[q + hb];
-          v[q] = __fadd2_rn(a, c);
-          v[q + hb] = __ffma2_rn(c, neg1, a);  // a - c, one rounding
-        }
-      }
-    }
-    float m = 0.0f;
-#pragma unroll
-    for (int q = 0; q < 64; ++q) m = max3_abs(m, v[q].x, v[q].y);
+    load_scaled_block(team_base + s * in_bytes, box_bytes, b, r, sv4, v);
+    wht128_thread(v);
+    const float m = absmax_thread(v);
     if (active) atomicMax(&row_max[buf * R + r], __float_as_uint(m));
     if (tt == 0) bulk_wait_group_read<0>();  // the previous tile's store has finished reading the staging tile
     team_barrier(team, team_threads);        // row maxima complete; every thread of the team has read stage s
@@ -186,22 +122,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) rotate_quantize_team_kernel
 
     const float amax = __uint_as_float(row_max[buf * R + r]);
     const float inv = amax > 0.0f ? __fdiv_rn(127.0f, amax) : 0.0f;
-    const float2 inv2 = make_float2(inv, inv);
-    const float2 magic2 = make_float2(kRoundMagic, kRoundMagic);
-    // The product must be rounded to fp32 before the magic addition rounds it to an integer.  A packed multiply feeding
-    // a packed add is contracted into one fused operation by the assembler, so the product is written as
-    // fma(v, inv, zero) with `zero` a kernel argument equal to 0.0f.
-    const float2 zero2 = make_float2(p.zero, p.zero);
     if (active) {
-      const uint32_t out_row = out_base + b * box_bytes + r * 128;
-      const uint32_t oswz = (out_row >> 7) & 7u;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {  // 16 codes = 8 pairs per 16-byte chunk
-        float2 q[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) q[i] = __fadd2_rn(__ffma2_rn(v[c * 8 + i], inv2, zero2), magic2);
-        st_shared_v4(out_row + ((c ^ oswz) << 4), pack4(q[0], q[1]), pack4(q[2], q[3]), pack4(q[4], q[5]), pack4(q[6], q[7]));
-      }
+      quantize_store_block(v, inv, p.zero, out_base + b * box_bytes + r * 128);
       const int64_t row = static_cast<int64_t>(tile) * R + r;
       if (b == 0 && row < p.M) p.scales[row] = __fdiv_rn(amax, 127.0f);
     }
@@ -236,11 +158,11 @@ bool team_shape_for(int K, int tw, TeamShape* out) {
   int rows = tw * 32 / nb;
   if (rows < 1) return false;
   if (rows > 32) rows = 32;
-  int teams = kMaxWarps / tw;
+  int teams = kTeamMaxWarps / tw;
   while (teams > 0 && team_smem_bytes(K, rows, teams) > 227u * 1024u) --teams;
   if (teams < 2) return false;
   *out = TeamShape{rows, tw, teams, team_smem_bytes(K, rows, teams),
-                   static_cast<double>(rows) * nb / (tw * 32) * (static_cast<double>(teams * tw) / kMaxWarps)};
+                   static_cast<double>(rows) * nb / (tw * 32) * (static_cast<double>(teams * tw) / kTeamMaxWarps)};
   return true;
 }
 
@@ -250,7 +172,7 @@ bool team_shape_for(int K, int tw, TeamShape* out) {
 // 6.7 us, measured).
 bool choose_team_shape(int M, int K, int sms, TeamShape* out) {
   TeamShape best = {0, 0, 0, 0, 0.0};
-  for (int tw = 1; tw <= kMaxWarps / 2; ++tw) {
+  for (int tw = 1; tw <= kTeamMaxWarps / 2; ++tw) {
     TeamShape s;
     if (team_shape_for(K, tw, &s) && s.use > best.use + 1e-9) best = s;
   }
