@@ -526,7 +526,7 @@ trdq_status trdq_rotate_quantize(const trdq_rotation* rot, int32_t t, const void
     return finish(e2 == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA, stream);
   }
   if (rotate_quantize_prefers_team(M, rot->K))
-    return finish(launch_rotate_quantize_team(X_bf16, ldx, M, rot->K, vec, codes, scales, static_cast<cudaStream_t>(stream)), stream);
+    return finish(launch_rotate_quantize_team(X_bf16, ldx, M, rot->K, vec, codes, scales, nullptr, static_cast<cudaStream_t>(stream)), stream);
   const cudaError_t e = launch_rotate_quantize(X_bf16, ldx, M, rot->K, vec, 0, codes, scales, static_cast<cudaStream_t>(stream));
   return finish(e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA, stream);
 }
@@ -657,6 +657,10 @@ trdq_status trdq_rotate_quantize_asym(const trdq_rotation* rot, int32_t t, const
       (reinterpret_cast<uintptr_t>(zero_points) & 3u))
     return TRDQ_ERR_ALIGN;
   if (!on_current_device(rot->device)) return TRDQ_ERR_MISMATCH;
+  if (rotate_quantize_asym_prefers_team(M, rot->K))
+    return finish(launch_rotate_quantize_team(X_bf16, ldx, M, rot->K, rot->act_vec + static_cast<size_t>(g) * rot->K, codes, scales, zero_points,
+                                              static_cast<cudaStream_t>(stream)),
+                  stream);
   const cudaError_t e = launch_rotate_quantize_asym(X_bf16, ldx, M, rot->K, rot->act_vec + static_cast<size_t>(g) * rot->K, codes, scales,
                                                     zero_points, static_cast<cudaStream_t>(stream));
   return finish(e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA, stream);

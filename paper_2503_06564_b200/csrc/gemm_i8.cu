@@ -353,23 +353,28 @@ int choose_tile_n(int64_t tiles_m, int N, int sms) {
 
 }  // namespace
 
-// Row count from which the CTA-pair kernel is used (two SMs per 256-row tile, a third less operand traffic per SM).
-static int pair_min_rows() {
-  static const int rows = [] {
+// Whether the CTA-pair kernel (two SMs per 256-row tile, a third less operand traffic per SM) runs M rows against [N, K] weights:
+// from 2048 rows, once the output is large enough that its fewer, larger tiles fill the SMs.  Microseconds, pair / single CTA:
+// 1152 -> 1152 at M = 2048 6.5 / 5.5, 3072 7.5 / 6.6, 4096 8.8 / 8.2; 1152 -> 3456 at 2048 9.8 / 9.4, 3072 12.5 / 12.6; 1152 -> 4608 at 2048
+// 11.3 / 11.3; 384 -> 384 at 4096 4.8 / 4.2.  With a long reduction the operand traffic counts earlier: 4608 -> 1152 at 2048 11.1 / 10.6,
+// 3072 13.6 / 13.5, 4096 18.3 / 19.3.  TRDQ_PAIR_MIN_M (read once per process) replaces the rule by a row count.
+static bool use_pair(int64_t M, int32_t K, int32_t N) {
+  static const int forced = [] {
     const char* e = getenv("TRDQ_PAIR_MIN_M");
-    return e ? atoi(e) : 2048;
+    return e ? atoi(e) : -1;
   }();
-  return rows;
+  if (forced >= 0) return M >= forced;
+  const int64_t least = (K >= 2304 ? 64 : 110) * 65536ll;  // output values: tiles of 256 x 256
+  return M >= 2048 && M * N >= least;
 }
 
 // Name of the kernel trdq_linear runs for M rows against [N, K] weights of `wbits` bits (one row segment).
 void describe_gemm_kernel(int32_t M, int32_t K, int32_t N, int32_t wbits, char* name, size_t cap) {
-  (void)K;
   if (wbits == 4) {
     snprintf(name, cap, "gemm_w4a8_kernel");
     return;
   }
-  if (M >= pair_min_rows()) {
+  if (use_pair(M, K, N)) {
     const int bn = gemm_w8_pair_tile_width((static_cast<int64_t>(M) + 2 * kTileM - 1) / (2 * kTileM), N);
     if (bn > 0) {
       snprintf(name, cap, "gemm_w8a8_pair_kernel<%d>", bn);
@@ -384,8 +389,8 @@ void describe_gemm_kernel(int32_t M, int32_t K, int32_t N, int32_t wbits, char* 
 static trdq_status launch_gemm_w8_mode(const trdq_weights* w, int g, const GemmSegment seg[2], const void* bias_bf16, int mode,
                                        const int32_t* const zp[2], cudaStream_t stream, int act = 0) {
   const bool raw_i32 = mode == 1;
-  if (mode == 0 && static_cast<int64_t>(seg[0].M) + seg[1].M >= pair_min_rows()) {
-    const trdq_status st = launch_gemm_w8_pair(w, g, seg, bias_bf16, stream, act);
+  if (mode != 1 && use_pair(static_cast<int64_t>(seg[0].M) + seg[1].M, w->K, w->N)) {
+    const trdq_status st = launch_gemm_w8_pair(w, g, seg, mode == 2 ? zp : nullptr, bias_bf16, stream, act);
     if (st != TRDQ_ERR_SHAPE) return st;
   }
   int dev = 0, sms = 148;

@@ -17,6 +17,8 @@
 // at a time (a 32 x 64 bf16 tile per TMA store: whole 128-byte lines).  No TMA multicast is used.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "epilogue.cuh"
 #include "internal.h"
 #include "ptx.cuh"
@@ -38,7 +40,7 @@ struct Cfg2 {
   static constexpr int kABytes = kTileM * kTileKBytes;
   static constexpr int kBBytes = (BN / 2) * kTileKBytes;  // this CTA's half of the weight tile
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kParamBytes = 2 * ColumnParamLayout<BN>::kBytes;
+  static constexpr int kParamBytes = 2 * (ColumnParamLayout<BN>::kBytes + BN * 4);  // two sets: column parameters and (asymmetric mode) weight column sums
   static constexpr int kBarrierBytes = 256;
   static constexpr int kOutStageBytes = (kEpilogueThreads / 32) * 4096;  // one 32 x 64 bf16 tile per warp
   static constexpr int kStages = (kSmemBudget - 1024 - kOutStageBytes - kParamBytes - kBarrierBytes) / kStageBytes;
@@ -57,6 +59,8 @@ struct alignas(64) Gemm2Params {
   int32_t pair_tiles_m[2];  // 256-row tiles per segment
   const float* sw;
   const __nv_bfloat16* bias;
+  const int32_t* zp[2];   // asymmetric activation codes: zero point of every row, sum of every channel's weight codes
+  const int32_t* colsum;
   int32_t N, K, tiles_n;
   int32_t band;  // row tiles per band of the tile order; 0: column-block major over all row tiles
   uint32_t* status;
@@ -141,15 +145,18 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
                "h"(static_cast<uint16_t>(3))
                : "memory");
 }
-// kind::i8 instruction descriptor for the pair: M = 256.
-__host__ __device__ constexpr uint32_t umma_idesc_s8_pair(int n) {
-  return (2u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
+// kind::i8 instruction descriptor for the pair: M = 256, A unsigned or signed, B signed.
+__host__ __device__ constexpr uint32_t umma_idesc_s8_pair(int n, bool unsigned_a = false) {
+  return (2u << 4) | (unsigned_a ? 0u : 1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
 }
 
-// ACT: GELU (tanh form) on the dequantized value before the bf16 rounding.
-template <int BN, bool ACT>
+// MODE 0: dequantizing epilogue.  MODE 1: GELU (tanh form) on the dequantized value before the bf16 rounding.
+// MODE 2: unsigned activation codes with zero points (Eq. 1-3), acc - z[m] * colsum[n] in front of the epilogue of mode 0.
+enum PairMode { kPairPlain = 0, kPairGelu = 1, kPairAsym = 2 };
+template <int BN, int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8a8_pair_kernel(const __grid_constant__ Gemm2Params p) {
   using C = Cfg2<BN>;
+  constexpr bool ACT = MODE == kPairGelu;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -252,7 +259,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
     // ---------------------------------------------------- MMA issuer (leader only)
     if (leader && elect_one()) {
       BoundedWaiter w(p.status, kStatusTimeoutMma);
-      constexpr uint32_t idesc = umma_idesc_s8_pair(BN);
+      constexpr uint32_t idesc = umma_idesc_s8_pair(BN, MODE == kPairAsym);
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
@@ -300,9 +307,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
       const int m0 = tc.m0 + rank * kTileM;
       const ColumnParams cp =
           stage_column_params<BN>(param_buf + acc * ColumnParamLayout<BN>::kFloats, p.sw, p.bias, tc.n0, p.N, et, kEpilogueThreads);
+      int32_t* csum = reinterpret_cast<int32_t*>(param_buf + 2 * ColumnParamLayout<BN>::kFloats) + acc * BN;
+      if (MODE == kPairAsym)
+        for (int c = et; c < BN; c += kEpilogueThreads) csum[c] = tc.n0 + c < p.N ? __ldg(p.colsum + tc.n0 + c) : 0;
       asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory");
       const int row = m0 + q * 32 + lane;
       const float sxm = row < p.M[tc.seg] ? __ldg(p.sx[tc.seg] + row) : 0.0f;
+      const int32_t zrow = MODE == kPairAsym && row < p.M[tc.seg] ? __ldg(p.zp[tc.seg] + row) : 0;
+      // sum_k (q - z) * qw = sum_k q * qw - z * sum_k qw, for chunk c
+      auto subtract_zero = [&](uint32_t (&r)[32], int c) {
+        if (MODE == kPairAsym) {
+          const int4* cs = reinterpret_cast<const int4*>(csum + c * 32);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int4 v = cs[j];
+            r[4 * j] -= zrow * v.x, r[4 * j + 1] -= zrow * v.y, r[4 * j + 2] -= zrow * v.z, r[4 * j + 3] -= zrow * v.w;
+          }
+        }
+      };
 
       w.wait(bar_tfull + 8 * acc, acc_phase);
       __syncwarp();
@@ -317,6 +339,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
           uint32_t r[32];
           tmem_ld_32x32(t_row + (c + h2) * 32, r);
           tmem_wait_ld();
+          subtract_zero(r, c + h2);
           uint32_t packed[16];
           dequant_row32<ACT>(r, sxm, cp, c + h2, packed);
           if (h2 == 0) {
@@ -341,6 +364,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
         uint32_t r[32];
         tmem_ld_32x32(t_row + c * 32, r);
         tmem_wait_ld();
+        subtract_zero(r, c);
         uint32_t packed[16];
         dequant_row32<ACT>(r, sxm, cp, c, packed);
         if (lane == 0) bulk_wait_group_read<0>();
@@ -378,7 +402,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
   }
 }
 
-template <int BN, bool ACT>
+template <int BN, int MODE>
 cudaError_t launch_pair(const Gemm2Params& p, int clusters, cudaStream_t stream) {
   using C = Cfg2<BN>;
   cudaLaunchConfig_t cfg = {};
@@ -391,7 +415,7 @@ cudaError_t launch_pair(const Gemm2Params& p, int clusters, cudaStream_t stream)
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, gemm_w8a8_pair_kernel<BN, ACT>, p);
+  return cudaLaunchKernelEx(&cfg, gemm_w8a8_pair_kernel<BN, MODE>, p);
 }
 
 // Clusters of two CTAs that can be resident at once (at most SMs / 2; fewer if a GPC has an odd SM count).
@@ -402,8 +426,9 @@ int max_clusters(int dev) {
   int known = cached.get(dev);
   if (known == 0) {
     using C = Cfg2<BN>;
-    if (cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess) {
+    if (cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, kPairPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, kPairGelu>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, kPairAsym>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess) {
       cudaGetLastError();
       cached.set(dev, -1);
       return 0;
@@ -413,7 +438,7 @@ int max_clusters(int dev) {
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = C::kSmemBytes;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_w8a8_pair_kernel<BN, false>, &cfg) != cudaSuccess || n <= 0) {
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_w8a8_pair_kernel<BN, kPairPlain>, &cfg) != cudaSuccess || n <= 0) {
       cudaGetLastError();
       cached.set(dev, -1);
       return 0;
@@ -555,8 +580,8 @@ trdq_status launch_mma_ceiling(int32_t mmas_per_cluster, int32_t* clusters_out, 
 }
 
 // Returns TRDQ_ERR_SHAPE when the pair kernel does not apply (caller falls back to the single-CTA kernel).
-trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment seg[2], const void* bias_bf16, cudaStream_t stream,
-                                int act) {
+trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment seg[2], const int32_t* const zp[2], const void* bias_bf16,
+                                cudaStream_t stream, int act) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return TRDQ_ERR_CUDA;
   Gemm2Params p;
@@ -594,6 +619,9 @@ trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment 
   p.tmap_b = w->groups[g].tmap_b_half[best];
   p.sw = w->groups[g].scales;
   p.bias = static_cast<const __nv_bfloat16*>(bias_bf16);
+  p.zp[0] = zp ? zp[0] : nullptr;
+  p.zp[1] = zp ? zp[1] : nullptr;
+  p.colsum = w->groups[g].colsum;
   p.N = w->N;
   p.K = w->K;
   p.tiles_n = (w->N + bn - 1) / bn;
@@ -604,11 +632,13 @@ trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment 
   if (!p.status) return TRDQ_ERR_CUDA;
   const int64_t total = tiles_m * p.tiles_n;
   const int clusters = static_cast<int>(total < resident ? total : resident);
-  cudaError_t e;
-  if (act)
-    e = bn == 128 ? launch_pair<128, true>(p, clusters, stream) : bn == 192 ? launch_pair<192, true>(p, clusters, stream) : launch_pair<256, true>(p, clusters, stream);
-  else
-    e = bn == 128 ? launch_pair<128, false>(p, clusters, stream) : bn == 192 ? launch_pair<192, false>(p, clusters, stream) : launch_pair<256, false>(p, clusters, stream);
+  auto launch = [&](auto mode) {
+    constexpr int kMode = decltype(mode)::value;
+    return bn == 128 ? launch_pair<128, kMode>(p, clusters, stream) : bn == 192 ? launch_pair<192, kMode>(p, clusters, stream) : launch_pair<256, kMode>(p, clusters, stream);
+  };
+  const cudaError_t e = zp    ? launch(std::integral_constant<int, kPairAsym>())
+                        : act ? launch(std::integral_constant<int, kPairGelu>())
+                              : launch(std::integral_constant<int, kPairPlain>());
   return e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA;
 }
 

@@ -88,8 +88,10 @@ cudaError_t launch_rotate2_quantize(const void* x_bf16, int64_t ldx, int32_t M, 
 
 // rotate_quantize_team.cu: per-row int8 path, TMA-staged, one thread per block, independent teams of warps per CTA
 bool rotate_quantize_prefers_team(int32_t M, int32_t K);
-trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, int8_t* codes,
-                                        float* scales, cudaStream_t stream);
+bool rotate_quantize_asym_prefers_team(int32_t M, int32_t K);
+// zero_points == nullptr: symmetric int8 codes; otherwise unsigned codes with a zero point per row (Eq. 1-3)
+trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, void* codes,
+                                        float* scales, int32_t* zero_points, cudaStream_t stream);
 
 // rotate2_quantize_team.cu: full transform, per-row int8 path in the same form
 bool rotate2_prefers_team(int32_t M, int32_t K);
@@ -140,7 +142,8 @@ int gemm_w8_pair_tile_width(int64_t pair_tiles_m, int N);  // 0: the pair kernel
 // measurement aid: `mmas_per_cluster` back-to-back 256 x 256 x 32 int8 MMAs per CTA pair on resident operands
 trdq_status launch_mma_ceiling(int32_t mmas_per_cluster, int32_t* clusters_out, cudaStream_t stream);
 // gemm_i8_2cta.cu: CTA-pair kernel; TRDQ_ERR_SHAPE means "not applicable here, use the single-CTA kernel"
-trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment seg[2], const void* bias_bf16,
+// (zp: zero points of unsigned activation codes, or nullptr)
+trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment seg[2], const int32_t* const zp[2], const void* bias_bf16,
                                 cudaStream_t stream, int act = 0);
 // for `sets` time-step groups, the tables of one behind the other
 cudaError_t launch_w4_multipliers(const float* scales, int32_t N, int32_t groups, int32_t n_pad, int sets, int32_t* mult_t, float* base,

@@ -171,4 +171,13 @@ __device__ __forceinline__ void wht128_lanes4(float2 (&v)[16], int lane4) {
 
 }
 
+// Order-preserving integer image of a float, for shared-memory atomic minima and maxima.
+__device__ __forceinline__ unsigned int float_order_key(float f) {
+  const unsigned int b = __float_as_uint(f);
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float float_from_order_key(unsigned int k) {
+  return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
+}
+
 }  // namespace trdq

@@ -417,14 +417,6 @@ rotate2_quantize_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t ldx, i
 // (the lower clamp of Eq. 1 can never bind: rounding is monotone and z cancels the minimum's own code).
 // Same four-lanes-per-block layout and butterfly as rotate_quantize_rows_kernel; the row minimum and maximum
 // are combined through shared-memory atomics on an order-preserving integer image of the floats.
-__device__ __forceinline__ unsigned int float_order_key(float f) {
-  const unsigned int b = __float_as_uint(f);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float float_from_order_key(unsigned int k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
-}
-
 template <int MIN_CTAS>
 __global__ void __launch_bounds__(320, MIN_CTAS)
 rotate_quantize_rows_asym_kernel(const __nv_bfloat16* __restrict__ x, int64_t ldx, int32_t M, int32_t K, const float* __restrict__ vec,

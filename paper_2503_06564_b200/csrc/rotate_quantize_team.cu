@@ -27,6 +27,7 @@ struct alignas(64) TeamParams {
   CUtensorMap tmap_codes;  // int8: (128, M, K/128), box 128 x R x K/128
   const float* vec;        // fused vector of the group, K floats
   float* scales;           // [M]
+  int32_t* zero_points;    // [M], asymmetric form only
   int32_t M, K;
   int32_t R;               // rows per team tile
   int32_t team_warps;      // warps per team (R * K/128 <= 32 * team_warps)
@@ -35,6 +36,46 @@ struct alignas(64) TeamParams {
   uint32_t* status;
 };
 
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
+// Unsigned codes of the thread's block (Eq. 1-3): code = min(rne(fl(v * inv)) + z, 255); the lower clamp of Eq. 1 can never bind
+// (rounding is monotone and z cancels the minimum's own code).  fl(v * inv) + 1.5 * 2^23 leaves the rounded product in the low
+// mantissa bits; adding z and the clamp are exact there as long as |v * inv| < 2^22, which `small` says for the whole row.
+__device__ __forceinline__ void quantize_store_block_asym(const float2 (&v)[64], float inv, int z, bool small, float zero, uint32_t out_row) {
+  const uint32_t oswz = (out_row >> 7) & 7u;
+  const float2 inv2 = make_float2(inv, inv), magic2 = make_float2(kRoundMagic, kRoundMagic), zero2 = make_float2(zero, zero);
+  const float zf = static_cast<float>(z);
+  const float2 z2 = make_float2(zf, zf);
+  constexpr float top = kRoundMagic + 255.0f;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    float2 q[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float2 y = __ffma2_rn(v[c * 8 + i], inv2, zero2);
+      if (small) {
+        const float2 u = __fadd2_rn(__fadd2_rn(y, magic2), z2);
+        q[i] = make_float2(fminf(u.x, top), fminf(u.y, top));
+      } else {
+        q[i] = make_float2(__uint_as_float(static_cast<uint32_t>(min(__float2int_rn(y.x) + z, 255))),
+                           __uint_as_float(static_cast<uint32_t>(min(__float2int_rn(y.y) + z, 255))));
+      }
+    }
+    st_shared_v4(out_row + ((c ^ oswz) << 4), pack4(q[0], q[1]), pack4(q[2], q[3]), pack4(q[4], q[5]), pack4(q[6], q[7]));
+  }
+}
+
+// ASYM: the literal asymmetric quantizer of Eq. 1-3 (row minimum and maximum, unsigned codes, a zero point per row).
+template <bool ASYM>
 __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_kernel(const __grid_constant__ TeamParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 127u) & ~127u;  // TMA destinations need 128 bytes; the swizzle is a function of the address
@@ -47,7 +88,7 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_ke
   const uint32_t team_bytes = 2 * in_bytes + out_bytes;
   float* svec = reinterpret_cast<float*>(smem + p.teams * team_bytes);
   unsigned int* row_max_all = reinterpret_cast<unsigned int*>(svec + nb * (TRDQ_BLOCK + kVecPadFloats));  // [teams][3][R]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(row_max_all + ((p.teams * 3 * R + 1) & ~1));                  // [teams][2]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(row_max_all + (ASYM ? 2 * p.teams * 3 * R : (p.teams * 3 * R + 1) & ~1));  // [teams][2]
 
   const int tid = threadIdx.x;
   const int team_threads = p.team_warps * 32;
@@ -56,6 +97,7 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_ke
   const uint32_t team_base = smem_base + team * team_bytes;
   const uint32_t out_base = team_base + 2 * in_bytes;
   unsigned int* row_max = row_max_all + team * 3 * R;
+  unsigned int* row_min = row_max + p.teams * 3 * R;  // ASYM: keys of the minima behind those of the maxima
   const uint32_t bar_full = smem_u32(bars + 2 * team);  // [2]
 
   if (tt == 0) {
@@ -64,7 +106,10 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_ke
     fence_mbar_init();
   }
   stage_vector(svec, p.vec, p.K, tid, blockDim.x);
-  for (int i = tid; i < p.teams * 3 * R; i += blockDim.x) row_max_all[i] = 0u;
+  for (int i = tid; i < p.teams * 3 * R; i += blockDim.x) {
+    row_max_all[i] = 0u;
+    if (ASYM) row_max_all[p.teams * 3 * R + i] = 0xFFFFFFFFu;
+  }
   if (tid == 0) {
     prefetch_tensormap(&p.tmap_x);
     prefetch_tensormap(&p.tmap_codes);
@@ -97,7 +142,10 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_ke
     const int s = it & 1;
     const uint32_t phase = (it >> 1) & 1;
     const int buf = it % 3;
-    if (tt < R) row_max[((it + 1) % 3) * R + tt] = 0u;
+    if (tt < R) {
+      row_max[((it + 1) % 3) * R + tt] = 0u;
+      if (ASYM) row_min[((it + 1) % 3) * R + tt] = 0xFFFFFFFFu;
+    }
 
     w.wait(bar_full + 8 * s, phase);
     if (it == 0 && tt == 0 && tile + stride < num_tiles) {  // the team's second tile, into the other stage
@@ -107,8 +155,21 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_ke
     float2 v[64];
     load_scaled_block(team_base + s * in_bytes, box_bytes, b, r, sv4, v);
     wht128_thread(v);
-    const float m = absmax_thread(v);
-    if (active) atomicMax(&row_max[buf * R + r], __float_as_uint(m));
+    if (ASYM) {
+      float hi = v[0].x, lo = v[0].x;
+#pragma unroll
+      for (int q = 0; q < 64; ++q) {
+        hi = max3(hi, v[q].x, v[q].y);
+        lo = min3(lo, v[q].x, v[q].y);
+      }
+      if (active) {
+        atomicMax(&row_max[buf * R + r], float_order_key(hi));
+        atomicMin(&row_min[buf * R + r], float_order_key(lo));
+      }
+    } else {
+      const float m = absmax_thread(v);
+      if (active) atomicMax(&row_max[buf * R + r], __float_as_uint(m));
+    }
     if (tt == 0) bulk_wait_group_read<0>();  // the previous tile's store has finished reading the staging tile
     team_barrier(team, team_threads);        // row maxima complete; every thread of the team has read stage s
 
@@ -120,12 +181,30 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_ke
       }
     }
 
-    const float amax = __uint_as_float(row_max[buf * R + r]);
-    const float inv = amax > 0.0f ? __fdiv_rn(127.0f, amax) : 0.0f;
-    if (active) {
-      quantize_store_block(v, inv, p.zero, out_base + b * box_bytes + r * 128);
-      const int64_t row = static_cast<int64_t>(tile) * R + r;
-      if (b == 0 && row < p.M) p.scales[row] = __fdiv_rn(amax, 127.0f);
+    const int64_t row = static_cast<int64_t>(tile) * R + r;
+    const uint32_t out_row = out_base + b * box_bytes + r * 128;
+    if (ASYM) {
+      const float vmax = float_from_order_key(row_max[buf * R + r]);
+      const float vmin = float_from_order_key(row_min[buf * R + r]);
+      const float range = __fsub_rn(vmax, vmin);
+      const float inv = range > 0.0f ? __fdiv_rn(255.0f, range) : 0.0f;
+      const int z = -__float2int_rn(__fmul_rn(vmin, inv));
+      // false also where infinities or NaN took part (a NaN input makes the block's sum v[0].x one)
+      const bool small = fmaxf(fabsf(vmax), fabsf(vmin)) * inv < 4194303.0f && v[0].x == v[0].x;
+      if (active) {
+        quantize_store_block_asym(v, inv, z, small, p.zero, out_row);
+        if (b == 0 && row < p.M) {
+          p.scales[row] = __fdiv_rn(range, 255.0f);
+          p.zero_points[row] = z;
+        }
+      }
+    } else {
+      const float amax = __uint_as_float(row_max[buf * R + r]);
+      const float inv = amax > 0.0f ? __fdiv_rn(127.0f, amax) : 0.0f;
+      if (active) {
+        quantize_store_block(v, inv, p.zero, out_row);
+        if (b == 0 && row < p.M) p.scales[row] = __fdiv_rn(amax, 127.0f);
+      }
     }
     fence_proxy_async_smem();
     team_barrier(team, team_threads);
@@ -147,7 +226,7 @@ struct TeamShape {
 size_t team_smem_bytes(int K, int R, int teams) {
   const int nb = K / TRDQ_BLOCK;
   return 128 + static_cast<size_t>(teams) * 5 * R * K + static_cast<size_t>(nb) * (TRDQ_BLOCK + kVecPadFloats) * 4 +
-         (static_cast<size_t>(teams) * 3 * R + 2) * 4 + static_cast<size_t>(teams) * 16 + 16;
+         (static_cast<size_t>(teams) * 6 * R + 2) * 4 + static_cast<size_t>(teams) * 16 + 16;
 }
 
 // The team of `tw` warps for rows of K channels: as many whole rows as its lanes hold, as many teams as registers
@@ -203,8 +282,15 @@ bool rotate_quantize_prefers_team(int32_t M, int32_t K) {
   return (static_cast<int64_t>(M) + s.R - 1) / s.R >= sms;
 }
 
-trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, int8_t* codes,
-                                        float* scales, cudaStream_t stream) {
+// Asymmetric codes: the second reduction over the block (minimum beside maximum) and its exchange make a team's tile longer, so
+// the lane-group kernel keeps the smaller problems.  Microseconds, lane groups / teams: K = 1152 at M = 2048 3.3 / 4.2, 8192 10.7 / 11.3,
+// 16384 20.1 / 18.6, 32768 39.4 / 31.9; K = 2304 at 4096 11.9 / 11.5; K = 4608 at 2048 11.9 / 11.4, 4096 20.1 / 19.1, 8192 39.3 / 33.1.
+bool rotate_quantize_asym_prefers_team(int32_t M, int32_t K) {
+  return static_cast<int64_t>(M) * K >= (K >= 2048 ? 9ll << 20 : 18ll << 20) && rotate_quantize_prefers_team(M, K);
+}
+
+trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, void* codes,
+                                        float* scales, int32_t* zero_points, cudaStream_t stream) {
   int dev = 0;
   const int sms = device_sm_count(&dev);
   if (sms <= 0) return TRDQ_ERR_CUDA;
@@ -220,6 +306,7 @@ trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t
   if (st != TRDQ_OK) return st;
   p.vec = vec;
   p.scales = scales;
+  p.zero_points = zero_points;
   p.M = M;
   p.K = K;
   p.R = shape.R;
@@ -230,13 +317,14 @@ trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t
   if (!p.status) return TRDQ_ERR_CUDA;
   static PerDeviceFlag configured;
   if (!configured.get(dev)) {
-    if (cudaFuncSetAttribute(rotate_quantize_team_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
+    if (cudaFuncSetAttribute(rotate_quantize_team_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+        cudaFuncSetAttribute(rotate_quantize_team_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
       return TRDQ_ERR_CUDA;
     configured.set(dev, true);
   }
   const int num_tiles = (M + shape.R - 1) / shape.R;
   const int grid = num_tiles < sms ? num_tiles : sms;  // few tiles: spread them over the SMs, fewer busy teams on each
-  const cudaError_t e = launch_overlapped(rotate_quantize_team_kernel, dim3(grid), dim3(shape.teams * shape.team_warps * 32), shape.smem,
+  const cudaError_t e = launch_overlapped(zero_points ? rotate_quantize_team_kernel<true> : rotate_quantize_team_kernel<false>, dim3(grid), dim3(shape.teams * shape.team_warps * 32), shape.smem,
                                           stream, p);
   return e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA;
 }
