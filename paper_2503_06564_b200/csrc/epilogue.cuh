@@ -25,17 +25,11 @@ __device__ __forceinline__ float dequant_one(int32_t a, float sxm, float swn, fl
 // GELU in its tanh form, the activation between the two MLP linears of a DiT block, two values at a time:
 //   gelu(x) = 0.5 x (1 + tanh(u)) = x / (1 + exp(-2u)) = x exp(2u) / (1 + exp(2u)),   u = sqrt(2/pi) (x + 0.044715 x^3).
 // With e = exp(-|2u|) in [0, 1] the denominator d = 1 + e stays in [1, 2] on both sides, so nothing overflows and the
-// flush-to-zero forms of 2^x and 1 / x are in their defined range; they need no scaling around the special-function
-// instruction, which the forms that keep subnormals carry for every value.  Relative error near 1e-6, far inside a bf16
-// rounding step; results below about 1e-37 in magnitude (x < -10) flush to zero.
-// Over all 2^32 arguments the results equal those of the forms that keep subnormals (__expf and __fdividef), but for x in
-// -10.7 .. -10.0, where those give subnormal numbers and these zero.
-// 1152 -> 4608 with GELU at M = 4096: 30.3 us with a scalar form and the column-by-column epilogue, 25.8 with dequant_row32,
-// 23.9 with these (18.6 without GELU).  One reciprocal shared by four quotients was measured as well: one bf16 result in 10^5
-// then rounds the other way, and repairing exactly those costs more than is gained.
-__device__ __forceinline__ float exp2_ftz(float x) {
+// flush-to-zero form of 1 / x is in its defined range.  2^x keeps subnormal results: e is one from x = -10.0 down, and x e then
+// still is a number that bf16 holds (to x = -10.6).
+__device__ __forceinline__ float exp2_approx(float x) {
   float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 __device__ __forceinline__ float rcp_ftz(float x) {
@@ -48,7 +42,7 @@ __device__ __forceinline__ float2 gelu_tanh2(float2 x) {
   const float log2e = 1.4426950408889634f;
   const float2 t = __fmul2_rn(x, __ffma2_rn(__fmul2_rn(x, x), make_float2(0.044715f * k, 0.044715f * k), make_float2(k, k)));  // 2u, sign of x
   const float2 t2 = __fmul2_rn(t, make_float2(log2e, log2e));
-  const float2 e = make_float2(exp2_ftz(-fabsf(t2.x)), exp2_ftz(-fabsf(t2.y)));
+  const float2 e = make_float2(exp2_approx(-fabsf(t2.x)), exp2_approx(-fabsf(t2.y)));
   const float2 m = __fmul2_rn(x, e);
   const float2 d = __fadd2_rn(e, make_float2(1.0f, 1.0f));
   return __fmul2_rn(make_float2(t.x >= 0.0f ? x.x : m.x, t.y >= 0.0f ? x.y : m.y), make_float2(rcp_ftz(d.x), rcp_ftz(d.y)));

@@ -52,3 +52,25 @@ def test_special_values_stay_in_their_column(M, wbits):
     special = [1, 37, 70]
     assert np.all(np.isnan(got[:, [1, 37]])) and np.all(got[:, 70] == np.inf)
     assert np.array_equal(np.delete(got, special, axis=1), np.delete(clean, special, axis=1))
+
+
+@pytest.mark.parametrize("M,wbits", [(3, 8), (2304, 8), (3, 4)])  # one CTA per tile, CTA pairs, 4-bit weights
+def test_gelu_of_every_bf16_value(M, wbits):
+    """With zero weights the pre-activation is the bias, so one layer of 65536 columns meets every finite bf16 value, the ones whose
+    GELU is near the bottom of the float range among them.  fp32: the exponent of 2 (up to 150) has passed five
+    roundings, so the power is off by 150 * 5 * 2^-24 * ln 2 < 2^-14; then the rounding to bf16, 2^-8, and half its smallest
+    subnormal, 2^-134."""
+    from paper_2503_06564_b200 import trdq
+    K = 128
+    bits = np.arange(65536, dtype=np.uint32).astype(np.uint16)
+    bits[~np.isfinite(WL.bf16_bits_to_f32(bits))] = 0
+    v = WL.bf16_bits_to_f32(bits).astype(np.float64)
+    rot = trdq.Rotation(K, [0, 1000], np.ones((1, K), np.int8), None)
+    wts = trdq.trdq_prepare_weights(rot, to_dev_bf16(np.zeros((65536, K), np.uint16)), wbits)
+    codes, scales = trdq.trdq_rotate_quantize(rot, 0, to_dev_bf16(WL.to_bf16_bits(np.random.default_rng(1).standard_normal((M, K)))))
+    got = trdq.trdq_linear_act(wts, 0, codes, scales, to_dev_bf16(bits))
+    with np.errstate(over="ignore"):
+        want = v / (1.0 + np.exp(-2.0 * np.sqrt(2.0 / np.pi) * (v + 0.044715 * v ** 3)))
+    for row in (0, M - 1):
+        err = np.abs(bf16_to_f32_np(got[row]).astype(np.float64) - want)
+        assert np.all(err <= (2.0 ** -8 + 2.0 ** -14) * np.abs(want) + 1.01 * 2.0 ** -134)
