@@ -9,17 +9,17 @@ namespace trdq {
 // One output: y = acc * sx * sw + bias in fp32.  fp32 is accurate to 2^-23 of the product; only when
 // product and bias cancel below `thr` = 2^-10 |bias| can that exceed a bf16 rounding step of the result;
 // then the scale product is carried as an exact two-term sum and the part of the accumulator that
-// fp32 could not hold is added back.
-__device__ __forceinline__ float dequant_one(int32_t a, float sxm, float swn, float biasn, float thr) {
+// fp32 could not hold is added back (to v, the value without these two parts).
+__device__ __forceinline__ float repair_cancellation(int32_t a, float sxm, float swn, float v) {
   const float af = static_cast<float>(a);
   const float s_hi = __fmul_rn(sxm, swn);
-  float v = __fmaf_rn(af, s_hi, biasn);
-  if (fabsf(v) < thr) {
-    const float s_lo = __fmaf_rn(sxm, swn, -s_hi);
-    v = __fmaf_rn(af, s_lo, v);
-    v = __fmaf_rn(static_cast<float>(a - __float2int_rz(af)), s_hi, v);
-  }
-  return v;
+  const float s_lo = __fmaf_rn(sxm, swn, -s_hi);
+  v = __fmaf_rn(af, s_lo, v);
+  return __fmaf_rn(static_cast<float>(a - __float2int_rz(af)), s_hi, v);
+}
+__device__ __forceinline__ float dequant_one(int32_t a, float sxm, float swn, float biasn, float thr) {
+  const float v = __fmaf_rn(static_cast<float>(a), __fmul_rn(sxm, swn), biasn);
+  return fabsf(v) < thr ? repair_cancellation(a, sxm, swn, v) : v;
 }
 
 // GELU in its tanh form, the activation between the two MLP linears of a DiT block, two values at a time:
@@ -60,32 +60,34 @@ __device__ __forceinline__ float min3_abs(float a, float b, float c) {
   return r;
 }
 
-// Epilogue parameters of a tile in shared memory: per column the weight scale and the bias, per chunk of 32 columns the
-// largest cancellation threshold 2^-10 |bias| of the chunk.
+// Epilogue parameters of a tile in shared memory: per column the weight scale and the bias, per eight columns the
+// largest cancellation threshold 2^-10 |bias| among them.
 struct ColumnParams {
   const float* sw;
   const float* bias;
   const float* thr;
 };
 template <int BN>
-struct ColumnParamLayout {  // [sw BN][bias BN][thr BN / 32], 16-byte aligned
-  static constexpr int kFloats = 2 * BN + (BN / 32 + 3) / 4 * 4;
+struct ColumnParamLayout {  // [sw BN][bias BN][thr BN / 8], 16-byte aligned
+  static constexpr int kFloats = 2 * BN + BN / 8;
   static constexpr int kBytes = kFloats * 4;
 };
 
 // 32 consecutive columns (chunk c of the tile) of one output row: y = acc * sx * sw[n] + bias[n] (then GELU if ACT),
 // packed to bf16 pairs.  Packed fp32x2 arithmetic, the same roundings as dequant_one; the cancellation against the bias is
-// looked for once per row and chunk (smallest |y| against the chunk's largest threshold) and repaired column by column
-// only where it may have happened.  Per column: one conversion, 2.5 instructions of arithmetic and half a 16-byte
-// shared-memory read, against about 6 and 0.75 when every column is tested by itself: the 8-bit GEMM at M = 4096,
-// 1152 -> 3456 / 4608 / 1152 went from 16.2 / 19.1 / 9.2 to 14.9 / 17.9 / 8.7 us, at M = 16384, 1152 -> 3456 from 62 to 54 us.
+// looked for once per row and eight columns (smallest |y| against the largest threshold of the eight).  Where it may have
+// happened the eight are held against their own thresholds, and only those below are repaired: with a bias of the output's size a
+// value in 10^3 is below the largest threshold, so in a warp of 32 rows every third or fourth group of eight columns, but hardly one below its own.
+// Microseconds of the GEMM with each column tested by itself / one test per 32 columns that repairs all of them / this, for a bias
+// of a hundredth of the output's size and one of twice its size: M = 4096, 1152 -> 4608 19.1 / 17.1 / 17.4 and 19.1 / 20.7 / 18.4, M = 16384,
+// 1152 -> 3456 54.7 / 52.7 / 51.7 and 54.5 / 59.4 / 52.9.  One test per four columns costs more than it saves (17.3 and 19.8).
 template <bool ACT = false>
 __device__ __forceinline__ void dequant_row32(const uint32_t (&r)[32], float sxm, const ColumnParams& cp, int c, uint32_t (&packed)[16]) {
   const float4* sw4 = reinterpret_cast<const float4*>(cp.sw + c * 32);
   const float4* b4 = reinterpret_cast<const float4*>(cp.bias + c * 32);
   const float2 sx2 = make_float2(sxm, sxm);
   float2 v[16];
-  float lowest = __uint_as_float(0x7F800000u);
+  float low[4];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const float4 s = sw4[j], b = b4[j];
@@ -93,18 +95,28 @@ __device__ __forceinline__ void dequant_row32(const uint32_t (&r)[32], float sxm
     const float2 a1 = make_float2(static_cast<float>(static_cast<int32_t>(r[4 * j + 2])), static_cast<float>(static_cast<int32_t>(r[4 * j + 3])));
     v[2 * j] = __ffma2_rn(a0, __fmul2_rn(sx2, make_float2(s.x, s.y)), make_float2(b.x, b.y));
     v[2 * j + 1] = __ffma2_rn(a1, __fmul2_rn(sx2, make_float2(s.z, s.w)), make_float2(b.z, b.w));
-    lowest = min3_abs(lowest, v[2 * j].x, v[2 * j].y);
-    lowest = min3_abs(lowest, v[2 * j + 1].x, v[2 * j + 1].y);
+    low[j / 2] = min3_abs(j & 1 ? low[j / 2] : __uint_as_float(0x7F800000u), v[2 * j].x, v[2 * j].y);
+    low[j / 2] = min3_abs(low[j / 2], v[2 * j + 1].x, v[2 * j + 1].y);
   }
-  if (!(lowest >= cp.thr[c])) {  // also when a NaN bias made the threshold one
+  const float4 thr = *reinterpret_cast<const float4*>(cp.thr + c * 4);
+  // not "low < thr": also when a NaN bias made the threshold one
+  const bool cancels[4] = {!(low[0] >= thr.x), !(low[1] >= thr.y), !(low[2] >= thr.z), !(low[3] >= thr.w)};
+  if (cancels[0] || cancels[1] || cancels[2] || cancels[3]) {
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const float bn = cp.bias[c * 32 + j];
-      const float y = dequant_one(static_cast<int32_t>(r[j]), sxm, cp.sw[c * 32 + j], bn, fabsf(bn) * 0.0009765625f);
-      if (j & 1)
-        v[j / 2].y = y;
-      else
-        v[j / 2].x = y;
+    for (int g = 0; g < 4; ++g) {
+      if (!cancels[g]) continue;
+      const float4 b0 = b4[2 * g], b1 = b4[2 * g + 1];
+      const float bn[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      bool own = false;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) own |= fabsf(e & 1 ? v[4 * g + e / 2].y : v[4 * g + e / 2].x) < fabsf(bn[e]) * 0.0009765625f;
+      if (!own) continue;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int j = 8 * g + e;
+        float& y = j & 1 ? v[j / 2].y : v[j / 2].x;
+        if (fabsf(y) < fabsf(bn[e]) * 0.0009765625f) y = repair_cancellation(static_cast<int32_t>(r[j]), sxm, cp.sw[c * 32 + j], y);
+      }
     }
   }
 #pragma unroll
@@ -112,22 +124,27 @@ __device__ __forceinline__ void dequant_row32(const uint32_t (&r)[32], float sxm
 }
 
 // Stages the epilogue parameters of BN columns starting at n0 (see ColumnParamLayout).  Called by whole warps with
-// consecutive tid from 0 to nthreads - 1, nthreads a multiple of 32: a warp holds whole chunks.
+// consecutive tid from 0 to nthreads - 1, nthreads a multiple of 32: a warp holds whole groups of eight columns.
+// Columns from N on (their outputs are clipped by the store) get an infinite bias and no threshold: with zeros their outputs would be 0
+// and every row of a chunk that N ends in would look like a cancellation.
 template <int BN>
 __device__ __forceinline__ ColumnParams stage_column_params(float* dst, const float* sw, const __nv_bfloat16* bias, int n0, int N, int tid,
                                                             int nthreads) {
   for (int c = tid; c < BN; c += nthreads) {
     const int n = n0 + c;
-    float s = 0.0f, b = 0.0f;
+    float s = 0.0f, b = __uint_as_float(0x7F800000u);
+    unsigned int top = 0u;
     if (n < N) {
       s = __ldg(sw + n);
       b = bias ? __bfloat162float(bias[n]) : 0.0f;
+      // non-negative floats order like their bit patterns (a NaN bias gives a NaN threshold)
+      top = __float_as_uint(fabsf(b) * 0.0009765625f);
     }
     dst[c] = s;
     dst[BN + c] = b;
-    // non-negative floats order like their bit patterns (a NaN bias gives a NaN threshold)
-    const unsigned int top = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(b) * 0.0009765625f));
-    if ((c & 31) == 0) dst[2 * BN + c / 32] = __uint_as_float(top);
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, d));
+    if ((c & 7) == 0) dst[2 * BN + c / 8] = __uint_as_float(top);
   }
   return ColumnParams{dst, dst + BN, dst + 2 * BN};
 }
