@@ -50,8 +50,24 @@ __device__ __forceinline__ float min3(float a, float b, float c) {
 // Unsigned codes of the thread's block (Eq. 1-3): code = min(rne(fl(v * inv)) + z, 255); the lower clamp of Eq. 1 can never bind
 // (rounding is monotone and z cancels the minimum's own code).  fl(v * inv) + 1.5 * 2^23 leaves the rounded product in the low
 // mantissa bits; adding z and the clamp are exact there as long as |v * inv| < 2^22, which `small` says for the whole row.
+// Other rows (a range so narrow or so wide that 255 / range or the products leave the integers, NaN) take the integer form of the
+// lane-group kernel word for word: which of the two kernels a call runs depends on M and may not show in its codes.
 __device__ __forceinline__ void quantize_store_block_asym(const float2 (&v)[64], float inv, int z, bool small, float zero, uint32_t out_row) {
   const uint32_t oswz = (out_row >> 7) & 7u;
+  if (!small) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      uint32_t wd[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int q0 = min(__float2int_rn(__fmul_rn(v[c * 8 + i].x, inv)) + z, 255);
+        const int q1 = min(__float2int_rn(__fmul_rn(v[c * 8 + i].y, inv)) + z, 255);
+        wd[i / 2] |= (static_cast<uint32_t>(q0) | (static_cast<uint32_t>(q1) << 8)) << (16 * (i & 1));
+      }
+      st_shared_v4(out_row + ((c ^ oswz) << 4), wd[0], wd[1], wd[2], wd[3]);
+    }
+    return;
+  }
   const float2 inv2 = make_float2(inv, inv), magic2 = make_float2(kRoundMagic, kRoundMagic), zero2 = make_float2(zero, zero);
   const float zf = static_cast<float>(z);
   const float2 z2 = make_float2(zf, zf);
@@ -61,14 +77,8 @@ __device__ __forceinline__ void quantize_store_block_asym(const float2 (&v)[64],
     float2 q[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const float2 y = __ffma2_rn(v[c * 8 + i], inv2, zero2);
-      if (small) {
-        const float2 u = __fadd2_rn(__fadd2_rn(y, magic2), z2);
-        q[i] = make_float2(fminf(u.x, top), fminf(u.y, top));
-      } else {
-        q[i] = make_float2(__uint_as_float(static_cast<uint32_t>(min(__float2int_rn(y.x) + z, 255))),
-                           __uint_as_float(static_cast<uint32_t>(min(__float2int_rn(y.y) + z, 255))));
-      }
+      const float2 u = __fadd2_rn(__fadd2_rn(__ffma2_rn(v[c * 8 + i], inv2, zero2), magic2), z2);
+      q[i] = make_float2(fminf(u.x, top), fminf(u.y, top));
     }
     st_shared_v4(out_row + ((c ^ oswz) << 4), pack4(q[0], q[1]), pack4(q[2], q[3]), pack4(q[4], q[5]), pack4(q[6], q[7]));
   }

@@ -59,3 +59,30 @@ def test_linear_matches_oracle(M, N, K):
     y_ref = O.linear_asym_rows(c_ref, s_ref, z_ref, qw, sw, bias, np.arange(M))
     assert check_output(bf16_to_f32_np(y), y_ref)[1] <= 1.0
     assert trdq.trdq_device_status() == 0
+
+
+@pytest.mark.parametrize("M,K,part", [(16400, 1152, 4100), (2100, 4608, 700)])
+def test_special_rows_do_not_depend_on_the_row_count(M, K, part):
+    """Rows of infinities, NaN, overflowing sums and ranges so narrow that 255 / range overflows: the call over all rows (team kernel)
+    gives what calls over a part of them (lane-group kernel) give."""
+    import torch
+    from paper_2503_06564_b200 import trdq
+    rng = np.random.default_rng(K)
+    x = rng.standard_normal((M, K)) * 3.0
+    at = rng.permutation(M)[:16]
+    x[at[0], 3] = x[at[1], K - 1] = np.nan
+    x[at[2], 5], x[at[3], 5] = np.inf, -np.inf
+    x[at[4], 1:3] = np.inf
+    x[at[5], 1], x[at[5], 2] = np.inf, -np.inf
+    x[at[6]], x[at[7], 0] = 3e38, 3.3e38
+    x[at[8:12]] = 0.0
+    x[at[8]], x[at[9], K - 1], x[at[10], 130] = 1e-39, 1e-38, 2e-36
+    x[at[12:]] *= np.float64(2.0) ** np.array([-100, -126, -60, 100])[:, None]
+    xd = torch.from_numpy(x).cuda().to(torch.bfloat16)
+    rot = trdq.Rotation(K, [0, 1000], (rng.integers(0, 2, (1, K)) * 2 - 1).astype(np.int8), None)
+    whole = trdq.trdq_rotate_quantize_asym(rot, 0, xd)
+    parts = [trdq.trdq_rotate_quantize_asym(rot, 0, xd[i:i + part]) for i in range(0, M, part)]
+    for got, want in zip(whole, zip(*parts)):
+        assert torch.equal(got.view(torch.int32 if got.element_size() == 4 else torch.uint8),
+                           torch.cat(want).view(torch.int32 if got.element_size() == 4 else torch.uint8))
+    assert trdq.trdq_device_status() == 0
