@@ -83,6 +83,7 @@ cudaError_t launch_rotate_quantize(const void* x_bf16, int64_t ldx, int32_t M, i
 cudaError_t launch_rotate_quantize_groups(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, int groups, int mode,
                                           void* codes, float* scales, cudaStream_t stream);
 
+int rotate2_lane_group_rows(int32_t K);  // rows of a CTA of the four-lanes-per-block kernel (K <= 72 * 128), two CTAs per SM
 cudaError_t launch_rotate2_quantize(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec1, const int32_t* perm,
                                     const float* vec2, int mode, void* codes, float* scales, cudaStream_t stream);
 

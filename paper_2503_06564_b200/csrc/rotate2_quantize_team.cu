@@ -11,7 +11,8 @@
 // buffer is swizzled (16-byte chunk index xor block) and rows are 48 bytes apart modulo 128, so that the writes of a
 // quarter warp and the three rows of one channel fall into different banks.
 // One input stage (the next tile is requested as soon as this one is in registers, most of a tile's time before its use)
-// and codes staged in the row buffer after the last gather leave room for ten teams at K = 1152 and two at K = 4608.
+// and codes staged in the row buffer after the last gather leave room for 30 rows in flight at K = 1152 (three teams of ten) and six at
+// K = 4608 (two teams of three).
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -199,15 +200,29 @@ bool choose_team2_shape(int K, Team2Shape* out) {
 }  // namespace
 
 // The team kernel serves rows that keep at least 0.45 of the lanes of twelve warps busy (K = 7680: 72 -> 64 us at M = 4096;
-// K = 8192, 0.33 of the lanes: 75 against 84 us) once there is a tile per SM.  Below that the lane-group kernel, whose CTAs
-// are smaller and start sooner, finishes first (M = 256, K = 1152: 5.0 against 5.6 us; M = 448: 5.9 against 5.6).
-// M = 4096, K = 1152 / 4608: 14.2 / 44.3 -> 10.0 / 35.0 us; M = 16384: 43.8 / 166 -> 28.7 / 115 us.
+// K = 8192, 0.33 of the lanes: 75 against 84 us), from the row count on at which it stays ahead of the lane-group kernel.  With fewer
+// rows both take one pass and the shorter one wins: a thread of this kernel transforms a whole block twice and gathers 128
+// values, of that kernel a quarter of one.  So the line is drawn in rounds of that kernel, the rows its two CTAs per SM take
+// at once, over M in steps of 12 % from one row per SM to 24 million values:
+//   one block per row 0.94 rounds (K = 128: 5.6 / 6.3 us at M = 8024, lane groups / teams, 7.4 / 6.4 at 8987);
+//   rows of up to ten blocks 0.54 (the second CTA of an SM starts to count; K = 1024: 6.3 / 7.2 at M = 1306, 7.7 / 7.2 at 1463);
+//   rows of up to 36 blocks 1.1 (K = 2048: 6.9 / 8.0 at M = 1166, 9.2 / 8.1 at 1306);
+//   wider rows, one per lane-group CTA, 1.6 (K = 6144: 12.2 / 12.8 at M = 417, 12.9 / 12.7 at 468);
+//   and where a team's tile is a single row, eleven rows per SM (K = 4096: 12.4 / 14.0 at M = 1166, 17.4 / 14.8 at 1639;
+//   K = 7680: 22.1 / 24.2 at M = 1166, 31.5 / 29.3 at 1639).
+// Two of 958 points end up slower than the lane groups, by 2 %.  M = 4096, K = 1152 / 4608: 14.1 / 42.5 -> 9.0 / 33.3 us;
+// M = 16384: 42.6 / 166 -> 28.2 / 115 us.
 bool rotate2_prefers_team(int32_t M, int32_t K) {
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   Team2Shape s;
-  return choose_team2_shape(K, &s) && s.use >= 0.45 && (M + s.R - 1) / s.R >= sms;
+  if (!choose_team2_shape(K, &s) || s.use < 0.45 || (static_cast<int64_t>(M) + s.R - 1) / s.R < sms) return false;
+  if (s.R == 1) return M >= 11 * sms;
+  const int nb = K / TRDQ_BLOCK;
+  const int64_t round = 2ll * sms * rotate2_lane_group_rows(K);
+  const int percent = nb == 1 ? 94 : nb <= 10 ? 54 : nb <= 36 ? 110 : 160;
+  return static_cast<int64_t>(M) * 100 >= round * percent;
 }
 
 trdq_status launch_rotate2_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec1, const int32_t* perm,

@@ -579,6 +579,8 @@ cudaError_t launch_rotate_quantize_asym(const void* x_bf16, int64_t ldx, int32_t
 }
 
 // Full transform.  Rows of up to 128 blocks (K <= 16384); cudaErrorInvalidValue beyond that.
+int rotate2_lane_group_rows(int32_t K) { return min(32, 72 / (K / TRDQ_BLOCK)); }
+
 cudaError_t launch_rotate2_quantize(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec1, const int32_t* perm,
                                     const float* vec2, int mode, void* codes, float* scales, cudaStream_t stream) {
   if (M == 0) return cudaSuccess;
@@ -590,8 +592,7 @@ cudaError_t launch_rotate2_quantize(const void* x_bf16, int64_t ldx, int32_t M, 
                : cudaErrorUnknown;
   if (mode == 0 && nb <= 72) {
     // four lanes per block, packed arithmetic: about 72 lane groups per CTA, two CTAs per SM
-    int rows2 = 72 / nb;
-    if (rows2 > 32) rows2 = 32;
+    const int rows2 = rotate2_lane_group_rows(K);
     int threads2 = rows2 * nb * kFastLanes;
     threads2 = (threads2 + 31) / 32 * 32;
     const size_t smem2 = (static_cast<size_t>(K) + static_cast<size_t>(rows2) * K) * sizeof(float);
