@@ -353,19 +353,30 @@ int choose_tile_n(int64_t tiles_m, int N, int sms) {
 
 }  // namespace
 
-// Whether the CTA-pair kernel (two SMs per 256-row tile, a third less operand traffic per SM) runs M rows against [N, K] weights:
-// from 2048 rows, once the output is large enough that its fewer, larger tiles fill the SMs.  Microseconds, pair / single CTA:
-// 1152 -> 1152 at M = 2048 6.5 / 5.5, 3072 7.5 / 6.6, 4096 8.8 / 8.2; 1152 -> 3456 at 2048 9.8 / 9.4, 3072 12.5 / 12.6; 1152 -> 4608 at 2048
-// 11.3 / 11.3; 384 -> 384 at 4096 4.8 / 4.2.  With a long reduction the operand traffic counts earlier: 4608 -> 1152 at 2048 11.1 / 10.6,
-// 3072 13.6 / 13.5, 4096 18.3 / 19.3.  TRDQ_PAIR_MIN_M (read once per process) replaces the rule by a row count.
-static bool use_pair(int64_t M, int32_t K, int32_t N) {
+// Whether the CTA-pair kernel (two SMs per 256-row tile, a third less operand traffic per SM) runs M rows against [N, K] weights: from
+// 2048 rows, once the output holds enough tiles of 256 x 256 values.  Below that its fewer, larger tiles leave SMs idle; the
+// longer the reduction, the earlier the operand traffic outweighs that, and from K = 7168 on it always does.  Both kernels were
+// timed at nineteen K from 128 to 12288, eleven N from 128 to 4608 and M from 2048 to 32768 (1065 points, plain, GELU and asymmetric
+// epilogue).  Microseconds, pair / single CTA, at N x M: K = 128: 8.2 / 7.8 at 2304 x 4096 (144 tiles), 10.1 / 11.1 at 4608 x 2560 (180);
+// K = 1152: 10.1 / 9.4 at 3456 x 2048 (108), 10.8 / 11.2 at 3072 x 2560 (120);  K = 2304: 11.2 / 10.3 at 2304 x 2048 (72), 12.5 / 13.2 at
+// 2048 x 2560 (80);  K = 4608: 13.8 / 12.9 at 1152 x 3072 (54), 16.1 / 16.7 at 1536 x 2560 (60), 18.5 / 19.5 at 256 x 12288 (48);
+// K = 12288: 21.9 / 26.9 at 768 x 2560 (30).  The asymmetric correction and GELU make the epilogue longer and change over later at
+// short reductions.  Averaged over the points the rule is 0.1 % off the faster kernel, the pair kernel everywhere 4.6 %, the
+// other 3.4 %.  TRDQ_PAIR_MIN_M (read once per process) replaces the rule by a row count.
+static int pair_least_tiles(int32_t K, int32_t N, bool gelu, bool asym) {
+  if (K >= 7168) return 0;
+  if (K >= 6144) return 40;
+  if (K >= 4096) return N <= 256 ? 46 : 56;
+  if (K >= 1536) return gelu && K < 2304 ? 110 : 78;
+  return K < (asym ? 1280 : 1024) ? 165 : 110;
+}
+static bool use_pair(int64_t M, int32_t K, int32_t N, bool gelu, bool asym) {
   static const int forced = [] {
     const char* e = getenv("TRDQ_PAIR_MIN_M");
     return e ? atoi(e) : -1;
   }();
   if (forced >= 0) return M >= forced;
-  const int64_t least = (K >= 2304 ? 64 : 110) * 65536ll;  // output values: tiles of 256 x 256
-  return M >= 2048 && M * N >= least;
+  return M >= 2048 && M * N >= pair_least_tiles(K, N, gelu, asym) * 65536ll;
 }
 
 // Name of the kernel trdq_linear runs for M rows against [N, K] weights of `wbits` bits (one row segment).
@@ -374,7 +385,7 @@ void describe_gemm_kernel(int32_t M, int32_t K, int32_t N, int32_t wbits, char* 
     snprintf(name, cap, "gemm_w4a8_kernel");
     return;
   }
-  if (use_pair(M, K, N)) {
+  if (use_pair(M, K, N, false, false)) {
     const int bn = gemm_w8_pair_tile_width((static_cast<int64_t>(M) + 2 * kTileM - 1) / (2 * kTileM), N);
     if (bn > 0) {
       snprintf(name, cap, "gemm_w8a8_pair_kernel<%d>", bn);
@@ -389,7 +400,7 @@ void describe_gemm_kernel(int32_t M, int32_t K, int32_t N, int32_t wbits, char* 
 static trdq_status launch_gemm_w8_mode(const trdq_weights* w, int g, const GemmSegment seg[2], const void* bias_bf16, int mode,
                                        const int32_t* const zp[2], cudaStream_t stream, int act = 0) {
   const bool raw_i32 = mode == 1;
-  if (mode != 1 && use_pair(static_cast<int64_t>(seg[0].M) + seg[1].M, w->K, w->N)) {
+  if (mode != 1 && use_pair(static_cast<int64_t>(seg[0].M) + seg[1].M, w->K, w->N, act != 0, mode == 2)) {
     const trdq_status st = launch_gemm_w8_pair(w, g, seg, mode == 2 ? zp : nullptr, bias_bf16, stream, act);
     if (st != TRDQ_ERR_SHAPE) return st;
   }

@@ -20,7 +20,7 @@ def _layer(N, K, wbits, seed):
     return rot, trdq.trdq_prepare_weights(rot, to_dev_bf16(w), wbits), act, O.prepare_w8(w, wv) if wbits == 8 else O.prepare_w4(w, wv), rng
 
 
-@pytest.mark.parametrize("M,N", [(40, 16), (40, 208), (4700, 1552), (4700, 1584)])  # one CTA per tile, then CTA pairs
+@pytest.mark.parametrize("M,N", [(40, 16), (40, 208), (7100, 1552), (7100, 1584)])  # one CTA per tile, then CTA pairs
 def test_bias_larger_than_the_product(M, N):
     from paper_2503_06564_b200 import trdq
     K = 256
@@ -36,7 +36,7 @@ def test_bias_larger_than_the_product(M, N):
     check_output(bf16_to_f32_np(y), O.linear_w8_rows(q_ref, sx_ref, qw, sw, bits, np.arange(M)))
 
 
-@pytest.mark.parametrize("M,wbits", [(40, 8), (46000, 8), (70, 4)])
+@pytest.mark.parametrize("M,wbits", [(40, 8), (68000, 8), (70, 4)])  # one CTA per tile, CTA pairs, 4-bit weights
 def test_special_values_stay_in_their_column(M, wbits):
     """GELU and the cancellation test work on several columns at once: a NaN or an infinite bias may not show in the others."""
     from paper_2503_06564_b200 import trdq

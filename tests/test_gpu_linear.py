@@ -99,8 +99,11 @@ def test_int32_accumulators_extreme_codes():
     (200, 1152, 4608, True),
     (1, 16, 128, True),
     (77, 1040, 256, True),
-    (2304, 1152, 1152, True),    # enough rows for the CTA-pair kernel: nine 256-row tiles
-    (2100, 1040, 256, False),    # pair kernel, ragged: the last pair's second CTA has no valid row; N not a tile multiple
+    (2304, 1152, 1152, True),    # too small an output for CTA pairs
+    (2100, 1040, 256, False),
+    (6400, 1152, 1152, True),    # the CTA-pair kernel: 25 tiles of 256 rows
+    (10500, 1040, 256, False),   # pair kernel, ragged: the last pair's second CTA has no valid row; N not a tile multiple
+    (2100, 144, 7168, True),     # pair kernel: a reduction for which it runs outputs of any size
 ])
 def test_linear_matches_oracle(M, N, K, with_bias):
     import torch
@@ -174,15 +177,15 @@ def test_linear_strided_output_and_cfg_segments():
     assert empty[0].shape[0] == 0 and torch.equal(empty[1], y)
     # M == 0
     assert trdq.trdq_linear(wts, t, codes[:0], scales[:0], bias_d).shape == (0, N)
-    # the same through the CTA-pair kernel (>= 2048 rows in total): two segments of 1300 and 1100 rows
-    xl = _acts(2400, K, 8)
+    # the same through the CTA-pair kernel (chosen by the rows of both segments): two segments of 3500 and 2900 rows
+    xl = _acts(6400, K, 8)
     cl, sl = trdq.trdq_rotate_quantize(rot, t, to_dev_bf16(xl))
     yl = trdq.trdq_linear(wts, t, cl, sl, bias_d)
-    hl = trdq.trdq_linear_cfg(wts, t, [cl[:1300].contiguous(), cl[1300:].contiguous()], [sl[:1300].contiguous(), sl[1300:].contiguous()],
+    hl = trdq.trdq_linear_cfg(wts, t, [cl[:3500].contiguous(), cl[3500:].contiguous()], [sl[:3500].contiguous(), sl[3500:].contiguous()],
                               bias_d)
     assert torch.equal(torch.cat(hl), yl)
     act_l, qw_l, sw_l = ref[1]
-    rows = np.concatenate([np.arange(0, 300), np.arange(1200, 1400), np.arange(2300, 2400)])
+    rows = np.concatenate([np.arange(0, 300), np.arange(3400, 3600), np.arange(6300, 6400)])
     q_l, sx_l = O.rotate_quantize(xl, act_l)
     y_l_ref = O.linear_w8_rows(q_l, sx_l, qw_l, sw_l, bias, rows)
     check_output(bf16_to_f32_np(yl)[rows], y_l_ref, max_ulp=1.0)
@@ -252,8 +255,8 @@ def test_linear_w4a8_group_scales_of_very_different_size():
 
 
 def test_small_shapes_through_the_cta_pair_kernel():
-    """The CTA-pair kernel normally serves problems of >= 2048 rows.  Re-run this file's 8-bit cases in a
-    child process with the threshold lowered to one row (the library reads TRDQ_PAIR_MIN_M once), so that
+    """The CTA-pair kernel normally serves larger problems (at least 2048 rows).  Re-run this file's 8-bit cases in a
+    child process with the rule replaced by one row (the library reads TRDQ_PAIR_MIN_M once), so that
     every small and ragged shape above also goes through the pair kernel."""
     import os
     import subprocess
@@ -325,7 +328,7 @@ def test_an_expired_wait_is_reported_and_the_device_stays_usable():
 
 @pytest.mark.parametrize("M,K,N,wbits", [(300, 256, 400, 8), (4096, 1152, 4608, 8), (260, 384, 272, 4)])
 def test_linear_with_gelu_epilogue(M, K, N, wbits):
-    """trdq_linear_act: GELU (tanh form) folded into the epilogue, all three GEMM kernels (M >= 2048 takes the CTA-pair one),
+    """trdq_linear_act: GELU (tanh form) folded into the epilogue, all three GEMM kernels (M = 4096 takes the CTA-pair one),
     against the oracle's double evaluation on the same codes; act = 0 must equal trdq_linear bit for bit."""
     import torch
     from paper_2503_06564_b200 import trdq
@@ -464,7 +467,7 @@ def test_prepare_then_use_on_one_stream_without_synchronisation():
     import torch
     from paper_2503_06564_b200 import trdq
     rng = np.random.default_rng(77)
-    M, K = 2304, 1152                                   # enough rows for the CTA-pair kernel
+    M, K = 6400, 1152                                   # N = 1152 and 3456 go to the CTA-pair kernel, the others to the single-CTA one
     x_bits = _acts(M, K, 78)
     xd = to_dev_bf16(x_bits)
     rows = np.arange(0, M, 53, dtype=np.int64)
