@@ -442,8 +442,16 @@ __global__ void w4_multipliers_kernel(const float* __restrict__ scales, int32_t 
 
 cudaError_t launch_w4_multipliers(const float* scales, int32_t N, int32_t groups, int32_t n_pad, int sets, int32_t* mult_t, float* base,
                                   cudaStream_t stream) {
-  w4_multipliers_kernel<<<dim3((n_pad + 127) / 128, sets), 128, 0, stream>>>(scales, N, groups, n_pad, mult_t, base);
-  return cudaGetLastError();
+  constexpr int kMaxGridY = 65535;
+  for (int first = 0; first < sets; first += kMaxGridY) {
+    const int count = sets - first < kMaxGridY ? sets - first : kMaxGridY;
+    w4_multipliers_kernel<<<dim3((n_pad + 127) / 128, count), 128, 0, stream>>>(
+        scales + static_cast<int64_t>(first) * N * groups, N, groups, n_pad, mult_t + static_cast<int64_t>(first) * groups * n_pad,
+        base + static_cast<int64_t>(first) * n_pad);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 trdq_status launch_gemm_w4(const trdq_weights* w, int g, const GemmSegment seg[2], const void* bias_bf16, cudaStream_t stream, int act) {
