@@ -87,7 +87,15 @@ int rotate2_lane_group_rows(int32_t K);  // rows of a CTA of the four-lanes-per-
 cudaError_t launch_rotate2_quantize(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec1, const int32_t* perm,
                                     const float* vec2, int mode, void* codes, float* scales, cudaStream_t stream);
 
+// How a team kernel cuts its CTA: teams of `team_warps` warps, each on tiles of R whole rows.
+struct TeamShape {
+  int R, team_warps, teams;
+  size_t smem;
+  double use;  // fraction of the twelve warps' lanes that hold a block
+};
+
 // rotate_quantize_team.cu: per-row int8 path, TMA-staged, one thread per block, independent teams of warps per CTA
+bool rotate_quantize_team_shape(int M, int K, int sms, bool asym, TeamShape* out);  // false: rows too wide for two teams
 bool rotate_quantize_prefers_team(int32_t M, int32_t K);
 bool rotate_quantize_asym_prefers_team(int32_t M, int32_t K);
 // zero_points == nullptr: symmetric int8 codes; otherwise unsigned codes with a zero point per row (Eq. 1-3)

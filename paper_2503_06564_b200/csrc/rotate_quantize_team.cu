@@ -227,49 +227,27 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_ke
   w.settle();
 }
 
-struct TeamShape {
-  int R, team_warps, teams;
-  size_t smem;
-  double use;  // fraction of the twelve warps' lanes that hold a block
-};
-
-size_t team_smem_bytes(int K, int R, int teams) {
+// One row-exchange table (three buffers of the row maxima), in the asymmetric form two (the minima as well): charging both to the
+// symmetric form would cost it a team at K = 128, eleven against ten.
+size_t team_smem_bytes(int K, int R, int teams, bool asym) {
   const int nb = K / TRDQ_BLOCK;
   return 128 + static_cast<size_t>(teams) * 5 * R * K + static_cast<size_t>(nb) * (TRDQ_BLOCK + kVecPadFloats) * 4 +
-         (static_cast<size_t>(teams) * 6 * R + 2) * 4 + static_cast<size_t>(teams) * 16 + 16;
+         (static_cast<size_t>(teams) * (asym ? 6 : 3) * R + 2) * 4 + static_cast<size_t>(teams) * 16 + 16;
 }
 
 // The team of `tw` warps for rows of K channels: as many whole rows as its lanes hold, as many teams as registers
 // (twelve warps) and shared memory (two input stages and a code tile per team) allow.  At least two teams, so that one
 // can transform while another waits.
-bool team_shape_for(int K, int tw, TeamShape* out) {
+bool team_shape_for(int K, int tw, bool asym, TeamShape* out) {
   const int nb = K / TRDQ_BLOCK;
   int rows = tw * 32 / nb;
   if (rows < 1) return false;
   if (rows > 32) rows = 32;
   int teams = kTeamMaxWarps / tw;
-  while (teams > 0 && team_smem_bytes(K, rows, teams) > 227u * 1024u) --teams;
+  while (teams > 0 && team_smem_bytes(K, rows, teams, asym) > 227u * 1024u) --teams;
   if (teams < 2) return false;
-  *out = TeamShape{rows, tw, teams, team_smem_bytes(K, rows, teams),
+  *out = TeamShape{rows, tw, teams, team_smem_bytes(K, rows, teams, asym),
                    static_cast<double>(rows) * nb / (tw * 32) * (static_cast<double>(teams * tw) / kTeamMaxWarps)};
-  return true;
-}
-
-// Team size by lane use (K = 1152: one warp, 3 rows, 27 of 32 lanes, twelve teams; K = 4608: four warps, 3 rows, 108 of
-// 128 lanes, three teams).  With fewer than about one tile per team the next larger team is taken when the best one
-// is a single warp: fewer, fatter tiles finish sooner when nothing is left to overlap (K = 1152, M = 4096: 6.2 against
-// 6.7 us, measured).
-bool choose_team_shape(int M, int K, int sms, TeamShape* out) {
-  TeamShape best = {0, 0, 0, 0, 0.0};
-  for (int tw = 1; tw <= kTeamMaxWarps / 2; ++tw) {
-    TeamShape s;
-    if (team_shape_for(K, tw, &s) && s.use > best.use + 1e-9) best = s;
-  }
-  if (best.teams == 0) return false;
-  const int64_t tiles = (static_cast<int64_t>(M) + best.R - 1) / best.R;
-  TeamShape wider;
-  if (best.team_warps == 1 && 4 * tiles < 5ll * best.teams * sms && team_shape_for(K, 2, &wider)) best = wider;
-  *out = best;
   return true;
 }
 
@@ -283,20 +261,39 @@ int device_sm_count(int* dev_out) {
 
 }  // namespace
 
+// Team size by lane use (K = 1152: one warp, 3 rows, 27 of 32 lanes, twelve teams; K = 4608: four warps, 3 rows, 108 of
+// 128 lanes, three teams).  With fewer than about one tile per team the next larger team is taken when the best one
+// is a single warp: fewer, fatter tiles finish sooner when nothing is left to overlap (K = 1152, M = 4096: 6.2 against
+// 6.7 us, measured).
+bool rotate_quantize_team_shape(int M, int K, int sms, bool asym, TeamShape* out) {
+  TeamShape best = {0, 0, 0, 0, 0.0};
+  for (int tw = 1; tw <= kTeamMaxWarps / 2; ++tw) {
+    TeamShape s;
+    if (team_shape_for(K, tw, asym, &s) && s.use > best.use + 1e-9) best = s;
+  }
+  if (best.teams == 0) return false;
+  const int64_t tiles = (static_cast<int64_t>(M) + best.R - 1) / best.R;
+  TeamShape wider;
+  if (best.team_warps == 1 && 4 * tiles < 5ll * best.teams * sms && team_shape_for(K, 2, asym, &wider)) best = wider;
+  *out = best;
+  return true;
+}
+
 // The team kernel serves rows for which at least two teams fit in shared memory, once there is at least a tile per SM; below
 // that the lane-group kernel, whose CTAs are smaller and start sooner, finishes first (M = 256, K = 1024: 2.3 against 3.3 us).
-bool rotate_quantize_prefers_team(int32_t M, int32_t K) {
+static bool a_tile_per_sm(int32_t M, int32_t K, bool asym) {
   const int sms = device_sm_count(nullptr);
   TeamShape s;
-  if (sms <= 0 || !choose_team_shape(M, K, sms, &s)) return false;
+  if (sms <= 0 || !rotate_quantize_team_shape(M, K, sms, asym, &s)) return false;
   return (static_cast<int64_t>(M) + s.R - 1) / s.R >= sms;
 }
+bool rotate_quantize_prefers_team(int32_t M, int32_t K) { return a_tile_per_sm(M, K, false); }
 
 // Asymmetric codes: the second reduction over the block (minimum beside maximum) and its exchange make a team's tile longer, so
 // the lane-group kernel keeps the smaller problems.  Microseconds, lane groups / teams: K = 1152 at M = 2048 3.3 / 4.2, 8192 10.7 / 11.3,
 // 16384 20.1 / 18.6, 32768 39.4 / 31.9; K = 2304 at 4096 11.9 / 11.5; K = 4608 at 2048 11.9 / 11.4, 4096 20.1 / 19.1, 8192 39.3 / 33.1.
 bool rotate_quantize_asym_prefers_team(int32_t M, int32_t K) {
-  return static_cast<int64_t>(M) * K >= (K >= 2048 ? 9ll << 20 : 18ll << 20) && rotate_quantize_prefers_team(M, K);
+  return static_cast<int64_t>(M) * K >= (K >= 2048 ? 9ll << 20 : 18ll << 20) && a_tile_per_sm(M, K, true);
 }
 
 trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, void* codes,
@@ -305,7 +302,7 @@ trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t
   const int sms = device_sm_count(&dev);
   if (sms <= 0) return TRDQ_ERR_CUDA;
   TeamShape shape;
-  if (!choose_team_shape(M, K, sms, &shape)) return TRDQ_ERR_SHAPE;
+  if (!rotate_quantize_team_shape(M, K, sms, zero_points != nullptr, &shape)) return TRDQ_ERR_SHAPE;
   const int nb = K / TRDQ_BLOCK;
   TeamParams p;
   trdq_status st = encode_tmap_boxes(&p.tmap_x, x_bf16, 2, 64, static_cast<uint64_t>(M), static_cast<uint64_t>(ldx) * 2,
