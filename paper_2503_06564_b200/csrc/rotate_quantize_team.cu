@@ -290,10 +290,15 @@ static bool a_tile_per_sm(int32_t M, int32_t K, bool asym) {
 bool rotate_quantize_prefers_team(int32_t M, int32_t K) { return a_tile_per_sm(M, K, false); }
 
 // Asymmetric codes: the second reduction over the block (minimum beside maximum) and its exchange make a team's tile longer, so
-// the lane-group kernel keeps the smaller problems.  Microseconds, lane groups / teams: K = 1152 at M = 2048 3.3 / 4.2, 8192 10.7 / 11.3,
-// 16384 20.1 / 18.6, 32768 39.4 / 31.9; K = 2304 at 4096 11.9 / 11.5; K = 4608 at 2048 11.9 / 11.4, 4096 20.1 / 19.1, 8192 39.3 / 33.1.
+// the lane-group kernel keeps the smaller problems; and rows of more than 48 blocks, one or two to a team, need more of them still.
+// Microseconds, lane groups / teams: K = 1152 at M = 2048 3.3 / 4.2, 8192 10.7 / 11.3, 16384 20.1 / 18.6, 32768 39.4 / 31.9;
+// K = 2304 at 4096 11.9 / 11.5; K = 4608 at 2048 11.9 / 11.4, 4096 20.1 / 19.1, 8192 39.3 / 33.1; K = 6912 at 1639 13.5 / 14.2,
+// 2304 17.5 / 18.2, 2891 21.5 / 20.3; K = 9216 at 1480 14.8 / 15.7, 2800 27.8 / 26.7;
+// K = 9728 0.98 of the lane groups' speed from 2000 to 5000 rows and level at 12288, so from there on they keep every size.
 bool rotate_quantize_asym_prefers_team(int32_t M, int32_t K) {
-  return static_cast<int64_t>(M) * K >= (K >= 2048 ? 9ll << 20 : 18ll << 20) && a_tile_per_sm(M, K, true);
+  if (K > 9216) return false;
+  const int64_t least = K > 8192 ? 28ll << 20 : K > 6144 ? 16ll << 20 : K >= 2048 ? 9ll << 20 : 18ll << 20;
+  return static_cast<int64_t>(M) * K >= least && a_tile_per_sm(M, K, true);
 }
 
 trdq_status launch_rotate_quantize_team(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, void* codes,

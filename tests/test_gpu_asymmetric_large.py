@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
     (16400, 1152, 8),    # one-warp teams, three tiles each, a last tile of two rows; rows with a stride
     (2100, 4608, 0),     # four-warp teams
     (4100, 2304, 16),
-    (1030, 9216, 0),
+    (1030, 9216, 0),     # below the rule, wide rows
+    (3300, 9216, 0),     # three-warp teams of one row
     (147500, 128, 0),    # one block per row
     (8000, 1152, 0),     # below the rule: the lane-group kernel
 ])
@@ -36,6 +37,16 @@ def test_codes_match_oracle(M, K, pad):
     assert np.array_equal(zp.cpu().numpy(), z_ref)
     assert np.array_equal(codes.cpu().numpy(), c_ref)
     assert trdq.trdq_device_status() == 0
+
+
+@pytest.mark.parametrize("K,first", [(128, 147456), (1152, 16384), (2048, 4608), (4608, 2048), (6144, 1536), (6912, 2428), (8192, 2048), (9216, 3186)])
+def test_dispatch_line(K, first):
+    """From this row count on the team kernel is ahead (figures at the rule)."""
+    import ctypes
+    from paper_2503_06564_b200 import trdq
+    prefers = getattr(trdq.lib(), "_ZN4trdq33rotate_quantize_asym_prefers_teamEii")
+    prefers.restype, prefers.argtypes = ctypes.c_bool, [ctypes.c_int32, ctypes.c_int32]
+    assert prefers(first, K) and not prefers(first - 1, K)
 
 
 @pytest.mark.parametrize("M,N,K", [
