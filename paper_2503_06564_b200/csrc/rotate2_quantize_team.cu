@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate2_quantize_team_k
     mbar_init(bar_full, 1);
     fence_mbar_init();
   }
-  stage_vector(svec1, p.vec1, p.K, tid, blockDim.x);
+  stage_vector(svec1, p.vec1, p.K);
   for (int j = tid; j < p.K; j += blockDim.x) {
     const int c = __ldg(p.perm + j);
     svec2[(c >> 7) * (TRDQ_BLOCK + kVecPadFloats) + (c & 127)] = __ldg(p.vec2 + j);

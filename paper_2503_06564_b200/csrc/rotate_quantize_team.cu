@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate_quantize_team_ke
     mbar_init(bar_full + 8, 1);
     fence_mbar_init();
   }
-  stage_vector(svec, p.vec, p.K, tid, blockDim.x);
+  stage_vector(svec, p.vec, p.K);
   for (int i = tid; i < p.teams * 3 * R; i += blockDim.x) {
     row_max_all[i] = 0u;
     if (ASYM) row_max_all[p.teams * 3 * R + i] = 0xFFFFFFFFu;
