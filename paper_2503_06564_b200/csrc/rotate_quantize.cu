@@ -245,15 +245,18 @@ __global__ void __launch_bounds__(1024) rotate2_quantize_kernel(const __nv_bfloa
 // Rounding to the integer code uses the exact identity rne(y) = (y + 1.5 * 2^23) - 1.5 * 2^23 for
 // |y| < 2^22: after the addition the low byte of the fp32 pattern is the two's-complement code.
 // ---------------------------------------------------------------------------------------------
-template <int MIN_CTAS>
+// GROUPS: weight preparation, all time-step groups in one launch, blockIdx.y the group.  (A form of its own: the three offsets
+// cost the activation call 0.1 us of 2 to 3.)
+template <int MIN_CTAS, bool GROUPS>
 __global__ void __launch_bounds__(320, MIN_CTAS)
 rotate_quantize_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t ldx, int32_t M, int32_t K, const float* __restrict__ vec,
                             int8_t* __restrict__ codes, float* __restrict__ scales, int32_t rows_per_tile, float zero) {
   extern __shared__ float svec[];  // the group's fused vector, K floats
-  // weight preparation runs all time-step groups in one launch: blockIdx.y is the group
-  vec += static_cast<int64_t>(blockIdx.y) * K;
-  codes += static_cast<int64_t>(blockIdx.y) * M * K;
-  scales += static_cast<int64_t>(blockIdx.y) * M;
+  if (GROUPS) {
+    vec += static_cast<int64_t>(blockIdx.y) * K;
+    codes += static_cast<int64_t>(blockIdx.y) * M * K;
+    scales += static_cast<int64_t>(blockIdx.y) * M;
+  }
   __shared__ unsigned int row_max[3][32];
   const int nb = K / TRDQ_BLOCK;
   const int lane4 = threadIdx.x & (kFastLanes - 1);
@@ -520,8 +523,8 @@ cudaError_t launch_rows_fast(const void* x, int64_t ldx, int32_t M, int32_t K, c
   const int num_tiles = (M + rows - 1) / rows;
   const int grid = min(num_tiles, sms * 2);
   const size_t smem = static_cast<size_t>(K) * sizeof(float);
-  return launch_overlapped(rotate_quantize_rows_kernel<2>, dim3(grid, groups), dim3(threads), smem, stream, static_cast<const __nv_bfloat16*>(x),
-                           ldx, M, K, vec, static_cast<int8_t*>(codes), scales, rows, 0.0f);
+  return launch_overlapped(groups > 1 ? rotate_quantize_rows_kernel<2, true> : rotate_quantize_rows_kernel<2, false>, dim3(grid, groups),
+                           dim3(threads), smem, stream, static_cast<const __nv_bfloat16*>(x), ldx, M, K, vec, static_cast<int8_t*>(codes), scales, rows, 0.0f);
 }
 
 template <int MODE, int P>
