@@ -206,11 +206,12 @@ bool choose_team2_shape(int K, Team2Shape* out) {
 // at once, over M in steps of 12 % from one row per SM to 24 million values:
 //   one block per row 0.94 rounds (K = 128: 5.6 / 6.3 us at M = 8024, lane groups / teams, 7.4 / 6.4 at 8987);
 //   rows of up to ten blocks 0.54 (the second CTA of an SM starts to count; K = 1024: 6.3 / 7.2 at M = 1306, 7.7 / 7.2 at 1463);
-//   rows of up to 36 blocks 1.1 (K = 2048: 6.9 / 8.0 at M = 1166, 9.2 / 8.1 at 1306);
+//   rows of up to 24 blocks 1.1 (K = 2048: 6.9 / 8.0 at M = 1166, 9.2 / 8.1 at 1306), up to 36 blocks 1.3 (K = 4608: 10.4 / 10.5 at
+//   M = 740, 13.8 / 10.9 at 829);
 //   wider rows, one per lane-group CTA, 1.6 (K = 6144: 12.2 / 12.8 at M = 417, 12.9 / 12.7 at 468);
 //   and where a team's tile is a single row, eleven rows per SM (K = 4096: 12.4 / 14.0 at M = 1166, 17.4 / 14.8 at 1639;
 //   K = 7680: 22.1 / 24.2 at M = 1166, 31.5 / 29.3 at 1639).
-// Two of 958 points end up slower than the lane groups, by 2 %.  M = 4096, K = 1152 / 4608: 14.1 / 42.5 -> 9.0 / 33.3 us;
+// One of 958 points ends up slower than the lane groups, by 2 %; K = 6144 at M = 1480 = 5 x 296, where their last round is full, by 10 %.  M = 4096, K = 1152 / 4608: 14.1 / 42.5 -> 9.0 / 33.3 us;
 // M = 16384: 42.6 / 166 -> 28.2 / 115 us.
 bool rotate2_prefers_team(int32_t M, int32_t K) {
   int dev = 0, sms = 148;
@@ -221,7 +222,7 @@ bool rotate2_prefers_team(int32_t M, int32_t K) {
   if (s.R == 1) return M >= 11 * sms;
   const int nb = K / TRDQ_BLOCK;
   const int64_t round = 2ll * sms * rotate2_lane_group_rows(K);
-  const int percent = nb == 1 ? 94 : nb <= 10 ? 54 : nb <= 36 ? 110 : 160;
+  const int percent = nb == 1 ? 94 : nb <= 10 ? 54 : nb <= 24 ? 110 : nb <= 36 ? 130 : 160;
   return static_cast<int64_t>(M) * 100 >= round * percent;
 }
 

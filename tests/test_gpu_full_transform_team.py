@@ -21,7 +21,7 @@ def _prefers_team(M, K):
 
 @pytest.mark.parametrize("K,last,first", [    # rows: still the lane-group kernel, already the team kernel
     (128, 8903, 8904), (384, 4704, 4705), (1024, 1438, 1439), (1152, 1470, 1471), (1536, 1953, 1954), (2048, 1302, 1303), (4096, 1627, 1628),
-    (4608, 651, 652), (6144, 473, 474), (7680, 1627, 1628), (8192, 100000, None),
+    (4608, 769, 770), (6144, 473, 474), (7680, 1627, 1628), (8192, 100000, None),
 ])
 def test_dispatch_line(K, last, first):
     """Where the rule says the team kernel is ahead, on the 148 SMs it was measured on (figures at the rule)."""
@@ -50,7 +50,7 @@ def test_three_tiles_per_team(K):
     (2001, 1280, 8),    # fewer than a tile per SM: still the lane-group kernel
     (2101, 1280, 8),    # the team kernel: five-warp teams of fourteen rows, a last tile of one row
     (321, 4608, 0),
-    (700, 4608, 0),     # four-warp teams of three rows
+    (800, 4608, 0),     # four-warp teams of three rows
     (150, 6144, 24),
     (475, 6144, 24),    # three-warp teams of two rows, the last one alone
     (149, 7680, 0),
