@@ -27,6 +27,9 @@ __device__ __forceinline__ float dequant_one(int32_t a, float sxm, float swn, fl
 // With e = exp(-|2u|) in [0, 1] the denominator d = 1 + e stays in [1, 2] on both sides, so nothing overflows and the
 // flush-to-zero form of 1 / x is in its defined range.  2^x keeps subnormal results: e is one from x = -10.0 down, and x e then
 // still is a number that bf16 holds (to x = -10.6).
+// 1152 -> 4608 with GELU at M = 4096: 29.8 us in scalar form with the epilogue column by column, 25.1 now (17.4 without GELU); the form of
+// 2^x that flushes subnormals would give 23.4.  Testing a chunk's 32 values for x < -9.75 and flushing otherwise gains 0.5 % of that
+// back; one reciprocal shared by four quotients moves one bf16 result in 10^5, and repairing those costs more than is gained.
 __device__ __forceinline__ float exp2_approx(float x) {
   float r;
   asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
