@@ -42,7 +42,7 @@ struct Cfg {
   static constexpr int kABytes = kTileM * kTileKBytes;
   static constexpr int kBBytes = BN * kTileKBytes;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  // parameters staged for the epilogue: (sw, bias) and the cancellation threshold per column, one
+  // parameters staged for the epilogue: scale and bias per column, the cancellation threshold per eight columns, one
   // buffer per accumulator stage
   static constexpr int kParamBytes = 2 * (ColumnParamLayout<BN>::kBytes + BN * 4);  // two sets: column parameters and (asymmetric mode) weight column sums
   static constexpr int kBarrierBytes = 256;

@@ -6,8 +6,9 @@
 // stores, instead of at each gathered value: the product is the same), and every thread gathers its 128 permuted channels;
 // the table of byte offsets is 16 bits per channel, eight per load.
 //
-// What bounds it: shared memory.  Of about 27 wavefronts per block and row (tile in, vectors, row out, gather, codes) the
-// gather of 128 scalars at arbitrary banks takes 16; 15 instructions per element come to 0.6 of that time.  The row
+// What bounds it (K = 1152, M = 16384): 31.5 shared-memory wavefronts per block and row, 22.5 of them loads (for the most part the
+// gather of 128 scalars at arbitrary banks), 14 of them conflicts, keep that pipe 57 % busy and issue slots 37 %: between the two lies the chain
+// load - transform - barrier - gather - transform - maximum of a team, of which nine warps hold three.  The row
 // buffer is swizzled (16-byte chunk index xor block) and rows are 48 bytes apart modulo 128, so that the writes of a
 // quarter warp and the three rows of one channel fall into different banks.
 // One input stage (the next tile is requested as soon as this one is in registers, most of a tile's time before its use)
