@@ -27,8 +27,8 @@ __device__ __forceinline__ float dequant_one(int32_t a, float sxm, float swn, fl
 // With e = exp(-|2u|) in [0, 1] the denominator d = 1 + e stays in [1, 2] on both sides, so nothing overflows and the
 // flush-to-zero form of 1 / x is in its defined range.  2^x keeps subnormal results: e is one from x = -10.0 down, and x e then
 // still is a number that bf16 holds (to x = -10.6).
-// 1152 -> 4608 with GELU at M = 4096: 29.8 us in scalar form with the epilogue column by column, 25.1 now (17.4 without GELU); the form of
-// 2^x that flushes subnormals would give 23.4.  Testing a chunk's 32 values for x < -9.75 and flushing otherwise gains 0.5 % of that
+// 1152 -> 4608 with GELU at M = 4096: 29.8 us in scalar form with the epilogue column by column, 22.8 now (18.4 without GELU); the form of
+// 2^x that flushes subnormals gave 23.4 where this one gave 25.1.  Testing a chunk's 32 values for x < -9.75 and flushing otherwise gains 0.5 % of that
 // back; one reciprocal shared by four quotients moves one bf16 result in 10^5, and repairing those costs more than is gained.
 __device__ __forceinline__ float exp2_approx(float x) {
   float r;
@@ -76,7 +76,7 @@ struct ColumnParamLayout {  // [sw BN][bias BN][thr BN / 8], 16-byte aligned
   static constexpr int kBytes = kFloats * 4;
 };
 
-// 32 consecutive columns (chunk c of the tile) of one output row: y = acc * sx * sw[n] + bias[n] (then GELU if ACT),
+// COLS (16 or 32) consecutive columns (the c-th such group of the tile) of one output row: y = acc * sx * sw[n] + bias[n] (then GELU if ACT),
 // packed to bf16 pairs.  Packed fp32x2 arithmetic, the same roundings as dequant_one; the cancellation against the bias is
 // looked for once per row and eight columns (smallest |y| against the largest threshold of the eight).  Where it may have
 // happened the eight are held against their own thresholds, and only those below are repaired: with a bias of the output's size a
@@ -84,15 +84,16 @@ struct ColumnParamLayout {  // [sw BN][bias BN][thr BN / 8], 16-byte aligned
 // Microseconds of the GEMM with each column tested by itself / one test per 32 columns that repairs all of them / this, for a bias
 // of a hundredth of the output's size and one of twice its size: M = 4096, 1152 -> 4608 19.1 / 17.1 / 17.4 and 19.1 / 20.7 / 18.4, M = 16384,
 // 1152 -> 3456 54.7 / 52.7 / 51.7 and 54.5 / 59.4 / 52.9.  One test per four columns costs more than it saves (17.3 and 19.8).
-template <bool ACT = false>
-__device__ __forceinline__ void dequant_row32(const uint32_t (&r)[32], float sxm, const ColumnParams& cp, int c, uint32_t (&packed)[16]) {
-  const float4* sw4 = reinterpret_cast<const float4*>(cp.sw + c * 32);
-  const float4* b4 = reinterpret_cast<const float4*>(cp.bias + c * 32);
+template <int COLS, bool ACT>
+__device__ __forceinline__ void dequant_row(const uint32_t (&r)[COLS], float sxm, const ColumnParams& cp, int c, uint32_t (&packed)[COLS / 2]) {
+  static_assert(COLS == 16 || COLS == 32, "two or four tests");
+  const float4* sw4 = reinterpret_cast<const float4*>(cp.sw + c * COLS);
+  const float4* b4 = reinterpret_cast<const float4*>(cp.bias + c * COLS);
   const float2 sx2 = make_float2(sxm, sxm);
-  float2 v[16];
+  float2 v[COLS / 2];
   float low[4];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
+  for (int j = 0; j < COLS / 4; ++j) {
     const float4 s = sw4[j], b = b4[j];
     const float2 a0 = make_float2(static_cast<float>(static_cast<int32_t>(r[4 * j])), static_cast<float>(static_cast<int32_t>(r[4 * j + 1])));
     const float2 a1 = make_float2(static_cast<float>(static_cast<int32_t>(r[4 * j + 2])), static_cast<float>(static_cast<int32_t>(r[4 * j + 3])));
@@ -101,12 +102,18 @@ __device__ __forceinline__ void dequant_row32(const uint32_t (&r)[32], float sxm
     low[j / 2] = min3_abs(j & 1 ? low[j / 2] : __uint_as_float(0x7F800000u), v[2 * j].x, v[2 * j].y);
     low[j / 2] = min3_abs(low[j / 2], v[2 * j + 1].x, v[2 * j + 1].y);
   }
-  const float4 thr = *reinterpret_cast<const float4*>(cp.thr + c * 4);
+  float4 thr;
+  if constexpr (COLS == 32) {
+    thr = *reinterpret_cast<const float4*>(cp.thr + c * 4);
+  } else {
+    const float2 two = *reinterpret_cast<const float2*>(cp.thr + c * 2);
+    thr = make_float4(two.x, two.y, 0.0f, 0.0f);
+  }
   // not "low < thr": also when a NaN bias made the threshold one
-  const bool cancels[4] = {!(low[0] >= thr.x), !(low[1] >= thr.y), !(low[2] >= thr.z), !(low[3] >= thr.w)};
+  const bool cancels[4] = {!(low[0] >= thr.x), !(low[1] >= thr.y), COLS == 32 && !(low[2] >= thr.z), COLS == 32 && !(low[3] >= thr.w)};
   if (cancels[0] || cancels[1] || cancels[2] || cancels[3]) {
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
+    for (int g = 0; g < COLS / 8; ++g) {
       if (!cancels[g]) continue;
       const float4 b0 = b4[2 * g], b1 = b4[2 * g + 1];
       const float bn[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
@@ -118,37 +125,95 @@ __device__ __forceinline__ void dequant_row32(const uint32_t (&r)[32], float sxm
       for (int e = 0; e < 8; ++e) {
         const int j = 8 * g + e;
         float& y = j & 1 ? v[j / 2].y : v[j / 2].x;
-        if (fabsf(y) < fabsf(bn[e]) * 0.0009765625f) y = repair_cancellation(static_cast<int32_t>(r[j]), sxm, cp.sw[c * 32 + j], y);
+        if (fabsf(y) < fabsf(bn[e]) * 0.0009765625f) y = repair_cancellation(static_cast<int32_t>(r[j]), sxm, cp.sw[c * COLS + j], y);
       }
     }
   }
 #pragma unroll
-  for (int j = 0; j < 16; ++j) packed[j] = pack_bf16(ACT ? gelu_tanh2(v[j]) : v[j]);
+  for (int j = 0; j < COLS / 2; ++j) packed[j] = pack_bf16(ACT ? gelu_tanh2(v[j]) : v[j]);
 }
 
-// Stages the epilogue parameters of BN columns starting at n0 (see ColumnParamLayout).  Called by whole warps with
-// consecutive tid from 0 to nthreads - 1, nthreads a multiple of 32: a warp holds whole groups of eight columns.
+// Staging of the epilogue parameters of BN columns (see ColumnParamLayout): the scale and bias of column n, then their place c in the
+// tile's table.  store_column_param is called by whole warps with consecutive c: a warp holds whole groups of eight columns.
 // Columns from N on (their outputs are clipped by the store) get an infinite bias and no threshold: with zeros their outputs would be 0
 // and every row of a chunk that N ends in would look like a cancellation.
+struct ColumnParam {  // scale and bias of one column
+  float s, b;
+};
+__device__ __forceinline__ ColumnParam load_column_param(const float* sw, const __nv_bfloat16* bias, int n, int N) {
+  ColumnParam c{0.0f, __uint_as_float(0x7F800000u)};
+  if (n < N) {
+    c.s = __ldg(sw + n);
+    c.b = bias ? __bfloat162float(bias[n]) : 0.0f;
+  }
+  return c;
+}
+template <int BN>
+__device__ __forceinline__ void store_column_param(float* dst, const ColumnParam& v, bool inside, int c) {
+  // non-negative floats order like their bit patterns (a NaN bias gives a NaN threshold)
+  unsigned int top = inside ? __float_as_uint(fabsf(v.b) * 0.0009765625f) : 0u;
+  dst[c] = v.s;
+  dst[BN + c] = v.b;
+#pragma unroll
+  for (int d = 1; d < 8; d <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, d));
+  if ((c & 7) == 0) dst[2 * BN + c / 8] = __uint_as_float(top);
+}
+
+// The parameters of a tile of 128 rows and BN columns: [columns (ColumnParamLayout)][weight column sums BN][row scales 128][zero points 128].
+constexpr int kParamRows = 128;
+template <int BN>
+struct TileParams {
+  static constexpr int kBytes = ColumnParamLayout<BN>::kBytes + BN * 4 + 2 * kParamRows * 4;
+  ColumnParams columns;
+  int32_t* colsum;
+  float* sx;
+  int32_t* zp;
+  __device__ __forceinline__ explicit TileParams(uint8_t* base) {
+    float* const f = reinterpret_cast<float*>(base);
+    columns = ColumnParams{f, f + BN, f + 2 * BN};
+    colsum = reinterpret_cast<int32_t*>(f + ColumnParamLayout<BN>::kFloats);
+    sx = reinterpret_cast<float*>(colsum + BN);
+    zp = reinterpret_cast<int32_t*>(sx + kParamRows);
+  }
+};
+// Called by two whole warps, st = 0 .. 63; `wait_free` returns once the set may be overwritten, the loads are in flight meanwhile.
+template <int BN, bool ASYM, typename Wait>
+__device__ __forceinline__ void stage_tile_params(uint8_t* set, const float* sw, const __nv_bfloat16* bias, const int32_t* colsum, int n0, int N,
+                                                  const float* sx, const int32_t* zp, int m0, int M, int st, Wait&& wait_free) {
+  ColumnParam col[BN / 64];
+  int32_t csum[BN / 64], zr[kParamRows / 64];
+  float sxr[kParamRows / 64];
+#pragma unroll
+  for (int i = 0; i < BN / 64; ++i) {
+    const int n = n0 + 64 * i + st;
+    col[i] = load_column_param(sw, bias, n, N);
+    if (ASYM) csum[i] = n < N ? __ldg(colsum + n) : 0;
+  }
+#pragma unroll
+  for (int i = 0; i < kParamRows / 64; ++i) {
+    const int row = m0 + 64 * i + st;
+    sxr[i] = row < M ? __ldg(sx + row) : 0.0f;
+    if (ASYM) zr[i] = row < M ? __ldg(zp + row) : 0;
+  }
+  wait_free();
+  const TileParams<BN> t(set);
+#pragma unroll
+  for (int i = 0; i < BN / 64; ++i) {
+    store_column_param<BN>(reinterpret_cast<float*>(set), col[i], n0 + 64 * i + st < N, 64 * i + st);
+    if (ASYM) t.colsum[64 * i + st] = csum[i];
+  }
+#pragma unroll
+  for (int i = 0; i < kParamRows / 64; ++i) {
+    t.sx[64 * i + st] = sxr[i];
+    if (ASYM) t.zp[64 * i + st] = zr[i];
+  }
+}
+
+// The columns of a tile that starts at column n0, by the threads tid = 0 .. nthreads - 1, nthreads a multiple of 32.
 template <int BN>
 __device__ __forceinline__ ColumnParams stage_column_params(float* dst, const float* sw, const __nv_bfloat16* bias, int n0, int N, int tid,
                                                             int nthreads) {
-  for (int c = tid; c < BN; c += nthreads) {
-    const int n = n0 + c;
-    float s = 0.0f, b = __uint_as_float(0x7F800000u);
-    unsigned int top = 0u;
-    if (n < N) {
-      s = __ldg(sw + n);
-      b = bias ? __bfloat162float(bias[n]) : 0.0f;
-      // non-negative floats order like their bit patterns (a NaN bias gives a NaN threshold)
-      top = __float_as_uint(fabsf(b) * 0.0009765625f);
-    }
-    dst[c] = s;
-    dst[BN + c] = b;
-#pragma unroll
-    for (int d = 1; d < 8; d <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, d));
-    if ((c & 7) == 0) dst[2 * BN + c / 8] = __uint_as_float(top);
-  }
+  for (int c = tid; c < BN; c += nthreads) store_column_param<BN>(dst, load_column_param(sw, bias, n0 + c, N), n0 + c < N, c);
   return ColumnParams{dst, dst + BN, dst + 2 * BN};
 }
 

@@ -12,9 +12,10 @@
 //              complete on it (the copies carry .cta_group::2 so that they may signal the peer CTA)
 //   empty[s]   in each CTA: tcgen05.commit multicast to both CTAs when the MMAs reading stage s are done
 //   tfull[a]   in each CTA: tcgen05.commit multicast when accumulator a is complete
-//   tempty[a]  in the LEADER: the epilogue warps of both CTAs arrive (16 arrivals)
-// The epilogue is the single-CTA kernel's (one row per thread, eight warps per CTA), but stores two 32-column chunks
-// at a time (a 32 x 64 bf16 tile per TMA store: whole 128-byte lines).  No TMA multicast is used.
+//   tempty[a]  in the LEADER: the epilogue warps of both CTAs arrive
+//   pfull[a], pempty[a]  in each CTA: the epilogue parameters of a tile are in shared memory / have been used
+// The epilogue is the single-CTA kernel's (one row per thread), but stores 64 columns at a time (a 32 x 64 bf16 tile per TMA
+// store: whole 128-byte lines).  No TMA multicast is used.
 #include <cuda_bf16.h>
 
 #include <type_traits>
@@ -29,20 +30,39 @@ namespace {
 constexpr int kTileM = 128;       // rows per CTA; the pair covers 256
 constexpr int kTileKBytes = 128;
 constexpr int kUmmaK = 32;
-constexpr int kThreads = 384;
-constexpr int kEpilogueThreads = 256;
 constexpr int kAccStride = 256;
 constexpr int kTmemCols = 512;
 constexpr int kSmemBudget = 227 * 1024;
 
-template <int BN>
+// MODE 0: dequantizing epilogue.  MODE 1: GELU (tanh form) on the dequantized value before the bf16 rounding.
+// MODE 2: unsigned activation codes with zero points (Eq. 1-3), acc - z[m] * colsum[n] in front of the epilogue of mode 0.
+// MODE 3: mode 1 for long reductions (see kWarpPerTile).
+enum PairMode { kPairPlain = 0, kPairGelu = 1, kPairAsym = 2, kPairGeluLong = 3 };
+
+constexpr int kGeluShortK = 1792;  // mode 1 up to this reduction, mode 3 beyond
+
+template <int BN, int MODE>
 struct Cfg2 {
+  // Epilogue warps: eight, each with half of the tile's columns, or (mode 1) one per 32 x 64 piece of the tile: sixteen at BN = 256.
+  // GELU makes the epilogue longer than the main loop of a short reduction (two special-function instructions and some twenty
+  // others a value), and with two warps a scheduler half of the issue slots stay empty.  But the staging tiles of sixteen warps take the
+  // memory of a pipeline stage, which costs long reductions, and launches without GELU, 2 - 10 %.  Microseconds with eight / sixteen
+  // warps at M = 16384, N = 4608: K = 768 85.1 / 69.5, 1152 87.0 / 77.1, 1536 95.3 / 87.5, 1792 101.2 / 97.5, 2048 107.3 / 107.5,
+  // 2304 115.9 / 118.2, 4608 209.1 / 217.8; N = 768: K = 1152 21.9 / 20.2, 1792 24.0 / 24.8, 2304 26.4 / 28.9.
+  static constexpr bool kWarpPerTile = MODE == kPairGelu;
+  static constexpr int kEpilogueWarps = kWarpPerTile ? BN / 16 : 8;
+  static constexpr int kEpilogueThreads = 32 * kEpilogueWarps;
+  static constexpr int kThreads = 128 + kEpilogueThreads;
+  static constexpr bool kOddChunk = (BN / 32 / (kEpilogueWarps / 4)) % 2 != 0;
   static constexpr int kABytes = kTileM * kTileKBytes;
   static constexpr int kBBytes = (BN / 2) * kTileKBytes;  // this CTA's half of the weight tile
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kParamBytes = 2 * (ColumnParamLayout<BN>::kBytes + BN * 4);  // two sets: column parameters and (asymmetric mode) weight column sums
+  // epilogue parameters of a tile, two sets: per column (see ColumnParamLayout) and, in asymmetric mode, the weight column sums;
+  // per row the scale and the zero point
+  static constexpr int kSetBytes = TileParams<BN>::kBytes;
+  static constexpr int kParamBytes = 2 * kSetBytes;
   static constexpr int kBarrierBytes = 256;
-  static constexpr int kOutStageBytes = (kEpilogueThreads / 32) * 4096;  // one 32 x 64 bf16 tile per warp
+  static constexpr int kOutStageBytes = kEpilogueWarps * 4096;  // one 32 x 64 bf16 tile per warp
   static constexpr int kStages = (kSmemBudget - 1024 - kOutStageBytes - kParamBytes - kBarrierBytes) / kStageBytes;
   static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kOutStageBytes + kParamBytes + kBarrierBytes;
   static_assert(kStages >= 3 && kStages <= 10, "stage count out of range");
@@ -150,24 +170,23 @@ __host__ __device__ constexpr uint32_t umma_idesc_s8_pair(int n, bool unsigned_a
   return (2u << 4) | (unsigned_a ? 0u : 1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
 }
 
-// MODE 0: dequantizing epilogue.  MODE 1: GELU (tanh form) on the dequantized value before the bf16 rounding.
-// MODE 2: unsigned activation codes with zero points (Eq. 1-3), acc - z[m] * colsum[n] in front of the epilogue of mode 0.
-enum PairMode { kPairPlain = 0, kPairGelu = 1, kPairAsym = 2 };
 template <int BN, int MODE>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8a8_pair_kernel(const __grid_constant__ Gemm2Params p) {
-  using C = Cfg2<BN>;
-  constexpr bool ACT = MODE == kPairGelu;
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Cfg2<BN, MODE>::kThreads, 1) gemm_w8a8_pair_kernel(const __grid_constant__ Gemm2Params p) {
+  using C = Cfg2<BN, MODE>;
+  constexpr bool ACT = MODE == kPairGelu || MODE == kPairGeluLong;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
   const uint32_t out_stage_base = smem_base + C::kStages * C::kStageBytes;
-  float* param_buf = reinterpret_cast<float*>(smem + C::kStages * C::kStageBytes + C::kOutStageBytes);
+  uint8_t* const param_buf = smem + C::kStages * C::kStageBytes + C::kOutStageBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes + C::kOutStageBytes + C::kParamBytes);
   const uint32_t bar_full = smem_u32(bars);                  // [S]   used in the leader
   const uint32_t bar_empty = bar_full + 8 * C::kStages;      // [S]   each CTA's own
   const uint32_t bar_tfull = bar_empty + 8 * C::kStages;     // [2]   each CTA's own
   const uint32_t bar_tempty = bar_tfull + 16;                // [2]   used in the leader
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * C::kStages + 4);
+  const uint32_t bar_pfull = bar_tempty + 16;                // [2]   each CTA's own: a tile's epilogue parameters are in shared memory
+  const uint32_t bar_pempty = bar_pfull + 16;                // [2]   each CTA's own: the epilogue warps are done with them
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * C::kStages + 8);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -185,7 +204,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(bar_tfull + 8 * a, 1);
-      mbar_init(bar_tempty + 8 * a, 2 * (kEpilogueThreads / 32));  // epilogue warps of both CTAs
+      mbar_init(bar_tempty + 8 * a, 2 * C::kEpilogueWarps);  // epilogue warps of both CTAs
+      mbar_init(bar_pfull + 8 * a, 2);                       // the two staging warps
+      mbar_init(bar_pempty + 8 * a, C::kEpilogueWarps);
     }
     fence_mbar_init();
   }
@@ -204,7 +225,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
     prefetch_tensormap(&p.tmap_b);
     prefetch_tensormap(&p.tmap_out[0]);
     prefetch_tensormap(&p.tmap_out[1]);
-    if ((BN / 64) % 2) {
+    if (C::kOddChunk) {
       prefetch_tensormap(&p.tmap_out32[0]);
       prefetch_tensormap(&p.tmap_out32[1]);
     }
@@ -290,13 +311,37 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
       }
       w.settle();
     }
-  } else if (warp >= 4) {
+  } else if (warp < 4) {
+    // ---------------------------------------------------- warps 2, 3: the epilogue parameters of the next tile
+    // An L2 round trip beside the operand traffic takes about a thousand clocks.  When the epilogue warps loaded these themselves at the
+    // head of a tile, every tile waited for it and for a barrier between them.  Two warps that have nothing else to do run a
+    // tile ahead instead; microseconds before -> now: M = 4096, 1152 -> 3456 15.7 -> 14.7 (asymmetric 17.2 -> 15.2), 1152 -> 4608 with GELU
+    // and eight epilogue warps 25.9 -> 24.4; M = 16384, 1152 -> 1152 21.2 -> 19.7 (23.1 -> 20.1), 1152 -> 4608 63.5 -> 62.7.
+    BoundedWaiter w(p.status, kStatusTimeoutEpilogue);
+    const int st = threadIdx.x - 64;
+    int set = 0;
+    uint32_t phase = 0;
+    for (int tile = cluster_id; tile < total_tiles; tile += num_clusters) {
+      const TileCoord tc = pair_tile_coord(p, tile, BN);
+      stage_tile_params<BN, MODE == kPairAsym>(param_buf + set * C::kSetBytes, p.sw, p.bias, p.colsum, tc.n0, p.N, p.sx[tc.seg], p.zp[tc.seg],
+                                               tc.m0 + static_cast<int>(rank) * kTileM, p.M[tc.seg], st, [&] {
+                                                 w.wait(bar_pempty + 8 * set, phase ^ 1);
+                                                 __syncwarp();
+                                               });
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_pfull + 8 * set);
+      if (++set == 2) {
+        set = 0;
+        phase ^= 1;
+      }
+    }
+    w.settle();
+  } else {
     // ---------------------------------------------------- epilogue (both CTAs, own 128 rows)
     const int ew = warp - 4;
     const int q = ew & 3;
-    const int half = ew >> 2;
-    const int et = threadIdx.x - 4 * 32;
-    constexpr int kChunksPerWarp = BN / 64;
+    const int part = ew >> 2;
+    constexpr int kChunksPerWarp = BN / 32 / (C::kEpilogueWarps / 4);
     const uint32_t my_stage = out_stage_base + ew * 4096;
     const uint32_t leader_tempty = map_to_cta(bar_tempty, 0);
     BoundedWaiter w(p.status, kStatusTimeoutEpilogue);
@@ -305,21 +350,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
     for (int tile = cluster_id; tile < total_tiles; tile += num_clusters) {
       const TileCoord tc = pair_tile_coord(p, tile, BN);
       const int m0 = tc.m0 + rank * kTileM;
-      const ColumnParams cp =
-          stage_column_params<BN>(param_buf + acc * ColumnParamLayout<BN>::kFloats, p.sw, p.bias, tc.n0, p.N, et, kEpilogueThreads);
-      int32_t* csum = reinterpret_cast<int32_t*>(param_buf + 2 * ColumnParamLayout<BN>::kFloats) + acc * BN;
-      if (MODE == kPairAsym)
-        for (int c = et; c < BN; c += kEpilogueThreads) csum[c] = tc.n0 + c < p.N ? __ldg(p.colsum + tc.n0 + c) : 0;
-      asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory");
-      const int row = m0 + q * 32 + lane;
-      const float sxm = row < p.M[tc.seg] ? __ldg(p.sx[tc.seg] + row) : 0.0f;
-      const int32_t zrow = MODE == kPairAsym && row < p.M[tc.seg] ? __ldg(p.zp[tc.seg] + row) : 0;
-      // sum_k (q - z) * qw = sum_k q * qw - z * sum_k qw, for chunk c
-      auto subtract_zero = [&](uint32_t (&r)[32], int c) {
-        if (MODE == kPairAsym) {
-          const int4* cs = reinterpret_cast<const int4*>(csum + c * 32);
+      const TileParams<BN> tp(param_buf + acc * C::kSetBytes);
+      const ColumnParams cp = tp.columns;
+      const int32_t* const csum = tp.colsum;
+      w.wait(bar_pfull + 8 * acc, acc_phase);
+      __syncwarp();
+      const float sxm = tp.sx[q * 32 + lane];
+      const int32_t zrow = MODE == kPairAsym ? tp.zp[q * 32 + lane] : 0;
+      // sum_k (q - z) * qw = sum_k q * qw - z * sum_k qw, for the columns from `col` on
+      auto subtract_zero = [&](auto& r, int col) {
+        if constexpr (MODE == kPairAsym) {
+          const int4* cs = reinterpret_cast<const int4*>(csum + col);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
+          for (int j = 0; j < sizeof(r) / 16; ++j) {
             const int4 v = cs[j];
             r[4 * j] -= zrow * v.x, r[4 * j + 1] -= zrow * v.y, r[4 * j + 2] -= zrow * v.z, r[4 * j + 3] -= zrow * v.w;
           }
@@ -330,43 +373,69 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
       __syncwarp();
       tc_fence_after();
       const uint32_t t_row = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccStride;
-      // two 32-column chunks per store: a 32 x 64 bf16 tile (128-byte rows, 128-byte swizzle), full lines on the way out
-#pragma unroll 1
-      for (int cc = 0; cc + 1 < kChunksPerWarp; cc += 2) {
-        const int c = half * kChunksPerWarp + cc;
-#pragma unroll
-        for (int h2 = 0; h2 < 2; ++h2) {
-          uint32_t r[32];
-          tmem_ld_32x32(t_row + (c + h2) * 32, r);
-          tmem_wait_ld();
-          subtract_zero(r, c + h2);
-          uint32_t packed[16];
-          dequant_row32<ACT>(r, sxm, cp, c + h2, packed);
-          if (h2 == 0) {
-            if (lane == 0) bulk_wait_group_read<0>();  // the previous store has finished reading the tile
-            __syncwarp();
-          }
-#pragma unroll
-          for (int v = 0; v < 4; ++v)
-            st_shared_v4(my_stage + lane * 128 + (((4 * h2 + v) ^ (lane & 7)) << 4), packed[4 * v], packed[4 * v + 1], packed[4 * v + 2],
-                         packed[4 * v + 3]);
-        }
+      // 64 columns per store: a 32 x 64 bf16 tile (128-byte rows, 128-byte swizzle), full lines on the way out
+      auto store_tile = [&](int c) {
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
           tma_store_2d(&p.tmap_out[tc.seg], tc.n0 + c * 32, m0 + q * 32, my_stage);  // rows >= M and columns >= N are clipped
           bulk_commit_group();
         }
+      };
+      if constexpr (C::kWarpPerTile) {
+        // 16 columns at a time: what is live fits the registers of 640 threads
+        const int c = 2 * part;
+#pragma unroll 1
+        for (int step = 0; step < 4; ++step) {
+          uint32_t r[16];
+          tmem_ld_32x16(t_row + c * 32 + step * 16, r);
+          tmem_wait_ld();
+          subtract_zero(r, c * 32 + step * 16);
+          uint32_t packed[8];
+          dequant_row<16, ACT>(r, sxm, cp, 2 * c + step, packed);
+          if (step == 0) {
+            if (lane == 0) bulk_wait_group_read<0>();  // the previous store has finished reading the tile
+            __syncwarp();
+          }
+#pragma unroll
+          for (int v = 0; v < 2; ++v)
+            st_shared_v4(my_stage + lane * 128 + (((2 * step + v) ^ (lane & 7)) << 4), packed[4 * v], packed[4 * v + 1], packed[4 * v + 2],
+                         packed[4 * v + 3]);
+        }
+        store_tile(c);
+      } else {
+#pragma unroll 1
+        for (int cc = 0; cc + 1 < kChunksPerWarp; cc += 2) {
+          const int c = part * kChunksPerWarp + cc;
+#pragma unroll
+          for (int h2 = 0; h2 < 2; ++h2) {
+            uint32_t r[32];
+            tmem_ld_32x32(t_row + (c + h2) * 32, r);
+            tmem_wait_ld();
+            subtract_zero(r, (c + h2) * 32);
+            uint32_t packed[16];
+            dequant_row<32, ACT>(r, sxm, cp, c + h2, packed);
+            if (h2 == 0) {
+              if (lane == 0) bulk_wait_group_read<0>();
+              __syncwarp();
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+              st_shared_v4(my_stage + lane * 128 + (((4 * h2 + v) ^ (lane & 7)) << 4), packed[4 * v], packed[4 * v + 1], packed[4 * v + 2],
+                           packed[4 * v + 3]);
+          }
+          store_tile(c);
+        }
       }
-      if (kChunksPerWarp % 2) {
+      if constexpr (C::kOddChunk) {
         // the odd chunk (BN = 192): a 32 x 32 tile, 64-byte rows, chunk v stored at v ^ ((lane >> 1) & 3)
-        const int c = half * kChunksPerWarp + kChunksPerWarp - 1;
+        const int c = part * kChunksPerWarp + kChunksPerWarp - 1;
         uint32_t r[32];
         tmem_ld_32x32(t_row + c * 32, r);
         tmem_wait_ld();
-        subtract_zero(r, c);
+        subtract_zero(r, c * 32);
         uint32_t packed[16];
-        dequant_row32<ACT>(r, sxm, cp, c, packed);
+        dequant_row<32, ACT>(r, sxm, cp, c, packed);
         if (lane == 0) bulk_wait_group_read<0>();
         __syncwarp();
 #pragma unroll
@@ -382,7 +451,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_remote_arrive(leader_tempty + 8 * acc);
+      if (lane == 0) {
+        mbar_remote_arrive(leader_tempty + 8 * acc);
+        mbar_arrive(bar_pempty + 8 * acc);
+      }
       if (++acc == 2) {
         acc = 0;
         acc_phase ^= 1;
@@ -404,10 +476,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) gemm_w8
 
 template <int BN, int MODE>
 cudaError_t launch_pair(const Gemm2Params& p, int clusters, cudaStream_t stream) {
-  using C = Cfg2<BN>;
+  using C = Cfg2<BN, MODE>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * clusters);
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(C::kThreads);
   cfg.dynamicSmemBytes = C::kSmemBytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -425,17 +497,18 @@ int max_clusters(int dev) {
   if (dev < 0 || dev >= kMaxDevices) return 0;
   int known = cached.get(dev);
   if (known == 0) {
-    using C = Cfg2<BN>;
+    using C = Cfg2<BN, kPairPlain>;
     if (cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, kPairPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, kPairGelu>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, kPairAsym>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess) {
+        cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, kPairGelu>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg2<BN, kPairGelu>::kSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, kPairGeluLong>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg2<BN, kPairGeluLong>::kSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_w8a8_pair_kernel<BN, kPairAsym>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg2<BN, kPairAsym>::kSmemBytes) != cudaSuccess) {
       cudaGetLastError();
       cached.set(dev, -1);
       return 0;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(C::kThreads);
     cfg.dynamicSmemBytes = C::kSmemBytes;
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, gemm_w8a8_pair_kernel<BN, kPairPlain>, &cfg) != cudaSuccess || n <= 0) {
@@ -637,7 +710,7 @@ trdq_status launch_gemm_w8_pair(const trdq_weights* w, int g, const GemmSegment 
     return bn == 128 ? launch_pair<128, kMode>(p, clusters, stream) : bn == 192 ? launch_pair<192, kMode>(p, clusters, stream) : launch_pair<256, kMode>(p, clusters, stream);
   };
   const cudaError_t e = zp    ? launch(std::integral_constant<int, kPairAsym>())
-                        : act ? launch(std::integral_constant<int, kPairGelu>())
+                        : act ? (p.K <= kGeluShortK ? launch(std::integral_constant<int, kPairGelu>()) : launch(std::integral_constant<int, kPairGeluLong>()))
                               : launch(std::integral_constant<int, kPairPlain>());
   return e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA;
 }
