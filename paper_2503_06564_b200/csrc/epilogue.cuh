@@ -27,12 +27,16 @@ __device__ __forceinline__ float dequant_one(int32_t a, float sxm, float swn, fl
 // With e = exp(-|2u|) in [0, 1] the denominator d = 1 + e stays in [1, 2] on both sides, so nothing overflows and the
 // flush-to-zero form of 1 / x is in its defined range.  2^x keeps subnormal results: e is one from x = -10.0 down, and x e then
 // still is a number that bf16 holds (to x = -10.6).
-// 1152 -> 4608 with GELU at M = 4096: 29.8 us in scalar form with the epilogue column by column, 22.8 now (18.4 without GELU); the form of
-// 2^x that flushes subnormals gave 23.4 where this one gave 25.1.  Testing a chunk's 32 values for x < -9.75 and flushing otherwise gains 0.5 % of that
-// back; one reciprocal shared by four quotients moves one bf16 result in 10^5, and repairing those costs more than is gained.
+// (The form of 2^x that keeps subnormals takes three more instructions, so gelu_pack uses it only where it makes a difference.  One reciprocal
+// shared by four quotients would move one bf16 result in 10^5, and repairing those costs more than is gained.)
+template <bool FLUSH>
 __device__ __forceinline__ float exp2_approx(float x) {
   float r;
-  asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  if constexpr (FLUSH) {
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  } else {
+    asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  }
   return r;
 }
 __device__ __forceinline__ float rcp_ftz(float x) {
@@ -40,12 +44,13 @@ __device__ __forceinline__ float rcp_ftz(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
+template <bool FLUSH>
 __device__ __forceinline__ float2 gelu_tanh2(float2 x) {
   const float k = 1.5957691216057308f;  // 2 sqrt(2/pi)
   const float log2e = 1.4426950408889634f;
   const float2 t = __fmul2_rn(x, __ffma2_rn(__fmul2_rn(x, x), make_float2(0.044715f * k, 0.044715f * k), make_float2(k, k)));  // 2u, sign of x
   const float2 t2 = __fmul2_rn(t, make_float2(log2e, log2e));
-  const float2 e = make_float2(exp2_approx(-fabsf(t2.x)), exp2_approx(-fabsf(t2.y)));
+  const float2 e = make_float2(exp2_approx<FLUSH>(-fabsf(t2.x)), exp2_approx<FLUSH>(-fabsf(t2.y)));
   const float2 m = __fmul2_rn(x, e);
   const float2 d = __fadd2_rn(e, make_float2(1.0f, 1.0f));
   return __fmul2_rn(make_float2(t.x >= 0.0f ? x.x : m.x, t.y >= 0.0f ? x.y : m.y), make_float2(rcp_ftz(d.x), rcp_ftz(d.y)));
@@ -54,6 +59,23 @@ __device__ __forceinline__ float2 gelu_tanh2(float2 x) {
 __device__ __forceinline__ uint32_t pack_bf16(float2 v) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
   return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// GELU of 2 PAIRS values, packed to bf16.  One test for all of them: from -9.75 up 2^x is a normal number and both forms of it agree.
+// 1152 -> 4608 with GELU, without / with the test: 22.8 -> 22.1 us at M = 4096, 79.4 -> 76.7 at 16384 (before the epilogue had sixteen warps it
+// waited more than it issued, and the test gained nothing; nor does it in the 4-bit kernel, 264 against 269 us).
+template <int PAIRS>
+__device__ __forceinline__ void gelu_pack(const float2 (&v)[PAIRS], uint32_t (&packed)[PAIRS]) {
+  float lowest = v[0].x;
+#pragma unroll
+  for (int j = 0; j < PAIRS; ++j) asm("min.f32 %0, %0, %1, %2;" : "+f"(lowest) : "f"(v[j].x), "f"(v[j].y));
+  if (lowest < -9.75f) {
+#pragma unroll
+    for (int j = 0; j < PAIRS; ++j) packed[j] = pack_bf16(gelu_tanh2<false>(v[j]));
+  } else {
+#pragma unroll
+    for (int j = 0; j < PAIRS; ++j) packed[j] = pack_bf16(gelu_tanh2<true>(v[j]));
+  }
 }
 
 // min(|a|, |b|, |c|) in one instruction
@@ -129,8 +151,12 @@ __device__ __forceinline__ void dequant_row(const uint32_t (&r)[COLS], float sxm
       }
     }
   }
+  if constexpr (ACT) {
+    gelu_pack(v, packed);
+  } else {
 #pragma unroll
-  for (int j = 0; j < COLS / 2; ++j) packed[j] = pack_bf16(ACT ? gelu_tanh2(v[j]) : v[j]);
+    for (int j = 0; j < COLS / 2; ++j) packed[j] = pack_bf16(v[j]);
+  }
 }
 
 // Staging of the epilogue parameters of BN columns (see ColumnParamLayout): the scale and bias of column n, then their place c in the

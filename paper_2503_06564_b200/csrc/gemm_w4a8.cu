@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_con
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
           const float2 two = make_float2(v[2 * g], v[2 * g + 1]);
-          packed[g] = pack_bf16(ACT ? gelu_tanh2(two) : two);
+          packed[g] = pack_bf16(ACT ? gelu_tanh2<false>(two) : two);
         }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
