@@ -6,14 +6,15 @@
 // stores, instead of at each gathered value: the product is the same), and every thread gathers its 128 permuted channels;
 // the table of byte offsets is 16 bits per channel, eight per load.
 //
-// What bounds it (K = 1152, M = 16384): 31.5 shared-memory wavefronts per block and row, 22.5 of them loads (for the most part the
-// gather of 128 scalars at arbitrary banks), 14 of them conflicts, keep that pipe 57 % busy and issue slots 37 %: between the two lies the chain
-// load - transform - barrier - gather - transform - maximum of a team, of which nine warps hold three.  The row
-// buffer is swizzled (16-byte chunk index xor block) and rows are 48 bytes apart modulo 128, so that the writes of a
-// quarter warp and the three rows of one channel fall into different banks.
-// One input stage (the next tile is requested as soon as this one is in registers, most of a tile's time before its use)
-// and codes staged in the row buffer after the last gather leave room for 30 rows in flight at K = 1152 (three teams of ten) and six at
-// K = 4608 (two teams of three).
+// What bounds it: the shared-memory pipe (per block and row some 30 wavefronts, for the most part the gather of 128 scalars at arbitrary
+// banks) and the chain load - transform - barrier - gather - transform - maximum of a team, hidden only by other teams.  So it
+// is rows in flight that count, and one buffer per team has to do for everything: the input tile lies in its first half until it is
+// in registers, then the rotated rows take all of it, and the codes its last quarter, while the next input already arrives in the
+// first half.  A separate input tile (requested most of a tile's time ahead) left room for 0.55 - 0.75 of the lanes of twelve warps; now
+// it is 0.84 - 1.0.  Microseconds before -> now, M = 16384: K = 1152 28.7 -> 24.9, 1536 43.3 -> 28.9, 2304 58.5 -> 49.2, 3072 72.8 -> 58.8,
+// 4608 115 -> 102; M = 4096: K = 1152 9.4 -> 8.5, 4608 36.2 -> 31.8, 7680 68.0 -> 54.9.
+// The row buffer is swizzled (16-byte chunk index xor block) and rows are 48 bytes apart modulo 128, so that the writes of a
+// quarter warp and the rows of one channel fall into different banks.
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -59,7 +60,7 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate2_quantize_team_k
   const uint32_t box_bytes = R * 128;
   const uint32_t in_bytes = 2 * nb * box_bytes;
   const uint32_t row_stride = 4 * p.K + kRowPadBytes;
-  const uint32_t team_bytes = in_bytes + row_buffer_bytes(p.K, R);
+  const uint32_t team_bytes = row_buffer_bytes(p.K, R);
   const int vec_floats = nb * (TRDQ_BLOCK + kVecPadFloats);
   float* svec1 = reinterpret_cast<float*>(smem + p.teams * team_bytes);
   float* svec2 = svec1 + vec_floats;                                              // by SOURCE channel
@@ -72,7 +73,10 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate2_quantize_team_k
   const int team = tid / team_threads;
   const int tt = tid - team * team_threads;
   const uint32_t team_base = smem_base + team * team_bytes;
-  const uint32_t rows_base = team_base + in_bytes;  // row buffer, later the code tile
+  // One buffer per team takes turns: the input tile in its first half, then the rows, then the codes in its last quarter, so that
+  // the next input may arrive while the codes are formed and stored.
+  const uint32_t rows_base = team_base;
+  const uint32_t code_base = team_base + 3 * R * p.K;
   unsigned int* row_max = row_max_all + team * 3 * R;
   const uint32_t bar_full = smem_u32(bars + team);
 
@@ -121,12 +125,8 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate2_quantize_team_k
     load_scaled_block(team_base, box_bytes, b, r, sv1, v);
     wht128_thread(v);  // first rotation
 
-    if (tt == 0) bulk_wait_group_read<0>();  // the previous tile's codes have left the row buffer
-    team_barrier(team, team_threads);        // every thread of the team has read the input stage
-    if (tt == 0 && tile + stride < num_tiles) {
-      mbar_arrive_expect_tx(bar_full, in_bytes);
-      tma_load_3d(team_base, &p.tmap_x, 0, (tile + stride) * R, 0, bar_full);
-    }
+    if (tt == 0) bulk_wait_group_read<0>();  // the previous tile's codes have left the buffer
+    team_barrier(team, team_threads);        // every thread of the team has read the input tile
     if (active) {
 #pragma unroll
       for (int q = 0; q < 32; ++q) {
@@ -147,19 +147,24 @@ __global__ void __launch_bounds__(kTeamMaxWarps * 32, 1) rotate2_quantize_team_k
     wht128_thread(v);  // second rotation
     const float m = absmax_thread(v);
     if (active) atomicMax(&row_max[buf * R + r], __float_as_uint(m));
-    team_barrier(team, team_threads);  // row maxima complete; every gather of the tile is done, the row buffer takes the codes
+    fence_proxy_async_smem();
+    team_barrier(team, team_threads);  // row maxima complete; every gather of the tile is done: the buffer takes the next input and the codes
+    if (tt == 0 && tile + stride < num_tiles) {
+      mbar_arrive_expect_tx(bar_full, in_bytes);
+      tma_load_3d(team_base, &p.tmap_x, 0, (tile + stride) * R, 0, bar_full);
+    }
 
     const float amax = __uint_as_float(row_max[buf * R + r]);
     const float inv = amax > 0.0f ? __fdiv_rn(127.0f, amax) : 0.0f;
     if (active) {
-      quantize_store_block(v, inv, p.zero, rows_base + b * box_bytes + r * 128);
+      quantize_store_block(v, inv, p.zero, code_base + b * box_bytes + r * 128);
       const int64_t row = static_cast<int64_t>(tile) * R + r;
       if (b == 0 && row < p.M) p.scales[row] = __fdiv_rn(amax, 127.0f);
     }
     fence_proxy_async_smem();
     team_barrier(team, team_threads);
     if (tt == 0) {
-      tma_store_3d(&p.tmap_codes, 0, tile * R, 0, rows_base);  // all nb column boxes; rows >= M are clipped
+      tma_store_3d(&p.tmap_codes, 0, tile * R, 0, code_base);  // all nb column boxes; rows >= M are clipped
       bulk_commit_group();
     }
   }
@@ -173,29 +178,56 @@ struct Team2Shape {
   double use;  // fraction of the twelve warps' lanes that hold a block
 };
 
-size_t team2_smem_bytes(int K, int R, int teams) {
+size_t team2_smem_bytes(int K, int R, int teams, bool input_apart = false) {
   const size_t nb = K / TRDQ_BLOCK;
-  return 128 + teams * (static_cast<size_t>(2) * R * K + row_buffer_bytes(K, R)) + nb * (TRDQ_BLOCK + kVecPadFloats) * 8 + nb * (TRDQ_BLOCK + 8) * 2 +
+  return 128 + teams * ((input_apart ? static_cast<size_t>(2) * R * K : 0) + row_buffer_bytes(K, R)) + nb * (TRDQ_BLOCK + kVecPadFloats) * 8 + nb * (TRDQ_BLOCK + 8) * 2 +
          (static_cast<size_t>(teams) * 3 * R + 2) * 4 + static_cast<size_t>(teams) * 8 + 16;
 }
 
-// The team size with the best use of the lanes of twelve warps (the fuller teams of two that are alike); at least two teams, so that one can transform while
-// another waits (rows of up to 72 blocks; offsets of 16 bits would reach 128).
-bool choose_team2_shape(int K, Team2Shape* out) {
+// The team size, by the share of the twelve warps' lanes that hold a block, weighted by what else was seen to count over 2600 timings of all
+// shapes (K = 384 ... 8192, M = 600 ... 16384): rows are 48 bytes apart modulo 128, so eight of them fill the banks evenly, and tiles of a
+// multiple of eight rows gather with fewer conflicts (K = 1408 at M = 16384: 8 rows 28.9 us, 7 rows 36.9), even numbers are a
+// little ahead of odd ones; two teams overlap less than three; and warps that do not divide by the four schedulers leave some of
+// them idle.  The shapes taken are 1.4 % off the best ones on average, by lanes alone 5.3 %.  A tile is at most two thirds of an SM's share of the
+// rows, or an SM would have nothing to overlap.  At least two teams (rows of up to 72 blocks; offsets of 16 bits would reach 128).
+bool choose_team2_shape(int M, int K, int sms, Team2Shape* out) {
   const int nb = K / TRDQ_BLOCK;
   Team2Shape best = {0, 0, 0, 0, 0.0};
+  double best_score = 0.0;
   for (int tw = 1; tw <= kTeamMaxWarps / 2; ++tw)
     for (int rows = tw * 32 / nb < 32 ? tw * 32 / nb : 32; rows >= 1; --rows) {
       int teams = kTeamMaxWarps / tw;
       while (teams > 0 && team2_smem_bytes(K, rows, teams) > 227u * 1024u) --teams;
       if (teams < 2) continue;
+      if (rows > 1 && static_cast<int64_t>(rows) * 3 * sms > 2ll * M) continue;
       const double use = static_cast<double>(rows) * nb * teams / (32 * kTeamMaxWarps);
-      const double lanes = static_cast<double>(rows) * nb / (32 * tw), best_lanes = static_cast<double>(best.R) * nb / (32 * best.team_warps + 1e-9);
-      if (use > best.use + 1e-9 || (use > best.use - 1e-9 && lanes > best_lanes + 1e-9)) best = Team2Shape{rows, tw, teams, team2_smem_bytes(K, rows, teams), use};
+      const int idle = (4 - teams * tw % 4) % 4;
+      const double score = use * (rows % 8 == 0 ? 1.2 : rows % 2 == 0 ? 1.06 : 1.0) * (teams == 2 ? 0.95 : 1.0) * (1.0 - 0.3 * idle / kTeamMaxWarps);
+      if (score > best_score + 1e-9) {
+        best = Team2Shape{rows, tw, teams, team2_smem_bytes(K, rows, teams), use};
+        best_score = score;
+      }
     }
   if (best.teams == 0) return false;
   *out = best;
   return true;
+}
+
+// The cut the dispatch line below was drawn with: by lanes alone (the fuller teams of two that are alike), with an input tile of its own per team.
+bool line_team2_shape(int K, Team2Shape* out) {
+  const int nb = K / TRDQ_BLOCK;
+  Team2Shape best = {0, 0, 0, 0, 0.0};
+  for (int tw = 1; tw <= kTeamMaxWarps / 2; ++tw)
+    for (int rows = tw * 32 / nb < 32 ? tw * 32 / nb : 32; rows >= 1; --rows) {
+      int teams = kTeamMaxWarps / tw;
+      while (teams > 0 && team2_smem_bytes(K, rows, teams, true) > 227u * 1024u) --teams;
+      if (teams < 2) continue;
+      const double use = static_cast<double>(rows) * nb * teams / (32 * kTeamMaxWarps);
+      const double lanes = static_cast<double>(rows) * nb / (32 * tw), best_lanes = static_cast<double>(best.R) * nb / (32 * best.team_warps + 1e-9);
+      if (use > best.use + 1e-9 || (use > best.use - 1e-9 && lanes > best_lanes + 1e-9)) best = Team2Shape{rows, tw, teams, 0, use};
+    }
+  *out = best;
+  return best.teams != 0;
 }
 
 }  // namespace
@@ -209,17 +241,17 @@ bool choose_team2_shape(int K, Team2Shape* out) {
 //   rows of up to ten blocks 0.54 (the second CTA of an SM starts to count; K = 1024: 6.3 / 7.2 at M = 1306, 7.7 / 7.2 at 1463);
 //   rows of up to 24 blocks 1.1 (K = 2048: 6.9 / 8.0 at M = 1166, 9.2 / 8.1 at 1306), up to 36 blocks 1.3 (K = 4608: 10.4 / 10.5 at
 //   M = 740, 13.8 / 10.9 at 829);
-//   wider rows, one per lane-group CTA, 1.6 (K = 6144: 12.2 / 12.8 at M = 417, 12.9 / 12.7 at 468);
+//   wider rows, one per lane-group CTA, 1.6 (K = 6144: 12.2 / 12.8 at M = 417, 12.9 / 12.7 at 468));
 //   and where a team's tile is a single row, eleven rows per SM (K = 4096: 12.4 / 14.0 at M = 1166, 17.4 / 14.8 at 1639;
 //   K = 7680: 22.1 / 24.2 at M = 1166, 31.5 / 29.3 at 1639).
-// One of 958 points ends up slower than the lane groups, by 2 %; K = 6144 at M = 1480 = 5 x 296, where their last round is full, by 10 %.  M = 4096, K = 1152 / 4608: 14.1 / 42.5 -> 9.0 / 33.3 us;
-// M = 16384: 42.6 / 166 -> 28.2 / 115 us.
+// These are timings of the form with an input tile of its own, and the line is kept where they put it: above it the present form is the faster of
+// the two, below it the lane groups still are for most shapes (K = 8192 would change sides at about M = 1200).
 bool rotate2_prefers_team(int32_t M, int32_t K) {
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   Team2Shape s;
-  if (!choose_team2_shape(K, &s) || s.use < 0.45 || (static_cast<int64_t>(M) + s.R - 1) / s.R < sms) return false;
+  if (!line_team2_shape(K, &s) || s.use < 0.45 || (static_cast<int64_t>(M) + s.R - 1) / s.R < sms) return false;
   if (s.R == 1) return M >= 11 * sms;
   const int nb = K / TRDQ_BLOCK;
   const int64_t round = 2ll * sms * rotate2_lane_group_rows(K);
@@ -233,7 +265,7 @@ trdq_status launch_rotate2_quantize_team(const void* x_bf16, int64_t ldx, int32_
   if (cudaGetDevice(&dev) != cudaSuccess) return TRDQ_ERR_CUDA;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   Team2Shape shape;
-  if (!choose_team2_shape(K, &shape)) return TRDQ_ERR_SHAPE;
+  if (!choose_team2_shape(M, K, sms, &shape)) return TRDQ_ERR_SHAPE;
   const int nb = K / TRDQ_BLOCK;
   Team2Params p;
   trdq_status st = encode_tmap_boxes(&p.tmap_x, x_bf16, 2, 64, static_cast<uint64_t>(M), static_cast<uint64_t>(ldx) * 2,
