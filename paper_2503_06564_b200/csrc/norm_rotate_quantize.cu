@@ -11,6 +11,8 @@
 // them in the same fixed order (mean = average of the block means, M2 = sum of the block M2 + 128 sum (mean_b - mean)^2),
 // so the result does not depend on scheduling: the same input always gives the same codes.  One extra barrier per tile;
 // the shared statistics alternate between two copies so that none is needed before they are reused.
+// What bounds it: instruction issue (30 instructions per element, half of the slots used) and the waits between: statistics, barrier,
+// modulation, transform, barrier.  In the AHEAD form the modulation is on its way while the statistics are formed.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -32,10 +34,10 @@ __device__ __forceinline__ float2 bf16x2_to_float2(uint32_t w) {
   return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));  // exact widening
 }
 
-// blockDim.x = rows_per_tile * (K / 128) * 4 rounded up to a warp (at most 320);
+// blockDim.x = rows_per_tile * (K / 128) * 4 rounded up to a warp (at most THREADS);
 // dynamic shared memory: K floats (fused vector) + 2 copies x 2 arrays x rows_per_tile * (K / 128) floats.
-template <int MIN_CTAS>
-__global__ void __launch_bounds__(320, MIN_CTAS)
+template <int THREADS, bool AHEAD>
+__global__ void __launch_bounds__(THREADS, 2)
 norm_rotate_quantize_rows_kernel(const uint16_t* __restrict__ x, int64_t ldx, int32_t M, int32_t K, const float* __restrict__ vec,
                                  const uint16_t* __restrict__ shift, const uint16_t* __restrict__ scale, int32_t rows_per_sample, float eps,
                                  int8_t* __restrict__ codes, float* __restrict__ scales, int32_t rows_per_tile, float zero) {
@@ -86,6 +88,17 @@ norm_rotate_quantize_rows_kernel(const uint16_t* __restrict__ x, int64_t ldx, in
     float* mean_b = stats + (it & 1) * 2 * items;
     float* m2_b = mean_b + items;
 
+    // The modulation of the lane's columns, 16 bytes of scale and shift per chunk.
+    const int64_t sidx = AHEAD ? static_cast<int64_t>((valid ? row : 0) / rows_per_sample) * K + col0 : 0;
+    uint4 sc_ahead[AHEAD ? 4 : 1], sh_ahead[AHEAD ? 4 : 1];
+    if constexpr (AHEAD) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        sc_ahead[c] = scale ? __ldg(reinterpret_cast<const uint4*>(scale + sidx) + 4 * c) : make_uint4(0u, 0u, 0u, 0u);
+        sh_ahead[c] = shift ? __ldg(reinterpret_cast<const uint4*>(shift + sidx) + 4 * c) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+
     // v[4c + j] = elements (2j, 2j+1) of chunk c
     float2 v[16];
     widen_chunks_lanes4(raw, v);
@@ -124,12 +137,18 @@ norm_rotate_quantize_rows_kernel(const uint16_t* __restrict__ x, int64_t ldx, in
 
     if (valid) {
       // h = (x - mean) * rstd * (1 + scale) + shift, then the fused vector of the rotation
-      const int64_t sidx = static_cast<int64_t>(row / rows_per_sample) * K + col0;
+      const int64_t here = AHEAD ? sidx : static_cast<int64_t>(row / rows_per_sample) * K + col0;
       const float2 nmean = make_float2(-mean, -mean), rstd2 = make_float2(rstd, rstd), one2 = make_float2(1.0f, 1.0f);
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const uint4 sc_raw = scale ? __ldg(reinterpret_cast<const uint4*>(scale + sidx) + 4 * c) : make_uint4(0u, 0u, 0u, 0u);
-        const uint4 sh_raw = shift ? __ldg(reinterpret_cast<const uint4*>(shift + sidx) + 4 * c) : make_uint4(0u, 0u, 0u, 0u);
+        uint4 sc_raw, sh_raw;
+        if constexpr (AHEAD) {
+          sc_raw = sc_ahead[c];
+          sh_raw = sh_ahead[c];
+        } else {
+          sc_raw = scale ? __ldg(reinterpret_cast<const uint4*>(scale + here) + 4 * c) : make_uint4(0u, 0u, 0u, 0u);
+          sh_raw = shift ? __ldg(reinterpret_cast<const uint4*>(shift + here) + 4 * c) : make_uint4(0u, 0u, 0u, 0u);
+        }
         const uint32_t scw[4] = {sc_raw.x, sc_raw.y, sc_raw.z, sc_raw.w};
         const uint32_t shw[4] = {sh_raw.x, sh_raw.y, sh_raw.z, sh_raw.w};
 #pragma unroll
@@ -168,12 +187,20 @@ cudaError_t launch_norm_rotate_quantize(const void* x_bf16, int64_t ldx, int32_t
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int rows = rows_per_tile_by_rounds(M, std::max(1, std::min(32, 72 / nb)), sms);  // at most about 72 lane groups (288 threads) per CTA
+  // The form that requests the modulation ahead keeps 64 more bytes a thread and so at most 64 lane groups (256 threads of 128 registers) in a
+  // CTA, the other 72.  It is 4 - 25 % faster (K = 1152: 5.3 -> 4.7 us at M = 1037, 9.1 -> 8.5 at 4096, 17.3 -> 16.2 at 8192, 31.8 -> 30.1 at 16384)
+  // where its fewer rows do not cost a round; where they cost more than a tenth (K = 640, M = 4096: 6.3 -> 8.2), and for rows
+  // of more than 12 blocks (K = 4608: one row a CTA in place of two, 33 -> 49), the other one runs.
+  const int rows_plain = rows_per_tile_by_rounds(M, std::max(1, std::min(32, 72 / nb)), sms);
+  const int rows_ahead = rows_per_tile_by_rounds(M, std::max(1, std::min(32, 64 / nb)), sms);
+  const auto cost = [&](int r) { return static_cast<int64_t>(((M + r - 1) / r + 2 * sms - 1) / (2 * sms)) * (r + 2); };
+  const bool ahead = nb >= 3 && nb <= 12 && 9 * cost(rows_ahead) <= 10 * cost(rows_plain);
+  const int rows = ahead ? rows_ahead : rows_plain;
   const int threads = (rows * nb * kFastLanes + 31) / 32 * 32;
   const size_t smem = (static_cast<size_t>(K) + 4u * rows * nb) * sizeof(float);
   const int num_tiles = (M + rows - 1) / rows;
   const int grid = std::min(num_tiles, sms * 2);
-  return launch_overlapped(norm_rotate_quantize_rows_kernel<2>, dim3(grid), dim3(threads), smem, stream,
+  return launch_overlapped(ahead ? norm_rotate_quantize_rows_kernel<256, true> : norm_rotate_quantize_rows_kernel<320, false>, dim3(grid), dim3(threads), smem, stream,
                            static_cast<const uint16_t*>(x_bf16), ldx, M, K, vec, static_cast<const uint16_t*>(shift_bf16),
                            static_cast<const uint16_t*>(scale_bf16), rows_per_sample, eps, codes, scales, rows, 0.0f);
 }

@@ -1,0 +1,34 @@
+"""The two forms of the LayerNorm + rotation kernel (modulation requested ahead or where it is used) give the same bits: which one runs depends
+on the row count, and may not show."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,K,piece", [   # M rows take one form, pieces of them the other or another number of rows per CTA
+    (4097, 640, 1110),     # modulation where it is used (the other form would need a round more); pieces: ahead
+    (2500, 1024, 370),
+    (2479, 1152, 407),
+    (777, 384, 111),
+    (300, 1536, 37),       # the widest rows of the form ahead
+    (300, 1664, 37),
+])
+@pytest.mark.parametrize("modulated", [True, False])
+def test_same_bits_whatever_the_row_count(M, K, piece, modulated):
+    import torch
+    from paper_2503_06564_b200 import trdq
+    rng = np.random.default_rng(M + K)
+    rot = trdq.Rotation(K, [0, 1000], (rng.integers(0, 2, (1, K)) * 2 - 1).astype(np.int8), rng.uniform(0.5, 2.0, (1, K)).astype(np.float32))
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    sample = 37
+    x = (torch.randn((M, K), generator=g, device="cuda") * 3.0 + 1.0).to(torch.bfloat16)
+    x[M // 3] = 0.0
+    mod = [(torch.randn((-(-M // sample), K), generator=g, device="cuda") * 0.2).to(torch.bfloat16) if modulated else None for _ in range(2)]
+    codes, scales = trdq.trdq_norm_rotate_quantize(rot, 0, x, mod[0], mod[1], sample, 1e-6)
+    assert piece % sample == 0
+    for a in range(0, M, piece):
+        part = [m[a // sample:].contiguous() if modulated else None for m in mod]
+        c, s = trdq.trdq_norm_rotate_quantize(rot, 0, x[a:a + piece].contiguous(), part[0], part[1], sample, 1e-6)
+        assert torch.equal(c, codes[a:a + piece]) and torch.equal(s.view(torch.int32), scales[a:a + piece].view(torch.int32)), a
+    assert trdq.trdq_device_status() == 0
