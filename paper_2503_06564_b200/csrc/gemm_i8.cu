@@ -360,15 +360,19 @@ int choose_tile_n(int64_t tiles_m, int N, int sms) {
 // epilogue).  Microseconds, pair / single CTA, at N x M: K = 128: 8.2 / 7.8 at 2304 x 4096 (144 tiles), 10.1 / 11.1 at 4608 x 2560 (180);
 // K = 1152: 10.1 / 9.4 at 3456 x 2048 (108), 10.8 / 11.2 at 3072 x 2560 (120);  K = 2304: 11.2 / 10.3 at 2304 x 2048 (72), 12.5 / 13.2 at
 // 2048 x 2560 (80);  K = 4608: 13.8 / 12.9 at 1152 x 3072 (54), 16.1 / 16.7 at 1536 x 2560 (60), 18.5 / 19.5 at 256 x 12288 (48);
-// K = 12288: 21.9 / 26.9 at 768 x 2560 (30).  The asymmetric correction and GELU make the epilogue longer and change over later at
-// short reductions.  Averaged over the points the rule is 0.1 % off the faster kernel, the pair kernel everywhere 4.6 %, the
-// other 3.4 %.  TRDQ_PAIR_MIN_M (read once per process) replaces the rule by a row count.
+// K = 12288: 21.9 / 26.9 at 768 x 2560 (30).  Averaged over the points the rule is 0.1 % off the faster kernel, the pair kernel everywhere
+// 4.6 %, the other 3.4 %.  These are times of both kernels with epilogue parameters loaded tile by tile; with parameters staged ahead in
+// the pair kernel the longer epilogues change over earlier, and from half the rows on.  Mean pair / single CTA at 78 - 95, 95 - 110 and 135 - 165
+// tiles (sixteen K, six N, M from 1037 to 12288): GELU 0.95, 0.98, 0.92 at K = 640 ... 1023, 0.93, 0.97, 0.92 at 1024 ... 1279, 0.94, 0.96, 0.92
+// at 1536 ... 2303 and 0.89 ... 0.97 below 2048 rows; asymmetric codes 1.00, 1.02, 0.96 at K = 640 ... 1023, 0.96, 0.99, 0.94 at 1024 ... 1535 and
+// 0.92 ... 0.99 below 2048 rows; both 1.04 ... 1.10 at 56 - 78 tiles.
+// TRDQ_PAIR_MIN_M (read once per process) replaces the rule by a row count.
 static int pair_least_tiles(int32_t K, int32_t N, bool gelu, bool asym) {
   if (K >= 7168) return 0;
   if (K >= 6144) return 40;
   if (K >= 4096) return N <= 256 ? 46 : 56;
-  if (K >= 1536) return gelu && K < 2304 ? 110 : 78;
-  return K < (asym ? 1280 : 1024) ? 165 : 110;
+  if (K >= 1536 || gelu || (asym && K >= 1024)) return 78;
+  return asym ? 135 : K < 1024 ? 165 : 110;
 }
 static bool use_pair(int64_t M, int32_t K, int32_t N, bool gelu, bool asym) {
   static const int forced = [] {
@@ -376,7 +380,8 @@ static bool use_pair(int64_t M, int32_t K, int32_t N, bool gelu, bool asym) {
     return e ? atoi(e) : -1;
   }();
   if (forced >= 0) return M >= forced;
-  return M >= 2048 && M * N >= pair_least_tiles(K, N, gelu, asym) * 65536ll;
+  const bool long_epilogue = (gelu && K < 2304) || (asym && K >= 1024 && K < 2304);
+  return M >= (long_epilogue ? 1024 : 2048) && M * N >= pair_least_tiles(K, N, gelu, asym) * 65536ll;
 }
 
 // Name of the kernel trdq_linear runs for M rows against [N, K] weights of `wbits` bits (one row segment).

@@ -37,3 +37,23 @@ def test_same_bits_as_one_cta_per_tile(M, N, K, width, with_bias):
             part = slice(a, a + 2000)
             assert torch.equal(whole[part].view(torch.int16), call(codes[part].clone(), scales[part].clone(), zero[part].clone()).view(torch.int16))
     assert trdq.trdq_device_status() == 0
+
+
+@pytest.mark.parametrize("M,N,K", [(1100, 4656, 1152), (1999, 2576, 768), (1664, 3072, 768), (1400, 3680, 2176)])
+def test_long_epilogues_take_pairs_from_1024_rows_on(M, N, K):
+    """GELU and asymmetric codes change to CTA pairs earlier than the plain epilogue: the same bits as in pieces that do not."""
+    import torch
+    from paper_2503_06564_b200 import trdq
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    rot = trdq.Rotation(K, [0, 1000], np.ones((1, K), np.int8), None)
+    wts = trdq.trdq_prepare_weights(rot, (torch.randn((N, K), generator=g, device="cuda") * 0.02).to(torch.bfloat16), 8)
+    codes = torch.randint(-127, 128, (M, K), generator=g, device="cuda", dtype=torch.int8)
+    scales = torch.rand((M,), generator=g, device="cuda") * 0.01
+    zero = torch.randint(0, 256, (M,), generator=g, device="cuda", dtype=torch.int32)
+    bias = torch.randn((N,), generator=g, device="cuda").to(torch.bfloat16)
+    for call in (lambda c, s, z: trdq.trdq_linear_act(wts, 0, c, s, bias), lambda c, s, z: trdq.trdq_linear_asym(wts, 0, c.view(torch.uint8), s, z, bias)):
+        whole = call(codes, scales, zero)
+        for a in range(0, M, 700):
+            part = slice(a, min(a + 700, M))
+            assert torch.equal(whole[part].view(torch.int16), call(codes[part].clone(), scales[part].clone(), zero[part].clone()).view(torch.int16))
+    assert trdq.trdq_device_status() == 0
