@@ -36,7 +36,7 @@ uint32_t* device_status_word() {
 // caller that prepares layer after layer, or again after a change of the weights, gets the memory of the one it has just destroyed.
 //   bounded     kKeptMax bytes per device (a layer's worth: the widest one in use here is 106 MB); what does not fit is freed at once
 //   given back  when the last rotation and weights object is destroyed, and before an allocation is reported as failed
-//   safe        destroying waits for the device, as the cudaFree it replaces does, so nothing on any stream still reads the memory when it
+//   safe        destroying waits for the device as the cudaFree it replaces does, so nothing on any stream still reads the memory when it
 //               is handed out again; a stream that is being captured never gets kept memory (its preparation is refused, as before)
 namespace {
 constexpr size_t kKeptMax = size_t{256} << 20;
@@ -84,7 +84,10 @@ struct TableMemory {
   }
   void give(int dev, void* p, size_t bytes) {
     int current = -1;
-    bool keep = bytes <= kKeptMax && cudaGetDevice(&current) == cudaSuccess && current == dev && cudaDeviceSynchronize() == cudaSuccess;
+    // The wait is that of a cudaFree, of one byte: cudaDeviceSynchronize would break a capture that another thread has open.
+    void* one = nullptr;
+    bool keep = bytes <= kKeptMax && cudaGetDevice(&current) == cudaSuccess && current == dev && cudaMalloc(&one, 1) == cudaSuccess &&
+                cudaFree(one) == cudaSuccess;
     if (keep) {
       std::lock_guard<std::mutex> lock(mu);
       size_t total = bytes;
