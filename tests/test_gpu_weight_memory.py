@@ -89,6 +89,21 @@ except (trdq.TrdqError, RuntimeError):
     pass
 torch.cuda.synchronize()
 
+# another thread may destroy weights while this one captures (thread-local mode), and the capture holds
+w = trdq.trdq_prepare_weights(rot, x, 8)
+y = torch.zeros(1024, device="cuda")
+torch.cuda.synchronize()
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+    y += 1.0
+    t = threading.Thread(target=w.close)
+    t.start()
+    t.join()
+    y += 1.0
+graph.replay()
+torch.cuda.synchronize()
+assert float(y.sum()) == 2048.0
+
 # more than the bound is not kept, and the last object gives back everything
 big = rotation(4608, 4)
 x = weight(16384, 4608, 3)
