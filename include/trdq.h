@@ -129,6 +129,10 @@ trdq_status trdq_find_group(const int32_t* t_bounds, int32_t num_groups, int32_t
  * right away.  `*out` is set only on TRDQ_OK. */
 trdq_status trdq_prepare_weights(const trdq_rotation* rot, const void* W_bf16, int32_t N, int32_t wbits,
                                  trdq_weights** out, void* stream);
+/* Destroys the object and returns its device memory (cudaFree, as trdq_rotation_destroy does).  With the drivers the library was
+ * tried on the call returns when the work already enqueued on the device has ended; work enqueued later must not use the
+ * object, replays of a graph that captured its use included.  Not while a stream capture is open that forbids cudaFree: one in global
+ * mode by any thread, or the calling thread's own in thread-local mode.  That invalidates the capture, and the memory is not returned. */
 trdq_status trdq_weights_destroy(trdq_weights* w);
 
 /* Shape and format of a prepared layer (any output pointer may be NULL). */

@@ -31,86 +31,6 @@ uint32_t* device_status_word() {
   return addr;
 }
 
-// Table memory of destroyed weights, kept for the next preparation.  Preparing five groups of 4608 x 1152 takes the device 30 us, but
-// the cudaMalloc and the cudaFree of their 27 MB 0.65 ms of host time (738 -> 96 us for prepare, export of all groups and destroy).  A
-// caller that prepares layer after layer, or again after a change of the weights, gets the memory of the one it has just destroyed.
-//   bounded     kKeptMax bytes per device (a layer's worth: the widest one in use here is 106 MB); what does not fit is freed at once
-//   given back  when the last rotation and weights object is destroyed, and before an allocation is reported as failed
-//   safe        destroying waits for the device as the cudaFree it replaces does, so nothing on any stream still reads the memory when it
-//               is handed out again; a stream that is being captured never gets kept memory (its preparation is refused, as before)
-namespace {
-constexpr size_t kKeptMax = size_t{256} << 20;
-struct KeptTables {
-  void* p;
-  size_t bytes;
-  int device;
-};
-struct TableMemory {
-  std::mutex mu;
-  std::vector<KeptTables> kept;
-  int live = 0;
-
-  static TableMemory& get() {
-    static TableMemory* const m = new TableMemory;  // never destroyed: objects may outlive the library's static data
-    return *m;
-  }
-  void release_all() {  // mu held
-    for (const KeptTables& k : kept) cudaFree(k.p);
-    kept.clear();
-  }
-  // A block of at least `bytes` on the current device `dev`; *got is its size.
-  void* take(int dev, size_t bytes, cudaStream_t stream, size_t* got) {
-    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    const bool reuse = cudaStreamIsCapturing(stream, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone;
-    std::lock_guard<std::mutex> lock(mu);
-    int best = -1;
-    for (int i = 0; reuse && i < static_cast<int>(kept.size()); ++i)
-      if (kept[i].device == dev && kept[i].bytes >= bytes && kept[i].bytes / 2 <= bytes && (best < 0 || kept[i].bytes < kept[best].bytes)) best = i;
-    if (best >= 0) {
-      void* const p = kept[best].p;
-      *got = kept[best].bytes;
-      kept.erase(kept.begin() + best);
-      return p;
-    }
-    void* p = nullptr;
-    *got = bytes;
-    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
-    cudaGetLastError();
-    if (!reuse || kept.empty()) return nullptr;
-    release_all();
-    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
-    cudaGetLastError();
-    return nullptr;
-  }
-  void give(int dev, void* p, size_t bytes) {
-    int current = -1;
-    // The wait is that of a cudaFree, of one byte: cudaDeviceSynchronize would break a capture that another thread has open.
-    void* one = nullptr;
-    bool keep = bytes <= kKeptMax && cudaGetDevice(&current) == cudaSuccess && current == dev && cudaMalloc(&one, 1) == cudaSuccess &&
-                cudaFree(one) == cudaSuccess;
-    if (keep) {
-      std::lock_guard<std::mutex> lock(mu);
-      size_t total = bytes;
-      for (const KeptTables& k : kept) total += k.device == dev ? k.bytes : 0;
-      keep = total <= kKeptMax;
-      if (keep) kept.push_back(KeptTables{p, bytes, dev});
-    }
-    if (!keep) cudaFree(p);
-  }
-};
-}  // namespace
-
-LiveObject::LiveObject() {
-  TableMemory& m = TableMemory::get();
-  std::lock_guard<std::mutex> lock(m.mu);
-  ++m.live;
-}
-LiveObject::~LiveObject() {
-  TableMemory& m = TableMemory::get();
-  std::lock_guard<std::mutex> lock(m.mu);
-  if (--m.live == 0) m.release_all();
-}
-
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -466,9 +386,9 @@ trdq_status trdq_prepare_weights(const trdq_rotation* rot, const void* W_bf16, i
   const uint64_t row_bytes = eight ? K : K / 2;
   const uint32_t box_bytes = eight ? 128 : 64;
 
-  // ONE device allocation holds every table of every group, table after table, group after group, so that the kernels below
-  // run over all groups in one launch (an allocation that is not reused costs 0.1 - 0.3 ms, and freeing it as much: three a
-  // group made up nearly all of the 3 ms that five groups of 4608 x 1152 took).
+  // ONE device allocation holds every table of every group (a cudaMalloc and its cudaFree cost 0.1 - 0.3 ms each: three a
+  // group made up nearly all of the 3 ms that five groups of 4608 x 1152 took), table after table, group after group, so
+  // that the kernels below run over all groups in one launch.
   size_t total = 0;
   auto place = [&total](size_t bytes) {
     const size_t at = total;
@@ -480,8 +400,8 @@ trdq_status trdq_prepare_weights(const trdq_rotation* rot, const void* W_bf16, i
   const size_t colsum_at = eight ? place(static_cast<size_t>(G) * N * sizeof(int32_t)) : 0;
   const size_t mult_at = eight ? 0 : place(static_cast<size_t>(G) * scale_groups * n_pad * sizeof(int32_t));
   const size_t base_at = eight ? 0 : place(static_cast<size_t>(G) * n_pad * sizeof(float));
-  w->tables = TableMemory::get().take(w->device, total, static_cast<cudaStream_t>(stream), &w->table_bytes);
-  if (!w->tables) {
+  if (cudaMalloc(&w->tables, total) != cudaSuccess) {
+    cudaGetLastError();
     trdq_weights_destroy(w);
     return TRDQ_ERR_NOMEM;
   }
@@ -550,7 +470,7 @@ trdq_status trdq_prepare_weights(const trdq_rotation* rot, const void* W_bf16, i
 
 trdq_status trdq_weights_destroy(trdq_weights* w) {
   if (!w) return TRDQ_OK;
-  if (w->tables) TableMemory::get().give(w->device, w->tables, w->table_bytes);
+  if (w->tables) cudaFree(w->tables);
   delete w;
   return TRDQ_OK;
 }

@@ -9,18 +9,7 @@
 
 #include "../../include/trdq.h"
 
-namespace trdq {
-// Counts the rotations and weights that exist; with the last of them the table memory kept for reuse is given back.
-struct LiveObject {
-  LiveObject();
-  ~LiveObject();
-  LiveObject(const LiveObject&) = delete;
-  LiveObject& operator=(const LiveObject&) = delete;
-};
-}  // namespace trdq
-
 struct trdq_rotation {
-  trdq::LiveObject live;
   int32_t K = 0;
   int32_t num_groups = 0;
   int device = 0;
@@ -57,12 +46,10 @@ struct GroupWeights {
 }  // namespace trdq
 
 struct trdq_weights {
-  trdq::LiveObject live;
   int32_t N = 0, K = 0, wbits = 8, num_groups = 0;
   int device = 0;
   std::vector<int32_t> t_bounds;
   void* tables = nullptr;  // dev: the one allocation all tables of all groups point into
-  size_t table_bytes = 0;  // size of that allocation
   std::vector<trdq::GroupWeights> groups;
 };
 
