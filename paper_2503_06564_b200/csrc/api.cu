@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 #include <new>
 
@@ -199,6 +200,12 @@ __global__ void selftest_wait_expiry_kernel(uint32_t* status) {
   w.wait(smem_u32(&bar), 0);
 }
 
+// Device memory of an object that is destroyed.  A cudaFree that is refused (a stream capture is open that forbids it) leaves its error for the next
+// cudaGetLastError, with which the launchers check their launches: it is taken back here.
+static void free_device(void* p) {
+  if (p && cudaFree(p) != cudaSuccess) cudaGetLastError();
+}
+
 }  // namespace trdq
 
 using namespace trdq;
@@ -326,12 +333,7 @@ trdq_status trdq_zigzag_permutation(const float* magnitude, int32_t K, int32_t* 
 
 trdq_status trdq_rotation_destroy(trdq_rotation* rot) {
   if (!rot) return TRDQ_OK;
-  if (rot->act_vec) cudaFree(rot->act_vec);
-  if (rot->weight_vec) cudaFree(rot->weight_vec);
-  if (rot->perm) cudaFree(rot->perm);
-  if (rot->vec2) cudaFree(rot->vec2);
-  if (rot->dense) cudaFree(rot->dense);
-  if (rot->dense_inv_t) cudaFree(rot->dense_inv_t);
+  for (void* const p : std::initializer_list<void*>{rot->act_vec, rot->weight_vec, rot->perm, rot->vec2, rot->dense, rot->dense_inv_t}) free_device(p);
   delete rot;
   return TRDQ_OK;
 }
@@ -470,7 +472,7 @@ trdq_status trdq_prepare_weights(const trdq_rotation* rot, const void* W_bf16, i
 
 trdq_status trdq_weights_destroy(trdq_weights* w) {
   if (!w) return TRDQ_OK;
-  if (w->tables) cudaFree(w->tables);
+  free_device(w->tables);
   delete w;
   return TRDQ_OK;
 }

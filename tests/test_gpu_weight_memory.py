@@ -115,6 +115,19 @@ graph.replay()
 torch.cuda.synchronize()
 assert float(y.sum()) == 2048.0
 
+# objects destroyed by a thread that captures: the capture is lost, the next calls are not
+for bits in (8, 4):
+    for obj in (trdq.trdq_prepare_weights(rot, x, bits), rotation(256, 2)):
+        torch.cuda.synchronize()
+        try:
+            with torch.cuda.graph(torch.cuda.CUDAGraph(), capture_error_mode="thread_local"):
+                obj.close()
+            raise SystemExit("memory was freed inside a capture")
+        except RuntimeError:
+            pass
+        torch.cuda.synchronize()
+        trdq.trdq_prepare_weights(rot, x, bits).close()
+
 # everything is returned at once, with rotations and other weights alive: another allocator may want it
 big = [rotation(4608, 4), rotation(4608, 1)]
 x = weight(16384, 4608, 3)
