@@ -62,8 +62,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float2 v) {
 }
 
 // GELU of 2 PAIRS values, packed to bf16.  One test for all of them: from -9.75 up 2^x is a normal number and both forms of it agree.
-// 1152 -> 4608 with GELU, without / with the test: 22.8 -> 22.1 us at M = 4096, 79.4 -> 76.7 at 16384 (before the epilogue had sixteen warps it
-// waited more than it issued, and the test gained nothing; nor does it in the 4-bit kernel, 264 against 269 us).
+// For kernels that issue more than they wait, the CTA-pair GEMM: 1152 -> 4608 with GELU, without / with the test, 22.8 -> 22.1 us at M = 4096, 79.4 -> 76.7
+// at 16384.  Where a CTA has one or two tiles the test only adds to the last epilogue (single-CTA GEMM, N x M: K = 1152, 1152 x 700 5.74 -> 5.94 us,
+// K = 4608, 384 x 1400 9.84 -> 10.06), and the 4-bit kernel is no faster with it (264 -> 269).
 template <int PAIRS>
 __device__ __forceinline__ void gelu_pack(const float2 (&v)[PAIRS], uint32_t (&packed)[PAIRS]) {
   float lowest = v[0].x;
@@ -98,7 +99,9 @@ struct ColumnParamLayout {  // [sw BN][bias BN][thr BN / 8], 16-byte aligned
   static constexpr int kBytes = kFloats * 4;
 };
 
-// COLS (16 or 32) consecutive columns (the c-th such group of the tile) of one output row: y = acc * sx * sw[n] + bias[n] (then GELU if ACT),
+enum EpilogueAct { kActNone, kActGelu, kActGeluTested };  // kActGeluTested: through gelu_pack
+
+// COLS (16 or 32) consecutive columns (the c-th such group of the tile) of one output row: y = acc * sx * sw[n] + bias[n] (then GELU, see ACT),
 // packed to bf16 pairs.  Packed fp32x2 arithmetic, the same roundings as dequant_one; the cancellation against the bias is
 // looked for once per row and eight columns (smallest |y| against the largest threshold of the eight).  Where it may have
 // happened the eight are held against their own thresholds, and only those below are repaired: with a bias of the output's size a
@@ -106,7 +109,7 @@ struct ColumnParamLayout {  // [sw BN][bias BN][thr BN / 8], 16-byte aligned
 // Microseconds of the GEMM with each column tested by itself / one test per 32 columns that repairs all of them / this, for a bias
 // of a hundredth of the output's size and one of twice its size: M = 4096, 1152 -> 4608 19.1 / 17.1 / 17.4 and 19.1 / 20.7 / 18.4, M = 16384,
 // 1152 -> 3456 54.7 / 52.7 / 51.7 and 54.5 / 59.4 / 52.9.  One test per four columns costs more than it saves (17.3 and 19.8).
-template <int COLS, bool ACT>
+template <int COLS, EpilogueAct ACT>
 __device__ __forceinline__ void dequant_row(const uint32_t (&r)[COLS], float sxm, const ColumnParams& cp, int c, uint32_t (&packed)[COLS / 2]) {
   static_assert(COLS == 16 || COLS == 32, "two or four tests");
   const float4* sw4 = reinterpret_cast<const float4*>(cp.sw + c * COLS);
@@ -151,11 +154,11 @@ __device__ __forceinline__ void dequant_row(const uint32_t (&r)[COLS], float sxm
       }
     }
   }
-  if constexpr (ACT) {
+  if constexpr (ACT == kActGeluTested) {
     gelu_pack(v, packed);
   } else {
 #pragma unroll
-    for (int j = 0; j < COLS / 2; ++j) packed[j] = pack_bf16(v[j]);
+    for (int j = 0; j < COLS / 2; ++j) packed[j] = pack_bf16(ACT == kActGelu ? gelu_tanh2<false>(v[j]) : v[j]);
   }
 }
 

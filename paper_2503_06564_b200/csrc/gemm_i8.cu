@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w8a8_kernel(const __grid_con
         }
         if (MODE != 1) {
           uint32_t packed[16];
-          dequant_row<32, MODE == 3>(r, sxm, cp, c, packed);
+          dequant_row<32, MODE == 3 ? kActGelu : kActNone>(r, sxm, cp, c, packed);
           // staging tile: row = lane, 64 bytes per row, 16-byte chunk j stored at j ^ ((lane >> 1) & 3)
           if (lane == 0) bulk_wait_group_read<0>();  // the previous store has finished reading the tile
           __syncwarp();

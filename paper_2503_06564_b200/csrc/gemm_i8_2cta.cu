@@ -173,7 +173,7 @@ __host__ __device__ constexpr uint32_t umma_idesc_s8_pair(int n, bool unsigned_a
 template <int BN, int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Cfg2<BN, MODE>::kThreads, 1) gemm_w8a8_pair_kernel(const __grid_constant__ Gemm2Params p) {
   using C = Cfg2<BN, MODE>;
-  constexpr bool ACT = MODE == kPairGelu || MODE == kPairGeluLong;
+  constexpr EpilogueAct ACT = MODE == kPairGelu || MODE == kPairGeluLong ? kActGeluTested : kActNone;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
