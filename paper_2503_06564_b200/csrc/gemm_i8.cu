@@ -362,17 +362,33 @@ int choose_tile_n(int64_t tiles_m, int N, int sms) {
 // 2048 x 2560 (80);  K = 4608: 13.8 / 12.9 at 1152 x 3072 (54), 16.1 / 16.7 at 1536 x 2560 (60), 18.5 / 19.5 at 256 x 12288 (48);
 // K = 12288: 21.9 / 26.9 at 768 x 2560 (30).  Averaged over the points the rule is 0.1 % off the faster kernel, the pair kernel everywhere
 // 4.6 %, the other 3.4 %.  These are times of both kernels with epilogue parameters loaded tile by tile; with parameters staged ahead in
-// the pair kernel the longer epilogues change over earlier, and from half the rows on.  Mean pair / single CTA at 78 - 95, 95 - 110 and 135 - 165
-// tiles (sixteen K, six N, M from 1037 to 12288): GELU 0.95, 0.98, 0.92 at K = 640 ... 1023, 0.93, 0.97, 0.92 at 1024 ... 1279, 0.94, 0.96, 0.92
-// at 1536 ... 2303 and 0.89 ... 0.97 below 2048 rows; asymmetric codes 1.00, 1.02, 0.96 at K = 640 ... 1023, 0.96, 0.99, 0.94 at 1024 ... 1535 and
-// 0.92 ... 0.99 below 2048 rows; both 1.04 ... 1.10 at 56 - 78 tiles.
+// the pair kernel the longer epilogues change over earlier, see pair_earlier.
 // TRDQ_PAIR_MIN_M (read once per process) replaces the rule by a row count.
 static int pair_least_tiles(int32_t K, int32_t N, bool gelu, bool asym) {
   if (K >= 7168) return 0;
   if (K >= 6144) return 40;
   if (K >= 4096) return N <= 256 ? 46 : 56;
-  if (K >= 1536 || gelu || (asym && K >= 1024)) return 78;
-  return asym ? 135 : K < 1024 ? 165 : 110;
+  if (K >= 1536) return gelu && K < 2304 ? 110 : 78;
+  return K < (asym ? 1280 : 1024) ? 165 : 110;
+}
+// The same for GELU and asymmetric codes with reductions below 2304, where the single-CTA kernel's epilogue weighs most: from half the rows and 78
+// tiles on (asymmetric codes below K = 1024: 135 tiles and 2048 rows), unless the pair kernel's tiles fall into rounds that leave an SM with more
+// columns.  A round is charged its width and 80 columns for its start; when both kernels need two rounds, of 256 columns here and of 192 there, the pair
+// kernel took 1.02 - 1.18 of the other's time (GELU, N x M, single CTA / pair: 4096 x 1539 at K = 2048 14.4 / 17.0 us, 2704 x 2349 at K = 1152
+// 12.1 / 12.5; asymmetric 4096 x 1543 at K = 1408 10.5 / 11.5), with K < 384 also where it needs a third round (asymmetric 3456 x 2586 at K = 128
+// 8.4 / 9.0), beyond that a third round costs it nothing (0.98 on average).  Over 1058 points between the two lines the rule gives 0.95 of
+// the single-CTA kernel's time on average, 0.80 at best and 1.04 at worst (GELU at K = 1920 and 2048).
+static bool pair_earlier(int64_t M, int32_t K, int32_t N, bool asym, int sms) {
+  const bool later = asym && K < 1024;
+  if (M < (later ? 2048 : 1024) || M * N < (later ? 135 : 78) * 65536ll) return false;
+  int width = 0;
+  int64_t rounds = 0;
+  if (!gemm_w8_pair_rounds((M + 2 * kTileM - 1) / (2 * kTileM), N, &width, &rounds)) return false;
+  if (rounds > 2 && K >= 384) return true;
+  const int64_t tiles_m = (M + kTileM - 1) / kTileM;
+  const int single = kTileN[choose_tile_n(tiles_m, N, sms)];
+  const int64_t single_rounds = (tiles_m * ((N + single - 1) / single) + sms - 1) / sms;
+  return rounds * (width + 80) <= single_rounds * (single + 80);
 }
 static bool use_pair(int64_t M, int32_t K, int32_t N, bool gelu, bool asym) {
   static const int forced = [] {
@@ -380,8 +396,11 @@ static bool use_pair(int64_t M, int32_t K, int32_t N, bool gelu, bool asym) {
     return e ? atoi(e) : -1;
   }();
   if (forced >= 0) return M >= forced;
-  const bool long_epilogue = (gelu && K < 2304) || (asym && K >= 1024 && K < 2304);
-  return M >= (long_epilogue ? 1024 : 2048) && M * N >= pair_least_tiles(K, N, gelu, asym) * 65536ll;
+  if (M >= 2048 && M * N >= pair_least_tiles(K, N, gelu, asym) * 65536ll) return true;
+  if (!(gelu || asym) || K >= 2304) return false;
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return pair_earlier(M, K, N, asym, sms);
 }
 
 // Name of the kernel trdq_linear runs for M rows against [N, K] weights of `wbits` bits (one row segment).

@@ -612,11 +612,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCeilingThreads, 1) 
 
 }  // namespace
 
+bool gemm_w8_pair_rounds(int64_t tiles_m, int N, int* width, int64_t* rounds) {
+  int dev = 0, clusters = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  const int i = pair_tile_choice(tiles_m, N, dev, &clusters);
+  if (i < 0) return false;
+  *width = kTileN[i];
+  *rounds = (tiles_m * ((N + kTileN[i] - 1) / kTileN[i]) + clusters - 1) / clusters;
+  return true;
+}
+
 int gemm_w8_pair_tile_width(int64_t tiles_m, int N) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  const int i = pair_tile_choice(tiles_m, N, dev, nullptr);
-  return i < 0 ? 0 : kTileN[i];
+  int width = 0;
+  int64_t rounds = 0;
+  return gemm_w8_pair_rounds(tiles_m, N, &width, &rounds) ? width : 0;
 }
 
 trdq_status launch_mma_ceiling(int32_t mmas_per_cluster, int32_t* clusters_out, cudaStream_t stream) {

@@ -147,7 +147,9 @@ trdq_status launch_gemm_w8_splitk_static(const trdq_weights* w, int g, const Gem
 // which kernel a call would run (for reports; the launchers use the same functions)
 void describe_rotate_quantize_kernel(int32_t M, int32_t K, char* name, size_t cap);
 void describe_gemm_kernel(int32_t M, int32_t K, int32_t N, int32_t wbits, char* name, size_t cap);
-int gemm_w8_pair_tile_width(int64_t pair_tiles_m, int N);  // 0: the pair kernel cannot run on this device
+// tile width the pair kernel takes and rounds of tiles a CTA pair then has; false: it cannot run on this device
+bool gemm_w8_pair_rounds(int64_t pair_tiles_m, int N, int* width, int64_t* rounds);
+int gemm_w8_pair_tile_width(int64_t pair_tiles_m, int N);  // 0: it cannot
 // measurement aid: `mmas_per_cluster` back-to-back 256 x 256 x 32 int8 MMAs per CTA pair on resident operands
 trdq_status launch_mma_ceiling(int32_t mmas_per_cluster, int32_t* clusters_out, cudaStream_t stream);
 // gemm_i8_2cta.cu: CTA-pair kernel; TRDQ_ERR_SHAPE means "not applicable here, use the single-CTA kernel"

@@ -3,6 +3,8 @@ ahead by warps of their own, and with GELU a warp owns 64 columns of a tile."""
 import numpy as np
 import pytest
 
+from tests.util import launched_kernels
+
 pytestmark = pytest.mark.gpu
 
 
@@ -39,9 +41,20 @@ def test_same_bits_as_one_cta_per_tile(M, N, K, width, with_bias):
     assert trdq.trdq_device_status() == 0
 
 
-@pytest.mark.parametrize("M,N,K", [(1100, 4656, 1152), (1999, 2576, 768), (1664, 3072, 768), (1400, 3680, 2176)])
-def test_long_epilogues_take_pairs_from_1024_rows_on(M, N, K):
+GELU, ASYM = "gelu", "asym"
+
+
+@pytest.mark.parametrize("kind,M,N,K,pair", [
+    (GELU, 1100, 4656, 1152, True), (GELU, 1999, 2576, 768, True), (GELU, 1664, 3072, 768, True), (GELU, 1400, 3680, 2176, True),
+    (ASYM, 1100, 4656, 1152, True), (ASYM, 1400, 3680, 2176, True), (ASYM, 1999, 2576, 1024, True), (ASYM, 2900, 3072, 768, True),
+    (ASYM, 1999, 4608, 768, False),    # below 2048 rows
+    (GELU, 1999, 2416, 1152, False),   # below 78 tiles
+    (GELU, 2330, 2704, 1152, False), (GELU, 1550, 4096, 1792, False), (ASYM, 1543, 4096, 1408, False),   # two wide rounds against two narrower ones
+    (ASYM, 2574, 3456, 256, False), (ASYM, 2574, 3456, 384, True),     # a third round
+])
+def test_long_epilogues_take_pairs_from_1024_rows_on(kind, M, N, K, pair):
     """GELU and asymmetric codes change to CTA pairs earlier than the plain epilogue: the same bits as in pieces that do not."""
+    import os
     import torch
     from paper_2503_06564_b200 import trdq
     g = torch.Generator(device="cuda").manual_seed(M + N)
@@ -51,9 +64,17 @@ def test_long_epilogues_take_pairs_from_1024_rows_on(M, N, K):
     scales = torch.rand((M,), generator=g, device="cuda") * 0.01
     zero = torch.randint(0, 256, (M,), generator=g, device="cuda", dtype=torch.int32)
     bias = torch.randn((N,), generator=g, device="cuda").to(torch.bfloat16)
-    for call in (lambda c, s, z: trdq.trdq_linear_act(wts, 0, c, s, bias), lambda c, s, z: trdq.trdq_linear_asym(wts, 0, c.view(torch.uint8), s, z, bias)):
-        whole = call(codes, scales, zero)
-        for a in range(0, M, 700):
-            part = slice(a, min(a + 700, M))
-            assert torch.equal(whole[part].view(torch.int16), call(codes[part].clone(), scales[part].clone(), zero[part].clone()).view(torch.int16))
+    if kind == GELU:
+        call = lambda c, s, z: trdq.trdq_linear_act(wts, 0, c, s, bias)
+    else:
+        call = lambda c, s, z: trdq.trdq_linear_asym(wts, 0, c.view(torch.uint8), s, z, bias)
+    whole = call(codes, scales, zero)
+    for a in range(0, M, 700):
+        part = slice(a, min(a + 700, M))
+        piece = [t[part].clone() for t in (codes, scales, zero)]
+        assert torch.equal(whole[part].view(torch.int16), call(*piece).view(torch.int16))
+    if "TRDQ_PAIR_MIN_M" not in os.environ:
+        for args, expected in (((codes, scales, zero), pair), (piece, False)):
+            (name, _, _), = launched_kernels(lambda: call(*args))
+            assert ("gemm_w8a8_pair_kernel" if expected else "gemm_w8a8_kernel") in name, name
     assert trdq.trdq_device_status() == 0

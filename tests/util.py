@@ -1,4 +1,6 @@
 """Helpers shared by the GPU parity tests: tensor transport and the comparison rules."""
+import ctypes
+
 import numpy as np
 
 from paper_2503_06564_b200 import workloads as WL
@@ -78,3 +80,33 @@ def check_codes_with_tolerance(codes: np.ndarray, scales: np.ndarray, v_ref: np.
         assert np.all(dist[bad] <= du[bad]), "a differing code is not at a rounding boundary"
         assert bad.sum() <= max_fraction * codes.size, f"{bad.sum()} of {codes.size} codes differ"
     return int(bad.sum())
+
+
+class _KernelNodeParams(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS of the driver API
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3), ("shared", ctypes.c_uint),
+                ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p), ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def launched_kernels(call):
+    """(mangled name, grid, block) of every kernel that `call` launches on the current stream, read from a captured graph that is never run.
+    `call` must have run once before (kernels configured) and its outputs are not computed."""
+    import torch
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    cu = ctypes.CDLL("libcuda.so.1")
+    raw, count = ctypes.c_void_p(int(graph.raw_cuda_graph())), ctypes.c_size_t(0)
+    assert cu.cuGraphGetNodes(raw, None, ctypes.byref(count)) == 0
+    nodes = (ctypes.c_void_p * count.value)()
+    assert cu.cuGraphGetNodes(raw, nodes, ctypes.byref(count)) == 0
+    found = []
+    for node in nodes:
+        kind, p, name = ctypes.c_int(), _KernelNodeParams(), ctypes.c_char_p()
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value != 0:   # a kernel node
+            continue
+        assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)) == 0
+        get, handle = (cu.cuFuncGetName, p.func) if p.func else (cu.cuKernelGetName, p.kern)
+        assert get(ctypes.byref(name), ctypes.c_void_p(handle)) == 0
+        found.append((name.value.decode(), tuple(p.grid), tuple(p.block)))
+    return found
