@@ -188,13 +188,17 @@ cudaError_t launch_norm_rotate_quantize(const void* x_bf16, int64_t ldx, int32_t
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // The form that requests the modulation ahead keeps 64 more bytes a thread and so at most 64 lane groups (256 threads of 128 registers) in a
-  // CTA, the other 72.  It is 4 - 25 % faster (K = 1152: 5.3 -> 4.7 us at M = 1037, 9.1 -> 8.5 at 4096, 17.3 -> 16.2 at 8192, 31.8 -> 30.1 at 16384)
-  // where its fewer rows do not cost a round; where they cost more than a tenth (K = 640, M = 4096: 6.3 -> 8.2), and for rows
-  // of more than 12 blocks (K = 4608: one row a CTA in place of two, 33 -> 49), the other one runs.
+  // CTA, the other 72.  It runs where its fewer rows cost no round: followed by the GEMM that reads the codes (N = 1152), the two together took 0.95 of
+  // the time with the other form over 310 points (K = 1152: 9.8 -> 9.0 us at M = 800, 16.8 -> 16.4 at 4096, 29.1 -> 28.1 at 8192), at best 0.86 and at worst,
+  // one round of 150 - 200 tiles, 1.05; without modulation 0.97.  (Launched again and again by itself it takes 0.93, but 1.1 - 1.25 where its
+  // tiles are exactly one or two rounds: the next launch finds fewer free registers.)  From four rounds on it also pays for up to a tenth more cost (K = 1152, M = 16384: 53.9 -> 51.0
+  // in eight rounds in place of seven); with fewer it does not (K = 384, M = 7104: 13.9 -> 15.8 in two in place of one).  Rows
+  // of more than 12 blocks (K = 4608: one row a CTA in place of two, 33 -> 49) take the other form, and so do rows of one or two (0.95 with this one).
   const int rows_plain = rows_per_tile_by_rounds(M, std::max(1, std::min(32, 72 / nb)), sms);
   const int rows_ahead = rows_per_tile_by_rounds(M, std::max(1, std::min(32, 64 / nb)), sms);
-  const auto cost = [&](int r) { return static_cast<int64_t>(((M + r - 1) / r + 2 * sms - 1) / (2 * sms)) * (r + 2); };
-  const bool ahead = nb >= 3 && nb <= 12 && 9 * cost(rows_ahead) <= 10 * cost(rows_plain);
+  const auto rounds = [&](int r) { return static_cast<int64_t>(((M + r - 1) / r + 2 * sms - 1) / (2 * sms)); };
+  const int64_t cost_plain = rounds(rows_plain) * (rows_plain + 2), cost_ahead = rounds(rows_ahead) * (rows_ahead + 2);
+  const bool ahead = nb >= 3 && nb <= 12 && (cost_ahead <= cost_plain || (rounds(rows_plain) >= 4 && 9 * cost_ahead <= 10 * cost_plain));
   const int rows = ahead ? rows_ahead : rows_plain;
   const int threads = (rows * nb * kFastLanes + 31) / 32 * 32;
   const size_t smem = (static_cast<size_t>(K) + 4u * rows * nb) * sizeof(float);
