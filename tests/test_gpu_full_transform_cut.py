@@ -3,6 +3,8 @@ rows and the codes of a team taking turns in one buffer."""
 import numpy as np
 import pytest
 
+from tests.util import launched_kernels
+
 pytestmark = pytest.mark.gpu
 
 
@@ -32,7 +34,11 @@ def test_same_bits_as_lane_groups(M, K, piece, pad):
     x[M // 2] = 0.0
     x[M - 1, ::3] = float("inf")
     codes, scales = trdq.trdq_rotate_quantize(rot, 0, x)
+    (name, _, _), = launched_kernels(lambda: trdq.trdq_rotate_quantize(rot, 0, x, codes, scales))
+    assert "rotate2_quantize_team_kernel" in name, name
     for a in range(0, M, piece):
         c, s = trdq.trdq_rotate_quantize(rot, 0, x[a:a + piece])
+        (name, _, _), = launched_kernels(lambda: trdq.trdq_rotate_quantize(rot, 0, x[a:a + piece], c, s))
+        assert "rotate2_quantize_rows_kernel" in name, (a, name)
         assert torch.equal(c, codes[a:a + piece]) and torch.equal(s.view(torch.int32), scales[a:a + piece].view(torch.int32)), a
     assert trdq.trdq_device_status() == 0

@@ -33,8 +33,11 @@ def test_same_bits_as_one_cta_per_tile(M, N, K, width, with_bias):
     calls = [lambda c, s, z: trdq.trdq_linear(wts, 0, c, s, bias),
              lambda c, s, z: trdq.trdq_linear_act(wts, 0, c, s, bias),
              lambda c, s, z: trdq.trdq_linear_asym(wts, 0, c.view(torch.uint8), s, z, bias)]
-    for call in calls:
+    warps = [8, width // 16 if K <= 1792 else 8, 8]   # epilogue warps
+    for call, ew in zip(calls, warps):
         whole = call(codes, scales, zero)
+        (name, _, block), = launched_kernels(lambda: call(codes, scales, zero))
+        assert f"gemm_w8a8_pair_kernelILi{width}E" in name and block[0] == 128 + 32 * ew, (name, block)
         for a in (0, 4000, M - 2000):
             part = slice(a, a + 2000)
             assert torch.equal(whole[part].view(torch.int16), call(codes[part].clone(), scales[part].clone(), zero[part].clone()).view(torch.int16))
