@@ -46,9 +46,10 @@ struct Cfg2 {
   // Epilogue warps: eight, each with half of the tile's columns, or (mode 1) one per 32 x 64 piece of the tile: sixteen at BN = 256.
   // GELU makes the epilogue longer than the main loop of a short reduction (two special-function instructions and some twenty
   // others a value), and with two warps a scheduler half of the issue slots stay empty.  But the staging tiles of sixteen warps take the
-  // memory of a pipeline stage, which costs long reductions, and launches without GELU, 2 - 10 %.  Microseconds with eight / sixteen
-  // warps at M = 16384, N = 4608: K = 768 85.1 / 69.5, 1152 87.0 / 77.1, 1536 95.3 / 87.5, 1792 101.2 / 97.5, 2048 107.3 / 107.5,
-  // 2304 115.9 / 118.2, 4608 209.1 / 217.8; N = 768: K = 1152 21.9 / 20.2, 1792 24.0 / 24.8, 2304 26.4 / 28.9.
+  // memory of a pipeline stage, which costs long reductions, and launches without GELU, 2 - 10 %.  Sixteen warps against eight over 44 points each,
+  // M = 1400 ... 16384: 0.94 of the time at K = 1664, 0.96 at 1792 (none slower; N = 768, M = 16384: 22.5 -> 21.8 us), 0.98 at 1920 (0.90 ... 1.04).  Microseconds with
+  // eight / sixteen at M = 16384, N = 4608: K = 1664 117 / 107, 1792 121.1 / 115.5, 1920 120.6 / 122.3; before GELU's test for subnormal powers: K = 768 85.1 / 69.5,
+  // 1152 87.0 / 77.1, 2304 115.9 / 118.2, 4608 209.1 / 217.8.
   static constexpr bool kWarpPerTile = MODE == kPairGelu;
   static constexpr int kEpilogueWarps = kWarpPerTile ? BN / 16 : 8;
   static constexpr int kEpilogueThreads = 32 * kEpilogueWarps;

@@ -191,7 +191,7 @@ cudaError_t launch_norm_rotate_quantize(const void* x_bf16, int64_t ldx, int32_t
   // CTA, the other 72.  It runs where its fewer rows cost no round: followed by the GEMM that reads the codes (N = 1152), the two together took 0.95 of
   // the time with the other form over 310 points (K = 1152: 9.8 -> 9.0 us at M = 800, 16.8 -> 16.4 at 4096, 29.1 -> 28.1 at 8192), at best 0.86 and at worst,
   // one round of 150 - 200 tiles, 1.05; without modulation 0.97.  (Launched again and again by itself it takes 0.93, but 1.1 - 1.25 where its
-  // tiles are exactly one or two rounds: the next launch finds fewer free registers.)  From four rounds on it also pays for up to a tenth more cost (K = 1152, M = 16384: 53.9 -> 51.0
+  // tiles are exactly one or two rounds of CTAs.)  From four rounds on it also pays for up to a tenth more cost (K = 1152, M = 16384: 53.9 -> 51.0
   // in eight rounds in place of seven); with fewer it does not (K = 384, M = 7104: 13.9 -> 15.8 in two in place of one).  Rows
   // of more than 12 blocks (K = 4608: one row a CTA in place of two, 33 -> 49) take the other form, and so do rows of one or two (0.95 with this one).
   const int rows_plain = rows_per_tile_by_rounds(M, std::max(1, std::min(32, 72 / nb)), sms);

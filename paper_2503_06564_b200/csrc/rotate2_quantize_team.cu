@@ -11,8 +11,9 @@
 // is rows in flight that count, and one buffer per team has to do for everything: the input tile lies in its first half until it is
 // in registers, then the rotated rows take all of it, and the codes its last quarter, while the next input already arrives in the
 // first half.  A separate input tile (requested most of a tile's time ahead) left room for 0.55 - 0.75 of the lanes of twelve warps; now
-// it is 0.84 - 1.0.  Microseconds before -> now, M = 16384: K = 1152 28.7 -> 24.9, 1536 43.3 -> 28.9, 2304 58.5 -> 49.2, 3072 72.8 -> 58.8,
-// 4608 115 -> 102; M = 4096: K = 1152 9.4 -> 8.5, 4608 36.2 -> 31.8, 7680 68.0 -> 54.9.
+// it is 0.84 - 1.0.  Microseconds before -> now, M = 16384: K = 1152 27.9 -> 22.4, 1536 42.0 -> 26.4, 2304 58.2 -> 49.0, 3072 72.7 -> 53.6,
+// 4608 115 -> 102; M = 4096: K = 1152 8.8 -> 7.8, 4608 33.4 -> 30.0, 7680 68.8 -> 54.5.  0.86 of the time over 401 points; five are slower by more than
+// 1.5 %, where the larger tiles used before filled the last round better (K = 640 at M = 5000: 7.2 -> 7.8, K = 512 at 16384: 12.3 -> 12.7).
 // The row buffer is swizzled (16-byte chunk index xor block) and rows are 48 bytes apart modulo 128, so that the writes of a
 // quarter warp and the rows of one channel fall into different banks.
 #include <cuda_bf16.h>
@@ -189,7 +190,7 @@ size_t team2_smem_bytes(int K, int R, int teams, bool input_apart = false) {
 // multiple of eight rows gather with fewer conflicts (K = 1408 at M = 16384: 8 rows 28.9 us, 7 rows 36.9), even numbers are a
 // little ahead of odd ones; two teams overlap less than three; and warps that do not divide by the four schedulers leave some of
 // them idle.  The shapes taken are 1.4 % off the best ones on average, by lanes alone 5.3 %.  A tile is at most two thirds of an SM's share of the
-// rows, or an SM would have nothing to overlap.  At least two teams (rows of up to 72 blocks; offsets of 16 bits would reach 128).
+// rows, or an SM would have nothing to overlap.  At least two teams (the memory allows it for rows of up to 98 blocks; offsets of 16 bits would reach 128).
 bool choose_team2_shape(int M, int K, int sms, Team2Shape* out) {
   const int nb = K / TRDQ_BLOCK;
   Team2Shape best = {0, 0, 0, 0, 0.0};
@@ -213,7 +214,8 @@ bool choose_team2_shape(int M, int K, int sms, Team2Shape* out) {
   return true;
 }
 
-// The cut the dispatch line below was drawn with: by lanes alone (the fuller teams of two that are alike), with an input tile of its own per team.
+// What the dispatch line below is drawn with: not the cut that is launched, but that of an earlier form of the kernel, by lanes alone (the fuller teams of two
+// that are alike) and with an input tile of its own per team.
 bool line_team2_shape(int K, Team2Shape* out) {
   const int nb = K / TRDQ_BLOCK;
   Team2Shape best = {0, 0, 0, 0, 0.0};
@@ -232,20 +234,14 @@ bool line_team2_shape(int K, Team2Shape* out) {
 
 }  // namespace
 
-// The team kernel serves rows that keep at least 0.45 of the lanes of twelve warps busy (K = 7680: 72 -> 64 us at M = 4096;
-// K = 8192, 0.33 of the lanes: 75 against 84 us), from the row count on at which it stays ahead of the lane-group kernel.  With fewer
-// rows both take one pass and the shorter one wins: a thread of this kernel transforms a whole block twice and gathers 128
-// values, of that kernel a quarter of one.  So the line is drawn in rounds of that kernel, the rows its two CTAs per SM take
-// at once, over M in steps of 12 % from one row per SM to 24 million values:
-//   one block per row 0.94 rounds (K = 128: 5.6 / 6.3 us at M = 8024, lane groups / teams, 7.4 / 6.4 at 8987);
-//   rows of up to ten blocks 0.54 (the second CTA of an SM starts to count; K = 1024: 6.3 / 7.2 at M = 1306, 7.7 / 7.2 at 1463);
-//   rows of up to 24 blocks 1.1 (K = 2048: 6.9 / 8.0 at M = 1166, 9.2 / 8.1 at 1306), up to 36 blocks 1.3 (K = 4608: 10.4 / 10.5 at
-//   M = 740, 13.8 / 10.9 at 829);
-//   wider rows, one per lane-group CTA, 1.6 (K = 6144: 12.2 / 12.8 at M = 417, 12.9 / 12.7 at 468));
-//   and where a team's tile is a single row, eleven rows per SM (K = 4096: 12.4 / 14.0 at M = 1166, 17.4 / 14.8 at 1639;
-//   K = 7680: 22.1 / 24.2 at M = 1166, 31.5 / 29.3 at 1639).
-// These are timings of the form with an input tile of its own, and the line is kept where they put it: above it the present form is the faster of
-// the two, below it the lane groups still are for most shapes (K = 8192 would change sides at about M = 1200).
+// From which row count on the team kernel serves rows of K channels.  With few rows both kernels take one pass and the shorter one wins: a thread of this
+// kernel transforms a whole block twice and gathers 128 values, of the lane-group kernel a quarter of one.  The line is drawn in rounds of that kernel,
+// the rows its two CTAs per SM take at once: 0.94 for one block per row, 0.54 up to ten blocks, 1.1 up to 24, 1.3 up to 36, 1.6 beyond, eleven
+// rows per SM where the earlier form held one row per team; and where that form used less than 0.45 of the lanes (K = 6784 ... 7296, 8192 and more) the
+// lane groups serve all row counts.  It lies where the earlier form changed sides, to the safe side of the present one: of 401 timed points above it
+// (K = 128 ... 9216, M = 300 ... 16384) none is slower than the lane groups, 0.66 of their time on average (K = 1024: 7.6 / 6.8 us at M = 1480, lane groups / teams;
+// K = 4096: 17.1 / 13.2 at 1639; K = 6144: 21.4 / 18.0 at 1480); of 471 below it the present form would be faster by more than 1.5 % at 214 (K = 4608: 10.1 / 9.6 at M = 740;
+// K = 4096: 11.9 / 9.2 at 829; K = 8192: 74.2 / 57.4 at 4096), and slower, up to twice, at the fewest rows.
 bool rotate2_prefers_team(int32_t M, int32_t K) {
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
