@@ -51,6 +51,7 @@ def main():
     ap.add_argument("--sets", type=int, default=4)
     ap.add_argument("--mmas", type=int, default=65536, help="ceiling: MMAs (256 x 256 x 32, int8) per CTA pair and launch")
     ap.add_argument("--full-transform", action="store_true", help="rq: rotation, zigzag permutation, second rotation (Eq. 9)")
+    ap.add_argument("--gelu", action="store_true", help="gemm: GELU in the epilogue (trdq_linear_act)")
     ap.add_argument("--splitk", action="store_true", help="gemm: use trdq_linear_splitk with a preallocated workspace")
     ap.add_argument("--no-graph", action="store_true", help="time individual launches issued from Python (profiler runs)")
     args = ap.parse_args()
@@ -108,6 +109,8 @@ def main():
             s = i % args.sets
             if args.splitk:
                 trdq.trdq_linear_splitk(wts, 0, codes[s], scales[s], bias, ys[s], ws)
+            elif args.gelu:
+                trdq.trdq_linear_act(wts, 0, codes[s], scales[s], bias, ys[s])
             else:
                 trdq.trdq_linear(wts, 0, codes[s], scales[s], bias, ys[s])
         work, unit = 2.0 * M * N * K / 1e12, "TOPS"
