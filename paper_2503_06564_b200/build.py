@@ -1,4 +1,4 @@
-"""Compile the CUDA library (sm_100a) into ``libtrdq.so`` next to this file.
+"""Compile the CUDA library (sm_100a) into ``libtrdq.so`` and the native part of its binding into ``_calls.so``, next to this file.
 
 nvcc cross-compiles without a GPU, so this runs on a CPU-only machine too.  The
 CUDA runtime is linked statically and the driver API is reached through the
@@ -14,6 +14,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libtrdq.so")
+CALLS = os.path.join(HERE, "_calls.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 FLAGS = [
@@ -28,6 +29,23 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def _calls_stale() -> bool:
+    deps = [os.path.join(CSRC, "calls.cpp"), os.path.join(HERE, "..", "include", "trdq.h"), __file__]
+    return not os.path.exists(CALLS) or any(os.path.getmtime(d) > os.path.getmtime(CALLS) for d in deps)
+
+
+def _calls_command() -> list:
+    import sysconfig
+
+    import torch
+    base = os.path.dirname(torch.__file__)
+    include = [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include"),
+               sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")]
+    return [os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            *(f"-I{d}" for d in include), os.path.join(CSRC, "calls.cpp"), "-o", CALLS,
+            "-L" + os.path.join(base, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+
+
 def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
@@ -37,11 +55,21 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _finish(procs) -> None:
+    for p, cmd in procs:
+        if p.wait() != 0:
+            raise RuntimeError("compiler failed: " + " ".join(cmd))
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    procs = []
+    if force or _calls_stale():
+        cmd = _calls_command()
+        procs.append((subprocess.Popen(cmd), cmd))
     if not force and not _stale():
+        _finish(procs)
         return LIB
     objs = []
-    procs = []
     for src in sources():
         obj = os.path.join(CSRC, os.path.basename(src)[:-3] + ".o")
         cmd = [NVCC, *FLAGS, "-c", src, "-o", obj]
@@ -50,9 +78,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             cmd.insert(2, "-v")
         procs.append((subprocess.Popen(cmd), cmd))
         objs.append(obj)
-    for p, cmd in procs:
-        if p.wait() != 0:
-            raise RuntimeError("nvcc failed: " + " ".join(cmd))
+    _finish(procs)
     subprocess.run([NVCC, "-shared", "-cudart", "static", "-o", LIB, *objs], check=True)
     return LIB
 

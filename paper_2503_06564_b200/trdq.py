@@ -1,8 +1,8 @@
-"""ctypes binding of ``libtrdq.so``: argument marshalling only.
+"""Binding of ``libtrdq.so``: argument marshalling only.
 
 Every function here has the name of the C entry point it calls (``include/trdq.h``)
 and does nothing but turn torch tensors into pointers, sizes and the current
-stream.  All arithmetic runs in the CUDA kernels of the library; if the shared
+stream, in native code (``_calls``) for the hot calls on plain CUDA tensors, through ctypes otherwise.  All arithmetic runs in the CUDA kernels of the library; if the shared
 object is missing the import of this module's library handle fails loudly, and
 there is no fallback of any kind.
 """
@@ -127,6 +127,34 @@ def _stream() -> int:
         get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
         _raw_stream = (lambda: get(dev())) if get and dev else (lambda: torch.cuda.current_stream().cuda_stream)
     return _raw_stream()
+
+
+_native = None
+
+
+def _calls():
+    """The native form of the calls below (``csrc/calls.cpp``): it returns None for arguments it leaves to the general way."""
+    global _native
+    if _native is None:
+        import torch  # noqa: F401  (its libraries have to be loaded first)
+        try:
+            from . import _calls as native
+        except ImportError as e:
+            raise ImportError(f"{os.path.join(_HERE, '_calls.so')} is missing or does not fit this torch: build it with "
+                              "`python -m paper_2503_06564_b200.build`") from e
+        l = lib()
+        native.bind(*(C.cast(f, C.c_void_p).value for f in (
+            l.trdq_rotate_quantize, l.trdq_norm_rotate_quantize, l.trdq_rotate_quantize_asym, l.trdq_linear_act, l.trdq_linear_cfg,
+            l.trdq_linear_asym, l.trdq_linear_splitk_workspace, l.trdq_linear_splitk)))
+        _native = native
+    return _native
+
+
+def _done(result, where: str):
+    """The outputs of a native call, or its status as an exception."""
+    if type(result) is int:
+        raise TrdqError(result, where)
+    return result
 
 
 def _plain_empty(like):
@@ -265,6 +293,9 @@ def trdq_prepare_weights(rot: Rotation, W_bf16, wbits: int = 8) -> Weights:
 
 def trdq_rotate_quantize(rot: Rotation, t: int, X_bf16, codes=None, scales=None):
     """codes int8 [M,K], scales fp32 [M] of the rotated activations at time-step t."""
+    done = (_native or _calls()).rotate_quantize(rot._h.value, rot.K, t, X_bf16, codes, scales)
+    if done is not None:
+        return _done(done, "trdq_rotate_quantize")
     import torch
     assert X_bf16.is_cuda and X_bf16.dim() == 2 and X_bf16.element_size() == 2 and X_bf16.stride(1) == 1
     M = int(X_bf16.shape[0])
@@ -282,6 +313,9 @@ def trdq_rotate_quantize(rot: Rotation, t: int, X_bf16, codes=None, scales=None)
 def trdq_norm_rotate_quantize(rot: Rotation, t: int, X_bf16, shift_bf16=None, scale_bf16=None, rows_per_sample: Optional[int] = None,
                               eps: float = 1e-6, codes=None, scales=None):
     """LayerNorm + per-sample modulation + rotation + per-token quantizer in one kernel."""
+    done = (_native or _calls()).norm_rotate_quantize(rot._h.value, rot.K, t, X_bf16, shift_bf16, scale_bf16, rows_per_sample, eps, codes, scales)
+    if done is not None:
+        return _done(done, "trdq_norm_rotate_quantize")
     import torch
     assert X_bf16.is_cuda and X_bf16.dim() == 2 and X_bf16.element_size() == 2 and X_bf16.stride(1) == 1
     M = int(X_bf16.shape[0])
@@ -339,6 +373,9 @@ def trdq_greedy_rotation_block(x_calib, gauss) -> Tuple[np.ndarray, int]:
 
 def trdq_linear(w: Weights, t: int, codes, scales, bias_bf16=None, out=None):
     """bf16 [M,N] output of the integer GEMM with the dequantizing epilogue."""
+    done = (_native or _calls()).linear(w._h.value, w.N, t, codes, scales, bias_bf16, out, ACT_NONE)
+    if done is not None:
+        return _done(done, "trdq_linear")
     import torch
     M = int(codes.shape[0])
     empty = codes.new_empty if type(codes) is torch.Tensor else _plain_empty(codes)
@@ -355,6 +392,9 @@ ACT_NONE, ACT_GELU_TANH = 0, 1
 
 def trdq_linear_act(w: Weights, t: int, codes, scales, bias_bf16=None, out=None, act: int = ACT_GELU_TANH):
     """trdq_linear with the following activation (GELU, tanh form) folded into the epilogue."""
+    done = (_native or _calls()).linear(w._h.value, w.N, t, codes, scales, bias_bf16, out, act)
+    if done is not None:
+        return _done(done, "trdq_linear_act")
     import torch
     M = int(codes.shape[0])
     empty = codes.new_empty if type(codes) is torch.Tensor else _plain_empty(codes)
@@ -368,6 +408,10 @@ def trdq_linear_act(w: Weights, t: int, codes, scales, bias_bf16=None, out=None,
 
 def trdq_linear_cfg(w: Weights, t: int, codes2, scales2, bias_bf16=None, out2=None):
     """Two row segments (conditional, unconditional) through one launch."""
+    if out2 is None:
+        done = (_native or _calls()).linear_cfg(w._h.value, w.N, t, codes2, scales2, bias_bf16)
+        if done is not None:
+            return _done(done, "trdq_linear_cfg")
     import torch
     Ms = [int(c.shape[0]) for c in codes2]
     empty = codes2[0].new_empty if type(codes2[0]) is torch.Tensor else _plain_empty(codes2[0])
@@ -391,6 +435,9 @@ def trdq_linear_splitk_workspace(w: Weights, M: int) -> Tuple[int, int]:
 def trdq_linear_splitk(w: Weights, t: int, codes, scales, bias_bf16=None, out=None, workspace=None):
     """trdq_linear with the reduction split over several CTAs per tile; `workspace` is a device tensor of at least
     the size trdq_linear_splitk_workspace reports (allocated here when omitted)."""
+    done = (_native or _calls()).linear_splitk(w._h.value, w.N, t, codes, scales, bias_bf16, out, workspace)
+    if done is not None:
+        return _done(done, "trdq_linear_splitk")
     import torch
     M = int(codes.shape[0])
     empty = codes.new_empty if type(codes) is torch.Tensor else _plain_empty(codes)
@@ -421,6 +468,9 @@ def trdq_linear_splitk_static(w: Weights, t: int, codes, scales, bias_bf16, out)
 
 def trdq_rotate_quantize_asym(rot: Rotation, t: int, X_bf16):
     """Asymmetric per-token quantizer of Eq. 1-3: (codes uint8 [M,K], scales fp32 [M], zero points int32 [M])."""
+    done = (_native or _calls()).rotate_quantize_asym(rot._h.value, rot.K, t, X_bf16)
+    if done is not None:
+        return _done(done, "trdq_rotate_quantize_asym")
     import torch
     M = int(X_bf16.shape[0])
     empty = X_bf16.new_empty if type(X_bf16) is torch.Tensor else _plain_empty(X_bf16)
@@ -434,6 +484,9 @@ def trdq_rotate_quantize_asym(rot: Rotation, t: int, X_bf16):
 
 
 def trdq_linear_asym(w: Weights, t: int, codes, scales, zero_points, bias_bf16=None, out=None):
+    done = (_native or _calls()).linear_asym(w._h.value, w.N, t, codes, scales, zero_points, bias_bf16, out)
+    if done is not None:
+        return _done(done, "trdq_linear_asym")
     import torch
     M = int(codes.shape[0])
     empty = codes.new_empty if type(codes) is torch.Tensor else _plain_empty(codes)
