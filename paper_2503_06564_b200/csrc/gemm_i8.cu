@@ -539,39 +539,43 @@ cudaError_t launch_weight_colsum(const int8_t* codes, int64_t rows, int32_t K, i
 // ---------------------------------------------------------------------------------------------
 namespace {
 
+constexpr int kMaxSplits = 8;
+
+// A thread adds four columns of one row.  The partial sums come from L2 and there is no second use for a thread, so what counts is that all its loads
+// are in flight at once: up to kMaxSplits of them, requested without a branch.  M = 128, N = 1152, eight ranges: from a cold start 5.6 us with eight columns a
+// thread and a loop over the ranges (72 blocks, two loads at a time), 4.4 now.
 __global__ void __launch_bounds__(256) splitk_reduce_epilogue_kernel(const int32_t* __restrict__ part, int splits, int64_t split_stride, int M,
                                                                      int N, const float* __restrict__ sx, const float* __restrict__ sw,
                                                                      const __nv_bfloat16* __restrict__ bias, __nv_bfloat16* __restrict__ y,
                                                                      int64_t ldy) {
   griddep_launch_dependents();
   griddep_wait();
-  const int vec_per_row = N / 8;  // N is a multiple of 16
+  const int vec_per_row = N / 4;  // N is a multiple of 16
   const int64_t total = static_cast<int64_t>(M) * vec_per_row;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int m = static_cast<int>(i / vec_per_row);
-    const int n = static_cast<int>(i - static_cast<int64_t>(m) * vec_per_row) * 8;
-    int32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int s = 0; s < splits; ++s) {
-      const int4* src = reinterpret_cast<const int4*>(part + s * split_stride + static_cast<int64_t>(m) * N + n);
-      const int4 a = src[0], b = src[1];
-      acc[0] += a.x; acc[1] += a.y; acc[2] += a.z; acc[3] += a.w;
-      acc[4] += b.x; acc[5] += b.y; acc[6] += b.z; acc[7] += b.w;
-    }
+    const int n = static_cast<int>(i - static_cast<int64_t>(m) * vec_per_row) * 4;
+    const int32_t* src = part + static_cast<int64_t>(m) * N + n;
+    int4 p[kMaxSplits];
+#pragma unroll
+    for (int s = 0; s < kMaxSplits; ++s) p[s] = s < splits ? *reinterpret_cast<const int4*>(src + s * split_stride) : make_int4(0, 0, 0, 0);
     const float sxm = __ldg(sx + m);
-    uint32_t packed[4];
+    const float4 sw4 = __ldg(reinterpret_cast<const float4*>(sw + n));
+    float b[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (bias) {
 #pragma unroll
-    for (int e = 0; e < 8; e += 2) {
-      float v2[2];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const float swn = __ldg(sw + n + e + u);
-        const float bn = bias ? __bfloat162float(bias[n + e + u]) : 0.0f;
-        v2[u] = dequant_one(acc[e + u], sxm, swn, bn, fabsf(bn) * 0.0009765625f);
-      }
-      const __nv_bfloat162 h = __floats2bfloat162_rn(v2[0], v2[1]);
-      packed[e / 2] = *reinterpret_cast<const uint32_t*>(&h);
+      for (int e = 0; e < 4; ++e) b[e] = __bfloat162float(bias[n + e]);
     }
-    *reinterpret_cast<uint4*>(y + static_cast<int64_t>(m) * ldy + n) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+#pragma unroll
+    for (int s = 1; s < kMaxSplits; ++s) {
+      p[0].x += p[s].x;
+      p[0].y += p[s].y;
+      p[0].z += p[s].z;
+      p[0].w += p[s].w;
+    }
+    const float v0 = dequant_one(p[0].x, sxm, sw4.x, b[0], fabsf(b[0]) * 0.0009765625f), v1 = dequant_one(p[0].y, sxm, sw4.y, b[1], fabsf(b[1]) * 0.0009765625f);
+    const float v2 = dequant_one(p[0].z, sxm, sw4.z, b[2], fabsf(b[2]) * 0.0009765625f), v3 = dequant_one(p[0].w, sxm, sw4.w, b[3], fabsf(b[3]) * 0.0009765625f);
+    *reinterpret_cast<uint2*>(y + static_cast<int64_t>(m) * ldy + n) = make_uint2(pack_bf16(make_float2(v0, v1)), pack_bf16(make_float2(v2, v3)));
   }
 }
 
@@ -587,7 +591,7 @@ int splitk_choose(const trdq_weights* w, int32_t M) {
   // splitting only pays when the reduction is long (K >= 8192) and the tiles fill less than half the SMs.
   if (w->wbits != 8 || tiles <= 0 || tiles * 2 > sms || num_kb < 64) return 1;
   int splits = static_cast<int>(sms / tiles);
-  if (splits > 8) splits = 8;
+  if (splits > kMaxSplits) splits = kMaxSplits;
   while (splits > 1 && num_kb / splits < 4) --splits;  // at least four k-blocks per range
   if (splits < 1) splits = 1;
   const int per = (num_kb + splits - 1) / splits;
@@ -612,24 +616,29 @@ trdq_status launch_gemm_w8_splitk(const trdq_weights* w, int g, const GemmSegmen
   if (st != TRDQ_OK) return st;
   p.tmap_a[1] = p.tmap_a[0];
   p.tmap_out[0] = p.tmap_out[1] = p.tmap_a[0];  // unused in the raw-accumulator mode
-  p.tmap_b = w->groups[g].tmap_b[0];             // 128-column tiles
   p.sw = nullptr;
   p.bias = nullptr;
   p.zp[0] = p.zp[1] = nullptr;
   p.colsum = nullptr;
   p.N = w->N;
   p.K = w->K;
-  p.tiles_n = (w->N + 127) / 128;
   const int num_kb = w->K / kTileKBytes;
   p.kb_per_split = (num_kb + splits - 1) / splits;
   p.splits = (num_kb + p.kb_per_split - 1) / p.kb_per_split;
+  // Tiles of 64 columns where they still fit in one round of the SMs: a CTA is bound by the bytes it pulls, and half-width tiles spread the
+  // weights over twice the SMs (M = 128, K = 16384, N = 1152, eight ranges, from a cold start: 72 CTAs 13.1 us, 144 CTAs 10.6; the call with both
+  // kernels 13.9 -> 10.3, and 0.76 - 0.96 of the time at 24 more points of 16 - 510 rows).
+  const int64_t narrow_tiles = static_cast<int64_t>(p.tiles_m[0]) * ((w->N + 63) / 64) * p.splits;
+  const bool narrow = narrow_tiles <= sms;
+  p.tiles_n = narrow ? (w->N + 63) / 64 : (w->N + 127) / 128;
+  p.tmap_b = narrow ? w->groups[g].tmap_b_half[0] : w->groups[g].tmap_b[0];  // boxes of 64 / 128 rows
   p.split_stride = static_cast<int64_t>(seg.M) * w->N;
   p.status = device_status_word();
   if (!p.status) return TRDQ_ERR_CUDA;
   const int64_t total = static_cast<int64_t>(p.tiles_m[0]) * p.tiles_n * p.splits;
   const int grid = static_cast<int>(total < sms ? total : sms);
-  if (launch_one<128, 1>(p, grid, stream) != cudaSuccess) return TRDQ_ERR_CUDA;
-  const int64_t vecs = static_cast<int64_t>(seg.M) * (w->N / 8);
+  if ((narrow ? launch_one<64, 1>(p, grid, stream) : launch_one<128, 1>(p, grid, stream)) != cudaSuccess) return TRDQ_ERR_CUDA;
+  const int64_t vecs = static_cast<int64_t>(seg.M) * (w->N / 4);
   int64_t rgrid = (vecs + 255) / 256;
   if (rgrid > static_cast<int64_t>(sms) * 8) rgrid = static_cast<int64_t>(sms) * 8;
   const cudaError_t e = launch_overlapped(splitk_reduce_epilogue_kernel, dim3(static_cast<unsigned>(rgrid)), dim3(256), 0, stream,
