@@ -508,6 +508,98 @@ rotate_quantize_rows_asym_kernel(const __nv_bfloat16* __restrict__ x, int64_t ld
   }
 }
 
+// Rows of 81 to 160 blocks, one row per CTA and one CTA per SM, four lanes per block, 64 bytes a lane in flight (the next row's during a transform).
+// What bounds the few rows of a long reduction is the chain of one row: load, transform, row maximum, store.  In the eight-lane kernel it is longer
+// (scalar butterfly, three shuffle stages, no overlap with the kernel before), and above 128 blocks a lane group has two blocks.
+// Microseconds, eight lanes / this: K = 10368 3.9 / 2.6 for one row, 4.2 / 2.8 for 128; K = 16384 5.1 / 3.4 and 5.3 / 3.5; K = 16512 6.8 / 3.6, 7.1 / 3.8, and 25.1 / 12.4
+// for 512 rows; K = 20480 7.5 / 3.9, 7.6 / 4.1, 27.1 / 14.0 and 139 / 84 for 4096.  (To 128 blocks the team kernel takes over from a row per SM on.)
+// 94 registers; a form of 64 for two CTAs per SM took 5.4 at M = 128, K = 16384.  Beyond 160 blocks the eight-lane kernel stays.  The codes are
+// formed as there, not by the magic addition, so that rows with infinities or NaN keep theirs.
+constexpr int kWideBlocks = 160;
+
+namespace wide {
+__global__ void __launch_bounds__(kWideBlocks* kFastLanes, 1)
+rotate_quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t ldx, int32_t M, int32_t K, const float* __restrict__ vec,
+                            int8_t* __restrict__ codes, float* __restrict__ scales) {
+  __shared__ unsigned int row_max[3];
+  const int lane4 = threadIdx.x & (kFastLanes - 1);
+  const int b = threadIdx.x / kFastLanes;
+  const bool active = b < K / TRDQ_BLOCK;
+  const int col0 = (active ? b : 0) * TRDQ_BLOCK + lane4 * 8;  // first element of chunk 0 of this lane; chunk c is 32 further
+  const float4* const vp = reinterpret_cast<const float4*>(vec + col0);
+
+  if (threadIdx.x < 3) row_max[threadIdx.x] = 0u;
+  __syncthreads();
+  griddep_launch_dependents();
+  griddep_wait();  // x may be written, and the code buffer still read, by the kernel before (the group vector is constant)
+
+  uint4 raw[4];
+  auto fetch = [&](int64_t row) {
+    if (active && row < M) {
+      const uint4* src = reinterpret_cast<const uint4*>(x + row * ldx + col0);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) raw[c] = __ldg(src + 4 * c);  // +32 elements = +4 uint4
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) raw[c] = make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  fetch(blockIdx.x);
+  int buf = 0;
+  for (int64_t row = blockIdx.x; row < M; row += gridDim.x) {
+    float2 v[16];
+    widen_chunks_lanes4(raw, v);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float4 f0 = __ldg(vp + 8 * c), f1 = __ldg(vp + 8 * c + 1);
+      v[4 * c] = __fmul2_rn(v[4 * c], make_float2(f0.x, f0.y));
+      v[4 * c + 1] = __fmul2_rn(v[4 * c + 1], make_float2(f0.z, f0.w));
+      v[4 * c + 2] = __fmul2_rn(v[4 * c + 2], make_float2(f1.x, f1.y));
+      v[4 * c + 3] = __fmul2_rn(v[4 * c + 3], make_float2(f1.z, f1.w));
+    }
+    fetch(row + gridDim.x);
+    wht128_lanes4(v, lane4);
+
+    // non-negative floats order like their bit patterns
+    const unsigned int top = __reduce_max_sync(0xffffffffu, __float_as_uint(absmax_lanes4(v)));
+    if ((threadIdx.x & 31) == 0) atomicMax(&row_max[buf], top);
+    __syncthreads();
+    const float amax = __uint_as_float(row_max[buf]);
+    if (++buf == 3) buf = 0;
+    if (threadIdx.x == 0) row_max[buf == 2 ? 0 : buf + 1] = 0u;  // that of the row after the next: nobody reads it any more
+    if (active) {
+      const float inv = amax > 0.0f ? __fdiv_rn(127.0f, amax) : 0.0f;
+      int8_t* dst = codes + row * K + col0;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        uint32_t w[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float2 a = v[4 * c + 2 * h], d = v[4 * c + 2 * h + 1];
+          uint32_t q[4] = {static_cast<uint32_t>(max(-127, min(127, quantize_one(a.x, inv)))), static_cast<uint32_t>(max(-127, min(127, quantize_one(a.y, inv)))),
+                           static_cast<uint32_t>(max(-127, min(127, quantize_one(d.x, inv)))), static_cast<uint32_t>(max(-127, min(127, quantize_one(d.y, inv))))};
+          w[h] = __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
+        }
+        *reinterpret_cast<uint2*>(dst + 32 * c) = make_uint2(w[0], w[1]);
+      }
+      if (threadIdx.x == 0) scales[row] = __fdiv_rn(amax, 127.0f);
+    }
+  }
+}
+
+}  // namespace wide
+
+bool rows_are_wide(int32_t K) { return K / TRDQ_BLOCK > 80 && K / TRDQ_BLOCK <= kWideBlocks; }
+
+cudaError_t launch_wide(const void* x, int64_t ldx, int32_t M, int32_t K, const float* vec, void* codes, float* scales, cudaStream_t stream) {
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int threads = (K / TRDQ_BLOCK * kFastLanes + 31) / 32 * 32;
+  return launch_overlapped(wide::rotate_quantize_kernel, dim3(min(M, sms)), dim3(threads), 0, stream, static_cast<const __nv_bfloat16*>(x), ldx, M, K,
+                           vec, static_cast<int8_t*>(codes), scales);
+}
+
 cudaError_t launch_rows_fast(const void* x, int64_t ldx, int32_t M, int32_t K, const float* vec, int groups, void* codes, float* scales,
                              cudaStream_t stream) {
   const int nb = K / TRDQ_BLOCK;
@@ -667,7 +759,9 @@ cudaError_t launch_rotate_quantize_groups(const void* x_bf16, int64_t ldx, int32
     const float* v = vec + static_cast<int64_t>(g) * K;
     uint8_t* c = static_cast<uint8_t*>(codes) + g * code_bytes;
     float* s = scales + g * scale_count;
-    const cudaError_t e = mode == 0 ? dispatch<0>(x_bf16, ldx, M, K, v, c, s, stream) : dispatch<1>(x_bf16, ldx, M, K, v, c, s, stream);
+    const cudaError_t e = mode != 0          ? dispatch<1>(x_bf16, ldx, M, K, v, c, s, stream)
+                          : rows_are_wide(K) ? launch_wide(x_bf16, ldx, M, K, v, c, s, stream)
+                                             : dispatch<0>(x_bf16, ldx, M, K, v, c, s, stream);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
