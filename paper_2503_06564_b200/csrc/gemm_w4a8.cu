@@ -35,6 +35,8 @@
 // 4000 more for conversion and output.  M = 16384, microseconds with 64-bit sums throughout -> now:
 // 1152 -> 4608 221 -> 203 (with GELU 260 -> 243), 1152 -> 3456 168 -> 155, 1152 -> 1152 58.0 -> 53.8; M = 1037, 1152 -> 3456 16.2 -> 15.3; 4608 -> 1152 170
 // either way.
+// With an epilogue for each form a kernel has 73 KB of instructions (98 with GELU, 40 and 53 with one form), more than stays cached when kernels alternate: in a
+// block's sequence of layers 34 us less by layer are 16 less in all (743 -> 727).  One epilogue for both forms: 61 and 73 KB, but 155 -> 159 by itself and 726 in all.
 // Measured and not better: a CTA pair sharing the codes and sixteen drain warps of 32 tokens (64-bit sums: 1152 -> 4608 221 -> 211 and 218, 1152 -> 1152
 // 59 -> 64 and 58); sums in fp64 (260 -> 358); weights unpacked into tensor memory with the codes of a token tile resident and one k-block
 // per hand-over (221 -> 238, 4608 -> 1152 170 -> 180: four unpack warps and one instruction cache for everything); nibbles unpacked to q4 instead of

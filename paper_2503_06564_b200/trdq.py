@@ -132,20 +132,30 @@ def _stream() -> int:
 _native = None
 
 
+class _GeneralWay:
+    """Stands in for the native calls where they have not been built for the torch at hand: every call goes the general way."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _calls():
     """The native form of the calls below (``csrc/calls.cpp``): it returns None for arguments it leaves to the general way."""
     global _native
     if _native is None:
+        import warnings
+
         import torch  # noqa: F401  (its libraries have to be loaded first)
+        l = lib()
         try:
             from . import _calls as native
+            native.bind(*(C.cast(f, C.c_void_p).value for f in (
+                l.trdq_rotate_quantize, l.trdq_norm_rotate_quantize, l.trdq_rotate_quantize_asym, l.trdq_linear_act, l.trdq_linear_cfg,
+                l.trdq_linear_asym, l.trdq_linear_splitk_workspace, l.trdq_linear_splitk)))
         except ImportError as e:
-            raise ImportError(f"{os.path.join(_HERE, '_calls.so')} is missing or does not fit this torch: build it with "
-                              "`python -m paper_2503_06564_b200.build`") from e
-        l = lib()
-        native.bind(*(C.cast(f, C.c_void_p).value for f in (
-            l.trdq_rotate_quantize, l.trdq_norm_rotate_quantize, l.trdq_rotate_quantize_asym, l.trdq_linear_act, l.trdq_linear_cfg,
-            l.trdq_linear_asym, l.trdq_linear_splitk_workspace, l.trdq_linear_splitk)))
+            warnings.warn(f"the native calls ({os.path.join(_HERE, '_calls.so')}) cannot be used, calls take about twice the host time: {e}; build them "
+                          "with `python -m paper_2503_06564_b200.build`")
+            native = _GeneralWay()
         _native = native
     return _native
 
