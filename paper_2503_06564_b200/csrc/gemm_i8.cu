@@ -333,6 +333,14 @@ cudaError_t launch_one(const GemmParams& p, int grid, cudaStream_t stream) {
   return launch_overlapped(gemm_w8a8_kernel<BN, MODE>, dim3(grid), dim3(kThreads), C::kSmemBytes, stream, p);
 }
 
+template <int MODE>
+cudaError_t launch_width(int bn, const GemmParams& p, int grid, cudaStream_t stream) {
+  return bn == 64    ? launch_one<64, MODE>(p, grid, stream)
+         : bn == 128 ? launch_one<128, MODE>(p, grid, stream)
+         : bn == 192 ? launch_one<192, MODE>(p, grid, stream)
+                     : launch_one<256, MODE>(p, grid, stream);
+}
+
 // Cost model for the tile width: waves of CTAs times the time of one tile (main loop grows
 // with BN; the 128-row operand and the fixed per-tile overhead do not).
 int choose_tile_n(int64_t tiles_m, int N, int sms) {
@@ -349,6 +357,18 @@ int choose_tile_n(int64_t tiles_m, int N, int sms) {
     }
   }
   return best;
+}
+
+// Tiles of kNarrowTile columns where all of them are one round of the SMs: a CTA is bound by the bytes that it pulls (24 KB per k-block in place of
+// 32 and more) and by its epilogue, which it does not overlap with another tile, and there are twice as many CTAs.  Microseconds, 128 columns and more / 64:
+// M = 256, K = N = 1024 4.4 / 3.9; K = 1152, 3456 x 128 4.6 / 4.0, GELU 4608 x 16 5.7 / 5.0; K = 4608, 1152 x 128 8.6 / 8.1; 0.77 - 1.0 of the time, 0.87 on
+// average, over 70 points from 1 to 1200 rows.  Where the tiles nearly fill the SMs, in more than four rows of tiles, the activation tiles that
+// twice the CTAs read again cost what is gained: K = 4096, 1152 x 960 (144 tiles) 8.14 / 8.22, K = 2304 1.02, but 132 tiles in eleven rows 0.99 and
+// 148 in four 0.99.
+constexpr int kNarrowTile = 64;
+bool narrow_tiles(int64_t tiles_m, int N, int sms, int splits = 1) {
+  const int64_t tiles = tiles_m * ((N + kNarrowTile - 1) / kNarrowTile) * splits;
+  return tiles <= sms && (10 * tiles <= 9 * sms || tiles_m <= 4);
 }
 
 }  // namespace
@@ -418,7 +438,8 @@ void describe_gemm_kernel(int32_t M, int32_t K, int32_t N, int32_t wbits, char* 
   }
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  snprintf(name, cap, "gemm_w8a8_kernel<%d>", kTileN[choose_tile_n((static_cast<int64_t>(M) + kTileM - 1) / kTileM, N, sms)]);
+  const int64_t tiles_m = (static_cast<int64_t>(M) + kTileM - 1) / kTileM;
+  snprintf(name, cap, "gemm_w8a8_kernel<%d>", narrow_tiles(tiles_m, N, sms) ? kNarrowTile : kTileN[choose_tile_n(tiles_m, N, sms)]);
 }
 
 static trdq_status launch_gemm_w8_mode(const trdq_weights* w, int g, const GemmSegment seg[2], const void* bias_bf16, int mode,
@@ -443,8 +464,9 @@ static trdq_status launch_gemm_w8_mode(const trdq_weights* w, int g, const GemmS
     tiles_m += p.tiles_m[s];
   }
   if (tiles_m == 0) return TRDQ_OK;
+  const bool narrow = narrow_tiles(tiles_m, w->N, sms);
   const int ti = choose_tile_n(tiles_m, w->N, sms);
-  const int bn = kTileN[ti];
+  const int bn = narrow ? kNarrowTile : kTileN[ti];
   for (int s = 0; s < 2; ++s) {
     if (seg[s].M == 0) continue;
     const GemmSegment& src = seg[s];
@@ -465,7 +487,7 @@ static trdq_status launch_gemm_w8_mode(const trdq_weights* w, int g, const GemmS
     p.tmap_out[s] = p.tmap_out[1 - s];
   }
   if (raw_i32) p.tmap_out[0] = p.tmap_out[1] = p.tmap_a[0];  // unused by the raw-accumulator mode
-  p.tmap_b = w->groups[g].tmap_b[ti];
+  p.tmap_b = narrow ? w->groups[g].tmap_b_half[0] : w->groups[g].tmap_b[ti];  // boxes of 64 rows / a tile width
   p.sw = w->groups[g].scales;
   p.bias = static_cast<const __nv_bfloat16*>(bias_bf16);
   p.N = w->N;
@@ -482,16 +504,8 @@ static trdq_status launch_gemm_w8_mode(const trdq_weights* w, int g, const GemmS
   const int64_t total = tiles_m * p.tiles_n;
   const int grid = static_cast<int>(total < sms ? total : sms);
 
-  cudaError_t e;
-  if (raw_i32) {
-    e = bn == 128 ? launch_one<128, 1>(p, grid, stream) : bn == 192 ? launch_one<192, 1>(p, grid, stream) : launch_one<256, 1>(p, grid, stream);
-  } else if (mode == 2) {
-    e = bn == 128 ? launch_one<128, 2>(p, grid, stream) : bn == 192 ? launch_one<192, 2>(p, grid, stream) : launch_one<256, 2>(p, grid, stream);
-  } else if (act) {
-    e = bn == 128 ? launch_one<128, 3>(p, grid, stream) : bn == 192 ? launch_one<192, 3>(p, grid, stream) : launch_one<256, 3>(p, grid, stream);
-  } else {
-    e = bn == 128 ? launch_one<128, 0>(p, grid, stream) : bn == 192 ? launch_one<192, 0>(p, grid, stream) : launch_one<256, 0>(p, grid, stream);
-  }
+  const cudaError_t e = raw_i32 ? launch_width<1>(bn, p, grid, stream) : mode == 2 ? launch_width<2>(bn, p, grid, stream)
+                        : act   ? launch_width<3>(bn, p, grid, stream) : launch_width<0>(bn, p, grid, stream);
   return e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA;
 }
 
@@ -628,8 +642,7 @@ trdq_status launch_gemm_w8_splitk(const trdq_weights* w, int g, const GemmSegmen
   // Tiles of 64 columns where they still fit in one round of the SMs: a CTA is bound by the bytes it pulls, and half-width tiles spread the
   // weights over twice the SMs (M = 128, K = 16384, N = 1152, eight ranges, from a cold start: 72 CTAs 13.1 us, 144 CTAs 10.6; the call with both
   // kernels 13.9 -> 10.3, and 0.76 - 0.96 of the time at 24 more points of 16 - 510 rows).
-  const int64_t narrow_tiles = static_cast<int64_t>(p.tiles_m[0]) * ((w->N + 63) / 64) * p.splits;
-  const bool narrow = narrow_tiles <= sms;
+  const bool narrow = narrow_tiles(p.tiles_m[0], w->N, sms, p.splits);
   p.tiles_n = narrow ? (w->N + 63) / 64 : (w->N + 127) / 128;
   p.tmap_b = narrow ? w->groups[g].tmap_b_half[0] : w->groups[g].tmap_b[0];  // boxes of 64 / 128 rows
   p.split_stride = static_cast<int64_t>(seg.M) * w->N;
