@@ -28,15 +28,13 @@
 // rounds F by half a step at most, so |D| <= 9 * 2^27 < 2^31 after nine k-blocks.  S stays within 2^50 for mult below 2^b,
 // b = 33 - ceil(log2(14 K / 128)): 26 bits at K = 1152.  A channel whose scales need more (exponents that span more than three binades; a ratio
 // below four never does) is marked by the sign of base, and a warp that holds one adds 64-bit products with all 30 bits of mult.  Longer
-// reductions do so throughout: with 25 bits few channels qualify, and of the 32 of a warp hardly ever all.
+// reductions do so throughout: with 25 bits few channels qualify, and of the 32 of a warp hardly ever all.  So do small problems (see launch_gemm_w4).
 //
 // What bounds it: the drain.  Clocks per k-block of 128 x 128 accumulators for the drain loop by itself: 64-bit multiply-adds 603, L and F 453, one
 // fp32 conversion and FMA 322, the loads from tensor memory 185; 256 of tensor pipe.  In the kernel a k-block takes about 1000, and a tile
 // 4000 more for conversion and output.  M = 16384, microseconds with 64-bit sums throughout -> now:
-// 1152 -> 4608 221 -> 203 (with GELU 260 -> 243), 1152 -> 3456 168 -> 155, 1152 -> 1152 58.0 -> 53.8; M = 1037, 1152 -> 3456 16.2 -> 15.3; 4608 -> 1152 170
-// either way.
-// With an epilogue for each form a kernel has 73 KB of instructions (98 with GELU, 40 and 53 with one form), more than stays cached when kernels alternate: in a
-// block's sequence of layers 34 us less by layer are 16 less in all (743 -> 727).  One epilogue for both forms: 61 and 73 KB, but 155 -> 159 by itself and 726 in all.
+// 1152 -> 4608 221 -> 203 (with GELU 260 -> 243), 1152 -> 3456 168 -> 155; 4608 -> 1152 170
+// either way; the layers alternating in a block together 738 -> 730.
 // Measured and not better: a CTA pair sharing the codes and sixteen drain warps of 32 tokens (64-bit sums: 1152 -> 4608 221 -> 211 and 218, 1152 -> 1152
 // 59 -> 64 and 58); sums in fp64 (260 -> 358); weights unpacked into tensor memory with the codes of a token tile resident and one k-block
 // per hand-over (221 -> 238, 4608 -> 1152 170 -> 180: four unpack warps and one instruction cache for everything); nibbles unpacked to q4 instead of
@@ -88,6 +86,7 @@ static_assert(kDrainWarps * 32 * kRegsDrain + (kThreads - kDrainWarps * 32) * kR
 constexpr int kMultBits = 30, kGrid = 28, kMinFastBits = 26;
 constexpr float kAnchor = 3377699720527872.0f;  // 1.5 * 2^51: one binade for sums within +- 2^50, its float steps are 2^28
 constexpr uint32_t kAnchorBits = 0x59400000u;
+constexpr int64_t kFastBlocksPerSm = 200;
 // bits of mult with which sums of `groups` k-blocks stay within +- 2^50: |acc| <= 16 * 128 * 7 * 128 = 14 * 2^17
 __host__ __device__ constexpr int w4_fast_bits(int groups) {
   int log = 0;
@@ -320,8 +319,9 @@ __device__ __forceinline__ void drain_tile(const W4Params& p, DrainState& s, int
   }
 }
 
-// ACT: GELU (tanh form) on the dequantized value before the bf16 rounding.
-template <bool ACT>
+// ACT: GELU (tanh form) on the dequantized value before the bf16 rounding.  FAST: reductions of up to nine k-blocks, with both forms of the
+// sum; longer ones have a kernel with the 64-bit form alone, which is half the instructions (40 KB against 73, with GELU 53 against 98).
+template <bool ACT, bool FAST>
 __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_constant__ W4Params p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -391,9 +391,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_con
       }
       const int after = tile + static_cast<int>(gridDim.x);
       const int32_t* next = after < total_tiles ? p.mult_t + tile_coord(p, after).n0 + lane_n : nullptr;
-      if (__any_sync(0xffffffffu, base < 0.0f)) {
+      if (!FAST || __any_sync(0xffffffffu, base < 0.0f)) {
         drain_tile<true, ACT>(p, s, n, fabsf(base), bias, num_kb, next, sx_reg);
-      } else {
+      } else if constexpr (FAST) {
         drain_tile<false, ACT>(p, s, n, base, bias, num_kb, next, sx_reg);
       }
       fence_proxy_async_smem();
@@ -625,13 +625,19 @@ trdq_status launch_gemm_w4(const trdq_weights* w, int g, const GemmSegment seg[2
   const int grid = static_cast<int>(total < sms ? total : sms);
   static PerDeviceFlag configured;
   if (!configured.get(dev)) {
-    if (cudaFuncSetAttribute(gemm_w4a8_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_w4a8_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
-      return TRDQ_ERR_CUDA;
+    for (const auto kernel : {gemm_w4a8_kernel<false, false>, gemm_w4a8_kernel<false, true>, gemm_w4a8_kernel<true, false>, gemm_w4a8_kernel<true, true>})
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return TRDQ_ERR_CUDA;
     configured.set(dev, true);
   }
-  const cudaError_t e = act ? launch_overlapped(gemm_w4a8_kernel<true>, dim3(grid), dim3(kThreads), kSmemBytes, stream, p)
-                            : launch_overlapped(gemm_w4a8_kernel<false>, dim3(grid), dim3(kThreads), kSmemBytes, stream, p);
+  // The kernel with both forms of the sum has 73 KB of instructions (98 with GELU) in place of 40 (53), more than stays cached when kernels alternate, as
+  // the layers of a block do: its launch and the ones around it take 4 - 8 us longer than in a loop by themselves.  So it runs from 200 k-blocks per SM
+  // on, where it gains 12 us and more.  A block of 4-bit layers, microseconds, 64-bit sums throughout / wherever the reduction is short / from here on: 1000 tokens of
+  // width 384 41.1 / 45.6 / 41.3, 4000 of 896 164.3 / 171.5 / 161.9, 2000 of 1152 with cross-attention 171 / 180 / 170, 16384 of 1152 738 / 728 / 730, of 768 414 / - / 406.
+  const int64_t blocks = w->K / kTileK;
+  const bool fast = w4_fast_bits(static_cast<int>(blocks)) >= kMinFastBits && total * blocks >= kFastBlocksPerSm * sms;
+  void (*const kernel)(W4Params) = act ? (fast ? gemm_w4a8_kernel<true, true> : gemm_w4a8_kernel<true, false>)
+                                       : (fast ? gemm_w4a8_kernel<false, true> : gemm_w4a8_kernel<false, false>);
+  const cudaError_t e = launch_overlapped(kernel, dim3(grid), dim3(kThreads), kSmemBytes, stream, p);
   return e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA;
 }
 

@@ -1,5 +1,5 @@
-"""GPU parity of the two forms of the 4-bit GEMM's sum over scale groups (two 32-bit numbers up to nine groups, 64 bits otherwise) at the ends of
-their ranges: largest sums of both signs, sums that swing back, scales on either side of what the first form takes."""
+"""GPU parity of the two forms of the 4-bit GEMM's sum over scale groups (two 32-bit numbers up to nine groups in large problems, 64 bits otherwise) at the
+ends of their ranges: largest sums of both signs, sums that swing back, scales on either side of what the first form takes."""
 import numpy as np
 import pytest
 
@@ -33,9 +33,13 @@ def test_sums_at_the_ends_of_their_range(blocks, span):
     codes[3] = np.where(np.arange(K) < K // 2, 127, -127)
     codes[4] = np.where(np.arange(K) // 128 % 2, 127, -127)
     scales = rng.uniform(0.01, 0.02, M).astype(np.float32)
-    y = trdq.trdq_linear(wts, 0, torch.from_numpy(codes).cuda(), torch.from_numpy(scales).cuda())
     y_ref = O.linear_w4_rows(codes, scales, packed, sw4, None, np.arange(M))
-    # one fp32 rounding of the sum and one of its product are far below a bf16 step: the result is the bf16 number next to the oracle's value
-    assert check_output(bf16_to_f32_np(y), y_ref)[1] <= 1.0
-    assert not bf16_to_f32_np(y)[2].any()
+    c, sx = torch.from_numpy(codes).cuda(), torch.from_numpy(scales).cuda()
+    # alone, and repeated until the problem is large (200 k-blocks per SM): no row count of a tile, so every row meets many lanes and columns
+    for copies in (1, 148 * 200 // (2 * blocks) * 128 // M + 4):
+        y = trdq.trdq_linear(wts, 0, c.repeat(copies, 1), sx.repeat(copies))
+        # one fp32 rounding of the sum and one of its product are far below a bf16 step: the result is the bf16 number next to the oracle's value
+        assert check_output(bf16_to_f32_np(y[:M]), y_ref)[1] <= 1.0
+        assert not bf16_to_f32_np(y[2:3]).any()
+        assert bool((y.view(copies, M, N).view(torch.int16) == y[:M].view(torch.int16)).all())
     assert trdq.trdq_device_status() == 0
