@@ -21,24 +21,16 @@
 // with the same cancellation check against the bias as the 8-bit kernel, transposed through a staging tile in shared
 // memory and written by TMA stores.  Every wait is bounded.
 //
-// The drain holds S, up to 2^50, as two 32-bit numbers instead of multiplying 32 x 32 -> 64 bits:
-//   L = S mod 2^32          (one 32-bit multiply-add)
-//   F = S within 2^31       (one conversion and one fp32 FMA; F moves in one binade, so that every addition rounds to a multiple of 2^kGrid)
-// and S = f 2^kGrid + D with f the steps that F has moved and D the signed 32-bit remainder of L: as exact as the 64-bit sum.  An addition
-// rounds F by half a step at most, so |D| <= 9 * 2^27 < 2^31 after nine k-blocks.  S stays within 2^50 for mult below 2^b,
-// b = 33 - ceil(log2(14 K / 128)): 26 bits at K = 1152.  A channel whose scales need more (exponents that span more than three binades; a ratio
-// below four never does) is marked by the sign of base, and a warp that holds one adds 64-bit products with all 30 bits of mult.  Longer
-// reductions do so throughout: with 25 bits few channels qualify, and of the 32 of a warp hardly ever all.  So do small problems (see launch_gemm_w4).
-//
-// What bounds it: the drain.  Clocks per k-block of 128 x 128 accumulators for the drain loop by itself: 64-bit multiply-adds 603, L and F 453, one
-// fp32 conversion and FMA 322, the loads from tensor memory 185; 256 of tensor pipe.  In the kernel a k-block takes about 1000, and a tile
-// 4000 more for conversion and output.  M = 16384, microseconds with 64-bit sums throughout -> now:
-// 1152 -> 4608 221 -> 203 (with GELU 260 -> 243), 1152 -> 3456 168 -> 155; 4608 -> 1152 170
-// either way; the layers alternating in a block together 738 -> 730.
-// Measured and not better: a CTA pair sharing the codes and sixteen drain warps of 32 tokens (64-bit sums: 1152 -> 4608 221 -> 211 and 218, 1152 -> 1152
-// 59 -> 64 and 58); sums in fp64 (260 -> 358); weights unpacked into tensor memory with the codes of a token tile resident and one k-block
+// What bounds it: the drain.  A 32 x 32 -> 64-bit multiply-add issues at a quarter of the fp32 rate: the drain loop by itself takes 603 clocks per k-block of
+// 128 x 128 accumulators, 185 of them the loads from tensor memory, against 256 of tensor pipe.  In the kernel a k-block takes about 1100, and a tile 4000
+// more for conversion and output.  M = 16384, microseconds with the weights as the N operand (multipliers read from a shared-memory table per
+// column, one k-block per hand-over) -> now: 1152 -> 4608 323 -> 215 (with GELU 253), 4608 -> 1152 247 -> 166, 1152 -> 1152 84 -> 56, 1152 -> 3456 244 -> 163.
+// Measured and not better: a CTA pair sharing the codes (1152 -> 4608 221 -> 211, but 1152 -> 1152 59 -> 64: the 256-channel tile pads N = 1152 by 11 %);
+// sixteen drain warps of 32 tokens (218, 58); sums in fp64 (260 -> 358); weights unpacked into tensor memory with the codes of a token tile resident and one k-block
 // per hand-over (221 -> 238, 4608 -> 1152 170 -> 180: four unpack warps and one instruction cache for everything); nibbles unpacked to q4 instead of
-// 16 q4, which would give b four more bits (four more instructions per eight weights: 4608 -> 1152 170 -> 190).
+// 16 q4 (four more instructions per eight weights: 4608 -> 1152 170 -> 190).  The sum as two 32-bit numbers, its value modulo 2^32 and an fp32 sum
+// in one binade (453 clocks), is exact to nine k-blocks and faster in a loop by itself (1152 -> 3456 163 -> 153), but only if its float is rounded twice; converted with one
+// rounding it gives 159 - 168, and a block of four layers takes 743 - 771 in place of 731 (73 KB of instructions against 40).
 #include <cuda_bf16.h>
 
 #include "epilogue.cuh"
@@ -82,19 +74,7 @@ static_assert(kSlots * kHandoff * kTileTok <= kTmemCols, "tensor memory");
 constexpr int kRegsLaunch = 128, kRegsDrain = 192, kRegsOther = 64;
 static_assert(kDrainWarps * 32 * kRegsDrain + (kThreads - kDrainWarps * 32) * kRegsOther <= kThreads * kRegsLaunch, "register split exceeds the launch's allocation");
 
-// The drain's numbers: mult has kMultBits bits, a step of F is 2^kGrid.
-constexpr int kMultBits = 30, kGrid = 28, kMinFastBits = 26;
-constexpr float kAnchor = 3377699720527872.0f;  // 1.5 * 2^51: one binade for sums within +- 2^50, its float steps are 2^28
-constexpr uint32_t kAnchorBits = 0x59400000u;
-constexpr int64_t kFastBlocksPerSm = 200;
-// bits of mult with which sums of `groups` k-blocks stay within +- 2^50: |acc| <= 16 * 128 * 7 * 128 = 14 * 2^17
-__host__ __device__ constexpr int w4_fast_bits(int groups) {
-  int log = 0;
-  while (static_cast<int64_t>(1) << log < static_cast<int64_t>(14) * groups) ++log;
-  return 33 - log < kMultBits ? 33 - log : kMultBits;
-}
-// kMinFastBits: at most nine additions, so the remainder stays below 9 * 2^(kGrid - 1)
-static_assert(w4_fast_bits(9) >= kMinFastBits && w4_fast_bits(10) < kMinFastBits && 9 < (1 << (32 - kGrid)), "the remainder has to fit 32 signed bits");
+constexpr int kMultBits = 30;
 
 struct alignas(64) W4Params {
   CUtensorMap tmap_a[2];    // codes of each segment, box 128 B x 128 rows, 128-byte swizzle
@@ -104,10 +84,9 @@ struct alignas(64) W4Params {
   int32_t M[2];
   int32_t tiles_m[2];
   const int32_t* mult_t;  // [K/128][n_pad]
-  const float* base;      // [n_pad], negative: the channel needs more than w4_fast_bits
+  const float* base;      // [n_pad]
   const __nv_bfloat16* bias;
   int32_t N, K, tiles_n, n_pad;
-  int32_t fast_shift;     // kMultBits - w4_fast_bits
   uint32_t* status;
 };
 
@@ -144,73 +123,6 @@ __device__ __forceinline__ void tmem_wait_ld_regs(uint32_t (&r)[16]) {
   for (int i = 0; i < 16; ++i) asm volatile("" : "+r"(r[i]));
 }
 
-// What a drain thread adds up for its channel, a sum for each of its tokens.
-template <bool WIDE>
-struct ChannelSums;
-template <>
-struct ChannelSums<false> {
-  uint32_t L[kTokPerWarp];
-  float F[kTokPerWarp];
-  uint32_t mult;
-  float multf;
-  __device__ __forceinline__ void clear() {
-#pragma unroll
-    for (int j = 0; j < kTokPerWarp; ++j) {
-      L[j] = 0;
-      F[j] = kAnchor;
-    }
-  }
-  __device__ __forceinline__ void set_mult(int32_t m, int shift) {
-    mult = static_cast<uint32_t>(m >> shift);
-    multf = __int2float_rn(m >> shift);  // exact: 24 significant bits
-  }
-  __device__ __forceinline__ void add(int j, uint32_t acc) {
-    L[j] += acc * mult;
-    F[j] = __fmaf_rn(__int2float_rn(static_cast<int32_t>(acc)), multf, F[j]);
-  }
-  __device__ __forceinline__ int32_t rest(int j) const {  // (the anchor's low bits are zero)
-    return static_cast<int32_t>(L[j] - (__float_as_uint(F[j]) << kGrid));
-  }
-  __device__ __forceinline__ long long whole(int j) const {
-    return (static_cast<long long>(static_cast<int32_t>(__float_as_uint(F[j]) - kAnchorBits)) << kGrid) + rest(j);
-  }
-  // eight sums as floats
-  __device__ __forceinline__ void to_float(int j0, float (&v)[8]) const {
-    float low = __uint_as_float(0x7F800000u);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      v[e] = __fadd_rn(__fsub_rn(F[j0 + e], kAnchor), __int2float_rn(rest(j0 + e)));
-      if (e & 1) low = min3_abs(low, v[e - 1], v[e]);
-    }
-    if (low < 1073741824.0f) {  // below 2^30 the sum is L itself: no rounding of the remainder on the way
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        if (fabsf(v[e]) < 1073741824.0f) v[e] = __int2float_rn(static_cast<int32_t>(L[j0 + e]));
-    }
-  }
-};
-template <>
-struct ChannelSums<true> {
-  long long sum[kTokPerWarp];
-  int32_t mult;
-  __device__ __forceinline__ void clear() {
-#pragma unroll
-    for (int j = 0; j < kTokPerWarp; ++j) sum[j] = 0;
-  }
-  __device__ __forceinline__ void set_mult(int32_t m, int) {
-    mult = m;
-    asm volatile("" : "+r"(mult));  // stays a 32-bit factor: widened ahead of the loop it would cost a 64 x 64 product
-  }
-  __device__ __forceinline__ void add(int j, uint32_t acc) {
-    sum[j] += static_cast<long long>(static_cast<int32_t>(acc)) * static_cast<long long>(mult);
-  }
-  __device__ __forceinline__ long long whole(int j) const { return sum[j]; }
-  __device__ __forceinline__ void to_float(int j0, float (&v)[8]) const {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = __ll2float_rn(sum[j0 + e]);
-  }
-};
-
 // State of a drain warp that lasts from tile to tile.
 struct DrainState {
   BoundedWaiter w;
@@ -225,13 +137,13 @@ struct DrainState {
 
 // One tile of one drain warp: sums over the k-blocks, then y = float(S) * (sx * base) + bias (base is a power of two: the product is
 // exact) into the staging tile.  `next`: first multiplier of the warp's next tile.
-// WIDE: a channel of the warp needs all bits of mult.  ACT: GELU (tanh form) on the dequantized value before the bf16 rounding.
-template <bool WIDE, bool ACT>
+// ACT: GELU (tanh form) on the dequantized value before the bf16 rounding.
+template <bool ACT>
 __device__ __forceinline__ void drain_tile(const W4Params& p, DrainState& s, int n, float base, float bias, int num_kb, const int32_t* next,
                                            const float (&sx_reg)[kTokPerWarp / 32]) {
-  ChannelSums<WIDE> acc;
-  acc.clear();
-  const int shift = WIDE ? 0 : p.fast_shift;
+  long long sum[kTokPerWarp];
+#pragma unroll
+  for (int j = 0; j < kTokPerWarp; ++j) sum[j] = 0;
   const int32_t* mp = p.mult_t + n;
   // Two register buffers: a tensor-memory load is always in flight behind the multiply-adds, across k-blocks too.
   uint32_t r[2][16];
@@ -242,7 +154,8 @@ __device__ __forceinline__ void drain_tile(const W4Params& p, DrainState& s, int
   tmem_ld_32x16(t_row, r[0]);
 #pragma unroll 1
   for (int kb = 0; kb < num_kb; ++kb) {
-    acc.set_mult(s.m_next, shift);
+    int32_t mult = s.m_next;
+    asm volatile("" : "+r"(mult));  // stays a 32-bit factor: widened ahead of the loop it would cost a 64 x 64 product
     if (kb + 1 < num_kb) {
       mp += p.n_pad;
       s.m_next = __ldg(mp);
@@ -270,12 +183,12 @@ __device__ __forceinline__ void drain_tile(const W4Params& p, DrainState& s, int
         }
       }
 #pragma unroll
-      for (int j = 0; j < 16; ++j) acc.add(ch * 16 + j, r[ch & 1][j]);
+      for (int j = 0; j < 16; ++j)
+        sum[ch * 16 + j] += static_cast<long long>(static_cast<int32_t>(r[ch & 1][j])) * static_cast<long long>(mult);
     }
   }
 
   if (next) s.m_next = __ldg(next);
-  const float unit = __fmul_rn(base, static_cast<float>(1 << shift));
   const float thr = fabsf(bias) * 0.0009765625f;
   // byte of this lane's channel inside a staging row (64 bytes, 64-byte swizzle: 16-byte chunk index xor row bits 1..2)
   const uint32_t lane_chunk = s.lane >> 3, lane_byte = (s.lane & 7) * 2;
@@ -288,20 +201,21 @@ __device__ __forceinline__ void drain_tile(const W4Params& p, DrainState& s, int
 #pragma unroll
   for (int j0 = 0; j0 < kTokPerWarp; j0 += 8) {
     float v[8], y[8];
-    acc.to_float(j0, v);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = __ll2float_rn(sum[j0 + e]);
     const float4 sa = *reinterpret_cast<const float4*>(s.sx + j0), sb = *reinterpret_cast<const float4*>(s.sx + j0 + 4);
     const float sx8[8] = {sa.x, sa.y, sa.z, sa.w, sb.x, sb.y, sb.z, sb.w};
     bool cancels = false;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      y[e] = __fmaf_rn(v[e], __fmul_rn(sx8[e], unit), bias);
+      y[e] = __fmaf_rn(v[e], __fmul_rn(sx8[e], base), bias);
       cancels |= fabsf(y[e]) < thr;
     }
     if (cancels) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         // the part of the sum that fp32 dropped
-        if (fabsf(y[e]) < thr) y[e] = __fmaf_rn(__ll2float_rn(acc.whole(j0 + e) - __float2ll_rz(v[e])), __fmul_rn(sx8[e], unit), y[e]);
+        if (fabsf(y[e]) < thr) y[e] = __fmaf_rn(__ll2float_rn(sum[j0 + e] - __float2ll_rz(v[e])), __fmul_rn(sx8[e], base), y[e]);
       }
     }
     uint32_t packed[4];
@@ -319,9 +233,8 @@ __device__ __forceinline__ void drain_tile(const W4Params& p, DrainState& s, int
   }
 }
 
-// ACT: GELU (tanh form) on the dequantized value before the bf16 rounding.  FAST: reductions of up to nine k-blocks, with both forms of the
-// sum; longer ones have a kernel with the 64-bit form alone, which is half the instructions (40 KB against 73, with GELU 53 against 98).
-template <bool ACT, bool FAST>
+// ACT: GELU (tanh form) on the dequantized value before the bf16 rounding.
+template <bool ACT>
 __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_constant__ W4Params p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -391,11 +304,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a8_kernel(const __grid_con
       }
       const int after = tile + static_cast<int>(gridDim.x);
       const int32_t* next = after < total_tiles ? p.mult_t + tile_coord(p, after).n0 + lane_n : nullptr;
-      if (!FAST || __any_sync(0xffffffffu, base < 0.0f)) {
-        drain_tile<true, ACT>(p, s, n, fabsf(base), bias, num_kb, next, sx_reg);
-      } else if constexpr (FAST) {
-        drain_tile<false, ACT>(p, s, n, base, bias, num_kb, next, sx_reg);
-      }
+      drain_tile<ACT>(p, s, n, base, bias, num_kb, next, sx_reg);
       fence_proxy_async_smem();
       __syncwarp();  // (the reads of my_sx are done as well)
       if (lane == 0) {
@@ -552,18 +461,12 @@ __global__ void w4_multipliers_kernel(const float* __restrict__ scales, int32_t 
   int e_max = 0;
   frexpf(smax, &e_max);  // smax = f * 2^e_max, f in [0.5, 1); smax == 0 gives e_max = 0
   if (e_max < -90) e_max = -90;  // keeps base a normal number; such channels are numerically zero anyway
-  int32_t all = 0;
   for (int g = 0; g < groups; ++g) {
     const float s = scales[static_cast<int64_t>(n) * groups + g];
-    const int32_t m = __float2int_rn(ldexpf(s, kMultBits - e_max));  // < 2^30, exact if the exponents span < 7 bits
-    mult_t[static_cast<int64_t>(g) * n_pad + n] = m;
-    all |= m;
+    mult_t[static_cast<int64_t>(g) * n_pad + n] = __float2int_rn(ldexpf(s, kMultBits - e_max));  // < 2^30, exact if the exponents span < 7 bits
   }
-  // (a scale that is not a finite number gives a mult past 2^30)
-  const bool wide = w4_fast_bits(groups) < kMinFastBits || (all >> kMultBits) != 0 || (all & ((1 << (kMultBits - w4_fast_bits(groups))) - 1)) != 0;
   // the tensor core sees 16 * q4 (the nibble sits in the high half of the byte): fold the 1/16 here
-  const float unit = ldexpf(1.0f, e_max - kMultBits - 4);
-  base[n] = wide ? -unit : unit;
+  base[n] = ldexpf(1.0f, e_max - kMultBits - 4);
 }
 
 }  // namespace
@@ -618,26 +521,18 @@ trdq_status launch_gemm_w4(const trdq_weights* w, int g, const GemmSegment seg[2
   p.K = w->K;
   p.tiles_n = (w->N + kTileCh - 1) / kTileCh;
   p.n_pad = p.tiles_n * kTileCh;
-  p.fast_shift = kMultBits - w4_fast_bits(w->K / kTileK);
   p.status = device_status_word();
   if (!p.status) return TRDQ_ERR_CUDA;
   const int64_t total = tiles_m * p.tiles_n;
   const int grid = static_cast<int>(total < sms ? total : sms);
   static PerDeviceFlag configured;
   if (!configured.get(dev)) {
-    for (const auto kernel : {gemm_w4a8_kernel<false, false>, gemm_w4a8_kernel<false, true>, gemm_w4a8_kernel<true, false>, gemm_w4a8_kernel<true, true>})
+    for (const auto kernel : {gemm_w4a8_kernel<false>, gemm_w4a8_kernel<true>})
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return TRDQ_ERR_CUDA;
     configured.set(dev, true);
   }
-  // The kernel with both forms of the sum has 73 KB of instructions (98 with GELU) in place of 40 (53), more than stays cached when kernels alternate, as
-  // the layers of a block do: its launch and the ones around it take 4 - 8 us longer than in a loop by themselves.  So it runs from 200 k-blocks per SM
-  // on, where it gains 12 us and more.  A block of 4-bit layers, microseconds, 64-bit sums throughout / wherever the reduction is short / from here on: 1000 tokens of
-  // width 384 41.1 / 45.6 / 41.3, 4000 of 896 164.3 / 171.5 / 161.9, 2000 of 1152 with cross-attention 171 / 180 / 170, 16384 of 1152 738 / 728 / 730, of 768 414 / - / 406.
-  const int64_t blocks = w->K / kTileK;
-  const bool fast = w4_fast_bits(static_cast<int>(blocks)) >= kMinFastBits && total * blocks >= kFastBlocksPerSm * sms;
-  void (*const kernel)(W4Params) = act ? (fast ? gemm_w4a8_kernel<true, true> : gemm_w4a8_kernel<true, false>)
-                                       : (fast ? gemm_w4a8_kernel<false, true> : gemm_w4a8_kernel<false, false>);
-  const cudaError_t e = launch_overlapped(kernel, dim3(grid), dim3(kThreads), kSmemBytes, stream, p);
+  const cudaError_t e = act ? launch_overlapped(gemm_w4a8_kernel<true>, dim3(grid), dim3(kThreads), kSmemBytes, stream, p)
+                            : launch_overlapped(gemm_w4a8_kernel<false>, dim3(grid), dim3(kThreads), kSmemBytes, stream, p);
   return e == cudaSuccess ? TRDQ_OK : TRDQ_ERR_CUDA;
 }
 

@@ -40,7 +40,7 @@ struct GroupWeights {
   //   scales[n][kg] = mult_t[kg][n] * base[n]   (exact whenever the exponents of a channel span < 7 bits)
   int32_t* colsum = nullptr;            // 8-bit only: dev int32 [N], sum over k of the codes (for asymmetric activations)
   int32_t* mult_t = nullptr;            // dev int32 [K/128][n_pad], n_pad = N rounded up to 128
-  float* base = nullptr;                // dev fp32 [n_pad], a power of two (already divided by 16), negative where the sum needs all bits of mult (see gemm_w4a8.cu)
+  float* base = nullptr;                // dev fp32 [n_pad], a power of two (already divided by 16, see gemm_w4a8.cu)
 };
 
 }  // namespace trdq
