@@ -1,0 +1,75 @@
+"""Host tests of the build: the library needs nvcc alone, the native part of the binding is left out where it cannot be compiled."""
+import importlib.util
+import os
+import shutil
+import sys
+import warnings
+
+import pytest
+
+PACKAGE = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2503_06564_b200")
+
+
+def _tool(path, body):
+    path.write_text("#!/bin/sh\n" + body)
+    path.chmod(0o755)
+    return str(path)
+
+
+WRITES_ITS_OUTPUT = 'while [ $# -gt 0 ]; do if [ "$1" = -o ]; then echo made > "$2"; fi; shift; done\n'
+
+
+@pytest.fixture
+def tree(tmp_path, monkeypatch):
+    """build.py in a package of its own, with one source of each kind and an nvcc that only writes its output."""
+    package = tmp_path / "package"
+    (package / "csrc").mkdir(parents=True)
+    (tmp_path / "include").mkdir()
+    for name in ("csrc/one.cu", "csrc/calls.cpp", "../include/trdq.h"):
+        (package / name).write_text("")
+    shutil.copy(os.path.join(PACKAGE, "build.py"), package)
+    monkeypatch.setenv("NVCC", _tool(tmp_path / "nvcc", WRITES_ITS_OUTPUT))
+    monkeypatch.setenv("CXX", _tool(tmp_path / "cxx", WRITES_ITS_OUTPUT))
+    return package
+
+
+def _load(package):
+    spec = importlib.util.spec_from_file_location("build_under_test", package / "build.py")
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    return module
+
+
+def test_both_are_built(tree):
+    build = _load(tree)
+    with warnings.catch_warnings():
+        warnings.simplefilter("error")
+        assert build.build() == build.LIB
+    assert os.path.exists(build.LIB) and os.path.exists(build.CALLS)
+    os.remove(build.CALLS)
+    build.build()   # the library is up to date, the calls are not
+    assert os.path.exists(build.CALLS)
+
+
+@pytest.mark.parametrize("missing", ["torch", "compiler", "compiler fails"])
+def test_the_library_does_not_need_what_the_native_calls_need(tree, tmp_path, monkeypatch, missing):
+    build = _load(tree)
+    build.build()
+    before = os.path.getmtime(build.LIB)
+    if missing == "torch":
+        monkeypatch.setitem(sys.modules, "torch", None)   # importing it raises ImportError
+    else:
+        monkeypatch.setenv("CXX", str(tmp_path / "nowhere") if missing == "compiler" else _tool(tmp_path / "fails", "exit 1\n"))
+    os.remove(build.LIB)
+    with pytest.warns(UserWarning, match="native calls"):
+        assert build.build(force=True) == build.LIB
+    assert os.path.getmtime(build.LIB) >= before
+    assert not os.path.exists(build.CALLS)   # the one made from other sources is gone
+    with pytest.warns(UserWarning, match="native calls"):
+        assert build.build() == build.LIB    # nothing to do for the library
+
+
+def test_a_failing_nvcc_raises(tree, tmp_path, monkeypatch):
+    monkeypatch.setenv("NVCC", _tool(tmp_path / "fails", "exit 1\n"))
+    with pytest.raises(RuntimeError, match="failed"):
+        _load(tree).build()
