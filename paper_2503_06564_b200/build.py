@@ -1,10 +1,10 @@
-"""Compile the CUDA library (sm_100a) into ``libtrdq.so`` and the native part of its binding into ``_calls.so``, next to this file.
+"""Compile the CUDA library (sm_100a) into ``libtrdq.so`` and the native part of its binding into ``_calls.<torch>.<python>.so``, next to this file.
 
 nvcc cross-compiles without a GPU, so this runs on a CPU-only machine too.  The
 CUDA runtime is linked statically and the driver API is reached through the
 runtime at run time, so the shared object loads on a machine without a driver.
-``libtrdq.so`` needs nvcc alone; ``_calls.so`` needs torch and a C++ compiler, and where
-they are missing it is left out with a warning.
+``libtrdq.so`` needs nvcc alone; the native calls need torch and a C++ compiler, and where
+they are missing the calls are left out with a warning.
 """
 from __future__ import annotations
 
@@ -17,7 +17,6 @@ import warnings
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libtrdq.so")
-CALLS = os.path.join(HERE, "_calls.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 FLAGS = [
@@ -32,20 +31,29 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _calls_stale() -> bool:
+def calls_path() -> str:
+    """The native calls for the torch and the Python at hand.  They have the class layouts of both compiled in, so the file name says which
+    they are: under another torch or Python the file is not found, rather than loaded and wrong."""
+    import sysconfig
+
+    import torch
+    return os.path.join(HERE, f"_calls.torch-{torch.__version__}-abi{int(torch.compiled_with_cxx11_abi())}.{sysconfig.get_config_var('SOABI')}.so")
+
+
+def _calls_stale(path: str) -> bool:
     deps = [os.path.join(CSRC, "calls.cpp"), os.path.join(HERE, "..", "include", "trdq.h"), __file__]
-    return not os.path.exists(CALLS) or any(os.path.getmtime(d) > os.path.getmtime(CALLS) for d in deps)
+    return not os.path.exists(path) or any(os.path.getmtime(d) > os.path.getmtime(path) for d in deps)
 
 
-def _calls_command() -> list:
+def _calls_command(out: str) -> list:
     import sysconfig
 
     import torch
     base = os.path.dirname(torch.__file__)
     include = [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include"),
                sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")]
-    return [os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-            *(f"-I{d}" for d in include), os.path.join(CSRC, "calls.cpp"), "-o", CALLS + ".new",
+    return [os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+            *(f"-I{d}" for d in include), os.path.join(CSRC, "calls.cpp"), "-o", out,
             "-L" + os.path.join(base, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
 
 
@@ -58,14 +66,18 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def _start_calls():
-    """The compiler of the native calls at work, or None if it cannot even be started.  The binding does without them (with a warning), so this never
-    keeps the library from being built."""
+def _start_calls(force: bool):
+    """The compiler of the native calls at work and what it makes, or None if there is nothing to do or it cannot even be started.  The binding
+    does without them (with a warning), so this never keeps the library from being built."""
     try:
-        if os.path.exists(CALLS):
-            os.remove(CALLS)   # whatever happens next: it was made from other sources
-        cmd = _calls_command()
-        return subprocess.Popen(cmd), cmd
+        for old in glob.glob(os.path.join(HERE, "_calls*.so")):
+            if _calls_stale(old):
+                os.remove(old)   # whatever happens next: it was made from other sources, for whichever torch
+        path = calls_path()
+        if not force and os.path.exists(path):
+            return None
+        cmd = _calls_command(path + ".new")
+        return subprocess.Popen(cmd), cmd, path
     except (ImportError, OSError) as e:
         warnings.warn(f"the native calls of the binding are not built: {e}")
         return None
@@ -74,10 +86,11 @@ def _start_calls():
 def _finish_calls(started) -> None:
     if not started:
         return
-    if started[0].wait() == 0:
-        os.replace(CALLS + ".new", CALLS)
+    process, cmd, path = started
+    if process.wait() == 0:
+        os.replace(path + ".new", path)
     else:
-        warnings.warn("the native calls of the binding are not built, compiler failed: " + " ".join(started[1]))
+        warnings.warn("the native calls of the binding are not built, compiler failed: " + " ".join(cmd))
 
 
 def _build_library(verbose: bool) -> None:
@@ -98,7 +111,7 @@ def _build_library(verbose: bool) -> None:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    started = _start_calls() if force or _calls_stale() else None
+    started = _start_calls(force)
     try:
         if force or _stale():
             _build_library(verbose)

@@ -9,6 +9,7 @@ there is no fallback of any kind.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from functools import partial
 from typing import Optional, Sequence, Tuple
@@ -145,16 +146,18 @@ def _calls():
     if _native is None:
         import warnings
 
-        import torch  # noqa: F401  (its libraries have to be loaded first)
         l = lib()
         try:
-            from . import _calls as native
+            from .build import calls_path
+            spec = importlib.util.spec_from_file_location(f"{__package__}._calls", calls_path())   # (torch, whose libraries it needs, is loaded by now)
+            native = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(native)
             native.bind(*(C.cast(f, C.c_void_p).value for f in (
                 l.trdq_rotate_quantize, l.trdq_norm_rotate_quantize, l.trdq_rotate_quantize_asym, l.trdq_linear_act, l.trdq_linear_cfg,
                 l.trdq_linear_asym, l.trdq_linear_splitk_workspace, l.trdq_linear_splitk)))
         except ImportError as e:
-            warnings.warn(f"the native calls ({os.path.join(_HERE, '_calls.so')}) cannot be used, calls take about twice the host time: {e}; build them "
-                          "with `python -m paper_2503_06564_b200.build`")
+            warnings.warn(f"the native calls cannot be used, calls take about twice the host time: {e}; build them with "
+                          "`python -m paper_2503_06564_b200.build`")
             native = _GeneralWay()
         _native = native
     return _native

@@ -45,10 +45,10 @@ def test_both_are_built(tree):
     with warnings.catch_warnings():
         warnings.simplefilter("error")
         assert build.build() == build.LIB
-    assert os.path.exists(build.LIB) and os.path.exists(build.CALLS)
-    os.remove(build.CALLS)
+    assert os.path.exists(build.LIB) and os.path.exists(build.calls_path())
+    os.remove(build.calls_path())
     build.build()   # the library is up to date, the calls are not
-    assert os.path.exists(build.CALLS)
+    assert os.path.exists(build.calls_path())
 
 
 @pytest.mark.parametrize("missing", ["torch", "compiler", "compiler fails"])
@@ -56,15 +56,17 @@ def test_the_library_does_not_need_what_the_native_calls_need(tree, tmp_path, mo
     build = _load(tree)
     build.build()
     before = os.path.getmtime(build.LIB)
+    calls = build.calls_path()
     if missing == "torch":
         monkeypatch.setitem(sys.modules, "torch", None)   # importing it raises ImportError
     else:
         monkeypatch.setenv("CXX", str(tmp_path / "nowhere") if missing == "compiler" else _tool(tmp_path / "fails", "exit 1\n"))
     os.remove(build.LIB)
+    os.utime(calls, (1, 1))
     with pytest.warns(UserWarning, match="native calls"):
         assert build.build(force=True) == build.LIB
     assert os.path.getmtime(build.LIB) >= before
-    assert not os.path.exists(build.CALLS)   # the one made from other sources is gone
+    assert not os.path.exists(calls)   # the one made from other sources is gone
     with pytest.warns(UserWarning, match="native calls"):
         assert build.build() == build.LIB    # nothing to do for the library
 
@@ -73,3 +75,32 @@ def test_a_failing_nvcc_raises(tree, tmp_path, monkeypatch):
     monkeypatch.setenv("NVCC", _tool(tmp_path / "fails", "exit 1\n"))
     with pytest.raises(RuntimeError, match="failed"):
         _load(tree).build()
+
+
+def test_another_torch_has_native_calls_of_its_own(tree, monkeypatch):
+    import torch
+    build = _load(tree)
+    build.build()
+    first = build.calls_path()
+    monkeypatch.setattr(torch, "__version__", "0.0.0+other")
+    assert build.calls_path() != first and not os.path.exists(build.calls_path())
+    build.build()
+    assert os.path.exists(build.calls_path()) and os.path.exists(first)
+    os.utime(first, (1, 1))   # older than the sources: of no use to either
+    build.build()
+    assert os.path.exists(build.calls_path()) and not os.path.exists(first)
+
+
+def test_native_calls_made_for_another_torch_are_not_loaded(monkeypatch):
+    import torch
+    from paper_2503_06564_b200 import trdq
+    monkeypatch.setattr(trdq, "_native", None)
+    monkeypatch.setattr(torch, "__version__", "0.0.0+other")
+    with pytest.warns(UserWarning, match="native calls"):
+        assert trdq._calls().rotate_quantize(None, 128, 0, None, None, None) is None
+    assert type(trdq._native) is trdq._GeneralWay
+    monkeypatch.undo()
+    monkeypatch.setattr(trdq, "_native", None)
+    with warnings.catch_warnings():
+        warnings.simplefilter("error")
+        assert type(trdq._calls()) is not trdq._GeneralWay
