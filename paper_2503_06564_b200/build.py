@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import glob
 import os
+import shutil
 import subprocess
 import sys
 import warnings
@@ -50,8 +51,9 @@ def _calls_command(out: str) -> list:
 
     import torch
     base = os.path.dirname(torch.__file__)
+    toolkit = os.path.dirname(os.path.dirname(shutil.which(NVCC) or NVCC))   # (NVCC may be a name on PATH)
     include = [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include"),
-               sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")]
+               sysconfig.get_paths()["include"], os.path.join(toolkit, "include")]
     return [os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
             *(f"-I{d}" for d in include), os.path.join(CSRC, "calls.cpp"), "-o", out,
             "-L" + os.path.join(base, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]

@@ -77,6 +77,15 @@ def test_a_failing_nvcc_raises(tree, tmp_path, monkeypatch):
         _load(tree).build()
 
 
+def test_headers_of_an_nvcc_on_the_path(tree, tmp_path, monkeypatch):
+    bin_ = tmp_path / "toolkit" / "bin"
+    bin_.mkdir(parents=True)
+    _tool(bin_ / "nvcc", WRITES_ITS_OUTPUT)
+    monkeypatch.setenv("PATH", str(bin_), prepend=os.pathsep)
+    monkeypatch.setenv("NVCC", "nvcc")
+    assert f"-I{tmp_path / 'toolkit' / 'include'}" in _load(tree)._calls_command("out.so")
+
+
 def test_another_torch_has_native_calls_of_its_own(tree, monkeypatch):
     import torch
     build = _load(tree)
