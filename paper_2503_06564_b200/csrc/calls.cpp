@@ -89,51 +89,82 @@ bool output(PyObject* o, int32_t M, int64_t N, int64_t* ld) {
   return true;
 }
 
-// A new reference to `given`, or to a new tensor on the device of `like`.
-PyObject* given_or_empty(PyObject* given, PyObject* like, at::IntArrayRef sizes, at::ScalarType type) {
-  if (given != Py_None) {
-    Py_INCREF(given);
-    return given;
-  }
-  return THPVariable_Wrap(at::empty(sizes, THPVariable_Unpack(like).options().dtype(type)));
-}
-
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// Runs a library call without the GIL (as ctypes does) and returns the outputs in a tuple, or alone, or the status.
-struct Outputs {
-  PyObject* o[4] = {nullptr, nullptr, nullptr, nullptr};
-  int n = 0;
-  ~Outputs() {
-    for (int i = 0; i < n; ++i) Py_DECREF(o[i]);
-  }
-  PyObject* add(PyObject* p) {
-    if (!p) throw python_error();
-    return o[n++] = p;
-  }
+struct WithoutGil {
+  PyThreadState* const state = PyEval_SaveThread();
+  ~WithoutGil() { PyEval_RestoreThread(state); }
+};
+
+// The outputs of a call: given by the caller or new tensors on the device of `like`.
+class Outputs {
+ public:
+  explicit Outputs(PyObject* like) : options_(THPVariable_Unpack(like).options()) {}
+  void add(PyObject* given, int32_t rows, int64_t columns, at::ScalarType type) { put(given, rows, columns, 2, type); }
+  void add(PyObject* given, int32_t rows, at::ScalarType type) { put(given, rows, 0, 1, type); }
+
+  // Makes the new ones, runs the library call (it gets the pointers) and returns the outputs in a tuple, a list or alone, or the status.  All
+  // of it without the GIL: an allocation may wait for the device, and for other threads' work on it.
   template <typename Call>
   PyObject* run(Call&& call, bool list = false) {
     trdq_status st;
-    Py_BEGIN_ALLOW_THREADS
-    st = call();
-    Py_END_ALLOW_THREADS
-    if (st != TRDQ_OK) return PyLong_FromLong(st);
-    if (n == 1) {
-      Py_INCREF(o[0]);
-      return o[0];
+    {
+      WithoutGil released;
+      void* pointers[kMost];
+      for (int i = 0; i < n_; ++i) {
+        Item& o = item_[i];
+        if (!o.given) o.made = at::empty(at::IntArrayRef(o.sizes, o.dims), options_.dtype(o.type));
+        pointers[i] = o.given ? o.pointer : o.made.data_ptr();
+      }
+      st = call(pointers);
     }
-    PyObject* const r = list ? PyList_New(n) : PyTuple_New(n);
+    if (st != TRDQ_OK) return PyLong_FromLong(st);
+    if (n_ == 1) return wrap(item_[0]);
+    PyObject* const r = list ? PyList_New(n_) : PyTuple_New(n_);
     if (!r) return nullptr;
-    for (int i = 0; i < n; ++i) {
-      Py_INCREF(o[i]);
+    for (int i = 0; i < n_; ++i) {
+      PyObject* const o = wrap(item_[i]);
+      if (!o) {
+        Py_DECREF(r);
+        return nullptr;
+      }
       if (list) {
-        PyList_SET_ITEM(r, i, o[i]);
+        PyList_SET_ITEM(r, i, o);
       } else {
-        PyTuple_SET_ITEM(r, i, o[i]);
+        PyTuple_SET_ITEM(r, i, o);
       }
     }
     return r;
   }
+
+ private:
+  static constexpr int kMost = 3;
+  struct Item {
+    PyObject* given;  // borrowed from the caller's arguments
+    void* pointer;    // of the given one
+    int64_t sizes[2];
+    int dims;
+    at::ScalarType type;
+    at::Tensor made;
+  };
+  void put(PyObject* given, int64_t rows, int64_t columns, int dims, at::ScalarType type) {
+    Item& o = item_[n_++];
+    o.given = given == Py_None ? nullptr : given;
+    o.pointer = pointer(given);
+    o.sizes[0] = rows;
+    o.sizes[1] = columns;
+    o.dims = dims;
+    o.type = type;
+  }
+  static PyObject* wrap(Item& o) {
+    if (!o.given) return THPVariable_Wrap(std::move(o.made));
+    Py_INCREF(o.given);
+    return o.given;
+  }
+
+  at::TensorOptions options_;
+  Item item_[kMost];
+  int n_ = 0;
 };
 
 #define GENERAL_WAY_UNLESS(condition) \
@@ -147,12 +178,12 @@ PyObject* rotate_quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
   int32_t t, M;
   GENERAL_WAY_UNLESS(n == 6 && handle(a[0], &rot) && number(a[1], &K) && number(a[2], &t) && activations(a[3], K, &M, &ldx) &&
                      plain_or_none(a[4]) && plain_or_none(a[5]) && no_modes());
-  Outputs out;
-  void* const codes = pointer(out.add(given_or_empty(a[4], a[3], {M, K}, at::kChar)));
-  void* const scales = pointer(out.add(given_or_empty(a[5], a[3], {M}, at::kFloat)));
+  Outputs out(a[3]);
+  out.add(a[4], M, K, at::kChar);
+  out.add(a[5], M, at::kFloat);
   void* const x = pointer(a[3]);
   void* const s = stream();
-  return out.run([&] { return entry.rotate_quantize(static_cast<trdq_rotation*>(rot), t, x, ldx, M, static_cast<int8_t*>(codes), static_cast<float*>(scales), s); });
+  return out.run([&](void** o) { return entry.rotate_quantize(static_cast<trdq_rotation*>(rot), t, x, ldx, M, static_cast<int8_t*>(o[0]), static_cast<float*>(o[1]), s); });
   END_HANDLE_TH_ERRORS
 }
 
@@ -170,14 +201,14 @@ PyObject* norm_rotate_quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
     GENERAL_WAY_UNLESS(number(a[6], &per_sample));
   }
   const float eps = static_cast<float>(PyFloat_AS_DOUBLE(a[7]));
-  Outputs out;
-  void* const codes = pointer(out.add(given_or_empty(a[8], a[3], {M, K}, at::kChar)));
-  void* const scales = pointer(out.add(given_or_empty(a[9], a[3], {M}, at::kFloat)));
+  Outputs out(a[3]);
+  out.add(a[8], M, K, at::kChar);
+  out.add(a[9], M, at::kFloat);
   void *const x = pointer(a[3]), *const shift = pointer(a[4]), *const scale = pointer(a[5]);
   void* const s = stream();
-  return out.run([&] {
-    return entry.norm_rotate_quantize(static_cast<trdq_rotation*>(rot), t, x, ldx, M, shift, scale, per_sample, eps, static_cast<int8_t*>(codes),
-                                      static_cast<float*>(scales), s);
+  return out.run([&](void** o) {
+    return entry.norm_rotate_quantize(static_cast<trdq_rotation*>(rot), t, x, ldx, M, shift, scale, per_sample, eps, static_cast<int8_t*>(o[0]),
+                                      static_cast<float*>(o[1]), s);
   });
   END_HANDLE_TH_ERRORS
 }
@@ -189,15 +220,15 @@ PyObject* rotate_quantize_asym(PyObject*, PyObject* const* a, Py_ssize_t n) {
   int64_t K, ldx;
   int32_t t, M;
   GENERAL_WAY_UNLESS(n == 4 && handle(a[0], &rot) && number(a[1], &K) && number(a[2], &t) && activations(a[3], K, &M, &ldx) && no_modes());
-  Outputs out;
-  void* const codes = pointer(out.add(given_or_empty(Py_None, a[3], {M, K}, at::kByte)));
-  void* const scales = pointer(out.add(given_or_empty(Py_None, a[3], {M}, at::kFloat)));
-  void* const zero = pointer(out.add(given_or_empty(Py_None, a[3], {M}, at::kInt)));
+  Outputs out(a[3]);
+  out.add(Py_None, M, K, at::kByte);
+  out.add(Py_None, M, at::kFloat);
+  out.add(Py_None, M, at::kInt);
   void* const x = pointer(a[3]);
   void* const s = stream();
-  return out.run([&] {
-    return entry.rotate_quantize_asym(static_cast<trdq_rotation*>(rot), t, x, ldx, M, static_cast<uint8_t*>(codes), static_cast<float*>(scales),
-                                      static_cast<int32_t*>(zero), s);
+  return out.run([&](void** o) {
+    return entry.rotate_quantize_asym(static_cast<trdq_rotation*>(rot), t, x, ldx, M, static_cast<uint8_t*>(o[0]), static_cast<float*>(o[1]),
+                                      static_cast<int32_t*>(o[2]), s);
   });
   END_HANDLE_TH_ERRORS
 }
@@ -210,12 +241,12 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
   int32_t t, M, act;
   GENERAL_WAY_UNLESS(n == 8 && handle(a[0], &w) && number(a[1], &N) && number(a[2], &t) && rows(a[3], &M) && plain(a[4]) && plain_or_none(a[5]) &&
                      output(a[6], M, N, &ldy) && number(a[7], &act) && no_modes());
-  Outputs out;
-  void* const y = pointer(out.add(given_or_empty(a[6], a[3], {M, N}, at::kBFloat16)));
+  Outputs out(a[3]);
+  out.add(a[6], M, N, at::kBFloat16);
   void *const codes = pointer(a[3]), *const scales = pointer(a[4]), *const bias = pointer(a[5]);
   void* const s = stream();
-  return out.run([&] {
-    return entry.linear_act(static_cast<trdq_weights*>(w), t, static_cast<int8_t*>(codes), static_cast<float*>(scales), M, bias, y, ldy, act, s);
+  return out.run([&](void** o) {
+    return entry.linear_act(static_cast<trdq_weights*>(w), t, static_cast<int8_t*>(codes), static_cast<float*>(scales), M, bias, o[0], ldy, act, s);
   });
   END_HANDLE_TH_ERRORS
 }
@@ -228,13 +259,13 @@ PyObject* linear_asym(PyObject*, PyObject* const* a, Py_ssize_t n) {
   int32_t t, M;
   GENERAL_WAY_UNLESS(n == 8 && handle(a[0], &w) && number(a[1], &N) && number(a[2], &t) && rows(a[3], &M) && plain(a[4]) && plain(a[5]) &&
                      plain_or_none(a[6]) && output(a[7], M, N, &ldy) && no_modes());
-  Outputs out;
-  void* const y = pointer(out.add(given_or_empty(a[7], a[3], {M, N}, at::kBFloat16)));
+  Outputs out(a[3]);
+  out.add(a[7], M, N, at::kBFloat16);
   void *const codes = pointer(a[3]), *const scales = pointer(a[4]), *const zero = pointer(a[5]), *const bias = pointer(a[6]);
   void* const s = stream();
-  return out.run([&] {
+  return out.run([&](void** o) {
     return entry.linear_asym(static_cast<trdq_weights*>(w), t, static_cast<uint8_t*>(codes), static_cast<float*>(scales), static_cast<int32_t*>(zero), M,
-                             bias, y, ldy, s);
+                             bias, o[0], ldy, s);
   });
   END_HANDLE_TH_ERRORS
 }
@@ -249,20 +280,18 @@ PyObject* linear_splitk(PyObject*, PyObject* const* a, Py_ssize_t n) {
   GENERAL_WAY_UNLESS(n == 8 && handle(a[0], &w) && number(a[1], &N) && number(a[2], &t) && rows(a[3], &M) && plain(a[4]) && plain_or_none(a[5]) &&
                      output(a[6], M, N, &ldy) && plain_or_none(a[7]) && no_modes() &&
                      entry.splitk_workspace(static_cast<trdq_weights*>(w), M, &splits, &bytes) == TRDQ_OK);
-  Outputs out;
-  void* const y = pointer(out.add(given_or_empty(a[6], a[3], {M, N}, at::kBFloat16)));
-  at::Tensor workspace;
-  if (a[7] != Py_None) {
-    workspace = THPVariable_Unpack(a[7]);
-  } else if (bytes) {
-    workspace = at::empty({static_cast<int64_t>(bytes)}, THPVariable_Unpack(a[3]).options().dtype(at::kByte));
-  }
-  void* const ws = workspace.defined() ? workspace.data_ptr() : nullptr;
-  const uint64_t ws_bytes = workspace.defined() ? static_cast<uint64_t>(workspace.numel() * workspace.element_size()) : 0;
-  void *const codes = pointer(a[3]), *const scales = pointer(a[4]), *const bias = pointer(a[5]);
+  Outputs out(a[3]);
+  out.add(a[6], M, N, at::kBFloat16);
+  void *const codes = pointer(a[3]), *const scales = pointer(a[4]), *const bias = pointer(a[5]), *const given = pointer(a[7]);
+  const at::TensorOptions options = THPVariable_Unpack(a[3]).options().dtype(at::kByte);
+  const bool make = a[7] == Py_None && bytes;
+  if (a[7] != Py_None) bytes = static_cast<uint64_t>(THPVariable_Unpack(a[7]).numel() * THPVariable_Unpack(a[7]).element_size());
   void* const s = stream();
-  return out.run([&] {
-    return entry.linear_splitk(static_cast<trdq_weights*>(w), t, static_cast<int8_t*>(codes), static_cast<float*>(scales), M, bias, y, ldy, ws, ws_bytes, s);
+  return out.run([&](void** o) {
+    at::Tensor made;
+    if (make) made = at::empty({static_cast<int64_t>(bytes)}, options);
+    return entry.linear_splitk(static_cast<trdq_weights*>(w), t, static_cast<int8_t*>(codes), static_cast<float*>(scales), M, bias, o[0], ldy,
+                               make ? made.data_ptr() : given, bytes, s);
   });
   END_HANDLE_TH_ERRORS
 }
@@ -287,22 +316,21 @@ PyObject* linear_cfg(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return true;
   };
   GENERAL_WAY_UNLESS(two(a[3], codes) && two(a[4], scales) && rows(codes[0], &M[0]) && rows(codes[1], &M[1]) && plain(scales[0]) && plain(scales[1]));
-  Outputs out;
-  const void* c[2];
+  Outputs out(codes[0]);
+  at::Tensor held[4];  // the caller's lists may change while the GIL is released
+  const int8_t* c[2];
   const float* sx[2];
-  void* y[2];
-  int64_t ldy[2];
+  const int64_t ldy[2] = {N, N};
   for (int i = 0; i < 2; ++i) {
-    const at::Tensor& cond = THPVariable_Unpack(codes[i]);
-    c[i] = cond.data_ptr();
-    sx[i] = static_cast<const float*>(pointer(scales[i]));
-    y[i] = pointer(out.add(given_or_empty(Py_None, codes[0], {M[i], N}, at::kBFloat16)));
-    ldy[i] = N;
+    held[2 * i] = THPVariable_Unpack(codes[i]);
+    held[2 * i + 1] = THPVariable_Unpack(scales[i]);
+    c[i] = static_cast<const int8_t*>(held[2 * i].data_ptr());
+    sx[i] = static_cast<const float*>(held[2 * i + 1].data_ptr());
+    out.add(Py_None, M[i], N, at::kBFloat16);
   }
   void* const bias = pointer(a[5]);
   void* const s = stream();
-  const int8_t* const c8[2] = {static_cast<const int8_t*>(c[0]), static_cast<const int8_t*>(c[1])};
-  return out.run([&] { return entry.linear_cfg(static_cast<trdq_weights*>(w), t, c8, sx, M, bias, y, ldy, s); }, true);
+  return out.run([&](void** y) { return entry.linear_cfg(static_cast<trdq_weights*>(w), t, c, sx, M, bias, y, ldy, s); }, true);
   END_HANDLE_TH_ERRORS
 }
 
