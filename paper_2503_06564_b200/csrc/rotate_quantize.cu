@@ -512,7 +512,8 @@ rotate_quantize_rows_asym_kernel(const __nv_bfloat16* __restrict__ x, int64_t ld
 // What bounds the few rows of a long reduction is the chain of one row: load, transform, row maximum, store.  In the eight-lane kernel it is longer
 // (scalar butterfly, three shuffle stages, no overlap with the kernel before), and above 128 blocks a lane group has two blocks.
 // Microseconds, eight lanes / this: K = 10368 3.9 / 2.6 for one row, 4.2 / 2.8 for 128; K = 16384 5.1 / 3.4 and 5.3 / 3.5; K = 16512 6.8 / 3.6, 7.1 / 3.8, and 25.1 / 12.4
-// for 512 rows; K = 20480 7.5 / 3.9, 7.6 / 4.1, 27.1 / 14.0 and 139 / 84 for 4096.  (To 128 blocks the team kernel takes over from a row per SM on.)
+// for 512 rows; K = 20480 7.5 / 3.9, 7.6 / 4.1, 27.1 / 14.0 and 139 / 84 for 4096.  To 128 blocks the team kernel takes over from a row per SM on for
+// activations; 8-bit weights come here whatever their rows (16 to 4096 of them take 0.72 - 0.94 of the eight lanes' time to 128 blocks, 0.52 - 0.69 above).
 // 94 registers; a form of 64 for two CTAs per SM took 5.4 at M = 128, K = 16384.  Beyond 160 blocks the eight-lane kernel stays.  The codes are
 // formed as there, not by the magic addition, so that rows with infinities or NaN keep theirs.
 constexpr int kWideBlocks = 160;
@@ -640,12 +641,12 @@ template <int MODE>
 cudaError_t dispatch(const void* x, int64_t ldx, int32_t M, int32_t K, const float* vec, void* codes, float* scales,
                      cudaStream_t stream) {
   const int nb = K / TRDQ_BLOCK;
-  if (nb <= 128) {
+  if (MODE == 1 && nb <= 128) {  // (int8 rows of up to 160 blocks have kernels of their own)
     // about 32 lane groups (256 threads) per CTA, whole rows only, at most 32 rows per tile
     int rows = 32 / nb;
     if (rows < 1) rows = 1;
     if (rows > 32) rows = 32;
-    return launch<MODE, 1>(x, ldx, M, K, vec, codes, scales, rows, rows * nb, stream);
+    return launch<1, 1>(x, ldx, M, K, vec, codes, scales, rows, rows * nb, stream);
   }
   const int p = (nb + 127) / 128;  // nb <= 1024 -> p <= 8
   if (p <= 2) return launch<MODE, 2>(x, ldx, M, K, vec, codes, scales, 1, (nb + 1) / 2, stream);
@@ -733,6 +734,7 @@ cudaError_t launch_rotate2_quantize(const void* x_bf16, int64_t ldx, int32_t M, 
 }
 
 // Name of the kernel trdq_rotate_quantize runs for M rows of K channels (single rotation, symmetric codes).
+// "rotate_quantize_kernel" is wide::rotate_quantize_kernel up to kWideBlocks blocks and the eight-lane kernel beyond.
 void describe_rotate_quantize_kernel(int32_t M, int32_t K, char* name, size_t cap) {
   if (rotate_quantize_prefers_team(M, K))
     snprintf(name, cap, "rotate_quantize_team_kernel");
@@ -750,11 +752,18 @@ cudaError_t launch_rotate_quantize(const void* x_bf16, int64_t ldx, int32_t M, i
 cudaError_t launch_rotate_quantize_groups(const void* x_bf16, int64_t ldx, int32_t M, int32_t K, const float* vec, int groups, int mode,
                                           void* codes, float* scales, cudaStream_t stream) {
   if (M == 0) return cudaSuccess;
-  // fast path: the whole tile of a CTA fits 320 threads and the vector fits the default shared memory
-  if (mode == 0 && K / TRDQ_BLOCK <= 80 && static_cast<size_t>(K) * sizeof(float) <= 40 * 1024 && groups <= 65535)
-    return launch_rows_fast(x_bf16, ldx, M, K, vec, groups, codes, scales, stream);
   const int64_t code_bytes = mode == 0 ? static_cast<int64_t>(M) * K : static_cast<int64_t>(M) * K / 2;
   const int64_t scale_count = mode == 0 ? M : static_cast<int64_t>(M) * (K / TRDQ_BLOCK);
+  // fast path: the whole tile of a CTA fits 320 threads and the vector fits the default shared memory; as many groups to a launch as a grid dimension holds
+  if (mode == 0 && K / TRDQ_BLOCK <= 80 && static_cast<size_t>(K) * sizeof(float) <= 40 * 1024) {
+    constexpr int kMaxGridY = 65535;
+    for (int g = 0; g < groups; g += kMaxGridY) {
+      const cudaError_t e = launch_rows_fast(x_bf16, ldx, M, K, vec + static_cast<int64_t>(g) * K, std::min(groups - g, kMaxGridY),
+                                             static_cast<uint8_t*>(codes) + g * code_bytes, scales + g * scale_count, stream);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
   for (int g = 0; g < groups; ++g) {
     const float* v = vec + static_cast<int64_t>(g) * K;
     uint8_t* c = static_cast<uint8_t*>(codes) + g * code_bytes;
