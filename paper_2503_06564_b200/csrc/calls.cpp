@@ -4,8 +4,9 @@
 // (two calls, 7 us on the GPU) 19.3 us, now 10.3; three calls for two ragged row segments 37.4, now 22.6.
 //
 // Every function returns None for arguments it does not handle: tensor subclasses, tensors of other devices or layouts, wrapped tensors
-// (functorch, functional, fake), numbers that are not Python ints, an active function or dispatch mode.  The caller then goes its general
-// way, which also is where wrong arguments are reported.  A status other than TRDQ_OK is returned as an int.
+// (functorch, functional, fake), numbers that are not Python ints, an active function or dispatch mode (torch.set_default_device is one).  The caller
+// then goes its general way, which costs what it did and 0.15 us for the question, and is where wrong arguments are reported.  A status other than
+// TRDQ_OK is returned as an int.
 #include <Python.h>
 
 #include <ATen/ATen.h>

@@ -375,7 +375,9 @@ bool narrow_tiles(int64_t tiles_m, int N, int sms, int splits = 1) {
 
 // Whether the CTA-pair kernel (two SMs per 256-row tile, a third less operand traffic per SM) runs M rows against [N, K] weights: from
 // 2048 rows, once the output holds enough tiles of 256 x 256 values.  Below that its fewer, larger tiles leave SMs idle; the
-// longer the reduction, the earlier the operand traffic outweighs that, and from K = 7168 on it always does.  Both kernels were
+// longer the reduction, the earlier the operand traffic outweighs that, and from K = 7168 on it always does against tiles of 128 columns and more.
+// (Those of narrow_tiles came later and the line has not been drawn against them: where they would fit they are faster there up to 4096 rows, microseconds,
+// pair / 64 columns: 512 x 2048 at K = 7168 12.8 / 11.8, at 12288 19.6 / 18.0, at 16384 24.9 / 22.9; 128 x 8192 level to 5 %.)  Both kernels were
 // timed at nineteen K from 128 to 12288, eleven N from 128 to 4608 and M from 2048 to 32768 (1065 points, plain, GELU and asymmetric
 // epilogue).  Microseconds, pair / single CTA, at N x M: K = 128: 8.2 / 7.8 at 2304 x 4096 (144 tiles), 10.1 / 11.1 at 4608 x 2560 (180);
 // K = 1152: 10.1 / 9.4 at 3456 x 2048 (108), 10.8 / 11.2 at 3072 x 2560 (120);  K = 2304: 11.2 / 10.3 at 2304 x 2048 (72), 12.5 / 13.2 at

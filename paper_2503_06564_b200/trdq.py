@@ -2,9 +2,9 @@
 
 Every function here has the name of the C entry point it calls (``include/trdq.h``)
 and does nothing but turn torch tensors into pointers, sizes and the current
-stream, in native code (``_calls``) for the hot calls on plain CUDA tensors, through ctypes otherwise.  All arithmetic runs in the CUDA kernels of the library; if the shared
-object is missing the import of this module's library handle fails loudly, and
-there is no fallback of any kind.
+stream, in native code (``_calls``) for the hot calls on plain CUDA tensors, through ctypes otherwise and where the native
+calls have not been built (with a warning).  All arithmetic runs in the CUDA kernels of the library; if ``libtrdq.so``
+is missing the import of this module's library handle fails loudly, and there is no fallback for it of any kind.
 """
 from __future__ import annotations
 

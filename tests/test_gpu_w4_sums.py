@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("blocks", [1, 8, 9, 10])
-@pytest.mark.parametrize("span", [1.0, 2.0 ** -2, 2.0 ** -9])   # smallest scale of a channel over its largest: one binade, three, too many
+@pytest.mark.parametrize("span", [1.0, 2.0 ** -2, 2.0 ** -9])   # smallest scale of a channel over its largest: one binade, three, ten
 def test_sums_at_the_ends_of_their_range(blocks, span):
     import torch
     from paper_2503_06564_b200 import trdq
